@@ -103,11 +103,18 @@ void restrict_vec_multi(const TransferOp& T, int nrhs, float* out_c, size_t cstr
                         bool even_only, cudaStream_t s);
 void prolong_vec_multi(const TransferOp& T, int nrhs, float* v, size_t vstride, const float* in_c, size_t cstride,
                        bool even_only, cudaStream_t s);
-// p = column (chir, k) of P as a whole-lattice vector of the fine level
-void extract_column(const TransferOp& T, float* p, int chir, int k, cudaStream_t s);
-// Galerkin accumulation of one column: W[0..7] directional hops of u = M^{-1} p,
-// W[8] the identity-slot vector; writes column `col` of Y (faces) and X.
-void restrict9(const TransferOp& T, CoarseOp& C, const float* const W[9], int col, cudaStream_t s);
+// columns column0 .. column0 + ncol - 1 of P (column = chirality * Nv + k) as
+// whole-lattice vectors of the fine level, vstride floats apart
+void extract_columns(const TransferOp& T, float* p, size_t vstride, int column0, int ncol, cudaStream_t s);
+// Sh + Sl (float pairs) = slot + the hops W[d] that stay inside their block, for
+// ncol columns of a coarse level (the fine level sums them in galerkin_hops)
+void interior_sum(const TransferOp& T, const float* const W[8], const float* slot, float* Sh, float* Sl,
+                  size_t vstride, int ncol, cudaStream_t s);
+// Galerkin projection of ncol (even) columns: P^dag of the interior sums into X
+// and of the face hops W[d] (read on the block faces only) into Y_d, columns
+// col0 .. col0 + ncol - 1.
+void galerkin_project(const TransferOp& T, CoarseOp& C, const float* const W[8], const float* Sh, const float* Sl,
+                      size_t vstride, int col0, int ncol, cudaStream_t s);
 
 // ---- coarse stencil kernels
 // out[s] = epi(sum_{d in mask} Y_d(s) in[nbr_d(s)]) for storage sites

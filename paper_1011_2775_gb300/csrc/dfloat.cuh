@@ -24,6 +24,13 @@ __device__ __forceinline__ df df_add(df a, df b) {
   const float e = (a.h - (s - bb)) + (b.h - bb) + (a.l + b.l);
   return df_norm(s, e);
 }
+// h + l <- h + l + x, the rounding error of the sum kept in l (not renormalised)
+__device__ __forceinline__ void df_acc(float& h, float& l, float x) {
+  const float s = __fadd_rn(h, x);
+  const float bb = __fsub_rn(s, h);
+  l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+  h = s;
+}
 __device__ __forceinline__ df df_neg(df a) { return df{-a.h, -a.l}; }
 __device__ __forceinline__ df df_mul(df a, df b) {
   const float p = a.h * b.h;

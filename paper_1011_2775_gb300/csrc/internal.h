@@ -142,10 +142,14 @@ std::vector<int> dslash_mrhs_configs(bool fp32);
 int dslash_mrhs_default(bool fp32);
 template <typename T>
 void clover_apply_mrhs(const Geom& g, int nrhs, size_t stride, T* out, const T* in, const T* clov, cudaStream_t s);
-// the 8 directional terms H_d in (without summation), written to out[d]
-// (whole-lattice FP32 vectors, [even half][odd half] each)
-void hop_directions(const Geom& g, float* const out[8], const float* in_even, const float* in_odd,
-                    const float* gauge, cudaStream_t s);
+// The directional terms W_d = H_d u of ncol whole-lattice FP32 columns ([even
+// half][odd half], vstride floats apart) for blocks of `block` sites on a
+// coarse lattice of `cdims`: terms that cross a block face go to W[d] (other
+// sites of W[d] are left alone), the rest are added to `slot` into the float
+// pairs Sh + Sl.
+void galerkin_hops(const Geom& g, const int block[4], const int cdims[4], const float* u, const float* slot,
+                   float* const W[8], float* Sh, float* Sl, size_t vstride, int ncol, const float* gauge,
+                   cudaStream_t s);
 // Philox4x32-10 Gaussian start vector (see the generator's definition in coarse.cu)
 void philox_fine_vector(const Geom& g, uint64_t seed, int level, int k, float* even, float* odd, cudaStream_t s);
 

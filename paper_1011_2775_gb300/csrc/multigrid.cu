@@ -16,6 +16,7 @@
 // D_p = [[1, X], [Y, 1]] the solution of D_p u = (r_e, 0) has
 // u_e = D_r^{-1} r_e, which is why a coarse space of D_p serves D_r.
 // The whole preconditioner runs in FP32.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 
@@ -446,37 +447,44 @@ void build_coarse_links(Ctx* c, Hierarchy& H, int l) {
     MG_CUDA(cudaMemcpyAsync(C.Yscale.get(), ones.data(), sizeof(float) * ones.size(), cudaMemcpyHostToDevice, s));
     c->sync();
   }
-  DBuf pb(sizeof(float) * 2 * n), ub(sizeof(float) * 2 * n), mb(sizeof(float) * 2 * n);
-  std::vector<DBuf> Wb(8);
-  for (auto& b : Wb) b.alloc(sizeof(float) * 2 * n);
+  // columns are taken in batches: as many (an even number) as keep the
+  // batch's vectors within about the L2 capacity, so small lattices fill the
+  // GPU with several columns and large ones hold two
+  const size_t vs = 2 * n;   // floats per column vector
+  const size_t per = sizeof(float) * vs * 12;
+  const int ncol = (int)std::min<size_t>(nc, std::max<size_t>(2, ((size_t)128 << 20) / per / 2 * 2));
+  DBuf pb(sizeof(float) * vs * ncol), ub(sizeof(float) * vs * ncol), sb(sizeof(float) * vs * ncol * 2);
+  DBuf Wb(sizeof(float) * vs * ncol * 8);
   float* pv = pb.as<float>();
-  float* u = ub.as<float>();
-  float* mp = mb.as<float>();
+  float* mp = ub.as<float>();   // M^{-1} p (M p when the operator is the projection of D)
+  float* Sh = sb.as<float>();
+  float* Sl = Sh + vs * ncol;
   float* Wp[8];
-  for (int d = 0; d < 8; d++) Wp[d] = Wb[d].as<float>();
+  for (int d = 0; d < 8; d++) Wp[d] = Wb.as<float>() + (size_t)d * vs * ncol;
   const bool galerkin_dp = p.coarse_op != MG_COARSE_D;
-  for (int ch = 0; ch < 2; ch++)
-    for (int k = 0; k < nv; k++) {
-      extract_column(T, pv, ch, k, s);
-      const float* slot8 = pv;
-      const float* hop_in = pv;
-      if (galerkin_dp) {
-        Minv_level(c, H, l, u, pv, true);
-        hop_in = u;
-      } else {
-        Minv_level(c, H, l, mp, pv, false);
-        slot8 = mp;
-      }
-      if (l == 0) {
-        hop_directions(c->g, Wp, hop_in, hop_in + 24 * c->Vh, c->gauge<float>(), s);
-      } else {
-        const LevelGeom& G = H.geo[l];
+  for (int col = 0; col < nc; col += ncol) {
+    const int nq = std::min(ncol, nc - col);
+    extract_columns(T, pv, vs, col, nq, s);
+    // D_p p = p + H M^{-1} p, or D p = M p + H p
+    const float* slot = galerkin_dp ? pv : mp;
+    const float* hop_in = galerkin_dp ? mp : pv;
+    if (l == 0) {
+      const size_t half = 24 * c->Vh;
+      for (int par = 0; par < 2; par++)
+        clover_apply_mrhs<float>(c->g, nq, vs, mp + par * half, pv + par * half,
+                                 galerkin_dp ? c->Ainv<float>(par) : c->A<float>(par), s);
+      galerkin_hops(c->g, T.block, T.cdims, hop_in, slot, Wp, Sh, Sl, vs, nq, c->gauge<float>(), s);
+    } else {
+      const LevelGeom& G = H.geo[l];
+      for (int q = 0; q < nq; q++) {
+        Minv_level(c, H, l, mp + q * vs, pv + q * vs, galerkin_dp);
         for (int d = 0; d < 8; d++)
-          coarse_hop(G, H.cop[l], EPI_H, false, 0, G.nsites, Wp[d], hop_in, nullptr, 0.f, 1 << d, s);
+          coarse_hop(G, H.cop[l], EPI_H, false, 0, G.nsites, Wp[d] + q * vs, hop_in + q * vs, nullptr, 0.f, 1 << d, s);
       }
-      const float* W9[9] = {Wp[0], Wp[1], Wp[2], Wp[3], Wp[4], Wp[5], Wp[6], Wp[7], slot8};
-      restrict9(T, C, W9, ch * nv + k, s);
+      interior_sum(T, Wp, slot, Sh, Sl, vs, nq, s);
     }
+    galerkin_project(T, C, Wp, Sh, Sl, vs, col, nq, s);
+  }
   coarse_invert(Gc, C, c->ws.flags.as<int>(), s);
   if (c->read_flag(FLAG_SINGULAR, true)) raise(MG_ERR_SINGULAR_CLOVER, "singular coarse diagonal block");
   quantize_links(Gc, C, T.store, s);               // 16-bit storage of Y (FP32: no-op)

@@ -21,6 +21,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "dfloat.cuh"
 #include "internal.h"
 #include "philox.cuh"
 #include "wilson_dev.cuh"
@@ -863,46 +864,87 @@ template void clover_apply_mrhs<float>(const Geom&, int, size_t, float*, const f
 template void clover_apply_mrhs<double>(const Geom&, int, size_t, double*, const double*, const double*, cudaStream_t);
 
 // --------------------------------------------------------------------------- directional terms
-struct DirOut {
-  float* p[8];
+// Directional hops of the Galerkin construction, sorted while they are in
+// registers: a term that crosses a block face is stored for its own
+// projection, all others are added (with the identity-slot vector) into a
+// float pair, so a column writes 2 vectors and the faces instead of 8 vectors.
+struct GalerkinOut {
+  float* W[8];
+  float* Sh;
+  float* Sl;
+  int b[4];
+  int split[4];   // the coarse lattice has more than one site in this direction
 };
 
 template <int MU, bool FWD>
-__device__ __forceinline__ void one_dir(const Geom& g, const float* in, const float* gauge, int par, int i,
-                                        const int c[4], float* out_full) {
+__device__ __forceinline__ void one_dir(const Geom& g, const GalerkinOut& o, const float* in, const float* gauge,
+                                        int par, int i, const int c[4], size_t v, float sh[24], float sl[24]) {
   cx<float> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; k++) acc[k] = mkc(0.f, 0.f);
   hop_term<float, MU, FWD>(g, in, gauge, par, i, c, acc);
 #pragma unroll
   for (int k = 0; k < 12; k++) acc[k] = -0.5f * acc[k];
-  SpinorIO<float>::store(out_full + (size_t)par * 24 * g.Vh, g.Vh, i, acc);
+  const int l = c[MU] % o.b[MU];
+  if (o.split[MU] && (FWD ? l == o.b[MU] - 1 : l == 0)) {
+    SpinorIO<float>::store(o.W[MU + (FWD ? 0 : 4)] + v + (size_t)par * 24 * g.Vh, g.Vh, i, acc);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      df_acc(sh[2 * k], sl[2 * k], acc[k].re);
+      df_acc(sh[2 * k + 1], sl[2 * k + 1], acc[k].im);
+    }
+  }
 }
 
-__global__ void k_hop_directions(Geom g, DirOut o, const float* __restrict__ in_even, const float* __restrict__ in_odd,
-                                 const float* __restrict__ gauge) {
+__global__ void __launch_bounds__(128) k_galerkin_hops(Geom g, GalerkinOut o, const float* __restrict__ u,
+                                                       const float* __restrict__ slot,
+                                                       const float* __restrict__ gauge, size_t vstride) {
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= 2 * g.Vh) return;
   const int par = gid / g.Vh, i = gid % g.Vh;
+  const size_t v = blockIdx.y * vstride, half = (size_t)24 * g.Vh;
   int c[4];
   cb_coords(g, i, par, c);
-  const float* in = par ? in_even : in_odd;  // neighbours have the other parity
-  one_dir<0, true>(g, in, gauge, par, i, c, o.p[0]);
-  one_dir<1, true>(g, in, gauge, par, i, c, o.p[1]);
-  one_dir<2, true>(g, in, gauge, par, i, c, o.p[2]);
-  one_dir<3, true>(g, in, gauge, par, i, c, o.p[3]);
-  one_dir<0, false>(g, in, gauge, par, i, c, o.p[4]);
-  one_dir<1, false>(g, in, gauge, par, i, c, o.p[5]);
-  one_dir<2, false>(g, in, gauge, par, i, c, o.p[6]);
-  one_dir<3, false>(g, in, gauge, par, i, c, o.p[7]);
+  const float* in = u + v + (par ? 0 : half);  // neighbours have the other parity
+  cx<float> s[12];
+  SpinorIO<float>::load(slot + v + par * half, g.Vh, i, s);
+  float sh[24], sl[24];
+#pragma unroll
+  for (int k = 0; k < 12; k++) {
+    sh[2 * k] = s[k].re;
+    sh[2 * k + 1] = s[k].im;
+    sl[2 * k] = sl[2 * k + 1] = 0.f;
+  }
+  one_dir<0, true>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<1, true>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<2, true>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<3, true>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<0, false>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<1, false>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<2, false>(g, o, in, gauge, par, i, c, v, sh, sl);
+  one_dir<3, false>(g, o, in, gauge, par, i, c, v, sh, sl);
+#pragma unroll
+  for (int k = 0; k < 12; k++) s[k] = mkc(sh[2 * k], sh[2 * k + 1]);
+  SpinorIO<float>::store(o.Sh + v + par * half, g.Vh, i, s);
+#pragma unroll
+  for (int k = 0; k < 12; k++) s[k] = mkc(sl[2 * k], sl[2 * k + 1]);
+  SpinorIO<float>::store(o.Sl + v + par * half, g.Vh, i, s);
 }
 
-void hop_directions(const Geom& g, float* const out[8], const float* in_even, const float* in_odd, const float* gauge,
-                    cudaStream_t s) {
-  DirOut o;
-  for (int d = 0; d < 8; d++) o.p[d] = out[d];
+void galerkin_hops(const Geom& g, const int block[4], const int cdims[4], const float* u, const float* slot,
+                   float* const W[8], float* Sh, float* Sl, size_t vstride, int ncol, const float* gauge,
+                   cudaStream_t s) {
+  GalerkinOut o;
+  for (int d = 0; d < 8; d++) o.W[d] = W[d];
+  o.Sh = Sh;
+  o.Sl = Sl;
+  for (int m = 0; m < 4; m++) {
+    o.b[m] = block[m];
+    o.split[m] = cdims[m] > 1;
+  }
   const int n = 2 * g.Vh, bs = 128;
-  k_hop_directions<<<(n + bs - 1) / bs, bs, 0, s>>>(g, o, in_even, in_odd, gauge);
+  k_galerkin_hops<<<dim3((n + bs - 1) / bs, ncol), bs, 0, s>>>(g, o, u, slot, gauge, vstride);
   MG_LAUNCH();
 }
 
