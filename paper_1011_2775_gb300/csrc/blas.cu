@@ -5,10 +5,11 @@
 // All inner products accumulate in FP64 regardless of the vector precision.
 // Reductions are deterministic: a fixed grid (a function of n only), per-block
 // partials written to the workspace, and an ordered final sum by the last
-// block to finish (threadfence + atomic ticket).  The GCR kernels fuse the
+// block to finish (grid_sum in dfloat.cuh).  The GCR kernels fuse the
 // orthogonalisation update with the norms it needs and read their
 // coefficients from device memory, so a GCR iteration needs no host round
 // trip except the optional convergence check.
+#include "dfloat.cuh"
 #include "internal.h"
 
 namespace mg {
@@ -29,53 +30,28 @@ inline int ew_grid(size_t n) {
   return (int)b;
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// the grid's sums of NR per-thread values (see grid_sum)
+template <int NR, typename T>
+__device__ __forceinline__ void grid_reduce(const T (&v)[NR], double* partials, unsigned* counter, double* out) {
+  grid_sum<kBS, NR>(v, partials, counter, out);
 }
 
-// Block-reduce v[0..NR) then finish the grid reduction deterministically.
-template <int NR>
-__device__ __forceinline__ void grid_reduce(double (&v)[NR], double* partials, unsigned* counter, double* out) {
-  __shared__ double sm[NR > 0 ? NR : 1][kBS / 32];
-  __shared__ bool is_last;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int r = 0; r < NR; r++) {
-    double t = warp_sum(v[r]);
-    if (lane == 0) sm[r][wid] = t;
+// K complex coefficients read from FP64 device scalars, times `scale`: one
+// thread per value converts, all threads read them from shared memory (a
+// conversion per thread would queue on the FP64 pipe).
+template <int K>
+struct Coefs {
+  float h[2 * (K > 0 ? K : 1)], l[2 * (K > 0 ? K : 1)];
+};
+template <int K>
+__device__ __forceinline__ void load_coefs(Coefs<K>& s, const double* __restrict__ c, double scale) {
+  if (threadIdx.x < 2 * K) {
+    const double v = scale * c[threadIdx.x];
+    const float h = (float)v;
+    s.h[threadIdx.x] = h;
+    s.l[threadIdx.x] = (float)(v - (double)h);
   }
   __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-      double t = lane < nw ? sm[r][lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) partials[(size_t)blockIdx.x * NR + r] = t;
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-#pragma unroll
-  for (int r = 0; r < NR; r++) {
-    double t = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(&partials[(size_t)b * NR + r]);
-    t = warp_sum(t);
-    __syncthreads();
-    if (lane == 0) sm[r][wid] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < nw; w++) s += sm[r][w];
-      out[r] = s;
-    }
-  }
-  if (threadIdx.x == 0) *counter = 0u;
 }
 
 template <typename T>
@@ -136,7 +112,7 @@ __global__ void k_norm2(const cx<T>* __restrict__ x, size_t n, double* partials,
     s = fma((acc_t<T>)a.re, (acc_t<T>)a.re, s);
     s = fma((acc_t<T>)a.im, (acc_t<T>)a.im, s);
   }
-  double v[1] = {(double)s};
+  const acc_t<T> v[1] = {s};
   grid_reduce<1>(v, partials, counter, out);
 }
 template <typename T>
@@ -156,7 +132,7 @@ __global__ void k_cdot(const cx<T>* __restrict__ x, const cx<T>* __restrict__ y,
     s1 = fma((acc_t<T>)a.re, (acc_t<T>)b.im, s1);
     s1 = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s1);
   }
-  double v[2] = {(double)s0, (double)s1};
+  const acc_t<T> v[2] = {s0, s1};
   grid_reduce<2>(v, partials, counter, out);
 }
 template <typename T>
@@ -179,7 +155,7 @@ __global__ void k_dot2(const cx<T>* __restrict__ w, const cx<T>* __restrict__ r,
     s2 = fma((acc_t<T>)a.re, (acc_t<T>)b.im, s2);
     s2 = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s2);
   }
-  double v[3] = {(double)s0, (double)s1, (double)s2};
+  const acc_t<T> v[3] = {s0, s1, s2};
   grid_reduce<3>(v, partials, counter, out);
 }
 // nrhs pairs (w_q, r_q) at `stride` complex apart: d_out[4q .. 4q+2] per pair,
@@ -200,7 +176,7 @@ __global__ void k_dot2_multi(const cx<T>* __restrict__ w, const cx<T>* __restric
     s2 = fma((acc_t<T>)a.re, (acc_t<T>)b.im, s2);
     s2 = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s2);
   }
-  double v[3] = {(double)s0, (double)s1, (double)s2};
+  const acc_t<T> v[3] = {s0, s1, s2};
   grid_reduce<3>(v, partials + (size_t)q * gridDim.x * 3, counters + q, out + 4 * q);
 }
 template <typename T>
@@ -223,8 +199,10 @@ __global__ void k_mr_update_multi(cx<T>* e, cx<T>* r, const cx<T>* __restrict__ 
   r += q * stride;
   w += q * stride;
   in += 4 * q;
-  const double ww = in[0] > 0 ? in[0] : 1.0;
-  const T ar = (T)(in[1] / ww), ai = (T)(in[2] / ww);
+  __shared__ T s_al[2];
+  if (threadIdx.x < 2) s_al[threadIdx.x] = (T)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
+  __syncthreads();
+  const T ar = s_al[0], ai = s_al[1];
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> rv = r[i], wv = w[i], ev = e[i];
     ev.re += ar * rv.re - ai * rv.im;
@@ -272,10 +250,7 @@ __global__ void k_multidot(VecPtrs<T> V, const cx<T>* __restrict__ w, size_t n, 
       s[2 * j + 1] = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s[2 * j + 1]);
     }
   }
-  double v[2 * K];
-#pragma unroll
-  for (int r = 0; r < 2 * K; r++) v[r] = (double)s[r];
-  grid_reduce<2 * K>(v, partials, counter, out);
+  grid_reduce<2 * K>(s, partials, counter, out);
 }
 
 template <typename T>
@@ -308,10 +283,20 @@ template <typename T, int K, bool RED>
 __global__ void k_orth_update(cx<T>* w, VecPtrs<T> V, const double* __restrict__ beta, const cx<T>* __restrict__ r,
                               size_t n, double* partials, unsigned* counter, double* out) {
   T br[K > 0 ? K : 1], bi[K > 0 ? K : 1];
+  if constexpr (sizeof(T) == 4) {
+    __shared__ Coefs<K> sb;
+    if (K > 0) load_coefs<K>(sb, beta, 1.0);
 #pragma unroll
-  for (int j = 0; j < K; j++) {
-    br[j] = (T)beta[2 * j];
-    bi[j] = (T)beta[2 * j + 1];
+    for (int j = 0; j < K; j++) {
+      br[j] = sb.h[2 * j];
+      bi[j] = sb.h[2 * j + 1];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      br[j] = (T)beta[2 * j];
+      bi[j] = (T)beta[2 * j + 1];
+    }
   }
   acc_t<T> s0 = 0, s1 = 0, s2 = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -333,7 +318,7 @@ __global__ void k_orth_update(cx<T>* w, VecPtrs<T> V, const double* __restrict__
       s2 = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s2);
     }
   }
-  double v[3] = {(double)s0, (double)s1, (double)s2};
+  const acc_t<T> v[3] = {s0, s1, s2};
   if (RED) grid_reduce<3>(v, partials, counter, out);
 }
 
@@ -386,15 +371,25 @@ void blas_orth_update(T* w, const T* const* V, const double* d_beta, int k, cons
 template <typename T>
 __global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restrict__ in, double* alpha_out,
                            double* gamma_out, double* partials, unsigned* counter, double* out) {
-  const double g2 = in[0];
-  const double gam = g2 > 0 ? sqrt(g2) : 1.0;
-  const double ar = in[1] / gam, ai = in[2] / gam;  // alpha = <w/gamma, r>
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    alpha_out[0] = ar;
-    alpha_out[1] = ai;
-    gamma_out[0] = gam;
+  // the square root and the divisions by one thread of the block: in every
+  // thread they took longer than the pass over the vectors (29.8 us of which
+  // about 15 at 0.79 M complex FP64)
+  __shared__ T s_ga[3];
+  if (threadIdx.x == 0) {
+    const double g2 = in[0];
+    const double gam = g2 > 0 ? sqrt(g2) : 1.0;
+    const double ar = in[1] / gam, ai = in[2] / gam;  // alpha = <w/gamma, r>
+    if (blockIdx.x == 0) {
+      alpha_out[0] = ar;
+      alpha_out[1] = ai;
+      gamma_out[0] = gam;
+    }
+    s_ga[0] = (T)(1.0 / gam);
+    s_ga[1] = (T)ar;
+    s_ga[2] = (T)ai;
   }
-  const T ig = (T)(1.0 / gam), a_r = (T)ar, a_i = (T)ai;
+  __syncthreads();
+  const T ig = s_ga[0], a_r = s_ga[1], a_i = s_ga[2];
   acc_t<T> s = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> q = w[i];
@@ -408,7 +403,7 @@ __global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restric
     s = fma((acc_t<T>)b.re, (acc_t<T>)b.re, s);
     s = fma((acc_t<T>)b.im, (acc_t<T>)b.im, s);
   }
-  double v[1] = {(double)s};
+  const acc_t<T> v[1] = {s};
   grid_reduce<1>(v, partials, counter, out);
 }
 
@@ -420,24 +415,52 @@ void blas_r_update(T* w, T* r, size_t n, const double* d_in, double* d_alpha, do
   MG_LAUNCH();
 }
 
+// FP64 results are accumulated in FP64.  FP32 results (FP32 vectors, FP64
+// coefficients) are accumulated in compensated FP32 -- about 48 bits before the
+// rounding to FP32 -- with the coefficients as float pairs: in FP64 arithmetic
+// the pass took ten times its memory time (221 us for eight vectors of 1.57 M
+// complex, against 126 MB of traffic).
 template <typename T, typename TZ, int K>
 __global__ void k_lincomb(cx<T>* x, VecPtrs<TZ> Z, const double* __restrict__ c, double scale, size_t n) {
-  double cr[K], ci[K];
+  if constexpr (sizeof(T) == 4) {
+    __shared__ Coefs<K> sc;
+    load_coefs<K>(sc, c, scale);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+      cx<float> z[K];
 #pragma unroll
-  for (int j = 0; j < K; j++) {
-    cr[j] = scale * c[2 * j];
-    ci[j] = scale * c[2 * j + 1];
-  }
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    cx<T> a = x[i];
-    double re = (double)a.re, im = (double)a.im;
+      for (int j = 0; j < K; j++) z[j] = Z.p[j][i];
+      const cx<T> a = x[i];
+      float rh = a.re, rl = 0.f, ih = a.im, il = 0.f;
+#pragma unroll
+      for (int j = 0; j < K; j++) {
+        const float cr = sc.h[2 * j], ci = sc.h[2 * j + 1], lr = sc.l[2 * j], li = sc.l[2 * j + 1];
+        dot2_acc(rh, rl, cr, z[j].re);
+        dot2_acc(rh, rl, -ci, z[j].im);
+        rl = fmaf(lr, z[j].re, fmaf(-li, z[j].im, rl));
+        dot2_acc(ih, il, cr, z[j].im);
+        dot2_acc(ih, il, ci, z[j].re);
+        il = fmaf(lr, z[j].im, fmaf(li, z[j].re, il));
+      }
+      x[i] = mkc<T>(rh + rl, ih + il);
+    }
+  } else {
+    double cr[K], ci[K];
 #pragma unroll
     for (int j = 0; j < K; j++) {
-      cx<TZ> z = Z.p[j][i];
-      re += cr[j] * (double)z.re - ci[j] * (double)z.im;
-      im += cr[j] * (double)z.im + ci[j] * (double)z.re;
+      cr[j] = scale * c[2 * j];
+      ci[j] = scale * c[2 * j + 1];
     }
-    x[i] = mkc<T>((T)re, (T)im);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+      cx<T> a = x[i];
+      double re = (double)a.re, im = (double)a.im;
+#pragma unroll
+      for (int j = 0; j < K; j++) {
+        cx<TZ> z = Z.p[j][i];
+        re += cr[j] * (double)z.re - ci[j] * (double)z.im;
+        im += cr[j] * (double)z.im + ci[j] * (double)z.re;
+      }
+      x[i] = mkc<T>((T)re, (T)im);
+    }
   }
 }
 
@@ -487,8 +510,10 @@ void gcr_backsub(const double* d_beta, int ld, const double* d_alpha, const doub
 
 template <typename T>
 __global__ void k_mr_update(cx<T>* e, cx<T>* r, const cx<T>* __restrict__ w, const double* __restrict__ in, size_t n) {
-  const double ww = in[0] > 0 ? in[0] : 1.0;
-  const T ar = (T)(in[1] / ww), ai = (T)(in[2] / ww);
+  __shared__ T s_al[2];
+  if (threadIdx.x < 2) s_al[threadIdx.x] = (T)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
+  __syncthreads();
+  const T ar = s_al[0], ai = s_al[1];
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> rv = r[i], wv = w[i], ev = e[i];
     ev.re += ar * rv.re - ai * rv.im;
@@ -507,7 +532,10 @@ void blas_mr_update(T* e, T* r, const T* w, const double* d_in, size_t n, cudaSt
 
 template <typename T>
 __global__ void k_normalize(cx<T>* x, const double* __restrict__ nrm2, size_t n) {
-  const T f = (T)(nrm2[0] > 0 ? 1.0 / sqrt(nrm2[0]) : 1.0);
+  __shared__ T s_f;
+  if (threadIdx.x == 0) s_f = (T)(nrm2[0] > 0 ? 1.0 / sqrt(nrm2[0]) : 1.0);
+  __syncthreads();
+  const T f = s_f;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> a = x[i];
     x[i] = mkc<T>(a.re * f, a.im * f);

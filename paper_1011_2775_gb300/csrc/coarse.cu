@@ -677,16 +677,6 @@ void extract_columns(const TransferOp& T, float* p, size_t vstride, int column0,
 // FP64 projections per site, 15.2 ms now (24 launches of two columns), the
 // hops and column extraction around them 2.2 ms.
 
-// h + l <- h + l + a b with the rounding errors of the product and the sum kept in l
-__device__ __forceinline__ void dot2_acc(float& h, float& l, float a, float b) {
-  const float p = __fmul_rn(a, b);
-  const float e = fmaf(a, b, -p);
-  const float s = __fadd_rn(h, p);
-  const float bb = __fsub_rn(s, h);
-  const float t = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  l = __fadd_rn(l, __fadd_rn(t, e));
-  h = s;
-}
 // complex conj(p) w
 __device__ __forceinline__ void dot2_cacc(float (&a)[4], cx<float> p, float wr, float wi) {
   dot2_acc(a[0], a[1], p.re, wr);

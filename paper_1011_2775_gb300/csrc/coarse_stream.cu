@@ -184,53 +184,6 @@ __device__ void gather(const SArgs& a, int i0, int i1, int ips, int site_base, c
   __syncthreads();
 }
 
-// Sum over the warp of V per-lane values (V = 2, 4, 8, 16): each of the first
-// log2 V levels keeps half of the values and passes the other half to its
-// partner, the remaining levels add whole values.  Afterwards lane l holds the
-// total of value (l >> log2(32 / V)) & (V - 1).
-template <int V>
-__device__ __forceinline__ float reduce_values(float v[V]) {
-  const int lane = threadIdx.x & 31;
-  int off = 16;
-#pragma unroll
-  for (int half = V / 2; half >= 1; half /= 2, off /= 2) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < half; i++) {
-      const float send = up ? v[i] : v[i + half];
-      const float keep = up ? v[i + half] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-  float t = v[0];
-#pragma unroll
-  for (int o = 16 / V; o >= 1; o /= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
-}
-
-// reduce_values for double-float sums: lane l ends with the warp total of
-// v[(l >> (5 - log2 V)) & (V - 1)], added in a fixed order.
-template <int V>
-__device__ __forceinline__ df reduce_df(df v[V]) {
-  const int lane = threadIdx.x & 31;
-  int off = 16;
-#pragma unroll
-  for (int half = V / 2; half >= 1; half /= 2, off /= 2) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < half; i++) {
-      const df send = up ? v[i] : v[i + half];
-      const df keep = up ? v[i + half] : v[i];
-      v[i] = df_add(keep, df{__shfl_xor_sync(0xffffffffu, send.h, off), __shfl_xor_sync(0xffffffffu, send.l, off)});
-    }
-  }
-  df t = v[0];
-#pragma unroll
-  for (int o = 16 / V; o >= 1; o /= 2)
-    t = df_add(t, df{__shfl_xor_sync(0xffffffffu, t.h, o), __shfl_xor_sync(0xffffffffu, t.l, o)});
-  return t;
-}
-
 // out[row] = sum_k L[row][k] v[k] for the NR rows of a staged item (row-major,
 // K complex per row, storage format ST).  Every lane strides along the rows
 // two float4 steps at a time, loading the vector element once for all rows.
@@ -270,7 +223,7 @@ __device__ __forceinline__ bool item_rows(const unsigned char* stage, int K, con
     step(q + 32);
   }
   if (q < K2) step(q);
-  const float t = reduce_values<V>(acc);                       // lane l: value (l >> SH) & (V - 1)
+  const float t = warp_transpose_sum<V>(acc);                       // lane l: value (l >> SH) & (V - 1)
   const float im = __shfl_down_sync(0xffffffffu, t, 1 << SH);  // value 2 row + 1
   res = make_float2(t, im);
   row = lane >> (SH + 1);
@@ -375,7 +328,7 @@ __device__ void grid_totals(const SArgs& a, int q0, int nq, df* out) {
 #pragma unroll
         for (int i = 1; i < kTotG / 32; i++) sv[u] = df_add(sv[u], df{t[u][i].x, t[u][i].y});
       }
-      const df s = reduce_df<kTotU>(sv);   // lane l: slot qb + (l >> 3) * kWarps
+      const df s = warp_transpose_sum<kTotU>(sv);   // lane l: slot qb + (l >> 3) * kWarps
       const int q = qb + (lane >> 3) * kWarps;
       if ((lane & 7) == 0 && q < nq) out[q] = s;
     }
@@ -518,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
           sv[2 * u] = df_of(re[u]);
           sv[2 * u + 1] = df_of(im[u]);
         }
-        const df sr = reduce_df<8>(sv);   // lane l: sum (l >> 2) = 2 u + {re, im}
+        const df sr = warp_transpose_sum<8>(sv);   // lane l: sum (l >> 2) = 2 u + {re, im}
         const int j = jb + (lane >> 3) * kWarps;
         if ((lane & 3) == 0 && j < k) a.partials[(size_t)(RA + 2 * j + ((lane >> 2) & 1)) * G + bid] = make_float2(sr.h, sr.l);
       }

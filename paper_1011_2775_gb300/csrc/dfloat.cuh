@@ -50,6 +50,17 @@ __device__ __forceinline__ df df_sqrt(df a) {
   const df r = df_add(a, df_neg(df_mul(df_of(s), df_of(s))));
   return df_norm(s, r.h / (2.f * s));
 }
+// a b added to h + l with the rounding errors of the product and of the sum
+// kept in l (Ogita, Rump and Oishi's Dot2, not renormalised)
+__device__ __forceinline__ void dot2_acc(float& h, float& l, float a, float b) {
+  const float p = __fmul_rn(a, b);
+  const float e = fmaf(a, b, -p);
+  const float s = __fadd_rn(h, p);
+  const float bb = __fsub_rn(s, h);
+  const float t = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  l = __fadd_rn(l, __fadd_rn(t, e));
+  h = s;
+}
 __device__ __forceinline__ df df_wsum(df v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -59,5 +70,97 @@ __device__ __forceinline__ df df_wsum(df v) {
   return v;
 }
 
+// Sums over the warp of V (2, 4, 8, 16) values per lane by transposition: each
+// of the first log2 V levels keeps half of the values and passes the other half
+// to its partner, the remaining levels add whole values, so V values cost
+// V - 1 + log2(32 / V) additions per lane instead of 5 V.  Lane l ends with the
+// warp total of v[(l >> (5 - log2 V)) & (V - 1)], added in a fixed order.
+__device__ __forceinline__ float shfl_x(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double shfl_x(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ df shfl_x(df v, int o) { return df{shfl_x(v.h, o), shfl_x(v.l, o)}; }
+__device__ __forceinline__ float add_x(float a, float b) { return a + b; }
+__device__ __forceinline__ double add_x(double a, double b) { return a + b; }
+__device__ __forceinline__ df add_x(df a, df b) { return df_add(a, b); }
+template <int V, typename S>
+__device__ __forceinline__ S warp_transpose_sum(S (&v)[V]) {
+  const int lane = threadIdx.x & 31;
+  int off = 16;
+#pragma unroll
+  for (int half = V / 2; half >= 1; half /= 2, off /= 2) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < half; i++) {
+      const S send = up ? v[i] : v[i + half];
+      const S keep = up ? v[i + half] : v[i];
+      v[i] = add_x(keep, shfl_x(send, off));
+    }
+  }
+  S t = v[0];
+#pragma unroll
+  for (int o = 16 / V; o >= 1; o /= 2) t = add_x(t, shfl_x(t, o));
+  return t;
+}
+
+// Deterministic sum over the grid of NR values per thread into out[0 .. NR):
+// transposed warp sums -- double-float for FP32 sums, FP64 for FP64 ones --, the
+// warps of a block added in order, block sums in partials[r][block], and the
+// last block to finish adds them, one warp per value.  FP64 additions are the
+// scarce resource here (1/62 of the FP32 rate): with a whole butterfly per
+// value the tree took longer than the memory pass it closes.  THREADS = block
+// size; the counter is 0 at launch and left at 0.
+__device__ __forceinline__ double sum_to_double(double v) { return v; }
+__device__ __forceinline__ double sum_to_double(df v) { return (double)v.h + (double)v.l; }
+__device__ __forceinline__ double sum_of(double v) { return v; }
+__device__ __forceinline__ df sum_of(float v) { return df_of(v); }
+__device__ __forceinline__ df sum_of(df v) { return v; }
+template <int THREADS, int NR, typename T>
+__device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, unsigned* counter, double* out) {
+  using S = decltype(sum_of(T{}));
+  constexpr int W = THREADS / 32;
+  constexpr int V = NR <= 1 ? 1 : NR <= 2 ? 2 : NR <= 4 ? 4 : NR <= 8 ? 8 : 16;
+  static_assert(NR <= 16, "at most 16 values");
+  __shared__ S sm[NR][W];
+  __shared__ bool is_last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  S t[V];
+#pragma unroll
+  for (int r = 0; r < V; r++) t[r] = r < NR ? sum_of(v[r < NR ? r : 0]) : sum_of(T{});
+  S sum;
+  if constexpr (V == 1) {
+    sum = t[0];
+#pragma unroll
+    for (int o = 16; o >= 1; o /= 2) sum = add_x(sum, shfl_x(sum, o));
+    if (lane == 0) sm[0][wid] = sum;
+  } else {
+    sum = warp_transpose_sum<V>(t);
+    constexpr int per = 32 / V;   // lanes holding one value
+    const int r = lane / per;
+    if (lane % per == 0 && r < NR) sm[r][wid] = sum;
+  }
+  __syncthreads();
+  if (threadIdx.x < NR) {
+    S s = sm[threadIdx.x][0];
+#pragma unroll
+    for (int w = 1; w < W; w++) s = add_x(s, sm[threadIdx.x][w]);
+    partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = sum_to_double(s);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();   // the block's partials before its ticket
+    is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!is_last) return;
+  __threadfence();
+  for (int r = wid; r < NR; r += W) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(&partials[(size_t)r * gridDim.x + b]);
+#pragma unroll
+    for (int o = 16; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[r] = s;
+  }
+  if (threadIdx.x == 0) *counter = 0u;
+}
 
 }  // namespace mg

@@ -10,9 +10,10 @@
 //   k_mr_update_clover             e += alpha r, r -= alpha w, s_e = A_e^{-1} r_e
 // The clover product A_e^{-1} r of the next step is taken from the update
 // (site-local), and the two inner products from the dslash epilogue (w and r
-// are in registers there).  Sums: FP32 per site (12 components), FP64 across
-// sites, per-block partials added by the last block in a fixed order, so the
+// are in registers there).  Sums: FP32 per site (12 components), double-float
+// across the sites of a block, FP64 across blocks, in a fixed order, so the
 // result does not depend on block scheduling.
+#include "dfloat.cuh"
 #include "internal.h"
 #include "wilson_dev.cuh"
 
@@ -21,62 +22,13 @@ namespace {
 
 constexpr int kMRThreads = 256;
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// the three sums of the CTA into partials[blockIdx.x][0..2]; the last CTA to
-// finish adds all partials in block order into out[0..2] and resets the counter
-__device__ void mr_reduce3(double v0, double v1, double v2, double* partials, unsigned* counter, double* out) {
-  __shared__ double sm[3][kMRThreads / 32];
-  __shared__ bool last;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double v[3] = {v0, v1, v2};
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-    const double t = warp_sum_d(v[q]);
-    if (lane == 0) sm[q][wid] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double t = 0.0;
-    for (int w = 0; w < kMRThreads / 32; w++) t += sm[threadIdx.x][w];
-    partials[(size_t)blockIdx.x * 3 + threadIdx.x] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double t[3] = {0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < 3; q++) t[q] += __ldcg(&partials[(size_t)b * 3 + q]);
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-    const double s = warp_sum_d(t[q]);
-    if (lane == 0) sm[q][wid] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int w = 0; w < kMRThreads / 32; w++) s += sm[threadIdx.x][w];
-    out[threadIdx.x] = s;
-  }
-  if (threadIdx.x == 0) *counter = 0u;
-}
-
 // w_e = r_e - H_eo t_o on even sites (grid-stride over sites), with
 // out[0] = <w, w>, out[1] + i out[2] = <w, r> = sum conj(w) r
 __global__ void __launch_bounds__(kMRThreads) k_mr_dslash_dot(Geom g, float* __restrict__ w, const float* __restrict__ t,
                                                               const float* __restrict__ gauge,
                                                               const float* __restrict__ r, double* partials,
                                                               unsigned* counter, double* out) {
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+  df s0 = df_of(0.f), s1 = df_of(0.f), s2 = df_of(0.f);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.Vh; i += gridDim.x * blockDim.x) {
     int c[4];
     cb_coords(g, i, 0, c);
@@ -96,11 +48,12 @@ __global__ void __launch_bounds__(kMRThreads) k_mr_dslash_dot(Geom g, float* __r
       a2 = fmaf(wv[k].re, rv[k].im, fmaf(-wv[k].im, rv[k].re, a2));
     }
     SpinorIO<float>::store(w, g.Vh, i, wv);
-    s0 += a0;
-    s1 += a1;
-    s2 += a2;
+    s0 = df_add(s0, df_of(a0));
+    s1 = df_add(s1, df_of(a1));
+    s2 = df_add(s2, df_of(a2));
   }
-  mr_reduce3(s0, s1, s2, partials, counter, out);
+  const df v[3] = {s0, s1, s2};
+  grid_sum<kMRThreads, 3>(v, partials, counter, out);
 }
 
 // e += alpha r, r -= alpha w (alpha = in[1..2] / in[0]), and s = A_e^{-1} r
@@ -108,10 +61,12 @@ __global__ void __launch_bounds__(kMRThreads) k_mr_dslash_dot(Geom g, float* __r
 __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restrict__ e, float* __restrict__ r,
                                                           const float* __restrict__ w, const double* __restrict__ in,
                                                           const float* __restrict__ clov, float* __restrict__ s) {
+  __shared__ float s_al[2];   // two FP64 divisions per block, not per thread
+  if (threadIdx.x < 2) s_al[threadIdx.x] = (float)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.Vh) return;
-  const double ww = in[0] > 0 ? in[0] : 1.0;
-  const float ar = (float)(in[1] / ww), ai = (float)(in[2] / ww);
+  const float ar = s_al[0], ai = s_al[1];
   cx<float> ev[12], rv[12], wv[12], sv[12];
   SpinorIO<float>::load(e, g.Vh, i, ev);
   SpinorIO<float>::load(r, g.Vh, i, rv);
