@@ -13,12 +13,13 @@
 //    epilogues as the fine dslash, which give the coarse even-odd operators
 //    (the coarse system is solved by its reduced even-odd form)
 //  * FP64 batched Gauss-Jordan for X^{-1}
-//  * block Gram-Schmidt (FP64 accumulation) and coarse-vector packing
+//  * block Gram-Schmidt (float-pair vectors and sums) and coarse-vector packing
 //
 // Coarse operators look like a staggered operator with Nc = 2 Nv colours
 // ("Implementation"); a CTA owns one coarse site, its warps own rows of the
 // 2Nv x 8*2Nv link block, and the neighbour vectors are staged in shared
 // memory so each link row is read once, coalesced.
+#include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -108,12 +109,6 @@ TArgs targs(const TransferOp& T) {
   a.Ps = T.Pscale.as<float>();
   a.flags = T.flags;
   return a;
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 }  // namespace
 
@@ -1317,7 +1312,7 @@ struct GSArgs {
   TArgs a;
   const float* V;       // nv level vectors, vector k at V + k * vstride
   size_t vstride;       // floats between consecutive vectors
-  double2* Q;           // [ncoarse][2][nv][L]
+  float4* Q;            // [ncoarse][2][nv][L] complex float pairs {re.h, re.l, im.h, im.l}
   int L;                // nb * ndof / 2
 };
 
@@ -1332,77 +1327,129 @@ __global__ void k_gs_gather(GSArgs g) {
     const int i = l / hd, c = ch * hd + l % hd;
     const int idx = g.a.blockmap[cc * g.a.nb + i];
     const cx<float> z = fget(g.a.fa, g.V + (size_t)k * g.vstride, idx, c);
-    g.Q[(size_t)cc * per + t] = make_double2(z.re, z.im);
+    g.Q[(size_t)cc * per + t] = make_float4(z.re, 0.f, z.im, 0.f);
   }
 }
 
-// one CTA per (coarse site, chirality): modified Gram-Schmidt, every vector
-// projected twice, FP64 accumulation; breakdown if the norm after projection
-// drops below kGSBreakdown of the norm before.  The vectors arrive in FP32,
-// so dependence is only resolvable to about 1e-7: the threshold is 1e-6
-// (the FP64 oracle uses 1e-10 on FP64 vectors).
+// one CTA per (coarse site, chirality): classical Gram-Schmidt with every
+// vector projected twice; breakdown if the norm after projection drops below
+// kGSBreakdown of the norm before.  The vectors arrive in FP32, so dependence
+// is only resolvable to about 1e-7: the threshold is 1e-6 (the FP64 oracle
+// uses 1e-10 on FP64 vectors).
+//
+// Arithmetic-bound in FP64 (11 ms at the FP64 rate for 512 blocks of 1536 x 24
+// x 2 chiralities) and, projected vector by vector, bound by one block barrier
+// per inner product (28.8 ms measured).  Here the vector being orthogonalised
+// stays in shared memory, all its inner products are taken before one
+// reduction, and vectors and sums are float pairs (about 48 bits, twelve FP32
+// operations per product against 62 operation slots of an FP64 FMA): 5.6 ms.  Large
+// problems run one CTA per SM so that the resident blocks' vectors (590 KB
+// each) are re-read from L2.
 constexpr double kGSBreakdown = 1e-6;
+constexpr int kGSThreads = 512;
+constexpr int kGSWarps = kGSThreads / 32;
+constexpr size_t kGSFixed = sizeof(df) * (64 * kGSWarps + 64) + 64;   // reduction and coefficients (nv <= 32)
 
-__global__ void k_block_gs(GSArgs g, int* flags) {
-  __shared__ double red[2][32];
+__global__ void __launch_bounds__(kGSThreads) k_block_gs(GSArgs g, int in_smem, int* flags) {
+  extern __shared__ __align__(16) unsigned char gsm[];
+  df* red = reinterpret_cast<df*>(gsm);            // [2 nv][warp]
+  df* coef = red + 64 * kGSWarps;                   // [2 nv]
+  float* bc = reinterpret_cast<float*>(coef + 64);  // broadcast values
+  float4* wbuf = reinterpret_cast<float4*>(gsm + kGSFixed);
   const int blk = blockIdx.x;  // cc * 2 + ch
   const int nv = g.a.nv, L = g.L;
-  double2* Q = g.Q + (size_t)blk * nv * L;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  auto block_sum2 = [&](double x, double y, double& ox, double& oy) {
-    x = warp_sum(x);
-    y = warp_sum(y);
-    __syncthreads();
-    if (lane == 0) {
-      red[0][wid] = x;
-      red[1][wid] = y;
+  float4* Q = g.Q + (size_t)blk * nv * L;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // ||w||^2 (every thread returns with the total in bc[0..1])
+  auto norm2 = [&](const float4* w) {
+    float h = 0.f, l = 0.f;
+    for (int e = threadIdx.x; e < L; e += kGSThreads) {
+      const float4 x = w[e];
+      df_dot_acc(h, l, df{x.x, x.y}, df{x.x, x.y});
+      df_dot_acc(h, l, df{x.z, x.w}, df{x.z, x.w});
     }
+    const df t = df_wsum(df_norm(h, l));
+    if (lane == 0) red[wid] = t;
     __syncthreads();
-    double sx = 0, sy = 0;
-    for (int q = 0; q < nw; q++) {
-      sx += red[0][q];
-      sy += red[1][q];
-    }
-    ox = sx;
-    oy = sy;
+    df s = red[0];
+#pragma unroll
+    for (int q = 1; q < kGSWarps; q++) s = df_add(s, red[q]);
+    __syncthreads();
+    return s;
   };
   for (int k = 0; k < nv; k++) {
-    double2* w = Q + (size_t)k * L;
-    double n0 = 0, dummy;
-    {
-      double a = 0;
-      for (int l = threadIdx.x; l < L; l += blockDim.x) a += w[l].x * w[l].x + w[l].y * w[l].y;
-      block_sum2(a, 0.0, n0, dummy);
-    }
-    for (int pass = 0; pass < 2; pass++)
-      for (int j = 0; j < k; j++) {
-        const double2* q = Q + (size_t)j * L;
-        double re = 0, im = 0;
-        for (int l = threadIdx.x; l < L; l += blockDim.x) {
-          re += q[l].x * w[l].x + q[l].y * w[l].y;
-          im += q[l].x * w[l].y - q[l].y * w[l].x;
+    float4* wk = Q + (size_t)k * L;
+    float4* w = in_smem ? wbuf : wk;
+    if (in_smem)   // a thread only ever touches its own elements of w
+      for (int e = threadIdx.x; e < L; e += kGSThreads) w[e] = wk[e];
+    const df n0 = norm2(w);
+    for (int pass = 0; pass < 2 && k > 0; pass++) {
+      for (int j0 = 0; j0 < k; j0 += 4) {
+        float acc[4][4] = {};
+        for (int e = threadIdx.x; e < L; e += kGSThreads) {
+          float4 q[4];
+#pragma unroll
+          for (int u = 0; u < 4; u++) q[u] = j0 + u < k ? Q[(size_t)(j0 + u) * L + e] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 x = w[e];
+          const df xr{x.x, x.y}, xi{x.z, x.w};
+#pragma unroll
+          for (int u = 0; u < 4; u++) {   // conj(q) x
+            const df qr{q[u].x, q[u].y}, qi{q[u].z, q[u].w};
+            df_dot_acc(acc[u][0], acc[u][1], qr, xr);
+            df_dot_acc(acc[u][0], acc[u][1], qi, xi);
+            df_dot_acc(acc[u][2], acc[u][3], qr, xi);
+            df_dot_acc(acc[u][2], acc[u][3], df_neg(qi), xr);
+          }
         }
-        double dre, dim;
-        block_sum2(re, im, dre, dim);
-        for (int l = threadIdx.x; l < L; l += blockDim.x) {
-          w[l].x -= dre * q[l].x - dim * q[l].y;
-          w[l].y -= dre * q[l].y + dim * q[l].x;
+        df v[8];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          v[2 * u] = df_norm(acc[u][0], acc[u][1]);
+          v[2 * u + 1] = df_norm(acc[u][2], acc[u][3]);
         }
-        __syncthreads();
+        const df t = warp_transpose_sum<8>(v);   // lane l: value l >> 2
+        const int q = 2 * j0 + (lane >> 2);
+        if ((lane & 3) == 0 && q < 2 * k) red[q * kGSWarps + wid] = t;
       }
-    double n1 = 0;
-    {
-      double a = 0;
-      for (int l = threadIdx.x; l < L; l += blockDim.x) a += w[l].x * w[l].x + w[l].y * w[l].y;
-      block_sum2(a, 0.0, n1, dummy);
+      __syncthreads();
+      if (threadIdx.x < 2 * k) {
+        df s = red[threadIdx.x * kGSWarps];
+#pragma unroll
+        for (int q = 1; q < kGSWarps; q++) s = df_add(s, red[threadIdx.x * kGSWarps + q]);
+        coef[threadIdx.x] = df_neg(s);
+      }
+      __syncthreads();
+      for (int e = threadIdx.x; e < L; e += kGSThreads) {
+        float4 x = w[e];
+#pragma unroll 4
+        for (int j = 0; j < k; j++) {   // x -= c q
+          const float4 q = Q[(size_t)j * L + e];
+          const df qr{q.x, q.y}, qi{q.z, q.w}, cr = coef[2 * j], ci = coef[2 * j + 1];
+          df_dot_acc(x.x, x.y, cr, qr);
+          df_dot_acc(x.x, x.y, df_neg(ci), qi);
+          df_dot_acc(x.z, x.w, cr, qi);
+          df_dot_acc(x.z, x.w, ci, qr);
+        }
+        const df re = df_norm(x.x, x.y), im = df_norm(x.z, x.w);
+        w[e] = make_float4(re.h, re.l, im.h, im.l);
+      }
     }
-    if (threadIdx.x == 0 && (!(n0 > 0) || !(sqrt(n1) >= kGSBreakdown * sqrt(n0)))) atomicExch(&flags[FLAG_GS_BREAKDOWN], 1);
-    const double f = n1 > 0 ? 1.0 / sqrt(n1) : 0.0;
-    for (int l = threadIdx.x; l < L; l += blockDim.x) {
-      w[l].x *= f;
-      w[l].y *= f;
+    const df n1 = norm2(w);
+    if (threadIdx.x == 0) {
+      const double a = (double)n0.h + (double)n0.l, b = (double)n1.h + (double)n1.l;
+      if (!(a > 0) || !(sqrt(b) >= kGSBreakdown * sqrt(a))) atomicExch(&flags[FLAG_GS_BREAKDOWN], 1);
+      const double f = b > 0 ? 1.0 / sqrt(b) : 0.0;
+      bc[0] = (float)f;
+      bc[1] = (float)(f - (double)bc[0]);
     }
     __syncthreads();
+    const df f{bc[0], bc[1]};
+    for (int e = threadIdx.x; e < L; e += kGSThreads) {
+      const float4 x = w[e];
+      const df re = df_mul(df{x.x, x.y}, f), im = df_mul(df{x.z, x.w}, f);
+      wk[e] = make_float4(re.h, re.l, im.h, im.l);
+    }
+    __syncthreads();   // q_k of this thread's elements is read by the same thread only; bc is reused
   }
 }
 
@@ -1415,14 +1462,14 @@ __global__ void k_gs_scatter(GSArgs g, void* P, float* Ps) {
   const int cc = blockIdx.x;
   const int nv = g.a.nv, hd = g.a.ndof / 2, L = g.L;
   const size_t per = (size_t)2 * nv * L;
-  const double2* Qc = g.Q + (size_t)cc * per;
+  const float4* Qc = g.Q + (size_t)cc * per;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   float m[2] = {0.f, 0.f};
   if (ST != STORE_F32)
     for (size_t t = threadIdx.x; t < per; t += blockDim.x) {
       const int ch = (int)(t / ((size_t)nv * L));
-      const double2 z = Qc[t];
-      m[ch] = fmaxf(m[ch], fmaxf(fabsf((float)z.x), fabsf((float)z.y)));
+      const float4 z = Qc[t];   // the high halves are the values rounded to FP32
+      m[ch] = fmaxf(m[ch], fmaxf(fabsf(z.x), fabsf(z.z)));
     }
   for (int ch = 0; ch < 2; ch++) {
     float v = m[ch];
@@ -1442,9 +1489,9 @@ __global__ void k_gs_scatter(GSArgs g, void* P, float* Ps) {
     const int k = (int)((t / L) % nv);
     const int l = (int)(t % L);
     const int i = l / hd, c = ch * hd + l % hd;
-    const double2 z = Qc[t];
+    const float4 z = Qc[t];
     const float inv = 1.f / scale_s[ch];
-    sput<ST>(P, ((size_t)(cc * g.a.nb + i) * g.a.ndof + c) * nv + k, mkc((float)z.x * inv, (float)z.y * inv));
+    sput<ST>(P, ((size_t)(cc * g.a.nb + i) * g.a.ndof + c) * nv + k, mkc(z.x * inv, z.z * inv));
   }
 }
 
@@ -1456,12 +1503,21 @@ void block_orthonormalize(TransferOp& T, const float* const* V, DBuf& scratch, i
   for (int k = 2; k < T.nv; k++)
     if ((size_t)(V[k] - V[0]) != k * g.vstride) raise(MG_ERR_ARG, "null vectors must be equally spaced");
   g.L = T.nb * T.fine_ndof / 2;
-  const size_t need = sizeof(double2) * (size_t)T.ncoarse * 2 * T.nv * g.L;
+  const size_t need = sizeof(float4) * (size_t)T.ncoarse * 2 * T.nv * g.L;
   if (scratch.bytes() < need) scratch.alloc(need);
-  g.Q = scratch.as<double2>();
+  g.Q = scratch.as<float4>();
   k_gs_gather<<<T.ncoarse, kBS, 0, s>>>(g);
   MG_LAUNCH();
-  k_block_gs<<<T.ncoarse * 2, kBS, 0, s>>>(g, flags);
+  int dev = 0, optin = 0;
+  MG_CUDA(cudaGetDevice(&dev));
+  MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  size_t sm = kGSFixed + sizeof(float4) * (size_t)g.L;
+  const int in_smem = sm <= (size_t)optin;   // a block too large for shared memory works in place
+  if (!in_smem) sm = kGSFixed;
+  // more than about the L2 capacity of vectors in all: one CTA per SM
+  if (need > ((size_t)96 << 20)) sm = std::max<size_t>(sm, (size_t)optin / 2 + 1024);
+  MG_CUDA(cudaFuncSetAttribute(k_block_gs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  k_block_gs<<<T.ncoarse * 2, kGSThreads, sm, s>>>(g, in_smem, flags);
   MG_LAUNCH();
   switch (T.store) {
     case STORE_F32: k_gs_scatter<STORE_F32><<<T.ncoarse, kBS, 0, s>>>(g, T.P.get(), T.Pscale.as<float>()); break;

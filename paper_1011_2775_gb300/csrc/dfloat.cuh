@@ -61,6 +61,16 @@ __device__ __forceinline__ void dot2_acc(float& h, float& l, float a, float b) {
   l = __fadd_rn(l, __fadd_rn(t, e));
   h = s;
 }
+// the same for a product of two double-floats (the l l term is below the sum's error)
+__device__ __forceinline__ void df_dot_acc(float& h, float& l, df a, df b) {
+  const float p = __fmul_rn(a.h, b.h);
+  const float e = fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)));
+  const float s = __fadd_rn(h, p);
+  const float bb = __fsub_rn(s, h);
+  const float t = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  l = __fadd_rn(l, __fadd_rn(t, e));
+  h = s;
+}
 __device__ __forceinline__ df df_wsum(df v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -1,4 +1,4 @@
-"""GPU parity of the Galerkin coarse links at the edges of their kernels.
+"""GPU parity of the Galerkin coarse links (and the block Gram-Schmidt) at the edges of their kernels.
 
 The projection takes two columns per thread, splits its threads into groups of
 Nv, and sums the hops inside a block apart from those that cross a face: odd
@@ -27,6 +27,7 @@ CASES = [
     ((4, 8, 4, 4), [(4, 2, 4, 2)], [32], 0),
     ((4, 4, 8, 4), [(2, 2, 4, 4)], [7], 1),
     ((8, 8, 4, 8), [(2, 2, 2, 2), (2, 4, 1, 2)], [6, 9], 0),
+    ((8, 8, 8, 8), [(8, 8, 8, 8)], [4], 0),   # a block too large for the Gram-Schmidt's shared memory
 ]
 
 
