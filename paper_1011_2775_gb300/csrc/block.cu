@@ -125,7 +125,9 @@ void read_norms(Run& R, const double* ve, const double* vo, const std::vector<ch
 // shared launches (the others solve their own)
 void precondition_all(std::vector<Run*>& runs, int k) {
   std::vector<Run*> joint, own;
-  for (Run* R : runs) (mg_batch_joinable(R->c) ? joint : own).push_back(R);
+  // a lattice whose systems the grouped solver takes together is faster by itself than
+  // in a launch shared with other lattices
+  for (Run* R : runs) (mg_batch_joinable(R->c) && !mg_batch_grouped(R->c, R->nb) ? joint : own).push_back(R);
   // runs that can share a launch: same device, coarse storage, restart, cap and even-odd structure
   std::vector<Run*> shared, alone = own;
   for (Run* R : joint) {

@@ -139,6 +139,8 @@ struct CoarseGCRBuffers {
   DBuf st_part, st_beta, st_sync;
   // tensor-core solve (coarse_tc.cu; grown on demand)
   DBuf tc_y, tc_r, tc_br, tc_s, tc_sy, tc_t, tc_tb, tc_W, tc_Z, tc_part, tc_sync;
+  // grouped solve (coarse_group.cu; grown on demand)
+  DBuf gp_v, gp_W, gp_R, gp_part, gp_sync;
   void init(const LevelGeom& G, int nc, int m);
 };
 // x = D_hat^{-1} b to ||b - D_hat x|| <= tol_rel ||b|| (or maxit iterations) by
@@ -206,6 +208,13 @@ void coarse_gcr_solve_multi(const std::vector<CoarseSystem>& sys, CoarseGCRBuffe
 // nb right-hand sides of one lattice (b, x: [nb][nsites nc] floats x 2)
 void coarse_gcr_solve_batch(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuffers& B, int m, int maxit,
                             double tol_rel, int nb, const float* b, float* x, long long* d_iters, int* flags,
+                            cudaStream_t s);
+
+// The same GCR for 1 to 16 systems of one lattice (even-odd or with an odd
+// extent, any link storage) with every link read once for all of them
+// (coarse_group.cu).  Raises FLAG_TIMEOUT if a wait runs out of time.
+bool coarse_gcr_group_ok(const LevelGeom& G, const CoarseOp& C, int nb);
+void coarse_gcr_group_solve(const std::vector<CoarseSystem>& sys, CoarseGCRBuffers& B, int m, int maxit, int* flags,
                             cudaStream_t s);
 
 // the coarsest systems of a context's batched cycle (2-level hierarchies; the

@@ -454,6 +454,8 @@ void mg_batch_pre(Ctx* c, float* z_e, const float* r_e, int nb);
 void mg_batch_coarse(Ctx* c, int nb);
 void mg_batch_post(Ctx* c, float* z_e, const float* r_e, int nb);
 bool mg_batch_joinable(Ctx* c);
+// the coarsest solves of nb right-hand sides of this context take the grouped solver by themselves
+bool mg_batch_grouped(Ctx* c, int nb);
 // MG_OP_CYCLE of level 0 for nb ABI vectors through mg_precondition_batch
 void mg_cycle_batch(Ctx* c, double* out_abi, const double* in_abi, int nb);
 void mg_apply_level(Ctx* c, int op, int level, double* out_abi, const double* in_abi);

@@ -278,8 +278,12 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
         coarse_gcr_stream_ok(G, H.cop[l]) ? coarse_gcr_stream_grids(G, H.cop[l]) : std::vector<int>();
     const std::vector<int> tensor =
         coarse_gcr_tc_ok(G, H.cop[l], 1) ? coarse_gcr_tc_grids(G, H.cop[l], 1) : std::vector<int>();
+    const bool grouped = coarse_gcr_group_ok(G, H.cop[l], 1);
     auto run = [&](int which, long long* it) {
-      if (which >= 200) {
+      if (which >= 300) {
+        coarse_gcr_group_solve({CoarseSystem{&G, &H.cop[l], b, x, p.tol_coarse, it}}, W.cg, restart, p.maxit_coarse,
+                               c->ws.flags.as<int>(), s);
+      } else if (which >= 200) {
         const double tol = p.tol_coarse;
         const size_t nf = G.vec_complex();
         coarse_gcr_tc_solve(G, H.cop[l], W.cg, restart, p.maxit_coarse, &tol, 1, b, nf, x, nf, it,
@@ -296,10 +300,13 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
     };
     if (W.coarse_impl < 0) {
       if (!W.tune_iters.get()) W.tune_iters.alloc(sizeof(long long));
-      TuneKey key{"coarse_gcr3", {G.L[0], G.L[1], G.L[2], G.L[3]}, H.cop[l].nc, H.cop[l].store};
+      TuneKey key{"coarse_gcr4", {G.L[0], G.L[1], G.L[2], G.L[3]}, H.cop[l].nc, H.cop[l].store};
       std::vector<int> cands = {0, 1};
       for (size_t k = 0; k < smaller.size(); k++) cands.push_back(2 + (int)k);
       for (size_t k = 0; k < streamed.size(); k++) cands.push_back(100 + (int)k);
+      // the grouped kernel with one system (candidate 300) also takes odd-extent lattices (3^3x6 sites, Nc = 48:
+      // 99 us against 243 us of the single-system kernel); on even-odd lattices it is timed against the streamed one
+      if (grouped) cands.push_back(300);
       const int forced = c->params.coarse_impl;
       // one system on tensor cores uses one column of eight of every MMA and
       // pays two site-inverse passes per iteration: measured slower than the
@@ -312,7 +319,7 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
         std::vector<int> f;
         for (int cnd : cands)
           if ((forced == 1 && (cnd == 0 || (cnd >= 2 && cnd < 100))) || (forced == 2 && cnd == 1) ||
-              (forced == 3 && cnd >= 100 && cnd < 200) || (forced == 4 && cnd >= 200))
+              (forced == 3 && cnd >= 100 && cnd < 200) || (forced == 4 && cnd >= 200 && cnd < 300))
             f.push_back(cnd);
         if (f.empty()) f.push_back(0);
         W.coarse_impl = f.size() == 1 ? f[0]
@@ -325,7 +332,8 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
       }
       const bool valid = (W.coarse_impl >= 0 && W.coarse_impl < 2 + (int)smaller.size()) ||
                          (W.coarse_impl >= 100 && W.coarse_impl < 100 + (int)streamed.size()) ||
-                         (W.coarse_impl >= 200 && W.coarse_impl < 200 + (int)tensor.size());
+                         (W.coarse_impl >= 200 && W.coarse_impl < 200 + (int)tensor.size()) ||
+                         (W.coarse_impl == 300 && grouped);
       if (!valid) W.coarse_impl = 0;  // a cached choice from other grids
     }
     run(W.coarse_impl, d_it);
@@ -696,6 +704,11 @@ void mg_batch_pre(Ctx* c, float* z, const float* r, int nb) {
 
 bool mg_batch_joinable(Ctx* c) { return c->mg && c->mg->L == 2; }
 
+bool mg_batch_grouped(Ctx* c, int nb) {
+  if (!mg_batch_joinable(c) || c->params.coarse_impl != 0) return false;
+  return coarse_gcr_group_ok(c->mg->geo[1], c->mg->cop[1], std::min(nb, coarse_gcr_batch_max()));
+}
+
 void mg_batch_systems(Ctx* c, int nb, std::vector<CoarseSystem>& out) {
   if (!mg_batch_joinable(c)) raise(MG_ERR_STATE, "only 2-level hierarchies join a shared coarsest solve");
   Hierarchy& H = *c->mg;
@@ -717,11 +730,18 @@ void mg_batch_coarse(Ctx* c, int nb) {
     mg_batch_systems(c, nb, sys);
     const LevelGeom& G1 = b.H.geo[1];
     const CoarseOp& C1 = b.H.cop[1];
-    const bool tc = b.p.coarse_impl == 0 || b.p.coarse_impl == 4;
+    // one launch for the group: the links read once for all systems.  Forced implementations: tensor
+    // cores (4, FP16 links), else the kernel that also takes systems of several lattices
+    const bool grouped = mg_batch_grouped(c, nb);
+    const bool tc = b.p.coarse_impl == 4;
     auto batched = [&]() {
       for (int q0 = 0; q0 < nb; q0 += gmax) {
         std::vector<CoarseSystem> part(sys.begin() + q0, sys.begin() + std::min(nb, q0 + gmax));
-        // tensor cores for FP16 links (the group's systems are consecutive vectors of this context)
+        if (grouped) {
+          coarse_gcr_group_solve(part, b.H.work[1].cg, restart, b.p.maxit_coarse, c->ws.flags.as<int>(), b.s);
+          continue;
+        }
+        // the group's systems are consecutive vectors of this context
         if (tc && coarse_gcr_tc_try(part, b.H.work[1].cg, restart, b.p.maxit_coarse, c->ws.flags.as<int>(), b.s))
           continue;
         coarse_gcr_solve_multi(part, b.H.work[1].cg, restart, b.p.maxit_coarse, c->ws.flags.as<int>(), b.s);
@@ -740,7 +760,7 @@ void mg_batch_coarse(Ctx* c, int nb) {
         long long* d_it = b.H.d_iters.as<long long>();
         DBuf keep(sizeof(long long) * MG_MAX_LEVELS);
         MG_CUDA(cudaMemcpyAsync(keep.get(), d_it, sizeof(long long) * MG_MAX_LEVELS, cudaMemcpyDeviceToDevice, b.s));
-        choice = tuned_block(TuneKey{"coarse_batch", {G1.L[0], G1.L[1], G1.L[2], G1.L[3]}, nb, C1.store}, {0, 1},
+        choice = tuned_block(TuneKey{"coarse_group", {G1.L[0], G1.L[1], G1.L[2], G1.L[3]}, nb, C1.store}, {0, 1},
                              [&](int which) {
                                if (which)
                                  one_by_one();
