@@ -352,8 +352,10 @@ template <typename T>
 void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double* psi_abi, int kind) {
   const Geom& g = c->g;
   const size_t half = 24 * c->Vh;   // reals per half vector
-  DBuf vec(sizeof(T) * 4 * half);
-  DBuf W(sizeof(T) * 2 * 6 * 9 * c->V);
+  DBuf& vec = c->force_vec;
+  DBuf& W = c->force_W;
+  if (vec.bytes() < sizeof(T) * 4 * half) vec.alloc(sizeof(T) * 4 * half);
+  if (W.bytes() < sizeof(T) * 2 * 6 * 9 * c->V) W.alloc(sizeof(T) * 2 * 6 * 9 * c->V);
   T* lam_e = vec.as<T>();
   T* lam_o = lam_e + half;
   T* psi_e = lam_o + half;
@@ -368,8 +370,7 @@ void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double*
   MG_LAUNCH();
   k_force_links<T><<<dim3(nb, 4), bs, 0, c->stream>>>(g, lam_e, lam_o, psi_e, psi_o, c->gauge<T>(), W.as<V2>(), kind,
                                                       (double2*)out_abi);
-  MG_LAUNCH();
-  c->sync();
+  MG_LAUNCH();   // the caller waits for the stream
 }
 
 void gauge_force(Ctx* c, double* out_abi, const double* lam_abi, const double* psi_abi, int kind) {

@@ -245,11 +245,14 @@ struct Ctx {
   mg_params params{};
   bool have_params = false;
   std::shared_ptr<Hierarchy> mg;         // null until mg_setup (shared_ptr: Hierarchy is incomplete here)
-  std::vector<std::vector<double>> injected;  // per transfer: injected raw null vectors (host, complex128)
-  std::vector<int> injected_nv;
+  // null vectors that replace the inverse iteration of a transfer: as given by the caller
+  // (host, complex128), or kept on the device from an earlier hierarchy (FP32, level layout)
+  std::vector<std::vector<double>> injected;
+  std::vector<std::shared_ptr<DBuf>> injected_dev;
 
-  // host I/O staging
-  DBuf stage_in, stage_out;              // complex128 whole-lattice staging
+  DBuf dagger_src;                       // gamma_5-rotated copy of a device source (adjoint solves)
+  DBuf force_vec, force_W;               // mg_force: packed vectors, insertions
+  std::shared_ptr<void> apply_work;      // mg_apply's buffers (api.cu), kept between calls
   long long dslash_launches = 0;
   // mg_params.level_timing: CUDA event pairs around each level's work, per level
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> level_events[MG_MAX_LEVELS];
@@ -303,6 +306,7 @@ struct FineOps {
   DBuf t1, t2;
   explicit FineOps(Ctx* ctx);
   size_t half_n() const { return 12 * c->Vh; }
+  size_t bytes() const { return t1.bytes() + t2.bytes() + m1.bytes() + m2.bytes(); }
   // D_r y = y - H_eo A_o^{-1} H_oe A_e^{-1} y
   void Dr(T* out_e, const T* in_e);
   // b_r = b_e - H_eo A_o^{-1} b_o
@@ -460,6 +464,8 @@ bool mg_batch_grouped(Ctx* c, int nb);
 void mg_cycle_batch(Ctx* c, double* out_abi, const double* in_abi, int nb);
 void mg_apply_level(Ctx* c, int op, int level, double* out_abi, const double* in_abi);
 void mg_get_vectors(Ctx* c, int level, double* V_abi, int nv);
+// the raw null vectors of every transfer of the current setup, as they lie on the device
+std::vector<std::shared_ptr<DBuf>> mg_keep_vectors(Ctx* c);
 // relaxes the null vectors of transfer `level` with the current solver (multigrid.cu)
 void mg_relax_null_vectors(Ctx* c, int level, int relax);
 // dequantised coarse links of level >= 1 (ABI layouts, see mg_get_coarse_links)

@@ -132,7 +132,8 @@ struct Hierarchy {
   std::vector<LevelGeom> geo;
   std::vector<CoarseOp> cop;
   std::vector<TransferOp> tr;
-  std::vector<DBuf> nullvecs;
+  // shared with Ctx::injected_dev when a rebuild keeps the vectors (cloned before they are changed)
+  std::vector<std::shared_ptr<DBuf>> nullvecs;
   std::vector<LevelWork> work;
   std::unique_ptr<FineOps<float>> F32;
   std::vector<long long> iters;
@@ -379,7 +380,15 @@ void find_null_vectors(Ctx* c, Hierarchy& H, int l, mg_setup_info* info) {
   const int nv = p.nv[l];
   const size_t n = full_n(H, l);
   cudaStream_t s = c->stream;
-  float* base = H.nullvecs[l].as<float>();
+  const size_t bytes = sizeof(float) * 2 * n * nv;
+  if (l < (int)c->injected_dev.size() && c->injected_dev[l] && c->injected_dev[l]->bytes() == bytes) {
+    H.nullvecs[l] = c->injected_dev[l];   // kept from an earlier hierarchy of this context
+    if (info) info->vectors[l] = nv;
+    return;
+  }
+  H.nullvecs[l] = std::make_shared<DBuf>(bytes);
+  float* base = H.nullvecs[l]->as<float>();
+  MG_CUDA(cudaMemset(base, 0, bytes));
   std::vector<const float*> found(nv);
   for (int k = 0; k < nv; k++) found[k] = base + (size_t)k * 2 * n;
   if (l < (int)c->injected.size() && !c->injected[l].empty()) {
@@ -625,12 +634,9 @@ void mg_build(Ctx* c, mg_setup_info* info) {
     const size_t esz = T.store == STORE_F32 ? sizeof(float2) : 4;
     T.P.alloc(esz * (size_t)T.ncoarse * T.nb * T.fine_ndof * T.nv);
     T.Pscale.alloc(sizeof(float) * 2 * (size_t)T.ncoarse);
-    H->nullvecs[l].alloc(sizeof(float) * 2 * full_n(*H, l) * T.nv);
-    MG_CUDA(cudaMemset(H->nullvecs[l].get(), 0, sizeof(float) * 2 * full_n(*H, l) * T.nv));
-
     find_null_vectors(c, *H, l, info);
     std::vector<const float*> V(T.nv);
-    for (int k = 0; k < T.nv; k++) V[k] = H->nullvecs[l].as<float>() + (size_t)k * 2 * full_n(*H, l);
+    for (int k = 0; k < T.nv; k++) V[k] = H->nullvecs[l]->as<float>() + (size_t)k * 2 * full_n(*H, l);
     block_orthonormalize(T, V.data(), H->gs_scratch, c->ws.flags.as<int>(), c->stream);
     if (c->read_flag(FLAG_GS_BREAKDOWN, true)) raise(MG_ERR_GS_BREAKDOWN, "block Gram-Schmidt breakdown");
     build_coarse_links(c, *H, l);
@@ -1074,7 +1080,12 @@ void mg_relax_null_vectors(Ctx* c, int level, int relax) {
   float* se = sb.as<float>();
   double* scr = c->ws.scalars.as<double>() + 1024;
   const int nv = H.tr[l].nv;
-  float* base = H.nullvecs[l].as<float>();
+  if (H.nullvecs[l].use_count() > 1) {   // also held for the next setup: change a copy
+    std::shared_ptr<DBuf> own = std::make_shared<DBuf>(H.nullvecs[l]->bytes());
+    MG_CUDA(cudaMemcpyAsync(own->get(), H.nullvecs[l]->get(), own->bytes(), cudaMemcpyDeviceToDevice, s));
+    H.nullvecs[l] = own;
+  }
+  float* base = H.nullvecs[l]->as<float>();
   std::vector<const float*> prev(nv);
   for (int k = 0; k < nv; k++) prev[k] = base + (size_t)k * 2 * nf;
   // inverse subspace iteration with the current solver of the level as the
@@ -1114,13 +1125,18 @@ void mg_relax_null_vectors(Ctx* c, int level, int relax) {
   c->sync();
 }
 
+std::vector<std::shared_ptr<DBuf>> mg_keep_vectors(Ctx* c) {
+  if (!c->mg) raise(MG_ERR_STATE, "multigrid not set up");
+  return c->mg->nullvecs;
+}
+
 void mg_get_vectors(Ctx* c, int level, double* V_abi, int nv) {
   if (!c->mg || level + 1 >= c->mg->L) raise(MG_ERR_STATE, "transfer not set up");
   Hierarchy& H = *c->mg;
   if (nv != H.tr[level].nv) raise(MG_ERR_NV, "nv does not match the setup");
   const size_t n = full_n(H, level);
   for (int k = 0; k < nv; k++) {
-    const float* v = H.nullvecs[level].as<float>() + (size_t)k * 2 * n;
+    const float* v = H.nullvecs[level]->as<float>() + (size_t)k * 2 * n;
     if (level == 0)
       unpack_spinor(c->g, v, v + 24 * c->Vh, true, V_abi + (size_t)k * 2 * n, c->stream);
     else
