@@ -753,13 +753,13 @@ int mg_apply(void* ctx, int op, int level, void* out, const void* in, int nrhs, 
       ApplyWork& aw = *static_cast<ApplyWork*>(c->apply_work.get());
       grow(aw.in, es * 2 * half * nrhs);
       grow(aw.out, es * 2 * half * nrhs);
-      MG_CUDA(cudaMemsetAsync(aw.out.get(), 0, es * 2 * half * nrhs, c->stream));
       char* ie = aw.in.as<char>();
       char* io = ie + es * half * nrhs;
       char* oe = aw.out.as<char>();
       char* oo = oe + es * half * nrhs;
-      for (int r = 0; r < nrhs; r++)
-        mg::pack_spinor(c->g, si.ptr + (size_t)r * 2 * nin, ie + es * half * r, io + es * half * r, f32, c->stream);
+      // D_r and its adjoint read the even sites only; they and b_r write the even sites and zeros
+      const bool reads_even = op == MG_OP_DR || op == MG_OP_DR_DAG, writes_even = reads_even || op == MG_OP_BR;
+      mg::pack_spinors(c->g, nrhs, si.ptr, ie, io, half, reads_even, f32, c->stream);
       auto run = [&](auto* tag) {
         using T = std::remove_pointer_t<decltype(tag)>;
         mg::FineOps<T>& F = aw.ops<T>(c);
@@ -797,8 +797,7 @@ int mg_apply(void* ctx, int op, int level, void* out, const void* in, int nrhs, 
         run((float*)nullptr);
       else
         run((double*)nullptr);
-      for (int r = 0; r < nrhs; r++)
-        mg::unpack_spinor(c->g, oe + es * half * r, oo + es * half * r, f32, so.ptr + (size_t)r * 2 * nout, c->stream);
+      mg::unpack_spinors(c->g, nrhs, oe, oo, half, writes_even, f32, so.ptr, c->stream);
       if (aw.bytes() > kApplyKeep) {
         c->sync();
         c->apply_work.reset();

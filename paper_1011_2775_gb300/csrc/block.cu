@@ -215,9 +215,7 @@ int solve_runs(std::vector<Run>& runs, double tol) {
   for (Run& R : runs) {
     BlockBuffers& B = *R.B;
     Ctx* c = R.c;
-    for (int q = 0; q < R.nb; q++)
-      pack_spinor(c->g, R.eta + (size_t)q * 24 * c->V, B.be.as<double>() + q * R.hs, B.bo.as<double>() + q * R.hs,
-                  false, c->stream);
+    pack_spinors(c->g, R.nb, R.eta, B.be.as<double>(), B.bo.as<double>(), R.hs, false, false, c->stream);
     read_norms(R, B.be.as<double>(), B.bo.as<double>(), std::vector<char>(R.nb, 1));
     for (int q = 0; q < R.nb; q++) {
       R.bnorm[q] = std::sqrt(R.h[2 * q] + R.h[2 * q + 1]);

@@ -162,13 +162,37 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, uns
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  for (int r = wid; r < NR; r += W) {
-    double s = 0.0;
-#pragma unroll 4
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(&partials[(size_t)r * gridDim.x + b]);
+  if constexpr (NR <= 4) {   // every thread takes blocks, all values in flight together
+    __shared__ double fin[NR][W];
+    double s[NR];
 #pragma unroll
-    for (int o = 16; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[r] = s;
+    for (int r = 0; r < NR; r++) s[r] = 0.0;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += THREADS)
+#pragma unroll
+      for (int r = 0; r < NR; r++) s[r] += __ldcg(&partials[(size_t)r * gridDim.x + b]);
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+#pragma unroll
+      for (int o = 16; o >= 1; o /= 2) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+      if (lane == 0) fin[r][wid] = s[r];
+    }
+    __syncthreads();
+    if (threadIdx.x < NR) {
+      double t = fin[threadIdx.x][0];
+#pragma unroll
+      for (int w = 1; w < W; w++) t += fin[threadIdx.x][w];
+      out[threadIdx.x] = t;
+    }
+  } else {
+    for (int r = wid; r < NR; r += W) {
+      double s = 0.0;
+#pragma unroll 8
+      for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(&partials[(size_t)r * gridDim.x + b]);
+#pragma unroll
+      for (int o = 16; o >= 1; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) out[r] = s;
+    }
   }
   if (threadIdx.x == 0) *counter = 0u;
 }

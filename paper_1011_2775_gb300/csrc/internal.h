@@ -118,6 +118,15 @@ enum Epilogue { EPI_H = 0, EPI_CH = 1, EPI_XPAY = 2, EPI_CX_PAY = 3, EPI_C_XPAY 
 //  EPI_CX_PAY: out = C x + a H in
 //  EPI_C_XPAY: out = C (x + a H in)
 
+// threads per CTA of the one-site-per-thread kernels (wilson.cu)
+int site_block(long long sites);
+// nrhs consecutive ABI vectors to and from packed half vectors `stride`
+// elements apart, one launch; even_only: odd sites are not read, zero_odd: odd
+// sites are written as zero
+void pack_spinors(const Geom& g, int nrhs, const double* abi, void* even, void* odd, size_t stride, bool even_only,
+                  bool fp32, cudaStream_t s);
+void unpack_spinors(const Geom& g, int nrhs, const void* even, const void* odd, size_t stride, bool zero_odd, bool fp32,
+                    double* abi, cudaStream_t s);
 void pack_spinor(const Geom& g, const double* abi, void* even, void* odd, bool fp32, cudaStream_t s);
 void unpack_spinor(const Geom& g, const void* even, const void* odd, bool fp32, double* abi, cudaStream_t s);
 void pack_gauge(const Geom& g, const double* abi, double* g64, float* g32, cudaStream_t s);
@@ -132,6 +141,10 @@ void clover_apply(const Geom& g, T* out, const T* in, const T* clov, cudaStream_
 template <typename T>
 void dslash(const Geom& g, Epilogue epi, int parity, T* out, const T* in, const T* gauge, const T* clov,
             const T* x, double a, int dirmask, cudaStream_t s);
+// both parities of out = epi(H in) in one launch (operands indexed e, o by output parity)
+template <typename T>
+void dslash_full(const Geom& g, Epilogue epi, T* oe, T* oo, const T* ie, const T* io, const T* gauge, const T* ce,
+                 const T* co, const T* xe, const T* xo, double a, cudaStream_t s);
 // nrhs right-hand sides at `stride` elements of T apart (out, in and x alike),
 // one launch; `config` = (right-hand sides per thread) * 1000 + CTA size, one
 // of dslash_mrhs_configs()

@@ -132,8 +132,7 @@ void FineOps<T>::reconstruct(T* x_e, T* x_o, const T* y_e, const T* b_o) {
 template <typename T>
 void FineOps<T>::D(T* oe, T* oo, const T* ie, const T* io) {
   const Geom& g = c->g;
-  dslash<T>(g, EPI_CX_PAY, 0, oe, io, c->gauge<T>(), c->A<T>(0), ie, 1.0, 0xff, c->stream);
-  dslash<T>(g, EPI_CX_PAY, 1, oo, ie, c->gauge<T>(), c->A<T>(1), io, 1.0, 0xff, c->stream);
+  dslash_full<T>(g, EPI_CX_PAY, oe, oo, ie, io, c->gauge<T>(), c->A<T>(0), c->A<T>(1), ie, io, 1.0, c->stream);
   c->dslash_launches += 2;
 }
 
@@ -144,16 +143,14 @@ void FineOps<T>::Dp(T* oe, T* oo, const T* ie, const T* io) {
   T* so = t2.as<T>();
   clover_apply<T>(g, se, ie, c->Ainv<T>(0), c->stream);
   clover_apply<T>(g, so, io, c->Ainv<T>(1), c->stream);
-  dslash<T>(g, EPI_XPAY, 0, oe, so, c->gauge<T>(), nullptr, ie, 1.0, 0xff, c->stream);
-  dslash<T>(g, EPI_XPAY, 1, oo, se, c->gauge<T>(), nullptr, io, 1.0, 0xff, c->stream);
+  dslash_full<T>(g, EPI_XPAY, oe, oo, se, so, c->gauge<T>(), nullptr, nullptr, ie, io, 1.0, c->stream);
   c->dslash_launches += 2;
 }
 
 template <typename T>
 void FineOps<T>::H(T* oe, T* oo, const T* ie, const T* io) {
   const Geom& g = c->g;
-  dslash<T>(g, EPI_H, 0, oe, io, c->gauge<T>(), nullptr, nullptr, 0.0, 0xff, c->stream);
-  dslash<T>(g, EPI_H, 1, oo, ie, c->gauge<T>(), nullptr, nullptr, 0.0, 0xff, c->stream);
+  dslash_full<T>(g, EPI_H, oe, oo, ie, io, c->gauge<T>(), nullptr, nullptr, nullptr, nullptr, 0.0, c->stream);
   c->dslash_launches += 2;
 }
 

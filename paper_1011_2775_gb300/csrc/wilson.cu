@@ -81,8 +81,10 @@ void upload_sigma() {
 }  // namespace
 
 // --------------------------------------------------------------------------- packing
+// nrhs ABI vectors (blockIdx.y) to packed half vectors `stride` elements of T
+// apart; even_only: the odd sites are not read.
 template <typename T>
-__global__ void k_pack_spinor(Geom g, const double2* __restrict__ abi, T* even, T* odd) {
+__global__ void k_pack_spinor(Geom g, const double2* __restrict__ abi, T* even, T* odd, size_t stride, int even_only) {
   const int lex = blockIdx.x * blockDim.x + threadIdx.x;
   if (lex >= 2 * g.Vh) return;
   int c[4];
@@ -91,48 +93,81 @@ __global__ void k_pack_spinor(Geom g, const double2* __restrict__ abi, T* even, 
   c[1] = r % g.L[1]; r /= g.L[1];
   c[2] = r % g.L[2]; c[3] = r / g.L[2];
   const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
+  if (par && even_only) return;
   const int cb = lex >> 1;
+  abi += (size_t)blockIdx.y * 24 * g.Vh;
   cx<T> s[12];
 #pragma unroll
   for (int k = 0; k < 12; k++) {
     double2 v = abi[(size_t)lex * 12 + k];
     s[k] = mkc<T>((T)v.x, (T)v.y);
   }
-  SpinorIO<T>::store(par ? odd : even, g.Vh, cb, s);
+  SpinorIO<T>::store((par ? odd : even) + blockIdx.y * stride, g.Vh, cb, s);
 }
 
+// Packed half vectors to ABI vectors; zero_odd: the odd sites become zero and
+// `odd` is not read.  A site's 192 bytes are gathered in shared memory and
+// written as one contiguous span per CTA: stored straight from the threads (16
+// bytes at a stride of 192) the writes reached 2.2 of 6.7 TB/s.
+constexpr int kUnpack = 128;   // sites per CTA; rows padded to 13 double2 against bank conflicts
 template <typename T>
-__global__ void k_unpack_spinor(Geom g, const T* even, const T* odd, double2* __restrict__ abi) {
-  const int lex = blockIdx.x * blockDim.x + threadIdx.x;
-  if (lex >= 2 * g.Vh) return;
-  int c[4];
-  int r = lex;
-  c[0] = r % g.L[0]; r /= g.L[0];
-  c[1] = r % g.L[1]; r /= g.L[1];
-  c[2] = r % g.L[2]; c[3] = r / g.L[2];
-  const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
-  cx<T> s[12];
-  SpinorIO<T>::load(par ? odd : even, g.Vh, lex >> 1, s);
+__global__ void __launch_bounds__(kUnpack) k_unpack_spinor(Geom g, const T* __restrict__ even,
+                                                           const T* __restrict__ odd, double2* __restrict__ abi,
+                                                           size_t stride, int zero_odd) {
+  __shared__ double2 sm[kUnpack * 13];
+  const int lex0 = blockIdx.x * kUnpack, lex = lex0 + threadIdx.x;
+  if (lex < 2 * g.Vh) {
+    int c[4];
+    int r = lex;
+    c[0] = r % g.L[0]; r /= g.L[0];
+    c[1] = r % g.L[1]; r /= g.L[1];
+    c[2] = r % g.L[2]; c[3] = r / g.L[2];
+    const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
+    cx<T> s[12];
+    if (par && zero_odd) {
 #pragma unroll
-  for (int k = 0; k < 12; k++) abi[(size_t)lex * 12 + k] = make_double2((double)s[k].re, (double)s[k].im);
+      for (int k = 0; k < 12; k++) s[k] = mkc<T>(0, 0);
+    } else {
+      SpinorIO<T>::load((par ? odd : even) + blockIdx.y * stride, g.Vh, lex >> 1, s);
+    }
+#pragma unroll
+    for (int k = 0; k < 12; k++) sm[threadIdx.x * 13 + k] = make_double2((double)s[k].re, (double)s[k].im);
+  }
+  __syncthreads();
+  const int n = 12 * min(kUnpack, 2 * g.Vh - lex0);
+  double2* dst = abi + (size_t)blockIdx.y * 24 * g.Vh + (size_t)lex0 * 12;
+  for (int t = threadIdx.x; t < n; t += kUnpack) dst[t] = sm[(t / 12) * 13 + t % 12];
+}
+
+void pack_spinors(const Geom& g, int nrhs, const double* abi, void* even, void* odd, size_t stride, bool even_only,
+                  bool fp32, cudaStream_t s) {
+  const int bs = 128;
+  const dim3 grid((2 * g.Vh + bs - 1) / bs, nrhs);
+  if (fp32)
+    k_pack_spinor<float><<<grid, bs, 0, s>>>(g, (const double2*)abi, (float*)even, (float*)odd, stride, even_only);
+  else
+    k_pack_spinor<double><<<grid, bs, 0, s>>>(g, (const double2*)abi, (double*)even, (double*)odd, stride, even_only);
+  MG_LAUNCH();
+}
+
+void unpack_spinors(const Geom& g, int nrhs, const void* even, const void* odd, size_t stride, bool zero_odd, bool fp32,
+                    double* abi, cudaStream_t s) {
+  const dim3 grid((2 * g.Vh + kUnpack - 1) / kUnpack, nrhs);
+  if (fp32)
+    k_unpack_spinor<float><<<grid, kUnpack, 0, s>>>(g, (const float*)even, (const float*)odd, (double2*)abi, stride,
+                                                    zero_odd);
+  else
+    k_unpack_spinor<double><<<grid, kUnpack, 0, s>>>(g, (const double*)even, (const double*)odd, (double2*)abi, stride,
+                                                     zero_odd);
+  MG_LAUNCH();
 }
 
 void pack_spinor(const Geom& g, const double* abi, void* even, void* odd, bool fp32, cudaStream_t s) {
-  const int n = 2 * g.Vh, bs = 128;
-  if (fp32)
-    k_pack_spinor<float><<<(n + bs - 1) / bs, bs, 0, s>>>(g, (const double2*)abi, (float*)even, (float*)odd);
-  else
-    k_pack_spinor<double><<<(n + bs - 1) / bs, bs, 0, s>>>(g, (const double2*)abi, (double*)even, (double*)odd);
-  MG_LAUNCH();
+  pack_spinors(g, 1, abi, even, odd, 0, false, fp32, s);
 }
 
 void unpack_spinor(const Geom& g, const void* even, const void* odd, bool fp32, double* abi, cudaStream_t s) {
-  const int n = 2 * g.Vh, bs = 128;
-  if (fp32)
-    k_unpack_spinor<float><<<(n + bs - 1) / bs, bs, 0, s>>>(g, (const float*)even, (const float*)odd, (double2*)abi);
-  else
-    k_unpack_spinor<double><<<(n + bs - 1) / bs, bs, 0, s>>>(g, (const double*)even, (const double*)odd, (double2*)abi);
-  MG_LAUNCH();
+  unpack_spinors(g, 1, even, odd, 0, false, fp32, abi, s);
 }
 
 __global__ void k_pack_gauge(Geom g, const double2* __restrict__ abi, double2* g64, float2* g32) {
@@ -378,7 +413,7 @@ __global__ void k_clover_apply(Geom g, T* out, const T* __restrict__ in, const T
 
 template <typename T>
 void clover_apply(const Geom& g, T* out, const T* in, const T* clov, cudaStream_t s) {
-  const int bs = 128;
+  const int bs = site_block(g.Vh);
   k_clover_apply<T><<<(g.Vh + bs - 1) / bs, bs, 0, s>>>(g, out, in, clov);
   MG_LAUNCH();
 }
@@ -430,13 +465,23 @@ __device__ __forceinline__ void dslash_site(const Geom& g, int par, int i, T* ou
   SpinorIO<T>::store(out, g.Vh, i, res);
 }
 
+// Operands of the output parities par0 + blockIdx.y, indexed by parity (`in`
+// is the half of the other parity).
+template <typename T>
+struct HalfArgs {
+  T* out[2];
+  const T* in[2];
+  const T* clov[2];
+  const T* x[2];
+};
 template <typename T, int EPI>
-__global__ void __launch_bounds__(128) k_dslash(Geom g, int par, T* out, const T* __restrict__ in,
-                                                 const T* __restrict__ gauge, const T* __restrict__ clov,
-                                                 const T* __restrict__ x, T a, int dirmask) {
+__global__ void __launch_bounds__(128) k_dslash(Geom g, int par0, HalfArgs<T> h, const T* __restrict__ gauge, T a,
+                                                int dirmask) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.Vh) return;
-  dslash_site<T, EPI>(g, par, i, out, in, gauge, clov, x, a, dirmask);
+  const int par = par0 + blockIdx.y;
+  dslash_site<T, EPI>(g, par, i, par ? h.out[1] : h.out[0], par ? h.in[1] : h.in[0], gauge,
+                      par ? h.clov[1] : h.clov[0], par ? h.x[1] : h.x[0], a, dirmask);
 }
 
 // The epilogues of the multi-RHS kernels for the nr <= NR right-hand sides
@@ -512,20 +557,46 @@ __global__ void __launch_bounds__(BS, MINB) k_dslash_mrhs(Geom g, int par, int n
   mrhs_epilogue<T, EPI, NR>(g, i, acc, nr, r0, stride, out, clov, x, a);
 }
 
+// Threads per CTA of the one-site-per-thread kernels for `ctas128` CTAs of 128
+// sites: the largest of 128, 64, 32 that gives every SM about six CTAs or more
+// (below that the last wave leaves SMs idle: 65536 sites in CTAs of 128 are 3.4
+// per SM, so some SMs take 4 and some 3; 4096 sites used 32 of 152 SMs, and in
+// FP64 a busy SM then runs at its FP64 rate while the others idle: 45 us for
+// 960 sites).
+int site_block(long long sites) { return sites >= 128 * 152 * 6 ? 128 : sites >= 64 * 152 * 6 ? 64 : 32; }
+
 template <typename T>
-void dslash(const Geom& g, Epilogue epi, int parity, T* out, const T* in, const T* gauge, const T* clov, const T* x,
-            double a, int dirmask, cudaStream_t s) {
-  const int bs = 128;
-  const int nb = (g.Vh + bs - 1) / bs;
+void dslash_halves(const Geom& g, Epilogue epi, int par0, int npar, const HalfArgs<T>& h, const T* gauge, double a,
+                   int dirmask, cudaStream_t s) {
+  const int bs = site_block((long long)g.Vh * npar);
+  const dim3 nb((g.Vh + bs - 1) / bs, npar);
   switch (epi) {
-    case EPI_H: k_dslash<T, EPI_H><<<nb, bs, 0, s>>>(g, parity, out, in, gauge, clov, x, (T)a, dirmask); break;
-    case EPI_CH: k_dslash<T, EPI_CH><<<nb, bs, 0, s>>>(g, parity, out, in, gauge, clov, x, (T)a, dirmask); break;
-    case EPI_XPAY: k_dslash<T, EPI_XPAY><<<nb, bs, 0, s>>>(g, parity, out, in, gauge, clov, x, (T)a, dirmask); break;
-    case EPI_CX_PAY: k_dslash<T, EPI_CX_PAY><<<nb, bs, 0, s>>>(g, parity, out, in, gauge, clov, x, (T)a, dirmask); break;
-    case EPI_C_XPAY: k_dslash<T, EPI_C_XPAY><<<nb, bs, 0, s>>>(g, parity, out, in, gauge, clov, x, (T)a, dirmask); break;
+    case EPI_H: k_dslash<T, EPI_H><<<nb, bs, 0, s>>>(g, par0, h, gauge, (T)a, dirmask); break;
+    case EPI_CH: k_dslash<T, EPI_CH><<<nb, bs, 0, s>>>(g, par0, h, gauge, (T)a, dirmask); break;
+    case EPI_XPAY: k_dslash<T, EPI_XPAY><<<nb, bs, 0, s>>>(g, par0, h, gauge, (T)a, dirmask); break;
+    case EPI_CX_PAY: k_dslash<T, EPI_CX_PAY><<<nb, bs, 0, s>>>(g, par0, h, gauge, (T)a, dirmask); break;
+    case EPI_C_XPAY: k_dslash<T, EPI_C_XPAY><<<nb, bs, 0, s>>>(g, par0, h, gauge, (T)a, dirmask); break;
   }
   MG_LAUNCH();
 }
+
+template <typename T>
+void dslash(const Geom& g, Epilogue epi, int parity, T* out, const T* in, const T* gauge, const T* clov, const T* x,
+            double a, int dirmask, cudaStream_t s) {
+  HalfArgs<T> h{{out, out}, {in, in}, {clov, clov}, {x, x}};
+  dslash_halves<T>(g, epi, parity, 1, h, gauge, a, dirmask, s);
+}
+
+template <typename T>
+void dslash_full(const Geom& g, Epilogue epi, T* oe, T* oo, const T* ie, const T* io, const T* gauge, const T* ce,
+                 const T* co, const T* xe, const T* xo, double a, cudaStream_t s) {
+  HalfArgs<T> h{{oe, oo}, {io, ie}, {ce, co}, {xe, xo}};
+  dslash_halves<T>(g, epi, 0, 2, h, gauge, a, 0xff, s);
+}
+template void dslash_full<float>(const Geom&, Epilogue, float*, float*, const float*, const float*, const float*,
+                                 const float*, const float*, const float*, const float*, double, cudaStream_t);
+template void dslash_full<double>(const Geom&, Epilogue, double*, double*, const double*, const double*, const double*,
+                                  const double*, const double*, const double*, const double*, double, cudaStream_t);
 template void dslash<float>(const Geom&, Epilogue, int, float*, const float*, const float*, const float*,
                             const float*, double, int, cudaStream_t);
 template void dslash<double>(const Geom&, Epilogue, int, double*, const double*, const double*, const double*,
