@@ -264,7 +264,7 @@ struct Ctx {
   std::vector<std::shared_ptr<DBuf>> injected_dev;
 
   DBuf dagger_src;                       // gamma_5-rotated copy of a device source (adjoint solves)
-  DBuf force_vec, force_W;               // mg_force: packed vectors, insertions
+  DBuf force_vec, force_W, force_R;      // mg_force: packed vectors, insertions, plaquette contributions
   std::shared_ptr<void> apply_work;      // mg_apply's buffers (api.cu), kept between calls
   long long dslash_launches = 0;
   // mg_params.level_timing: CUDA event pairs around each level's work, per level
