@@ -205,10 +205,10 @@ __global__ void k_mr_update_multi(cx<T>* e, cx<T>* r, const cx<T>* __restrict__ 
   const T ar = s_al[0], ai = s_al[1];
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> rv = r[i], wv = w[i], ev = e[i];
-    ev.re += ar * rv.re - ai * rv.im;
-    ev.im += ar * rv.im + ai * rv.re;
-    rv.re -= ar * wv.re - ai * wv.im;
-    rv.im -= ar * wv.im + ai * wv.re;
+    ev.re = fma(ar, rv.re, fma(-ai, rv.im, ev.re));
+    ev.im = fma(ar, rv.im, fma(ai, rv.re, ev.im));
+    rv.re = fma(-ar, wv.re, fma(ai, wv.im, rv.re));
+    rv.im = fma(-ar, wv.im, fma(-ai, wv.re, rv.im));
     e[i] = ev;
     r[i] = rv;
   }
@@ -304,8 +304,8 @@ __global__ void k_orth_update(cx<T>* w, VecPtrs<T> V, const double* __restrict__
 #pragma unroll
     for (int j = 0; j < K; j++) {
       cx<T> q = V.p[j][i];
-      a.re -= br[j] * q.re - bi[j] * q.im;
-      a.im -= br[j] * q.im + bi[j] * q.re;
+      a.re = fma(-br[j], q.re, fma(bi[j], q.im, a.re));   // four operations; written as a -= b q the compiler takes six
+      a.im = fma(-br[j], q.im, fma(-bi[j], q.re, a.im));
     }
     if (K > 0) w[i] = a;
     if (RED) {
@@ -397,8 +397,8 @@ __global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restric
     q.im *= ig;
     w[i] = q;
     cx<T> b = r[i];
-    b.re -= a_r * q.re - a_i * q.im;
-    b.im -= a_r * q.im + a_i * q.re;
+    b.re = fma(-a_r, q.re, fma(a_i, q.im, b.re));
+    b.im = fma(-a_r, q.im, fma(-a_i, q.re, b.im));
     r[i] = b;
     s = fma((acc_t<T>)b.re, (acc_t<T>)b.re, s);
     s = fma((acc_t<T>)b.im, (acc_t<T>)b.im, s);
@@ -455,9 +455,10 @@ __global__ void k_lincomb(cx<T>* x, VecPtrs<TZ> Z, const double* __restrict__ c,
       double re = (double)a.re, im = (double)a.im;
 #pragma unroll
       for (int j = 0; j < K; j++) {
-        cx<TZ> z = Z.p[j][i];
-        re += cr[j] * (double)z.re - ci[j] * (double)z.im;
-        im += cr[j] * (double)z.im + ci[j] * (double)z.re;
+        const cx<TZ> z = Z.p[j][i];
+        const double zr = (double)z.re, zi = (double)z.im;
+        re = fma(cr[j], zr, fma(-ci[j], zi, re));
+        im = fma(cr[j], zi, fma(ci[j], zr, im));
       }
       x[i] = mkc<T>((T)re, (T)im);
     }
@@ -516,10 +517,10 @@ __global__ void k_mr_update(cx<T>* e, cx<T>* r, const cx<T>* __restrict__ w, con
   const T ar = s_al[0], ai = s_al[1];
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
     cx<T> rv = r[i], wv = w[i], ev = e[i];
-    ev.re += ar * rv.re - ai * rv.im;
-    ev.im += ar * rv.im + ai * rv.re;
-    rv.re -= ar * wv.re - ai * wv.im;
-    rv.im -= ar * wv.im + ai * wv.re;
+    ev.re = fma(ar, rv.re, fma(-ai, rv.im, ev.re));
+    ev.im = fma(ar, rv.im, fma(ai, rv.re, ev.im));
+    rv.re = fma(-ar, wv.re, fma(ai, wv.im, rv.re));
+    rv.im = fma(-ar, wv.im, fma(-ai, wv.re, rv.im));
     e[i] = ev;
     r[i] = rv;
   }
