@@ -57,6 +57,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRestart = 64;
 constexpr int kMaxSys = 16;
 constexpr int kRows = 4;
+constexpr int kDeep = 6;   // link steps in flight with one system
 // reduction slots of a system: <w_j, w> (2 per j), then ||w||^2, Re and Im
 // <w, r>, the norm of a right-hand side or true residual, the exact
 // ||w''||^2, Re and Im <w'', r>
@@ -88,35 +89,33 @@ struct GArgs {
 
 // gathered vectors of `ns` sites from s0: gv[(site, p)][K] complex, times the
 // tile scale; nbd neighbours (8, or 9 with the site itself); in: element
-// (storage - base) nc of system p at in + p n
+// (storage - base) nc of system p at in + p n.  A warp takes one neighbour of
+// one site for all systems (lanes over its nc / 2 <= 32 pairs): no index
+// arithmetic per element, up to NS loads in flight per lane.
 template <int NS>
 __device__ void gather(const GArgs& a, size_t n, int store0, int s0, int ns, int nbd, int base, const float2* in,
                        const float* scale, float4* gv) {
-  const int nc = a.nc, hc = nc >> 1, K2 = nbd * hc;
-  const int total = ns * NS * K2;
-  constexpr int U = 8;   // loads in flight per thread
-  for (int t0 = threadIdx.x; t0 < total; t0 += U * kThreads) {
-    const float4* src[U];
-    float sc[U];
+  const int hc = a.nc >> 1, K2 = nbd * hc;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t n2 = n >> 1;
+  for (int t = w; t < ns * nbd; t += kWarps) {
+    const int sl = t / nbd, d = t - sl * nbd, st = store0 + s0 + sl;
+    const int from = d < 8 ? a.nbr[(size_t)st * 8 + d] : st;
+    const float sc = scale && d < 8 ? scale[(size_t)st * 8 + d] : 1.f;
+    if (lane >= hc) continue;
+    const float4* src = reinterpret_cast<const float4*>(in) + (size_t)(from - base) * hc + lane;
+    float4* dst = gv + (size_t)sl * NS * K2 + d * hc + lane;
+    constexpr int U = NS < 12 ? NS : 12;
 #pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int t = t0 + u * kThreads;
-      const int tt = t < total ? t : 0;
-      const int sp = tt / K2, rem = tt - sp * K2, d = rem / hc, j = rem - d * hc;
-      const int sl = sp / NS, p = sp - sl * NS;
-      const int st = store0 + s0 + sl;
-      const int from = d < 8 ? a.nbr[(size_t)st * 8 + d] : st;
-      src[u] = p < a.nb && t < total ? reinterpret_cast<const float4*>(in + (size_t)p * n + (size_t)(from - base) * nc) + j
-                                     : nullptr;
-      sc[u] = scale && d < 8 ? scale[(size_t)st * 8 + d] : 1.f;
-    }
-    float4 v[U];
+    for (int p0 = 0; p0 < NS; p0 += U) {
+      float4 v[U];
 #pragma unroll
-    for (int u = 0; u < U; u++) v[u] = src[u] ? __ldcg(src[u]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < U; u++)
+        v[u] = p0 + u < a.nb ? __ldcg(src + (size_t)(p0 + u) * n2) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int t = t0 + u * kThreads;
-      if (t < total) gv[t] = make_float4(sc[u] * v[u].x, sc[u] * v[u].y, sc[u] * v[u].z, sc[u] * v[u].w);
+      for (int u = 0; u < U; u++)
+        if (p0 + u < NS)
+          dst[(size_t)(p0 + u) * K2] = make_float4(sc * v[u].x, sc * v[u].y, sc * v[u].z, sc * v[u].w);
     }
   }
   __syncthreads();
@@ -146,17 +145,10 @@ __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int 
 #pragma unroll
         for (int p = 0; p < NS; p++) acc[r][p][0] = acc[r][p][1] = 0.f;
       const float4* v = gv + (size_t)(s - s0) * NS * K2;
-      typename LinkPair<ST>::raw nx[kRows];
-#pragma unroll
-      for (int r = 0; r < kRows; r++) nx[r] = lane < K2 ? LinkPair<ST>::load(row[r], lane) : LinkPair<ST>::zero();
-      for (int q = lane; q < K2; q += 32) {
+      auto step = [&](const typename LinkPair<ST>::raw (&raw)[kRows], int q) {
         float4 l[kRows];
 #pragma unroll
-        for (int r = 0; r < kRows; r++) l[r] = LinkPair<ST>::decode(nx[r]);
-        if (q + 32 < K2) {
-#pragma unroll
-          for (int r = 0; r < kRows; r++) nx[r] = LinkPair<ST>::load(row[r], q + 32);
-        }
+        for (int r = 0; r < kRows; r++) l[r] = LinkPair<ST>::decode(raw[r]);
 #pragma unroll
         for (int p = 0; p < NS; p++) {
           const float4 x = v[p * K2 + q];
@@ -171,6 +163,34 @@ __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int 
             acc[r][p][0] = fmaf(-l[r].w, x.w, acc[r][p][0]);
             acc[r][p][1] = fmaf(l[r].w, x.z, acc[r][p][1]);
           }
+        }
+      };
+      if constexpr (NS == 1) {
+        // one system: bound by the links' way from L2, so a lane keeps up to
+        // kDeep steps of all rows in flight (98 KB per SM)
+        for (int q0 = lane; q0 < K2; q0 += 32 * kDeep) {
+          typename LinkPair<ST>::raw raw[kDeep][kRows];
+#pragma unroll
+          for (int u = 0; u < kDeep; u++)
+#pragma unroll
+            for (int r = 0; r < kRows; r++)
+              raw[u][r] = q0 + 32 * u < K2 ? LinkPair<ST>::load(row[r], q0 + 32 * u) : LinkPair<ST>::zero();
+#pragma unroll
+          for (int u = 0; u < kDeep; u++)
+            if (q0 + 32 * u < K2) step(raw[u], q0 + 32 * u);
+        }
+      } else {
+        typename LinkPair<ST>::raw cur[kRows], nx[kRows];
+#pragma unroll
+        for (int r = 0; r < kRows; r++) nx[r] = lane < K2 ? LinkPair<ST>::load(row[r], lane) : LinkPair<ST>::zero();
+        for (int q = lane; q < K2; q += 32) {
+#pragma unroll
+          for (int r = 0; r < kRows; r++) cur[r] = nx[r];
+          if (q + 32 < K2) {
+#pragma unroll
+            for (int r = 0; r < kRows; r++) nx[r] = LinkPair<ST>::load(row[r], q + 32);
+          }
+          step(cur, q);
         }
       }
       // value f = (r NS + p) 2 + {re, im}: 32 at a time (8 with one system)
@@ -266,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
   const size_t n = (size_t)a.rows_sites * nc;
   const int i0 = (int)((long long)bid * a.items / G), i1 = (int)((long long)(bid + 1) * a.items / G);
   const size_t E0 = item_elem(a, i0), E1 = i1 == a.items ? n : item_elem(a, i1);
-  const int E = (int)(E1 - E0);
+  const int E = (int)(E1 - E0), E2 = E >> 1;   // both ends are even: pairs of elements, 16-byte accesses
   unsigned target = 0;
   bool ok = true;
   auto Wk = [&](int k, int p) { return a.W + ((size_t)k * nb + p) * n + E0; };
@@ -359,29 +379,37 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
               a.W[((size_t)k * nb + p) * n + e] = u;
             })))
         break;
-      // <w_j, w> (a warp takes eight j of one system), ||w||^2 and <w, r>
-      const int groups = (k + 7) >> 3;
-      for (int task = wid; task < nb * (groups + 1); task += kWarps) {
+      // <w_j, w> (a warp takes eight j of one system, two elements per load), ||w||^2 and <w, r>
+      const int groups = max(1, (k + 7) >> 3);
+      for (int task = wid; task < nb * groups; task += kWarps) {
         const int p = task % nb, gi = task / nb;
         if (!((run >> p) & 1u)) continue;
-        const float2* wk = Wk(k, p);
-        if (gi < groups) {
-          const int j0 = 8 * gi;
-          float re[8], im[8];
+        const float4* wk = reinterpret_cast<const float4*>(Wk(k, p));
+        const float4* rp = reinterpret_cast<const float4*>(a.r + (size_t)p * n + E0);
+        const int j0 = 8 * gi;
+        float re[8], im[8], s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll
-          for (int u = 0; u < 8; u++) re[u] = im[u] = 0.f;
+        for (int u = 0; u < 8; u++) re[u] = im[u] = 0.f;
 #pragma unroll 2
-          for (int e = lane; e < E; e += 32) {
-            float2 q[8];
+        for (int e = lane; e < E2; e += 32) {
+          float4 q[8];
 #pragma unroll
-            for (int u = 0; u < 8; u++) q[u] = j0 + u < k ? __ldcg(Wk(j0 + u, p) + e) : make_float2(0.f, 0.f);
-            const float2 x = __ldcg(wk + e);
-#pragma unroll
-            for (int u = 0; u < 8; u++) {
-              re[u] = fmaf(q[u].x, x.x, fmaf(q[u].y, x.y, re[u]));
-              im[u] = fmaf(q[u].x, x.y, fmaf(-q[u].y, x.x, im[u]));
-            }
+          for (int u = 0; u < 8; u++)
+            q[u] = j0 + u < k ? __ldcg(reinterpret_cast<const float4*>(Wk(j0 + u, p)) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 x = __ldcg(wk + e);
+          if (gi == 0) {
+            const float4 rr = __ldcg(rp + e);
+            s0 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, s0))));
+            s1 = fmaf(x.x, rr.x, fmaf(x.y, rr.y, fmaf(x.z, rr.z, fmaf(x.w, rr.w, s1))));
+            s2 = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, fmaf(x.z, rr.w, fmaf(-x.w, rr.z, s2))));
           }
+#pragma unroll
+          for (int u = 0; u < 8; u++) {
+            re[u] = fmaf(q[u].x, x.x, fmaf(q[u].y, x.y, fmaf(q[u].z, x.z, fmaf(q[u].w, x.w, re[u]))));
+            im[u] = fmaf(q[u].x, x.y, fmaf(-q[u].y, x.x, fmaf(q[u].z, x.w, fmaf(-q[u].w, x.z, im[u]))));
+          }
+        }
+        if (k > 0) {
           df v[16];
 #pragma unroll
           for (int u = 0; u < 8; u++) {
@@ -391,20 +419,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
           const df t = warp_transpose_sum<16>(v);   // lane l: value l >> 1
           const int q = 2 * j0 + (lane >> 1);
           if ((lane & 1) == 0 && q < 2 * k) partial(p, q, t);
-        } else {
-          df v[4];
-          float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-          const float2* rp = a.r + (size_t)p * n + E0;
-          for (int e = lane; e < E; e += 32) {
-            const float2 x = __ldcg(wk + e), rr = __ldcg(rp + e);
-            s0 = fmaf(x.x, x.x, fmaf(x.y, x.y, s0));
-            s1 = fmaf(x.x, rr.x, fmaf(x.y, rr.y, s1));
-            s2 = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, s2));
-          }
-          v[0] = df_of(s0);
-          v[1] = df_of(s1);
-          v[2] = df_of(s2);
-          v[3] = df_of(0.f);
+        }
+        if (gi == 0) {
+          df v[4] = {df_of(s0), df_of(s1), df_of(s2), df_of(0.f)};
           const df t = warp_transpose_sum<4>(v);   // lane l: value l >> 3
           if ((lane & 7) == 0 && (lane >> 3) < 3) partial(p, QW + (lane >> 3), t);
         }
@@ -433,16 +450,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
       }
       __syncthreads();
       const bool exact = s_exact != 0;   // uniform: from the same totals in every block
-      auto finish = [&](int p, int e, float2 x) {   // w_k = w'' / gamma, the direction r, r -= alpha w_k
-        const size_t i = (size_t)p * n + E0 + e;
-        x.x *= s_ig[p];
-        x.y *= s_ig[p];
-        Wk(k, p)[e] = x;
-        float2 rr = a.r[i];
-        Rk(k, p)[e] = rr;
-        rr.x -= s_ar[p] * x.x - s_ai[p] * x.y;
-        rr.y -= s_ar[p] * x.y + s_ai[p] * x.x;
-        a.r[i] = rr;
+      auto finish = [&](int p, int e, float4 x) {   // w_k = w'' / gamma, the direction r, r -= alpha w_k
+        float4* rp = reinterpret_cast<float4*>(a.r + (size_t)p * n + E0) + e;
+        const float ig = s_ig[p], ar = s_ar[p], ai = s_ai[p];
+        x.x *= ig;
+        x.y *= ig;
+        x.z *= ig;
+        x.w *= ig;
+        reinterpret_cast<float4*>(Wk(k, p))[e] = x;
+        float4 rr = *rp;
+        reinterpret_cast<float4*>(Rk(k, p))[e] = rr;
+        rr.x -= ar * x.x - ai * x.y;
+        rr.y -= ar * x.y + ai * x.x;
+        rr.z -= ar * x.z - ai * x.w;
+        rr.w -= ar * x.w + ai * x.z;
+        *rp = rr;
       };
       auto coefficients = [&]() {
         if (threadIdx.x < nb && ((run >> threadIdx.x) & 1u)) {
@@ -466,28 +488,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
         __syncthreads();
       };
       if (!exact) coefficients();
-      for (int q = threadIdx.x; q < nb * E; q += kThreads) {
-        const int p = q / E, e = q - p * E;
+      for (int q = threadIdx.x; q < nb * E2; q += kThreads) {
+        const int p = q / E2, e = q - p * E2;
         if (!((run >> p) & 1u)) continue;
-        float2 x = __ldcg(Wk(k, p) + e);
-        float sx[2] = {0.f, 0.f}, sy[2] = {0.f, 0.f};
+        float4 x = __ldcg(reinterpret_cast<const float4*>(Wk(k, p)) + e);
+        float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
         const float2* bp = sbeta + p * kMaxRestart;
+        const float4* hist = reinterpret_cast<const float4*>(Wk(0, p)) + e;
+        const size_t step = (size_t)nb * n >> 1;
+        auto add = [](float4& s, float2 b, float4 h) {
+          s.x = fmaf(b.x, h.x, fmaf(-b.y, h.y, s.x));
+          s.y = fmaf(b.x, h.y, fmaf(b.y, h.x, s.y));
+          s.z = fmaf(b.x, h.z, fmaf(-b.y, h.w, s.z));
+          s.w = fmaf(b.x, h.w, fmaf(b.y, h.z, s.w));
+        };
+        int j = 0;
         constexpr int U = 16;   // history loads in flight
-        for (int j0 = 0; j0 < k; j0 += U) {
-          float2 h[U];
+        for (; j + U <= k; j += U) {
+          float4 h[U];
 #pragma unroll
-          for (int u = 0; u < U; u++) h[u] = j0 + u < k ? __ldcg(Wk(j0 + u, p) + e) : make_float2(0.f, 0.f);
+          for (int u = 0; u < U; u++) h[u] = __ldcg(hist + (size_t)(j + u) * step);
 #pragma unroll
-          for (int u = 0; u < U; u++) {
-            const float2 bj = j0 + u < k ? bp[j0 + u] : make_float2(0.f, 0.f);
-            sx[u & 1] = fmaf(bj.x, h[u].x, fmaf(-bj.y, h[u].y, sx[u & 1]));
-            sy[u & 1] = fmaf(bj.x, h[u].y, fmaf(bj.y, h[u].x, sy[u & 1]));
+          for (int u = 0; u < U; u += 2) {
+            add(s0, bp[j + u], h[u]);
+            add(s1, bp[j + u + 1], h[u + 1]);
           }
         }
-        x.x -= sx[0] + sx[1];
-        x.y -= sy[0] + sy[1];
+        if (j < k) {
+          float4 h[U];
+#pragma unroll
+          for (int u = 0; u < U; u++) h[u] = j + u < k ? __ldcg(hist + (size_t)(j + u) * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < U; u++)
+            if (j + u < k) add(u & 1 ? s1 : s0, bp[j + u], h[u]);
+        }
+        x.x -= s0.x + s1.x;
+        x.y -= s0.y + s1.y;
+        x.z -= s0.z + s1.z;
+        x.w -= s0.w + s1.w;
         if (exact)
-          Wk(k, p)[e] = x;
+          reinterpret_cast<float4*>(Wk(k, p))[e] = x;
         else
           finish(p, e, x);
       }
@@ -510,9 +550,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
         if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
         if (!(ok = grid_totals<NS>(a, run, QE, 3, 0, 0, tot, target))) break;
         coefficients();
-        for (int q = threadIdx.x; q < nb * E; q += kThreads) {
-          const int p = q / E, e = q - p * E;
-          if ((run >> p) & 1u) finish(p, e, __ldcg(Wk(k, p) + e));
+        for (int q = threadIdx.x; q < nb * E2; q += kThreads) {
+          const int p = q / E2, e = q - p * E2;
+          if ((run >> p) & 1u) finish(p, e, __ldcg(reinterpret_cast<const float4*>(Wk(k, p)) + e));
         }
       }
       // r complete on every block before the next product reads it
