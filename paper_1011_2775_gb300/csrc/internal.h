@@ -389,8 +389,7 @@ class GCR {
 template <typename T>
 void dr_dagger(Ctx* c, FineOps<T>& F, T* out, const T* in, T* tmp);
 
-// BiCGStab and CGNR on n complex unknowns; the iteration scalars go through
-// the host (a few synchronisations per iteration)
+// BiCGStab (one synchronisation per iteration) and CGNR (two) on n complex unknowns
 template <typename T>
 class Krylov {
  public:
@@ -402,7 +401,6 @@ class Krylov {
     bool converged = false;
   };
   Krylov(Ctx* c, size_t n);
-  ~Krylov();
   Krylov(const Krylov&) = delete;
   Krylov& operator=(const Krylov&) = delete;
   // A x = b from x = 0 (x0_zero) or from x, until ||b - A x|| <= tol_abs
@@ -413,12 +411,10 @@ class Krylov {
   Result cgnr(const Op& A, const Op& Adag, T* x, const T* b, bool x0_zero, double tol_abs, int maxit);
 
  private:
-  const double* coefs(std::initializer_list<std::complex<double>> z);
   Ctx* c_;
   size_t n_;
-  DBuf r_, rh_, p_, v_, s_, t_, q_;
-  DBuf sc_, coef_;
-  double* hcoef_ = nullptr;  // pinned staging of lincomb coefficients
+  DBuf r_, rh_, p_, v_, s_, t_;
+  DBuf sc_;
 };
 
 // MR smoothing: e = MR_nu(A, r) from e = 0 (r is consumed as scratch)

@@ -2,9 +2,15 @@
 // BiCGStab, CG on the normal equations (CGNR) and, built on BiCGStab, a
 // mixed-precision solver by iterative refinement (driven from solver.cu).
 // They run on the even-odd reduced operator D_r with the same fine kernels as
-// the multigrid solve; the scalars of each iteration go through the host.
+// the multigrid solve.  BiCGStab's vector work is four fused passes per
+// iteration that form alpha and omega on the device, so the host waits once
+// per iteration, for the norms that decide convergence (separate copies,
+// linear combinations and three waits with coefficient uploads took 60 us of
+// passes and 75 us of gaps in a 280 us iteration of 16^3x32).
+#include <algorithm>
 #include <complex>
 
+#include "dfloat.cuh"
 #include "internal.h"
 
 namespace mg {
@@ -40,33 +46,179 @@ void dr_dagger(Ctx* c, FineOps<T>& F, T* out, const T* in, T* tmp) {
 
 template <typename T>
 Krylov<T>::Krylov(Ctx* c, size_t n) : c_(c), n_(n) {
-  for (DBuf* d : {&r_, &rh_, &p_, &v_, &s_, &t_, &q_}) {
+  for (DBuf* d : {&r_, &rh_, &p_, &v_, &s_, &t_}) {
     d->alloc(sizeof(T) * 2 * n);
     MG_CUDA(cudaMemsetAsync(d->get(), 0, sizeof(T) * 2 * n, c->stream));
   }
   sc_.alloc(sizeof(double) * 16);
-  coef_.alloc(sizeof(double) * 16);
-  MG_CUDA(cudaMallocHost(&hcoef_, sizeof(double) * 16));
 }
 
-template <typename T>
-Krylov<T>::~Krylov() {
-  if (hcoef_) cudaFreeHost(hcoef_);
+namespace {
+constexpr int kBS = 256;
+inline int sum_grid(size_t n) {   // blocks of the fused passes with sums
+  const size_t b = (n + kBS - 1) / kBS;
+  return (int)(b < 1 ? 1 : (b > (size_t)Workspace::kMaxBlocks ? (size_t)Workspace::kMaxBlocks : b));
 }
 
-// complex coefficients for blas_lincomb, through pinned memory: every caller
-// writes them after a host synchronisation, so the previous copy has run
+// device scalars of an iteration (doubles): <rh, v>; <t, t>, <t, s>, ||s||^2;
+// <rh, r>, <r, r>; alpha; omega
+enum { S_RV = 0, S_TT = 2, S_TS = 3, S_SS = 5, S_RHO = 6, S_RR = 8, S_AL = 10, S_OM = 12, S_COUNT = 14 };
+
+// a complex coefficient and a running sum c z: FP64, or for FP32 vectors the
+// coefficient as float pairs and the sum in compensated FP32 (about 48 bits,
+// rounded once), as blas_lincomb forms it
 template <typename T>
-const double* Krylov<T>::coefs(std::initializer_list<cplx> z) {
-  int k = 0;
-  for (const cplx& v : z) {
-    hcoef_[2 * k] = v.real();
-    hcoef_[2 * k + 1] = v.imag();
-    k++;
+struct Coef;
+template <>
+struct Coef<double> {
+  double re, im;
+  __host__ __device__ static Coef of(double r, double i) { return Coef{r, i}; }
+};
+template <>
+struct Coef<float> {
+  float rh, rl, ih, il;
+  __host__ __device__ static Coef of(double r, double i) {
+    const float a = (float)r, b = (float)i;
+    return Coef{a, (float)(r - (double)a), b, (float)(i - (double)b)};
   }
-  MG_CUDA(cudaMemcpyAsync(coef_.get(), hcoef_, sizeof(double) * 2 * k, cudaMemcpyHostToDevice, c_->stream));
-  return coef_.as<double>();
+};
+template <typename T>
+struct Sum;
+template <>
+struct Sum<double> {
+  double re, im;
+  __device__ explicit Sum(cx<double> z) : re(z.re), im(z.im) {}
+  __device__ void add(const Coef<double>& c, cx<double> z) {
+    re = fma(c.re, z.re, fma(-c.im, z.im, re));
+    im = fma(c.re, z.im, fma(c.im, z.re, im));
+  }
+  __device__ cx<double> value() const { return mkc(re, im); }
+};
+template <>
+struct Sum<float> {
+  float rh, rl, ih, il;
+  __device__ explicit Sum(cx<float> z) : rh(z.re), rl(0.f), ih(z.im), il(0.f) {}
+  __device__ void add(const Coef<float>& c, cx<float> z) {
+    dot2_acc(rh, rl, c.rh, z.re);
+    dot2_acc(rh, rl, -c.ih, z.im);
+    rl = fmaf(c.rl, z.re, fmaf(-c.il, z.im, rl));
+    dot2_acc(ih, il, c.rh, z.im);
+    dot2_acc(ih, il, c.ih, z.re);
+    il = fmaf(c.rl, z.im, fmaf(c.il, z.re, il));
+  }
+  __device__ cx<float> value() const { return mkc(rh + rl, ih + il); }
+};
+
+// |z|^2 <= 1e-60 rn^4, the breakdown test |z| <= 1e-30 rn^2 without a square root
+__device__ __forceinline__ bool tiny(double re, double im, double rn) {
+  return re * re + im * im <= 1e-60 * (rn * rn) * (rn * rn);
 }
+__device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double& re, double& im) {
+  const double d = 1.0 / (br * br + bi * bi);
+  re = (ar * br + ai * bi) * d;
+  im = (ai * br - ar * bi) * d;
+}
+
+// p = r + beta p - (beta omega) v
+template <typename T>
+__global__ void __launch_bounds__(kBS) k_bicg_p(cx<T>* __restrict__ p, const cx<T>* __restrict__ r,
+                                                const cx<T>* __restrict__ v, Coef<T> beta, Coef<T> mbo, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n; i += (size_t)gridDim.x * kBS) {
+    Sum<T> s(r[i]);
+    s.add(beta, p[i]);
+    s.add(mbo, v[i]);
+    p[i] = s.value();
+  }
+}
+
+// s = r - alpha v, alpha = rho / <rh, v> (0 on a breakdown, which the host sees too)
+template <typename T>
+__global__ void __launch_bounds__(kBS) k_bicg_s(cx<T>* __restrict__ sv, const cx<T>* __restrict__ r,
+                                                const cx<T>* __restrict__ v, double rho_re, double rho_im, double rn,
+                                                double* sc, size_t n) {
+  __shared__ Coef<T> ma;
+  if (threadIdx.x == 0) {
+    double re = 0.0, im = 0.0;
+    if (!tiny(sc[S_RV], sc[S_RV + 1], rn)) cdiv(rho_re, rho_im, sc[S_RV], sc[S_RV + 1], re, im);
+    ma = Coef<T>::of(-re, -im);
+    if (blockIdx.x == 0) {
+      sc[S_AL] = re;
+      sc[S_AL + 1] = im;
+    }
+  }
+  __syncthreads();
+  const Coef<T> c = ma;
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n; i += (size_t)gridDim.x * kBS) {
+    Sum<T> s(r[i]);
+    s.add(c, v[i]);
+    sv[i] = s.value();
+  }
+}
+
+// {<t, t>, Re <t, s>, Im <t, s>, ||s||^2} -> sc[S_TT ..]
+template <typename T>
+__global__ void __launch_bounds__(kBS) k_bicg_dots(const cx<T>* __restrict__ t, const cx<T>* __restrict__ sv, size_t n,
+                                                   double* partials, unsigned* counter, double* sc) {
+  T v[4] = {0, 0, 0, 0};
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n; i += (size_t)gridDim.x * kBS) {
+    const cx<T> a = t[i], b = sv[i];
+    v[0] = fma(a.re, a.re, fma(a.im, a.im, v[0]));
+    v[1] = fma(a.re, b.re, fma(a.im, b.im, v[1]));
+    v[2] = fma(a.re, b.im, fma(-a.im, b.re, v[2]));
+    v[3] = fma(b.re, b.re, fma(b.im, b.im, v[3]));
+  }
+  grid_sum<kBS, 4>(v, partials, counter, sc + S_TT);
+}
+
+// omega = <t, s> / <t, t>: x += alpha p + omega s, r = s - omega t; at the half
+// step (||s|| <= tol or t = 0) x += alpha p, r = s; on a breakdown nothing.
+// Then {<rh, r>, <r, r>} -> sc[S_RHO ..].
+template <typename T>
+__global__ void __launch_bounds__(kBS) k_bicg_xr(cx<T>* __restrict__ x, cx<T>* __restrict__ r,
+                                                 const cx<T>* __restrict__ p, const cx<T>* __restrict__ sv,
+                                                 const cx<T>* __restrict__ t, const cx<T>* __restrict__ rh, double rn,
+                                                 double tol_abs, size_t n, double* partials, unsigned* counter,
+                                                 double* sc) {
+  __shared__ Coef<T> s_al, s_om, s_mom;
+  __shared__ int s_skip;
+  if (threadIdx.x == 0) {
+    const bool half = sqrt(sc[S_SS]) <= tol_abs || sc[S_TT] == 0.0;
+    double re = 0.0, im = 0.0;
+    if (!half) {
+      const double d = 1.0 / sc[S_TT];
+      re = sc[S_TS] * d;
+      im = sc[S_TS + 1] * d;
+    }
+    s_skip = tiny(sc[S_RV], sc[S_RV + 1], rn);
+    s_al = Coef<T>::of(sc[S_AL], sc[S_AL + 1]);
+    s_om = Coef<T>::of(re, im);
+    s_mom = Coef<T>::of(-re, -im);
+    if (blockIdx.x == 0) {
+      sc[S_OM] = re;
+      sc[S_OM + 1] = im;
+    }
+  }
+  __syncthreads();
+  const Coef<T> al = s_al, om = s_om, mom = s_mom;
+  T v[3] = {0, 0, 0};
+  if (!s_skip)
+    for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n; i += (size_t)gridDim.x * kBS) {
+      const cx<T> si = sv[i];
+      Sum<T> a(x[i]);
+      a.add(al, p[i]);
+      a.add(om, si);
+      x[i] = a.value();
+      Sum<T> b(si);
+      b.add(mom, t[i]);
+      const cx<T> ri = b.value(), h = rh[i];
+      r[i] = ri;
+      v[0] = fma(h.re, ri.re, fma(h.im, ri.im, v[0]));
+      v[1] = fma(h.re, ri.im, fma(-h.im, ri.re, v[1]));
+      v[2] = fma(ri.re, ri.re, fma(ri.im, ri.im, v[2]));
+    }
+  grid_sum<kBS, 3>(v, partials, counter, sc + S_RHO);
+}
+}  // namespace
 
 // BiCGStab (van der Vorst) on A x = b.  Restarts (rh = r, p = v = 0) when
 // <rh, r> or <rh, A p> vanishes or omega does, and stops unconverged when the
@@ -85,7 +237,7 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
   T* sv = s_.as<T>();
   T* t = t_.as<T>();
   double* d = sc_.as<double>();
-  double h[8];
+  double h[S_COUNT];
   if (x0_zero) {
     blas_zero<T>(x, n, s);
     blas_convert<T, T>(r, b, n, s);
@@ -101,6 +253,11 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
     res.converged = true;
     return res;
   }
+  const int grid = sum_grid(n);
+  const unsigned wide = (unsigned)std::min<size_t>(152 * 8, (n + kBS - 1) / kBS);
+  double* part = c_->ws.partials.template as<double>();
+  unsigned* cnt = c_->ws.counter.template as<unsigned>();
+  auto cv = [](T* v) { return reinterpret_cast<cx<T>*>(v); };
   bool fresh = true;
   cplx rho(1.0, 0.0), alpha(1.0, 0.0), omega(1.0, 0.0), rho_new;
   while (res.iterations < maxit) {
@@ -110,20 +267,25 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
       blas_convert<T, T>(p, r, n, s);
       rho_new = cplx(rn * rn, 0.0);
     } else {
-      const cplx beta = (rho_new / rho) * (alpha / omega);
-      blas_convert<T, T>(q_.as<T>(), r, n, s);            // p = r + beta p - beta omega v
-      const T* Z[2] = {p, v};
-      blas_lincomb<T, T>(q_.as<T>(), Z, coefs({beta, -beta * omega}), 2, 1.0, n, s);
-      std::swap(p_, q_);
-      p = p_.as<T>();
+      const cplx beta = (rho_new / rho) * (alpha / omega), mbo = -beta * omega;
+      k_bicg_p<T><<<wide, kBS, 0, s>>>(cv(p), cv(r), cv(v), Coef<T>::of(beta.real(), beta.imag()),
+                                       Coef<T>::of(mbo.real(), mbo.imag()), n);
+      MG_LAUNCH();
     }
     fresh = false;
     A(v, p);
-    blas_cdot<T>(rh, v, n, d, c_->ws, s);
-    c_->read_scalars(d, h, 2);
-    const cplx rv(h[0], h[1]);
-    if (!std::isfinite(h[0]) || !std::isfinite(h[1])) raise(MG_ERR_NAN, "non-finite scalar in BiCGStab");
-    if (std::abs(rv) <= 1e-30 * rn * rn) {
+    blas_cdot<T>(rh, v, n, d + S_RV, c_->ws, s);
+    k_bicg_s<T><<<wide, kBS, 0, s>>>(cv(sv), cv(r), cv(v), rho_new.real(), rho_new.imag(), rn, d, n);
+    MG_LAUNCH();
+    A(t, sv);
+    k_bicg_dots<T><<<grid, kBS, 0, s>>>(cv(t), cv(sv), n, part, cnt, d);
+    MG_LAUNCH();
+    k_bicg_xr<T><<<grid, kBS, 0, s>>>(cv(x), cv(r), cv(p), cv(sv), cv(t), cv(rh), rn, tol_abs, n, part, cnt, d);
+    MG_LAUNCH();
+    c_->read_scalars(d, h, S_COUNT);
+    if (!std::isfinite(h[S_RV]) || !std::isfinite(h[S_RV + 1])) raise(MG_ERR_NAN, "non-finite scalar in BiCGStab");
+    const double rv2 = h[S_RV] * h[S_RV] + h[S_RV + 1] * h[S_RV + 1];
+    if (rv2 <= 1e-60 * (rn * rn) * (rn * rn)) {   // the kernels' breakdown test
       // breakdown: restart from the current residual, unless this step already
       // was the restart (<r, A r> = 0: no progress possible from here)
       if (restarted) break;
@@ -131,26 +293,10 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
       fresh = true;
       continue;
     }
-    alpha = rho_new / rv;
-    blas_convert<T, T>(sv, r, n, s);  // s = r - alpha v
-    {
-      const T* Z[1] = {v};
-      blas_lincomb<T, T>(sv, Z, coefs({-alpha}), 1, 1.0, n, s);
-    }
-    A(t, sv);
-    {
-      // {<t,t>, Re<t,s>, Im<t,s>} and ||s||^2
-      blas_dot2<T>(t, sv, n, d, c_->ws, s);
-      blas_norm2<T>(sv, n, d + 3, c_->ws, s);
-      c_->read_scalars(d, h, 4);
-    }
     res.iterations++;
-    const double sn = std::sqrt(h[3]);
-    if (!std::isfinite(sn) || !std::isfinite(h[0])) raise(MG_ERR_NAN, "non-finite scalar in BiCGStab");
-    if (sn <= tol_abs || h[0] == 0.0) {  // converged at the half step (or A s = 0: s is the exact residual)
-      const T* Z[1] = {p};
-      blas_lincomb<T, T>(x, Z, coefs({alpha}), 1, 1.0, n, s);
-      blas_convert<T, T>(r, sv, n, s);
+    const double sn = std::sqrt(h[S_SS]);
+    if (!std::isfinite(sn) || !std::isfinite(h[S_TT])) raise(MG_ERR_NAN, "non-finite scalar in BiCGStab");
+    if (sn <= tol_abs || h[S_TT] == 0.0) {  // converged at the half step (or A s = 0: s is the exact residual)
       res.rnorm = sn;
       res.converged = sn <= tol_abs;
       if (res.converged) break;
@@ -159,20 +305,9 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
       res.restarts++;
       continue;
     }
-    omega = cplx(h[1], h[2]) / h[0];
-    {
-      const T* Z[2] = {p, sv};  // x += alpha p + omega s
-      const double* cf = coefs({alpha, omega, -omega});
-      blas_lincomb<T, T>(x, Z, cf, 2, 1.0, n, s);
-      blas_convert<T, T>(r, sv, n, s);  // r = s - omega t
-      const T* Zt[1] = {t};
-      blas_lincomb<T, T>(r, Zt, cf + 4, 1, 1.0, n, s);
-    }
-    // <rh, r> for the next step and ||r||^2 in one reduction
-    const T* V[2] = {rh, r};
-    blas_multidot<T>(V, 2, r, n, d, c_->ws, s);
-    c_->read_scalars(d, h, 4);
-    rn = std::sqrt(h[2]);
+    alpha = cplx(h[S_AL], h[S_AL + 1]);
+    omega = cplx(h[S_OM], h[S_OM + 1]);
+    rn = std::sqrt(h[S_RR]);
     res.rnorm = rn;
     if (!std::isfinite(rn)) raise(MG_ERR_NAN, "non-finite residual in BiCGStab");
     if (rn <= tol_abs) {
@@ -180,7 +315,7 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
       break;
     }
     rho = rho_new;
-    rho_new = cplx(h[0], h[1]);
+    rho_new = cplx(h[S_RHO], h[S_RHO + 1]);
     if (std::abs(omega) == 0.0 || std::abs(rho_new) <= 1e-30 * rn * rn) {
       res.restarts++;
       fresh = true;
