@@ -88,10 +88,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, int* abort, unsign
     __threadfence();
     atomicAdd(count, 1u);
     const long long t0 = clock64();
-    while (true) {
+    for (unsigned poll = 1;; poll++) {
       unsigned c;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
       if ((int)(c - target) >= 0) break;
+      if (poll & 15u) continue;   // the abort flag is a second trip to L2: looked at on every sixteenth poll
       if (*(volatile int*)abort) {
         good = 0;
         break;
@@ -102,8 +103,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, int* abort, unsign
         break;
       }
     }
-    __threadfence();
-    ok = good;
+    ok = good;   // the acquire that saw the count orders the block's reads behind the other blocks' writes
   }
   __syncthreads();
   return ok != 0;

@@ -134,9 +134,9 @@ struct CoarseGCRBuffers {
   DBuf r, y, br, tA, tB, W, Z, partials, scal;
   // batched solves (coarse_batch.cu; grown on demand)
   DBuf bx_r, bx_y, bx_br, bx_tB, bx_W, bx_Z, bx_part, bx_scal;
-  // streamed solve (coarse_stream.cu; grown on demand): partial sums, the
-  // Gram-Schmidt coefficients, grid-barrier counter and abort flag
-  DBuf st_part, st_beta, st_sync;
+  // streamed solve (coarse_stream.cu; grown on demand): partial sums, X_o^{-1} b_o,
+  // grid-barrier counter and abort flag
+  DBuf st_part, st_to, st_sync;
   // tensor-core solve (coarse_tc.cu; grown on demand)
   DBuf tc_y, tc_r, tc_br, tc_s, tc_sy, tc_t, tc_tb, tc_W, tc_Z, tc_part, tc_sync;
   // grouped solve (coarse_group.cu; grown on demand)

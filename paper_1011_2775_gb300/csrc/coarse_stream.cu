@@ -11,7 +11,7 @@
 //    phase A uses the folded odd-site links X_o^{-1} Y_d X^{-1}(o + d) (FP32),
 //    phase B the even-site links Y_eo in their storage format.  Every block
 //    owns a fixed, contiguous range of A items and of B items, and warp w of
-//    the block takes every eighth item of each range.
+//    the block takes every sixteenth item of each range.
 //  * The links do not change during the solve, so the order in which a warp
 //    consumes them is known in advance: its B items (for b_r), then its A
 //    items and B items once per operator application.  Each warp keeps two
@@ -37,9 +37,17 @@
 //    times out raises an abort flag that releases the others, sets
 //    FLAG_TIMEOUT and the kernel returns after its copies in flight land.
 //
-// The site-local parts around it -- t_o = X_o^{-1} b_o before, and the
-// reconstruction x_e = X_e^{-1} y_e, x_o = X_o^{-1}(b_o - Y_oe x_e) after --
-// are separate launches of the coarse stencil kernels.
+// The site-local parts around it -- t_o = X_o^{-1} b_o before and x_e = X_e^{-1} y_e
+// after -- are separate launches.  The closing true residual has formed A y on
+// the odd sites, so x_o = X_o^{-1} (b_o - Y_oe x_e) = t_o - A y is written there
+// instead of by another pass over the links (17 us of a 16^3x32 solve, 112 of
+// 427 us at 24^3x48 with bf16 links).
+//
+// Measured (16^3x32, 4^4 blocks, Nc = 48, 256 reduced sites, 35 iterations):
+// 817 us per solve with 256 threads, neighbour indices read for every gather
+// and the coefficients formed before the sums; 744 us here.  An iteration is
+// 45k cycles: the stencil passes 9.4k and 10.1k, the gathers 1.4k each, the
+// barriers 9.3k, the inner products, totals and update 11k.
 #include <algorithm>
 #include <cstring>
 
@@ -52,11 +60,12 @@ namespace mg {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kStagesPerWarp = 2;
 constexpr int kStages = kWarps * kStagesPerWarp;
 constexpr int kMaxRows = 8;        // rows of one item (16 accumulators per lane)
+constexpr int kUpdThreads = kThreads - 32;   // warp 0 forms the coefficients meanwhile
 constexpr int kMaxGroups = 8;      // thread groups sharing the sum over j of the Gram-Schmidt update
 constexpr int kMaxRestart = 64;
 // reduction slots: [0, 2 kMaxRestart) <w_j, w>; then ||w||^2, Re/Im <w, r>;
@@ -78,10 +87,12 @@ struct SArgs {
   const float* Ys;            // their tile scales [e][8]
   const unsigned char* Af;    // folded odd-site links [o - half][nc][8][nc], FP32
   const float2* b;            // full right-hand side
+  const float2* to;           // full: the odd part holds X_o^{-1} b_o
+  float2* x;                  // full solution: the odd half is written here
   float2* y;                  // half: GCR iterate
   float2* r;                  // half: residual
   float2* br;                 // half: reduced right-hand side
-  float2* tB;                 // full: odd part holds X_o^{-1} b_o on entry, A outputs after
+  float2* tB;                 // full: the odd part holds the phase-A outputs
   float2* W;                  // [m][half nc] (when the slice is not in shared memory)
   float2* Z;                  // [m][half nc]
   float2* partials;           // [kNR][grid] double-float partial sums
@@ -148,39 +159,31 @@ __device__ __forceinline__ void issue(const SArgs& a, const Stream& st, long lon
   bulk_copy_g2s(st.ring + (size_t)stage * a.stage_bytes, src, bytes, &st.full[stage]);
 }
 
-// Gathers the vectors of the sites of items [i0, i1) (the whole block): for
-// each site, the 8 neighbours' nc components of `in`, times the tile scale of
-// Y (phase B).
-__device__ void gather(const SArgs& a, int i0, int i1, int ips, int site_base, const float2* in, const float* scale,
-                       float2* gv) {
-  if (i1 > i0) {
-    const int nc = a.nc, K = 8 * nc;
-    const int s0 = i0 / ips, s1 = (i1 - 1) / ips;
-    const int total = (s1 - s0 + 1) * K;
-    // four elements per thread and round: their neighbour indices, then their
-    // loads, are in flight together (two L2 round trips per round)
-    constexpr int U = 4;
-    for (int t0 = threadIdx.x; t0 < total; t0 += U * blockDim.x) {
-      int src[U];
-      float sc[U];
+// Gathers the vectors of the block's `ns` sites of a phase: for each site, the
+// 8 neighbours' nc components of `in` (neighbour indices in shared memory),
+// times the tile scale of Y (phase B).  A warp takes (site, direction) pairs,
+// 16 bytes per lane, the loads of kGather pairs in flight together: one L2
+// round trip for a block of up to eight sites.
+constexpr int kGather = 4;
+__device__ void gather(int nc, int ns, const int* nbr, const float* scale, const float2* in, float2* gv) {
+  const int nc2 = nc >> 1, np = 8 * ns, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float4* g4 = reinterpret_cast<float4*>(gv);
+  for (int p0 = w; p0 < np; p0 += kGather * kWarps)
+    for (int q = lane; q < nc2; q += 32) {
+      float4 v[kGather];
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        const int t = t0 + u * blockDim.x;
-        const int tt = t < total ? t : 0;
-        const int sl = tt / K, rem = tt % K, d = rem / nc, j = rem % nc;
-        src[u] = a.nbr[(size_t)(site_base + s0 + sl) * 8 + d] * nc + j;
-        sc[u] = scale ? scale[(size_t)(s0 + sl) * 8 + d] : 1.f;
+      for (int u = 0; u < kGather; u++) {
+        const int p = min(p0 + u * kWarps, np - 1);
+        v[u] = __ldcg(reinterpret_cast<const float4*>(in + (size_t)nbr[p] * nc) + q);
       }
-      float2 v[U];
 #pragma unroll
-      for (int u = 0; u < U; u++) v[u] = __ldcg(in + (size_t)src[u]);
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const int t = t0 + u * blockDim.x;
-        if (t < total) gv[t] = make_float2(sc[u] * v[u].x, sc[u] * v[u].y);
+      for (int u = 0; u < kGather; u++) {
+        const int p = p0 + u * kWarps;
+        if (p >= np) break;
+        const float c = scale ? scale[p] : 1.f;
+        g4[(size_t)p * nc2 + q] = make_float4(c * v[u].x, c * v[u].y, c * v[u].z, c * v[u].w);
       }
     }
-  }
   __syncthreads();
 }
 
@@ -281,57 +284,68 @@ __device__ bool run_items(const SArgs& a, Stream& st, int kind, const float2* gv
   return *(volatile int*)s_fail == 0;
 }
 
-// block partial sums of nq per-thread float values v[q]: warp sums, then the
-// eight warp sums added by one thread per slot; partials[q0 + q][block]
+// block partial sums of nq <= 4 per-thread float values v[q]: one transposed
+// warp reduction for the four, then warp q adds the warps' sums of value q;
+// partials[q0 + q][block]
 __device__ void block_partials(const SArgs& a, const float* v, int nq, int q0, df* sred) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int q = 0; q < nq; q++) {
-    const df t = df_wsum(df_of(v[q]));
-    if (lane == 0) sred[q * kWarps + wid] = t;
-  }
+  df t[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) t[q] = df_of(q < nq ? v[q] : 0.f);
+  const df ws = warp_transpose_sum<4>(t);   // lane l: value l >> 3
+  if ((lane & 7) == 0) sred[(lane >> 3) * kWarps + wid] = ws;
   __syncthreads();
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    df s = sred[q * kWarps];
-    for (int w = 1; w < kWarps; w++) s = df_add(s, sred[q * kWarps + w]);
-    a.partials[(size_t)(q0 + q) * gridDim.x + blockIdx.x] = make_float2(s.h, s.l);
+  if (wid < nq) {
+    const df s = df_wsum(lane < kWarps ? sred[wid * kWarps + lane] : df_of(0.f));
+    if (lane == 0) a.partials[(size_t)(q0 + wid) * gridDim.x + blockIdx.x] = make_float2(s.h, s.l);
   }
   __syncthreads();
 }
 
 // totals of slots [q0, q0 + nq) after a grid barrier, identical in every
-// block.  Warp w sums slots w, w + 8, ...; each round issues the loads of
-// kTotU slots (up to kTotG / 32 per lane and slot) before adding any, so that a
-// round costs one L2 round trip; the kTotU sums leave the warp through one
+// block.  Warp w sums slots w, w + 16, ...; each round issues the loads of U
+// slots (up to kTotG / 32 per lane and slot) before adding any, so that a
+// round costs one L2 round trip; the U sums leave the warp through one
 // transposing reduction.
 constexpr int kTotG = 160;   // grids up to this size take the one-pass path
-constexpr int kTotU = 4;     // slots per warp and round
+template <int U>
+__device__ __forceinline__ void totals_rounds(const SArgs& a, int q0, int nq, df* out) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int G = gridDim.x;
+  for (int qb = wid; qb < nq; qb += U * kWarps) {
+    float2 t[U][kTotG / 32];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int q = qb + u * kWarps;
+      const float2* p = a.partials + (size_t)(q0 + (q < nq ? q : 0)) * G;
+#pragma unroll
+      for (int i = 0; i < kTotG / 32; i++) {
+        const int g = lane + 32 * i;
+        t[u][i] = (q < nq && g < G) ? __ldcg(p + g) : make_float2(0.f, 0.f);
+      }
+    }
+    df sv[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      sv[u] = df{t[u][0].x, t[u][0].y};
+#pragma unroll
+      for (int i = 1; i < kTotG / 32; i++) sv[u] = df_add(sv[u], df{t[u][i].x, t[u][i].y});
+    }
+    const df s = warp_transpose_sum<U>(sv);   // lane l: slot qb + l / (32 / U) * kWarps
+    const int q = qb + lane / (32 / U) * kWarps;
+    if (lane % (32 / U) == 0 && q < nq) out[q] = s;
+  }
+}
 __device__ void grid_totals(const SArgs& a, int q0, int nq, df* out) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int G = gridDim.x;
   if (G <= kTotG) {
-    for (int qb = wid; qb < nq; qb += kTotU * kWarps) {
-      float2 t[kTotU][kTotG / 32];
-#pragma unroll
-      for (int u = 0; u < kTotU; u++) {
-        const int q = qb + u * kWarps;
-        const float2* p = a.partials + (size_t)(q0 + (q < nq ? q : 0)) * G;
-#pragma unroll
-        for (int i = 0; i < kTotG / 32; i++) {
-          const int g = lane + 32 * i;
-          t[u][i] = (q < nq && g < G) ? __ldcg(p + g) : make_float2(0.f, 0.f);
-        }
-      }
-      df sv[kTotU];
-#pragma unroll
-      for (int u = 0; u < kTotU; u++) {
-        sv[u] = df{t[u][0].x, t[u][0].y};
-#pragma unroll
-        for (int i = 1; i < kTotG / 32; i++) sv[u] = df_add(sv[u], df{t[u][i].x, t[u][i].y});
-      }
-      const df s = warp_transpose_sum<kTotU>(sv);   // lane l: slot qb + (l >> 3) * kWarps
-      const int q = qb + (lane >> 3) * kWarps;
-      if ((lane & 7) == 0 && q < nq) out[q] = s;
-    }
+    if (nq <= kWarps)
+      totals_rounds<1>(a, q0, nq, out);
+    else if (nq <= 4 * kWarps)
+      totals_rounds<4>(a, q0, nq, out);
+    else
+      totals_rounds<8>(a, q0, nq, out);
   } else {
     for (int q = wid; q < nq; q += kWarps) {
       const float2* p = a.partials + (size_t)(q0 + q) * G;
@@ -351,17 +365,19 @@ template <int ST>
 __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[kStages];
-  __shared__ float2 s_beta[kMaxRestart];   // <w_j, w> of this iteration, as floats
   __shared__ float s_coef[4];              // 1/gamma, Re alpha, Im alpha, exact flag
   __shared__ int s_fail;
   const int nc = a.nc, K = 8 * nc, m = a.m;
   const int G = gridDim.x, bid = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float2* gv = reinterpret_cast<float2*>(smem + (size_t)kStages * a.stage_bytes);
-  df* sred = reinterpret_cast<df*>(gv + (size_t)a.gmax * K);          // [kNR][kWarps]
-  df* tot = sred + kNR * kWarps;                                       // [kNR]
-  float2* upd = reinterpret_cast<float2*>(tot + kNR);                  // [2][kThreads] update partial sums
+  float2* upd = gv + (size_t)a.gmax * K;                               // [2][kThreads] update partial sums
   float2* wsm = upd + 2 * kThreads;                                    // [m][wsm_ld] when used
+  df* sred = reinterpret_cast<df*>(wsm + (size_t)m * a.wsm_ld);        // [4][kWarps]
+  df* tot = sred + 4 * kWarps;                                         // [kNR]
+  int* nbA = reinterpret_cast<int*>(tot + kNR);                        // [gmax][8] neighbours of the A sites,
+  int* nbB = nbA + 8 * a.gmax;                                         // of the B sites,
+  float* scB = reinterpret_cast<float*>(nbB + 8 * a.gmax);             // and the tile scales of the B sites
 
   Stream st;
   st.ring = smem;
@@ -382,9 +398,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
   const size_t wld = a.wsm_ld > 0 ? (size_t)a.wsm_ld : n;
   auto Wj = [&](int j) { return wbase + (size_t)j * wld; };
   auto Zj = [&](int j) { return a.Z + (size_t)j * n + E0; };
-  // the j sums of the Gram-Schmidt update are split over ngrp thread groups
-  // when the slice has at most one element per thread
-  const int ngrp = (E > 0 && E <= (int)blockDim.x) ? min((int)blockDim.x / E, kMaxGroups) : 0;
+  // the j sums of the Gram-Schmidt update are split over ngrp groups of the
+  // threads of warps 1 .. when the slice has at most one element per thread
+  const int ngrp = (E > 0 && E <= kUpdThreads) ? min(kUpdThreads / E, kMaxGroups) : 0;
   unsigned target = 0;
   bool ok = true;
   float v[4];
@@ -393,6 +409,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     for (int s = 0; s < kStages; s++) mbar_init(&full[s], 1);
     mbar_fence_init();
     s_fail = 0;
+  }
+  const int sA = st.a0 / a.ipsA, nA = st.a1 > st.a0 ? (st.a1 - 1) / a.ipsA - sA + 1 : 0;
+  const int sB = st.b0 / a.ipsB, nB = st.b1 > st.b0 ? (st.b1 - 1) / a.ipsB - sB + 1 : 0;
+  for (int i = threadIdx.x; i < 8 * nA; i += blockDim.x) nbA[i] = a.nbr[(size_t)(a.half + sA) * 8 + i];
+  for (int i = threadIdx.x; i < 8 * nB; i += blockDim.x) {
+    nbB[i] = a.nbr[(size_t)sB * 8 + i];
+    scB[i] = a.Ys[(size_t)sB * 8 + i];
   }
   __syncthreads();
   if (lane == 0)
@@ -411,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     block_partials(a, v, 1, RD, sred);
   }
   // b_r = b_e - Y_eo X_o^{-1} b_o on the owned rows; r = b_r, y = 0
-  gather(a, st.b0, st.b1, a.ipsB, 0, a.tB, a.Ys, gv);
+  gather(nc, nB, nbB, scB, a.to, gv);
   ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
     const float2 bb = a.b[i];
     const float2 o = make_float2(bb.x - u.x, bb.y - u.y);
@@ -441,11 +464,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     while (k < m && its < a.maxit) {
       float2* wk = Wj(k);
       // w = D_r r: phase A, barrier, phase B
-      gather(a, st.a0, st.a1, a.ipsA, a.half, a.r, nullptr, gv);
+      gather(nc, nA, nbA, nullptr, a.r, gv);
       if (!(ok = run_items<ST>(a, st, 0, gv, [&](size_t i, float2 u) { a.tB[(size_t)a.half * nc + i] = u; }, &s_fail)))
         break;
       if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-      gather(a, st.b0, st.b1, a.ipsB, 0, a.tB, a.Ys, gv);
+      gather(nc, nB, nbB, scB, a.tB, gv);
       if (!(ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
               const float2 rr = a.r[i];
               wk[i - E0] = make_float2(rr.x - u.x, rr.y - u.y);
@@ -485,38 +508,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
       block_partials(a, v, 3, RA + 2 * k, sred);   // after the beta slots: one pass reads all of them
       if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
       grid_totals(a, RA, 2 * k + 3, tot);
-      {  // move them to their own slots (the ranges may overlap: read all, then write)
-        df moved = df_of(0.f);
-        if (threadIdx.x < 3) moved = tot[2 * k + threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x < 3) tot[RB + threadIdx.x] = moved;
-        __syncthreads();
-      }
-      // sum_j |beta_j|^2 (warp 0, lanes over j) and the beta_j as floats
+      // warp 0: sum_j |beta_j|^2 and the coefficients; the other warps meanwhile
+      // S_w = sum_j beta_j w_j, S_z = sum_j beta_j z_j on the owned rows
+      auto beta = [&](int j) {
+        return make_float2(tot[2 * j].h + tot[2 * j].l, tot[2 * j + 1].h + tot[2 * j + 1].l);
+      };
+      // gamma = ||w''||, alpha = <w'', r> / gamma; with w_k = w'' / gamma of
+      // unit norm, ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2 (the running norm)
+      auto coefficients = [&](df g2, df wr, df wi) {
+        const df g = df_sqrt(g2);
+        const bool gz = !(g.h > 0.f);
+        s_coef[0] = gz ? 1.f : 1.f / g.h;
+        const df ar = gz ? wr : df_div(wr, g);
+        const df ai = gz ? wi : df_div(wi, g);
+        s_coef[1] = ar.h + ar.l;
+        s_coef[2] = ai.h + ai.l;
+        if (!gz) {
+          const df rn = df_add(tot[RC], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
+          tot[RC] = rn.h > 0.f ? rn : df_of(0.f);
+        }
+      };
       if (wid == 0) {
         df bb = df_of(0.f);
         for (int j = lane; j < k; j += 32) {
           bb = df_add(bb, df_mul(tot[2 * j], tot[2 * j]));
           bb = df_add(bb, df_mul(tot[2 * j + 1], tot[2 * j + 1]));
-          s_beta[j] = make_float2(tot[2 * j].h + tot[2 * j].l, tot[2 * j + 1].h + tot[2 * j + 1].l);
         }
         bb = df_wsum(bb);
         if (lane == 0) {
-          const df g2 = df_add(tot[RB], df_neg(bb));
-          s_coef[3] = (g2.h > 1e-3f * tot[RB].h) ? 0.f : 1.f;   // Pythagoras lost more than three digits
-          tot[RE] = g2;
+          const df ww = tot[2 * k], g2 = df_add(ww, df_neg(bb));
+          const bool fine = g2.h > 1e-3f * ww.h;   // otherwise Pythagoras lost more than three digits
+          s_coef[3] = fine ? 0.f : 1.f;
+          if (fine) coefficients(g2, tot[2 * k + 1], tot[2 * k + 2]);
         }
-      }
-      __syncthreads();
-      const bool exact = s_coef[3] != 0.f;
-      // S_w = sum_j beta_j w_j, S_z = sum_j beta_j z_j on the owned rows
-      if (ngrp) {
-        const int gi = threadIdx.x / E, ei = threadIdx.x - gi * E;
+      } else if (ngrp) {
+        const int t = threadIdx.x - 32, gi = t / E, ei = t - gi * E;
         if (gi < ngrp) {
           float swr = 0.f, swi = 0.f, szr = 0.f, szi = 0.f;
-#pragma unroll 4
+#pragma unroll 8
           for (int j = gi; j < k; j += ngrp) {
-            const float2 bj = s_beta[j];
+            const float2 bj = beta(j);
             const float2 p = Wj(j)[ei], q = Zj(j)[ei];
             swr = fmaf(bj.x, p.x, fmaf(-bj.y, p.y, swr));
             swi = fmaf(bj.x, p.y, fmaf(bj.y, p.x, swi));
@@ -526,11 +557,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
           upd[gi * E + ei] = make_float2(swr, swi);
           upd[kThreads + gi * E + ei] = make_float2(szr, szi);
         }
-        __syncthreads();
       }
-      // w'' = w - S_w kept in place; with the exact path its norm and <w'', r>
-      v[0] = v[1] = v[2] = 0.f;
-      for (int ei = threadIdx.x; ei < E; ei += blockDim.x) {
+      __syncthreads();
+      const bool exact = s_coef[3] != 0.f;
+      // w'' = w - S_w
+      auto w_orth = [&](int ei) {
         float2 x = wk[ei];
         if (ngrp) {
           for (int g = 0; g < ngrp; g++) {
@@ -541,48 +572,33 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
         } else {
 #pragma unroll 4
           for (int j = 0; j < k; j++) {
-            const float2 bj = s_beta[j], p = Wj(j)[ei];
+            const float2 bj = beta(j), p = Wj(j)[ei];
             x.x -= bj.x * p.x - bj.y * p.y;
             x.y -= bj.x * p.y + bj.y * p.x;
           }
         }
-        wk[ei] = x;
-        if (exact) {
-          const float2 rr = a.r[E0 + ei];
+        return x;
+      };
+      if (exact) {  // uniform: every block took the same decision from the same totals
+        v[0] = v[1] = v[2] = 0.f;
+        for (int ei = threadIdx.x; ei < E; ei += blockDim.x) {
+          const float2 x = w_orth(ei), rr = a.r[E0 + ei];
           v[0] = fmaf(x.x, x.x, fmaf(x.y, x.y, v[0]));
           v[1] = fmaf(x.x, rr.x, fmaf(x.y, rr.y, v[1]));
           v[2] = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, v[2]));
         }
-      }
-      if (exact) {  // uniform: every block took the same decision from the same totals
         block_partials(a, v, 3, RE, sred);
         if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
         grid_totals(a, RE, 3, tot + RB);   // the exact ||w''||^2, <w'', r> replace the estimates
-        if (threadIdx.x == 0) tot[RE] = tot[RB];
+        if (threadIdx.x == 0) coefficients(tot[RB], tot[RB + 1], tot[RB + 2]);
         __syncthreads();
       }
-      // gamma = ||w''||, alpha = <w'', r> / gamma; with w_k = w'' / gamma of
-      // unit norm, ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2 (the running norm)
-      if (threadIdx.x == 0) {
-        const df g = df_sqrt(tot[RE]);
-        const bool gz = !(g.h > 0.f);
-        s_coef[0] = gz ? 1.f : 1.f / g.h;
-        const df ar = gz ? tot[RB + 1] : df_div(tot[RB + 1], g);
-        const df ai = gz ? tot[RB + 2] : df_div(tot[RB + 2], g);
-        s_coef[1] = ar.h + ar.l;
-        s_coef[2] = ai.h + ai.l;
-        if (!gz) {
-          const df rn = df_add(tot[RC], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
-          tot[RC] = rn.h > 0.f ? rn : df_of(0.f);
-        }
-      }
-      __syncthreads();
       // w_k = w'' / gamma, z_k = (r - S_z) / gamma, y += alpha z_k, r -= alpha w_k
       const float ig = s_coef[0], far = s_coef[1], fai = s_coef[2];
       v[0] = 0.f;
       for (int ei = threadIdx.x; ei < E; ei += blockDim.x) {
         const size_t e = E0 + ei;
-        float2 x = wk[ei];
+        float2 x = w_orth(ei);
         x.x *= ig;
         x.y *= ig;
         wk[ei] = x;
@@ -597,7 +613,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
         } else {
 #pragma unroll 4
           for (int j = 0; j < k; j++) {
-            const float2 bj = s_beta[j], q = Zj(j)[ei];
+            const float2 bj = beta(j), q = Zj(j)[ei];
             z.x -= bj.x * q.x - bj.y * q.y;
             z.y -= bj.x * q.y + bj.y * q.x;
           }
@@ -627,11 +643,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     }
     if (!ok || done) break;
     // true residual r = b_r - D_r y (y complete on every block after the last barrier)
-    gather(a, st.a0, st.a1, a.ipsA, a.half, a.y, nullptr, gv);
-    if (!(ok = run_items<ST>(a, st, 0, gv, [&](size_t i, float2 u) { a.tB[(size_t)a.half * nc + i] = u; }, &s_fail)))
+    // and the odd half of the solution, x_o = X_o^{-1} b_o - A y
+    gather(nc, nA, nbA, nullptr, a.y, gv);
+    if (!(ok = run_items<ST>(a, st, 0, gv, [&](size_t i, float2 u) {
+            const float2 o = a.to[(size_t)a.half * nc + i];
+            a.tB[(size_t)a.half * nc + i] = u;
+            a.x[(size_t)a.half * nc + i] = make_float2(o.x - u.x, o.y - u.y);
+          }, &s_fail)))
       break;
     if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-    gather(a, st.b0, st.b1, a.ipsB, 0, a.tB, a.Ys, gv);
+    gather(nc, nB, nbB, scB, a.tB, gv);
     if (!(ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
             const float2 yy = a.y[i], bb = a.br[i];
             a.r[i] = make_float2(bb.x - (yy.x - u.x), bb.y - (yy.y - u.y));
@@ -648,6 +669,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     const df rn2 = tot[RC];
     if (rn2.h <= tol2.h || !(rn2.h == rn2.h)) done = true;
   }
+  if (ok && its == 0)   // b = 0: y = 0 and x_o = t_o
+    for (size_t e = (size_t)bid * kThreads + threadIdx.x; e < n; e += (size_t)G * kThreads) a.x[n + e] = a.to[n + e];
   if (!ok && threadIdx.x == 0) {
     atomicExch(&a.flags[FLAG_TIMEOUT], 1);
     atomicExch(a.abort, 1);
@@ -697,7 +720,8 @@ Plan make_plan(const LevelGeom& G, const CoarseOp& C, int grid, int m) {
   MG_CUDA(cudaGetDevice(&dev));
   MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t budget = (size_t)optin - 4096;   // static shared memory and slack
-  const size_t fixed = sizeof(float2) * (kNR * kWarps + kNR) + sizeof(float2) * 2 * kThreads;
+  const size_t fixed = sizeof(float2) * (4 * kWarps + kNR) + sizeof(float2) * 2 * kThreads;
+  const size_t per_site = sizeof(float2) * K + 24 * sizeof(int);   // gathered vector, neighbours, tile scales
   p.grid = grid;
   // the w_j slice in shared memory only when it is small (a sixteenth of the
   // budget): measured on GB300 at Nc = 48, m = 64, a deeper link ring gains
@@ -711,14 +735,14 @@ Plan make_plan(const LevelGeom& G, const CoarseOp& C, int grid, int m) {
   const size_t wbytes = wsmem ? (size_t)m * ebound * sizeof(float2) : 0;
   int gsites = 4;
   for (int pass = 0; pass < 3; pass++) {
-    const size_t other = fixed + wbytes + sizeof(float2) * (size_t)gsites * K;
+    const size_t other = fixed + wbytes + per_site * (size_t)gsites;
     p.stage_bytes = budget > other ? (int)(((budget - other) / kStages) / 16 * 16) : 0;
     plan_items(p, G.half, nc, esz);
     if (p.gmax <= gsites) break;
     gsites = p.gmax;
   }
   p.grid = std::min(grid, std::min(p.NA, p.NB));
-  p.smem = (size_t)kStages * p.stage_bytes + fixed + wbytes + sizeof(float2) * (size_t)std::max(gsites, p.gmax) * K;
+  p.smem = (size_t)kStages * p.stage_bytes + fixed + wbytes + per_site * (size_t)std::max(gsites, p.gmax);
   p.gmax = std::max(gsites, p.gmax);
   p.wsm_ld = wsmem ? ebound : 0;
   if (wsmem && p.emax > ebound) raise(MG_ERR_STATE, "streamed coarse GCR: Krylov slice larger than planned");
@@ -779,8 +803,8 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   need(B.st_sync, 256);
   if (B.W.bytes() < sizeof(float2) * n * m || B.Z.bytes() < sizeof(float2) * n * m)
     raise(MG_ERR_STATE, "coarse GCR buffers too small for this restart length");
-  float* tB = B.tB.as<float>();
-  coarse_site_mul(G, C, true, G.half, G.nsites, tB, b, s);     // t_o = X_o^{-1} b_o
+  need(B.st_to, sizeof(float2) * 2 * n);
+  coarse_site_mul(G, C, true, G.half, G.nsites, B.st_to.as<float>(), b, s);     // t_o = X_o^{-1} b_o
   MG_CUDA(cudaMemsetAsync(B.st_sync.get(), 0, 256, s));
   SArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -804,6 +828,8 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   a.Ys = C.Yscale.as<float>();
   a.Af = static_cast<const unsigned char*>(C.A.get());
   a.b = reinterpret_cast<const float2*>(b);
+  a.to = B.st_to.as<float2>();
+  a.x = reinterpret_cast<float2*>(x);
   a.y = B.y.as<float2>();
   a.r = B.r.as<float2>();
   a.br = B.br.as<float2>();
@@ -818,9 +844,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   void* params[] = {&a};
   MG_CUDA(cudaLaunchCooperativeKernel(kern, dim3(p.grid), dim3(kThreads), params, p.smem, s));
   MG_LAUNCH();
-  // reconstruction: x_e = X_e^{-1} y_e, x_o = X_o^{-1} (b_o - Y_oe x_e)
-  coarse_site_mul(G, C, true, 0, G.half, x, B.y.as<float>(), s);
-  coarse_hop(G, C, EPI_C_XPAY, true, G.half, G.nsites, x, x, b, -1.f, 0xff, s);
+  coarse_site_mul(G, C, true, 0, G.half, x, B.y.as<float>(), s);   // x_e = X_e^{-1} y_e; the kernel wrote x_o
 }
 
 }  // namespace mg
