@@ -120,6 +120,8 @@ enum Epilogue { EPI_H = 0, EPI_CH = 1, EPI_XPAY = 2, EPI_CX_PAY = 3, EPI_C_XPAY 
 
 // threads per CTA of the one-site-per-thread kernels (wilson.cu)
 int site_block(long long sites);
+// whether the FP32 single-vector kernels take four lanes per site at this half volume
+bool dslash_lanes_f32(int Vh);
 // nrhs consecutive ABI vectors to and from packed half vectors `stride`
 // elements apart, one launch; even_only: odd sites are not read, zero_odd: odd
 // sites are written as zero

@@ -484,6 +484,54 @@ __global__ void __launch_bounds__(128) k_dslash(Geom g, int par0, HalfArgs<T> h,
                       par ? h.clov[1] : h.clov[0], par ? h.x[1] : h.x[0], a, dirmask);
 }
 
+// The same for lattices that do not fill the GPU: four lanes per site
+// (wilson_dev.cuh), 32 sites and 128 threads or 8 and 32 per CTA.
+template <typename T, int EPI>
+__global__ void __launch_bounds__(128) k_dslash_lanes(Geom g, int par0, HalfArgs<T> h, const T* __restrict__ gauge,
+                                                       T a) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = t & 1, b = (t >> 1) & 1, s = 2 * b + k;
+  const bool live = (t >> 2) < g.Vh;
+  const int i = live ? t >> 2 : g.Vh - 1;   // every lane takes part in the shuffles
+  const int par = par0 + blockIdx.y;
+  const T* clov = par ? h.clov[1] : h.clov[0];
+  const T* x = par ? h.x[1] : h.x[0];
+  cx<T> acc[3], xv[3], res[3];
+  if (EPI != EPI_H && EPI != EPI_CH) {
+#pragma unroll
+    for (int r = 0; r < 3; r++) xv[r] = SpinorIO<T>::get(x, g.Vh, i, 3 * s + r);
+  }
+  lane_hop_sum<T>(g, par ? h.in[1] : h.in[0], gauge, par, i, k, b, acc);
+  const T half = (T)-0.5, f = half * a;
+  if (EPI == EPI_H || EPI == EPI_CH) {
+#pragma unroll
+    for (int r = 0; r < 3; r++) res[r] = half * acc[r];
+    if (EPI == EPI_CH) {
+#pragma unroll
+      for (int r = 0; r < 3; r++) acc[r] = res[r];
+      lane_clover<T>(clov, g.Vh, i, k, b, acc, res);
+    }
+  } else if (EPI == EPI_CX_PAY) {
+    lane_clover<T>(clov, g.Vh, i, k, b, xv, res);
+#pragma unroll
+    for (int r = 0; r < 3; r++) res[r] = res[r] + f * acc[r];
+  } else {
+#pragma unroll
+    for (int r = 0; r < 3; r++) xv[r] = xv[r] + f * acc[r];
+    if (EPI == EPI_C_XPAY) {
+      lane_clover<T>(clov, g.Vh, i, k, b, xv, res);
+    } else {
+#pragma unroll
+      for (int r = 0; r < 3; r++) res[r] = xv[r];
+    }
+  }
+  if (live) {
+    T* out = par ? h.out[1] : h.out[0];
+#pragma unroll
+    for (int r = 0; r < 3; r++) SpinorIO<T>::put(out, g.Vh, i, 3 * s + r, res[r]);
+  }
+}
+
 // The epilogues of the multi-RHS kernels for the nr <= NR right-hand sides
 // r0 .. r0 + nr - 1 of site i (acc: the hop sums without the -1/2).
 template <typename T, int EPI, int NR>
@@ -565,9 +613,39 @@ __global__ void __launch_bounds__(BS, MINB) k_dslash_mrhs(Geom g, int par, int n
 // 960 sites).
 int site_block(long long sites) { return sites >= 128 * 152 * 6 ? 128 : sites >= 64 * 152 * 6 ? 64 : 32; }
 
+// Four lanes per site: in FP64 by the length of the busiest scheduler's chain
+// (608 schedulers; a warp of 32 sites is about 1320 FP64 instructions of 64
+// cycles each, one of 8 sites and four lanes each about 366: 43.6 -> 15.8 us for
+// both parities of 6x4x8x10).  In FP32 up to kLanesF32 sites of a parity, where
+// latency and not bandwidth sets the time: A^{-1} H takes 6.2 us with a thread
+// per site and 4.8 with four lanes at 4096 sites, 7.3 and 6.7 at 20736, 8.8 and
+// 9.6 at 32768, 13.8 and 19.2 at 65536.
+constexpr int kLanesF32 = 24576;
+template <typename T>
+bool lanes_per_site(int Vh) {
+  if (sizeof(T) == 4) return Vh <= kLanesF32;
+  const int warps = (Vh + 31) / 32;
+  return ((4 * warps + 607) / 608) * 366 < ((warps + 607) / 608) * 1320;
+}
+
+bool dslash_lanes_f32(int Vh) { return lanes_per_site<float>(Vh); }
+
 template <typename T>
 void dslash_halves(const Geom& g, Epilogue epi, int par0, int npar, const HalfArgs<T>& h, const T* gauge, double a,
                    int dirmask, cudaStream_t s) {
+  if (dirmask == 0xff && lanes_per_site<T>(g.Vh)) {
+    const int bl = site_block((long long)g.Vh * 4);
+    const dim3 nl((4 * g.Vh + bl - 1) / bl, npar);
+    switch (epi) {
+      case EPI_H: k_dslash_lanes<T, EPI_H><<<nl, bl, 0, s>>>(g, par0, h, gauge, (T)a); break;
+      case EPI_CH: k_dslash_lanes<T, EPI_CH><<<nl, bl, 0, s>>>(g, par0, h, gauge, (T)a); break;
+      case EPI_XPAY: k_dslash_lanes<T, EPI_XPAY><<<nl, bl, 0, s>>>(g, par0, h, gauge, (T)a); break;
+      case EPI_CX_PAY: k_dslash_lanes<T, EPI_CX_PAY><<<nl, bl, 0, s>>>(g, par0, h, gauge, (T)a); break;
+      case EPI_C_XPAY: k_dslash_lanes<T, EPI_C_XPAY><<<nl, bl, 0, s>>>(g, par0, h, gauge, (T)a); break;
+    }
+    MG_LAUNCH();
+    return;
+  }
   const int bs = site_block((long long)g.Vh * npar);
   const dim3 nb((g.Vh + bs - 1) / bs, npar);
   switch (epi) {
