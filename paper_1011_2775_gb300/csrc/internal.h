@@ -419,11 +419,12 @@ class Krylov {
   DBuf sc_;
 };
 
+// post-smoothing of the fine level in FP32 with the fused kernels of mr.cu:
+// z += MR_nu(b - D_r z); e, r, w, s, t scratch half vectors; d_scr receives the
+// last step's inner products
+void mr_post_smooth_fine(Ctx* c, float* z, const float* b, float* e, float* r, float* w, float* s, float* t, int nu,
+                         double* d_scr);
 // MR smoothing: e = MR_nu(A, r) from e = 0 (r is consumed as scratch)
-// nu MR steps on the fine D_r in FP32 with the fused kernels of mr.cu: e = the
-// correction (zeroed first), r the residual (updated), w, s, t scratch half
-// vectors; d_scr receives the last step's inner products
-void mr_smooth_fine(Ctx* c, float* e, float* r, float* w, float* s, float* t, int nu, double* d_scr);
 template <typename T>
 void mr_smooth(Ctx* c, const std::function<void(T*, const T*)>& A, T* e, T* r, T* w, size_t n, int nu,
                double* d_scr);

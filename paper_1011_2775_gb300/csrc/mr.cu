@@ -1,13 +1,16 @@
 // Minimal-residual smoothing on the fine level, fused (section "Adaptive
 // multigrid": the cycle's smoother; FP32, like the rest of the cycle).
 //
-// One MR step on D_r y = y - H_eo A_o^{-1} H_oe A_e^{-1} y with residual r:
-//   w = D_r r,  alpha = <w, r> / <w, w>,  e += alpha r,  r -= alpha w.
-// The unfused step runs five kernels (clover apply, two dslash, the two-dot
-// reduction, the update).  Here it runs three:
+// The post-smoothing z += MR_nu(b - D_r z) starts from the residual r = b - D_r z
+// of D_r y = y - H_eo A_o^{-1} H_oe A_e^{-1} y and takes nu steps
+//   w = D_r r,  alpha = <w, r> / <w, w>,  e += alpha r,  r -= alpha w,   then z += e.
+// Unfused, the residual takes five passes and a step five kernels (clover
+// apply, two dslash, the two-dot reduction, the update).  Here:
+//   k_mr_residual                  r_e = b_e - z_e + H_eo t_o, s_e = A_e^{-1} r_e
 //   k_dslash<EPI_CH>               t_o = A_o^{-1} H_oe s_e       (s_e = A_e^{-1} r_e)
 //   k_mr_dslash_dot                w_e = r_e - H_eo t_o, and <w, w>, <w, r>
 //   k_mr_update_clover             e += alpha r, r -= alpha w, s_e = A_e^{-1} r_e
+//   k_mr_finish                    z += e + alpha r (last step; its r is not needed)
 // The clover product A_e^{-1} r of the next step is taken from the update
 // (site-local), and the two inner products from the dslash epilogue (w and r
 // are in registers there).  Sums: FP32 per site (12 components), double-float
@@ -22,10 +25,11 @@ namespace {
 
 
 // w_e = r_e - H_eo t_o on even sites, with out[0] = <w, w>, out[1] + i out[2] =
-// <w, r> = sum conj(w) r.  One site per thread in CTAs of BS sites (site_block;
+// <w, r> = sum conj(w) r.  One site per thread in CTAs of BS sites (128 or 64;
 // grid-stride only where the partial sums would not fit): with 256 threads and
-// 96 registers two CTAs fitted an SM and 331776 sites took 96 us, 77.5 us with
-// FP64 sums at 80 registers.
+// 96 registers two CTAs fitted an SM and 331776 sites took 96 us, 60 us here.
+// CTAs of 32 leave the last one too many partial sums: 49152 sites took 17.3 us,
+// 65536 sites in CTAs of 64 14.0 us.
 template <int BS>
 __global__ void __launch_bounds__(BS, 640 / BS) k_mr_dslash_dot(Geom g, float* __restrict__ w, const float* __restrict__ t,
                                                               const float* __restrict__ gauge,
@@ -59,8 +63,85 @@ __global__ void __launch_bounds__(BS, 640 / BS) k_mr_dslash_dot(Geom g, float* _
   grid_sum<BS, 3>(v, partials, counter, out);
 }
 
-// e += alpha r, r -= alpha w (alpha = in[1..2] / in[0]), and s = A_e^{-1} r
-// of the updated r on even sites
+// The same with four lanes per site (wilson_dev.cuh), for small lattices (8.0 ->
+// 6.4 us at 4096 sites): CTAs of 128 threads, since every CTA is a partial sum
+// for the last one to add (8.6 us in CTAs of 32).
+__global__ void __launch_bounds__(128) k_mr_dslash_dot_lanes(Geom g, float* __restrict__ w,
+                                                             const float* __restrict__ t,
+                                                             const float* __restrict__ gauge,
+                                                             const float* __restrict__ r, double* partials,
+                                                             unsigned* counter, double* out) {
+  const int l = blockIdx.x * 128 + threadIdx.x;
+  const int k = l & 1, b = (l >> 1) & 1, sp = 2 * b + k;
+  const bool live = (l >> 2) < g.Vh;
+  const int i = live ? l >> 2 : g.Vh - 1;
+  cx<float> acc[3];
+  lane_hop_sum<float>(g, t, gauge, 0, i, k, b, acc);
+  float v[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const cx<float> rv = SpinorIO<float>::get(r, g.Vh, i, 3 * sp + q);
+    const cx<float> wv = mkc(rv.re + 0.5f * acc[q].re, rv.im + 0.5f * acc[q].im);
+    if (live) {
+      v[0] = fmaf(wv.re, wv.re, fmaf(wv.im, wv.im, v[0]));
+      v[1] = fmaf(wv.re, rv.re, fmaf(wv.im, rv.im, v[1]));
+      v[2] = fmaf(wv.re, rv.im, fmaf(-wv.im, rv.re, v[2]));
+      SpinorIO<float>::put(w, g.Vh, i, 3 * sp + q, wv);
+    }
+  }
+  grid_sum<128, 3>(v, partials, counter, out);
+}
+
+// r_e = b_e - z_e + H_eo t_o and s_e = A_e^{-1} r_e
+__global__ void __launch_bounds__(128) k_mr_residual(Geom g, float* __restrict__ r, float* __restrict__ s,
+                                                     const float* __restrict__ t, const float* __restrict__ gauge,
+                                                     const float* __restrict__ z, const float* __restrict__ b,
+                                                     const float* __restrict__ clov) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.Vh) return;
+  int c[4];
+  cb_coords(g, i, 0, c);
+  cx<float> acc[12], zv[12], bv[12], sv[12];
+#pragma unroll
+  for (int k = 0; k < 12; k++) acc[k] = mkc<float>(0.f, 0.f);
+  hop_sum<float>(g, t, gauge, 0, i, c, 0xff, acc);
+  SpinorIO<float>::load(z, g.Vh, i, zv);
+  SpinorIO<float>::load(b, g.Vh, i, bv);
+#pragma unroll
+  for (int k = 0; k < 12; k++)
+    bv[k] = mkc(bv[k].re - (zv[k].re + 0.5f * acc[k].re), bv[k].im - (zv[k].im + 0.5f * acc[k].im));
+  SpinorIO<float>::store(r, g.Vh, i, bv);
+  clover_mul<float>(clov, g.Vh, i, bv, sv);
+  SpinorIO<float>::store(s, g.Vh, i, sv);
+}
+
+__global__ void __launch_bounds__(128) k_mr_residual_lanes(Geom g, float* __restrict__ r, float* __restrict__ s,
+                                                           const float* __restrict__ t, const float* __restrict__ gauge,
+                                                           const float* __restrict__ z, const float* __restrict__ bb,
+                                                           const float* __restrict__ clov) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = l & 1, b = (l >> 1) & 1, sp = 2 * b + k;
+  const bool live = (l >> 2) < g.Vh;
+  const int i = live ? l >> 2 : g.Vh - 1;
+  cx<float> acc[3], rv[3], sv[3];
+  lane_hop_sum<float>(g, t, gauge, 0, i, k, b, acc);
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    const cx<float> zv = SpinorIO<float>::get(z, g.Vh, i, 3 * sp + q), bv = SpinorIO<float>::get(bb, g.Vh, i, 3 * sp + q);
+    rv[q] = mkc(bv.re - (zv.re + 0.5f * acc[q].re), bv.im - (zv.im + 0.5f * acc[q].im));
+  }
+  lane_clover<float>(clov, g.Vh, i, k, b, rv, sv);
+  if (!live) return;
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    SpinorIO<float>::put(r, g.Vh, i, 3 * sp + q, rv[q]);
+    SpinorIO<float>::put(s, g.Vh, i, 3 * sp + q, sv[q]);
+  }
+}
+
+// e += alpha r (e = alpha r on the first step), r -= alpha w (alpha = in[1..2] /
+// in[0]), and s = A_e^{-1} r of the updated r on even sites
+template <bool FIRST>
 __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restrict__ e, float* __restrict__ r,
                                                           const float* __restrict__ w, const double* __restrict__ in,
                                                           const float* __restrict__ clov, float* __restrict__ s) {
@@ -71,11 +152,12 @@ __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restr
   if (i >= g.Vh) return;
   const float ar = s_al[0], ai = s_al[1];
   cx<float> ev[12], rv[12], wv[12], sv[12];
-  SpinorIO<float>::load(e, g.Vh, i, ev);
+  if (!FIRST) SpinorIO<float>::load(e, g.Vh, i, ev);
   SpinorIO<float>::load(r, g.Vh, i, rv);
   SpinorIO<float>::load(w, g.Vh, i, wv);
 #pragma unroll
   for (int k = 0; k < 12; k++) {
+    if (FIRST) ev[k] = mkc(0.f, 0.f);
     ev[k].re += ar * rv[k].re - ai * rv[k].im;
     ev[k].im += ar * rv[k].im + ai * rv[k].re;
     rv[k].re -= ar * wv[k].re - ai * wv[k].im;
@@ -87,40 +169,82 @@ __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restr
   SpinorIO<float>::store(s, g.Vh, i, sv);
 }
 
+// z += e + alpha r (without e when FIRST), pairs of complex numbers
+template <bool FIRST>
+__global__ void __launch_bounds__(256) k_mr_finish(float4* __restrict__ z, const float4* __restrict__ e,
+                                                   const float4* __restrict__ r, const double* __restrict__ in, int n2) {
+  __shared__ float s_al[2];
+  if (threadIdx.x < 2) s_al[threadIdx.x] = (float)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
+  __syncthreads();
+  const float ar = s_al[0], ai = s_al[1];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += gridDim.x * blockDim.x) {
+    const float4 rv = r[i];
+    float4 zv = z[i];
+    float4 ev = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!FIRST) ev = e[i];
+    ev.x += ar * rv.x - ai * rv.y;
+    ev.y += ar * rv.y + ai * rv.x;
+    ev.z += ar * rv.z - ai * rv.w;
+    ev.w += ar * rv.w + ai * rv.z;
+    z[i] = make_float4(zv.x + ev.x, zv.y + ev.y, zv.z + ev.z, zv.w + ev.w);
+  }
+}
+
 }  // namespace
 
-void mr_smooth_fine(Ctx* c, float* e, float* r, float* w, float* s, float* t, int nu, double* d_scr) {
+void mr_post_smooth_fine(Ctx* c, float* z, const float* b, float* e, float* r, float* w, float* s, float* t, int nu,
+                         double* d_scr) {
   const Geom& g = c->g;
-  const size_t n = 12 * c->Vh;
   cudaStream_t st = c->stream;
-  blas_zero<float>(e, n, st);
   if (nu <= 0) return;
-  clover_apply<float>(g, s, r, c->Ainv<float>(0), st);   // s_e = A_e^{-1} r_e
+  const float* U = c->gauge<float>();
   const int bs = site_block(c->Vh);
-  const long long most = Workspace::kMaxBlocks * (long long)Workspace::kMaxResults / 3;   // three partial sums per CTA
-  const unsigned grid_dot = (unsigned)std::min<long long>(most, ((long long)c->Vh + bs - 1) / bs);
+  const unsigned sites = (unsigned)((c->Vh + bs - 1) / bs);
+  // four lanes per site by the rule of the dslash; partial sums: three per CTA
+  const bool lanes = dslash_lanes_f32(g.Vh);
+  const int bl = site_block(4 * (long long)c->Vh);
+  const unsigned grid_l = (unsigned)((4 * c->Vh + bl - 1) / bl);
+  const long long most = Workspace::kMaxBlocks * (long long)Workspace::kMaxResults / 3;
+  const unsigned grid_dot = (unsigned)std::min<long long>(most, bs == 128 ? sites : (c->Vh + 63) / 64);
+  double* part = c->ws.partials.as<double>();
+  unsigned* cnt = c->ws.counter.as<unsigned>();
   auto dslash_dot = [&]() {
-    double* part = c->ws.partials.as<double>();
-    unsigned* cnt = c->ws.counter.as<unsigned>();
-    const float* U = c->gauge<float>();
-    if (bs == 128)
+    if (lanes) {
+      k_mr_dslash_dot_lanes<<<(unsigned)((4 * c->Vh + 127) / 128), 128, 0, st>>>(g, w, t, U, r, part, cnt, d_scr);
+    } else if (bs == 128) {
       k_mr_dslash_dot<128><<<grid_dot, 128, 0, st>>>(g, w, t, U, r, part, cnt, d_scr);
-    else if (bs == 64)
+    } else {
       k_mr_dslash_dot<64><<<grid_dot, 64, 0, st>>>(g, w, t, U, r, part, cnt, d_scr);
-    else
-      k_mr_dslash_dot<32><<<grid_dot, 32, 0, st>>>(g, w, t, U, r, part, cnt, d_scr);
+    }
     MG_LAUNCH();
   };
-  for (int it = 0; it < nu; it++) {
-    dslash<float>(g, EPI_CH, 1, t, s, c->gauge<float>(), c->Ainv<float>(1), nullptr, 0.0, 0xff, st);
-    dslash_dot();
+  auto half_dr = [&]() {   // t_o = A_o^{-1} H_oe s_e
+    dslash<float>(g, EPI_CH, 1, t, s, U, c->Ainv<float>(1), nullptr, 0.0, 0xff, st);
     c->dslash_launches += 2;
+  };
+  clover_apply<float>(g, s, z, c->Ainv<float>(0), st);
+  half_dr();
+  if (lanes)
+    k_mr_residual_lanes<<<grid_l, bl, 0, st>>>(g, r, s, t, U, z, b, c->Ainv<float>(0));
+  else
+    k_mr_residual<<<sites, bs, 0, st>>>(g, r, s, t, U, z, b, c->Ainv<float>(0));
+  MG_LAUNCH();
+  for (int it = 0; it < nu; it++) {
+    half_dr();
+    dslash_dot();
     if (it + 1 < nu) {
-      k_mr_update_clover<<<(c->Vh + bs - 1) / bs, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s);
-      MG_LAUNCH();
+      if (it == 0)
+        k_mr_update_clover<true><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s);
+      else
+        k_mr_update_clover<false><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s);
     } else {
-      blas_mr_update<float>(e, r, w, d_scr, n, st);
+      const int n2 = (int)(6 * c->Vh), grid = (int)std::min<long long>(152 * 8, (n2 + 255) / 256);
+      if (it == 0)
+        k_mr_finish<true><<<grid, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
+      else
+        k_mr_finish<false><<<grid, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
     }
+    MG_LAUNCH();
   }
 }
 

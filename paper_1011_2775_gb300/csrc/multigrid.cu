@@ -243,14 +243,13 @@ void cycle(Ctx* c, Hierarchy& H, int l, float* z, const float* r) {
   } else {
     prolong_vec(T, z, W.ec.as<float>(), true, s);
   }
-  if (p.nu_post > 0) {
+  if (p.nu_post > 0 && l == 0) {   // fused fine-level smoothing
+    mr_post_smooth_fine(c, z, r, e, res, w, H.F32->t1.as<float>(), H.F32->t2.as<float>(), p.nu_post, scr);
+  } else if (p.nu_post > 0) {
     Dr(w, z);
     blas_convert<float, float>(res, r, n, s);
     blas_axpby<float>(-1.0, w, 1.0, res, n, s);
-    if (l == 0)   // fused fine-level steps (three kernels per step)
-      mr_smooth_fine(c, e, res, w, H.F32->t1.as<float>(), H.F32->t2.as<float>(), p.nu_post, scr);
-    else
-      mr_smooth<float>(c, Dr, e, res, w, n, p.nu_post, scr);
+    mr_smooth<float>(c, Dr, e, res, w, n, p.nu_post, scr);
     blas_axpby<float>(1.0, e, 1.0, z, n, s);
   }
 }
