@@ -920,9 +920,145 @@ __global__ void __launch_bounds__(256) k_coarse_hop(HopArgs h) {
     }
 }
 
+// Rows of the link blocks without a site matrix: out = L in (+ x): CTA = (site,
+// 16 rows), a warp owns two rows.  The links do not depend on the gathered
+// vector, so their first steps are in flight before it is: two dependent trips
+// to L2 (neighbour index, vector) instead of three.  A single direction reads
+// that direction's columns only.
+struct RowArgs {
+  int nc, s0, lbase;         // link blocks of site s at (s - lbase) nc rows
+  int q0, q1;                // pairs of columns of a row to use
+  const int* nbr;
+  const void* L;
+  const float* Ls;           // tile scales, or null
+  float2* out;
+  const float2* in;
+  const float2* x;
+  float a;
+};
+constexpr int kRowSteps = 6;   // link steps in flight per lane and row (192 pairs: Nc = 48)
+template <int ST, bool XPAY>
+__global__ void __launch_bounds__(256) k_coarse_rows(RowArgs h) {
+  extern __shared__ __align__(16) float4 vp[];   // [4 nc] pairs of the gathered vector
+  using raw = typename LinkPair<ST>::raw;
+  const int nc = h.nc, hc = nc >> 1, K2 = 8 * hc, s = h.s0 + blockIdx.x;
+  const int lane = threadIdx.x & 31, i0 = blockIdx.y * 16 + 2 * (threadIdx.x >> 5);
+  const char* row[2];
+  raw m[kRowSteps][2];
+#pragma unroll
+  for (int r = 0; r < 2; r++)
+    row[r] = static_cast<const char*>(h.L) + ((size_t)(s - h.lbase) * nc + min(i0 + r, nc - 1)) * K2 * sizeof(raw);
+  auto load = [&](int qb) {
+#pragma unroll
+    for (int u = 0; u < kRowSteps; u++)
+#pragma unroll
+      for (int r = 0; r < 2; r++) {
+        const int q = qb + lane + 32 * u;
+        m[u][r] = q < h.q1 ? LinkPair<ST>::load(row[r], q) : LinkPair<ST>::zero();
+      }
+  };
+  load(h.q0);
+  for (int t = h.q0 + threadIdx.x; t < h.q1; t += blockDim.x) {
+    const int d = t / hc, j = t - d * hc;
+    const float sc = h.Ls ? h.Ls[(size_t)s * 8 + d] : 1.f;
+    const float4 v = reinterpret_cast<const float4*>(h.in + (size_t)h.nbr[(size_t)s * 8 + d] * nc)[j];
+    vp[t] = make_float4(sc * v.x, sc * v.y, sc * v.z, sc * v.w);
+  }
+  __syncthreads();
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int qb = h.q0; qb < h.q1; qb += 32 * kRowSteps) {
+    if (qb > h.q0) load(qb);
+#pragma unroll
+    for (int u = 0; u < kRowSteps; u++) {
+      const int q = qb + lane + 32 * u;
+      if (q < h.q1) {
+        const float4 x = vp[q];
+#pragma unroll
+        for (int r = 0; r < 2; r++) {
+          const float4 l = LinkPair<ST>::decode(m[u][r]);
+          acc[2 * r] = fmaf(l.x, x.x, fmaf(-l.y, x.y, fmaf(l.z, x.z, fmaf(-l.w, x.w, acc[2 * r]))));
+          acc[2 * r + 1] = fmaf(l.x, x.y, fmaf(l.y, x.x, fmaf(l.z, x.w, fmaf(l.w, x.z, acc[2 * r + 1]))));
+        }
+      }
+    }
+  }
+  const float t = warp_transpose_sum<4>(acc);   // lane l: value l >> 3 = 2 row + {re, im}
+  const float im = __shfl_down_sync(0xffffffffu, t, 8);
+  const int r = lane >> 4;
+  if ((lane & 15) == 0 && i0 + r < nc) {
+    const size_t i = (size_t)s * nc + i0 + r;
+    float2 o = make_float2(t, im);
+    if (XPAY) {
+      const float2 x = h.x[i];
+      o = make_float2(x.x + h.a * o.x, x.y + h.a * o.y);
+    }
+    h.out[i] = o;
+  }
+}
+
+namespace {
+void launch_rows(const RowArgs& h, int sites, int store, bool xpay, cudaStream_t s) {
+  const dim3 grid(sites, (h.nc + 15) / 16);
+  const size_t sm = sizeof(float2) * 8 * (size_t)h.nc;
+  auto run = [&](auto st) {
+    constexpr int ST = decltype(st)::value;
+    if (xpay)
+      k_coarse_rows<ST, true><<<grid, 256, sm, s>>>(h);
+    else
+      k_coarse_rows<ST, false><<<grid, 256, sm, s>>>(h);
+  };
+  switch (store) {
+    case STORE_F32: run(std::integral_constant<int, kStF32>()); break;
+    case STORE_F16: run(std::integral_constant<int, kStF16>()); break;
+    default: run(std::integral_constant<int, kStBF16>()); break;
+  }
+  MG_LAUNCH();
+}
+}  // namespace
+
+void coarse_folded(const LevelGeom& G, const CoarseOp& C, float* out, const float* in, const float* x, float a,
+                   cudaStream_t s) {
+  if (!G.eo || !C.A.get()) raise(MG_ERR_STATE, "no folded links on this level");
+  RowArgs h;
+  h.nc = C.nc;
+  h.s0 = h.lbase = G.half;
+  h.q0 = 0;
+  h.q1 = 4 * C.nc;
+  h.nbr = G.d_nbr.as<int>();
+  h.L = C.A.get();
+  h.Ls = nullptr;
+  h.out = (float2*)out;
+  h.in = (const float2*)in;
+  h.x = (const float2*)x;
+  h.a = a;
+  launch_rows(h, G.nsites - G.half, STORE_F32, x != nullptr, s);
+}
+
 void coarse_hop(const LevelGeom& G, const CoarseOp& C, Epilogue epi, bool use_inv, int s0, int s1, float* out,
                 const float* in, const float* x, float a, int dirmask, cudaStream_t s) {
   if (s1 <= s0) return;
+  if (epi == EPI_H || epi == EPI_XPAY) {
+    const bool single = (dirmask & (dirmask - 1)) == 0;
+    if (dirmask == 0xff || (single && dirmask)) {
+      RowArgs r;
+      r.nc = C.nc;
+      r.s0 = s0;
+      r.lbase = 0;
+      int d = 0;
+      while (single && dirmask >> (d + 1)) d++;
+      r.q0 = single ? d * (C.nc / 2) : 0;
+      r.q1 = single ? r.q0 + C.nc / 2 : 4 * C.nc;
+      r.nbr = G.d_nbr.as<int>();
+      r.L = C.Y.get();
+      r.Ls = C.Yscale.as<float>();
+      r.out = (float2*)out;
+      r.in = (const float2*)in;
+      r.x = (const float2*)x;
+      r.a = a;
+      launch_rows(r, s1 - s0, C.store, epi == EPI_XPAY, s);
+      return;
+    }
+  }
   HopArgs h;
   h.nc = C.nc;
   h.s0 = s0;

@@ -73,7 +73,8 @@ struct CoarseOp {
   DBuf Y;                  // [site][nc][8][nc] in `store` format
   DBuf Yscale;             // float[site][8]: per (site, direction) scale
   DBuf X, Xinv;            // [site][nc][nc] complex FP32
-  // Links with the site inverses folded in, for the persistent coarsest solve:
+  // Links with the site inverses folded in, for the persistent coarsest solve
+  // and the solver's D_r on intermediate levels:
   //  even-odd levels: A[o - half][nc][8][nc] = X_o^{-1} Y_d(o) X^{-1}(o + d) on odd
   //  sites, so that (X_o^{-1} Y_oe X_e^{-1} y)(o) = sum_d A_d(o) y(o + d);
   //  other levels: [site][nc][9][nc] = [Y_0 .. Y_7 | X], so D_hat v is one GEMV.
@@ -121,6 +122,10 @@ void galerkin_project(const TransferOp& T, CoarseOp& C, const float* const W[8],
 // s in [s0, s1); epilogues as the fine dslash (EPI_*), C = X or Xinv.
 void coarse_hop(const LevelGeom& G, const CoarseOp& C, Epilogue epi, bool use_inv, int s0, int s1, float* out,
                 const float* in, const float* x, float a, int dirmask, cudaStream_t s);
+// out_o = A in_e (+ x_o: out_o = x_o + a A in_e) on the odd sites of an even-odd
+// level with its folded links A = X_o^{-1} Y_oe X_e^{-1} (full-vector bases)
+void coarse_folded(const LevelGeom& G, const CoarseOp& C, float* out, const float* in, const float* x, float a,
+                   cudaStream_t s);
 // out[s] = C(s) in[s] (+ a x[s] if x) for s in [s0, s1)
 void coarse_site_mul(const LevelGeom& G, const CoarseOp& C, bool use_inv, int s0, int s1, float* out, const float* in,
                      cudaStream_t s);

@@ -150,11 +150,22 @@ size_t half_n(const Hierarchy& H, int l) {
 size_t full_n(const Hierarchy& H, int l) { return H.geo[l].vec_complex(); }
 
 // ----- level operators (FP32); vectors are full-vector base pointers, even sites first
+// D_r as the solver applies it: on coarse levels y_e - Y_eo (A y_e) with the
+// folded links A = X_o^{-1} Y_oe X_e^{-1} (two kernels, no site inverses)
 void Dr_level(Ctx* c, Hierarchy& H, int l, float* out, const float* in) {
   if (l == 0) {
     H.F32->Dr(out, in);
     return;
   }
+  const LevelGeom& G = H.geo[l];
+  const CoarseOp& C = H.cop[l];
+  float* tB = H.work[l].tB.as<float>();
+  coarse_folded(G, C, tB, in, nullptr, 0.f, c->stream);
+  coarse_hop(G, C, EPI_XPAY, false, 0, G.half, out, tB, in, -1.f, 0xff, c->stream);
+}
+
+// the same from the stored links and site inverses (mg_apply)
+void Dr_unfolded(Ctx* c, Hierarchy& H, int l, float* out, const float* in) {
   const LevelGeom& G = H.geo[l];
   const CoarseOp& C = H.cop[l];
   LevelWork& W = H.work[l];
@@ -504,7 +515,7 @@ void build_coarse_links(Ctx* c, Hierarchy& H, int l) {
   coarse_invert(Gc, C, c->ws.flags.as<int>(), s);
   if (c->read_flag(FLAG_SINGULAR, true)) raise(MG_ERR_SINGULAR_CLOVER, "singular coarse diagonal block");
   quantize_links(Gc, C, T.store, s);               // 16-bit storage of Y (FP32: no-op)
-  if (l + 2 == H.L) coarse_fold_links(Gc, C, s);  // the coarsest level runs the persistent solver
+  if (l + 2 == H.L || Gc.eo) coarse_fold_links(Gc, C, s);
 }
 
 void alloc_work(Ctx* c, Hierarchy& H) {
@@ -923,9 +934,9 @@ void mg_benchmark_coarse(Ctx* c, int warmup, int iters, double* avg_ms, double* 
   cudaEvent_t e0, e1;
   MG_CUDA(cudaEventCreate(&e0));
   MG_CUDA(cudaEventCreate(&e1));
-  for (int w = 0; w < warmup; w++) Dr_level(c, H, 1, ob.as<float>(), ib.as<float>());
+  for (int w = 0; w < warmup; w++) Dr_unfolded(c, H, 1, ob.as<float>(), ib.as<float>());
   MG_CUDA(cudaEventRecord(e0, c->stream));
-  for (int it = 0; it < iters; it++) Dr_level(c, H, 1, ob.as<float>(), ib.as<float>());
+  for (int it = 0; it < iters; it++) Dr_unfolded(c, H, 1, ob.as<float>(), ib.as<float>());
   MG_CUDA(cudaEventRecord(e1, c->stream));
   MG_CUDA(cudaEventSynchronize(e1));
   float t = 0;
@@ -1210,7 +1221,7 @@ void mg_apply_level(Ctx* c, int op, int level, double* out_abi, const double* in
     case MG_OP_HOP: coarse_hop(G, H.cop[level], EPI_H, false, 0, G.nsites, out, in, nullptr, 0.f, 0xff, s); break;
     case MG_OP_DR:
       if (!G.eo) raise(MG_ERR_DIMS, "level has an odd extent");
-      Dr_level(c, H, level, out, in);
+      Dr_unfolded(c, H, level, out, in);
       break;
     case MG_OP_BR:
       if (!G.eo) raise(MG_ERR_DIMS, "level has an odd extent");
