@@ -11,7 +11,7 @@
 //    phase A uses the folded odd-site links X_o^{-1} Y_d X^{-1}(o + d) (FP32),
 //    phase B the even-site links Y_eo in their storage format.  Every block
 //    owns a fixed, contiguous range of A items and of B items, and warp w of
-//    the block takes every sixteenth item of each range.
+//    the block takes every W-th item of each range (W = 16 or 8 warps).
 //  * The links do not change during the solve, so the order in which a warp
 //    consumes them is known in advance: its B items (for b_r), then its A
 //    items and B items once per operator application.  Each warp keeps two
@@ -44,10 +44,14 @@
 // 427 us at 24^3x48 with bf16 links).
 //
 // Measured (16^3x32, 4^4 blocks, Nc = 48, 256 reduced sites, 35 iterations):
-// 817 us per solve with 256 threads, neighbour indices read for every gather
-// and the coefficients formed before the sums; 744 us here.  An iteration is
-// 45k cycles: the stencil passes 9.4k and 10.1k, the gathers 1.4k each, the
-// barriers 9.3k, the inner products, totals and update 11k.
+// 817 us per solve with 256 threads, neighbour indices read for every gather,
+// the coefficients formed before the sums, divisions and a switch over the rows
+// of every item, and r and w read back from global memory; 640 us here.  Of the
+// 38k cycles of an iteration the stencil passes take 6.6k each (shared-memory
+// port: every link byte is written and read there, every gathered vector read
+// once per two rows), the gathers 1.5k each, the barriers 9k, inner products,
+// totals, coefficients and update 12k.  24^3x48 with bf16 links: 427 -> 290 us;
+// the links come from HBM and phase A runs at its rate (191 MB in 28.6 us).
 #include <algorithm>
 #include <cstring>
 
@@ -60,12 +64,8 @@ namespace mg {
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
 constexpr int kStagesPerWarp = 2;
-constexpr int kStages = kWarps * kStagesPerWarp;
 constexpr int kMaxRows = 8;        // rows of one item (16 accumulators per lane)
-constexpr int kUpdThreads = kThreads - 32;   // warp 0 forms the coefficients meanwhile
 constexpr int kMaxGroups = 8;      // thread groups sharing the sum over j of the Gram-Schmidt update
 constexpr int kMaxRestart = 64;
 // reduction slots: [0, 2 kMaxRestart) <w_j, w>; then ||w||^2, Re/Im <w, r>;
@@ -81,6 +81,7 @@ struct SArgs {
   int nc, half, m, maxit;
   int rowsA, rowsB, ipsA, ipsB, NA, NB, eszB;
   int stage_bytes, gmax, wsm_ld;   // wsm_ld > 0: the w_j slice in shared memory, leading dimension
+  int esm;                         // > 0: r and w of the owned rows in shared memory, their capacity
   double tol_rel;
   const int* nbr;
   const unsigned char* Y;     // even-site links [e][nc][8][nc], storage format
@@ -93,6 +94,7 @@ struct SArgs {
   float2* r;                  // half: residual
   float2* br;                 // half: reduced right-hand side
   float2* tB;                 // full: the odd part holds the phase-A outputs
+  float2* w;                  // half: D_r r, when the owned rows are not in shared memory
   float2* W;                  // [m][half nc] (when the slice is not in shared memory)
   float2* Z;                  // [m][half nc]
   float2* partials;           // [kNR][grid] double-float partial sums
@@ -107,56 +109,58 @@ __device__ __forceinline__ size_t item_elem(int i, int ips, int rows, int nc) {
   return (size_t)(i / ips) * nc + (size_t)(i % ips) * rows;
 }
 
-// Per-warp state of the link stream.
-struct Stream {
-  unsigned char* ring;
-  uint64_t* full;
-  int a0, a1, b0, b1;    // the block's item ranges
-  int cA, cB;            // this warp's items per A phase and per B phase
-  long long t;           // this warp's next sequence position (uniform in the warp)
+// A block's items [i0, i1) of one phase: this warp's are i0 + wid, i0 + wid + W,
+// ...; sl and rem: site (from the block's first) and item of the site of the
+// warp's first item, dq and dr their steps (no division per item).
+struct Items {
+  int i0, i1, ips, sl, rem, dq, dr;
+  __device__ Items(int b, int G, int n, int ips_, int W, int wid) : ips(ips_) {
+    i0 = (int)((long long)b * n / G);
+    i1 = (int)((long long)(b + 1) * n / G);
+    const int first = i0 + wid;
+    sl = first / ips - i0 / ips;
+    rem = first % ips;
+    dq = W / ips;
+    dr = W % ips;
+  }
+  __device__ int site0() const { return i0 / ips; }
+  __device__ int sites() const { return i1 > i0 ? (i1 - 1) / ips - i0 / ips + 1 : 0; }
 };
 
-// warp sequence position -> (kind 0: A, 1: B, item index)
-__device__ __forceinline__ void seq_item(const Stream& st, long long p, int& kind, int& it) {
-  const int w = threadIdx.x >> 5;
-  if (p < st.cB) {
-    kind = 1;
-    it = st.b0 + w + kWarps * (int)p;
-    return;
-  }
-  const long long q = p - st.cB;
-  const int off = (int)(q % (st.cA + st.cB));
-  if (off < st.cA) {
-    kind = 0;
-    it = st.a0 + w + kWarps * off;
-  } else {
-    kind = 1;
-    it = st.b0 + w + kWarps * (off - st.cA);
-  }
-}
+// rows of a phase-B item: the bytes of R rows of phase A
+__host__ __device__ constexpr int rows_b(int st, int R) { return st == kStF32 || R == 0 ? R : 2 * R < kMaxRows ? 2 * R : kMaxRows; }
 
-// lane 0: bulk copy of the item at warp position p into its stage
-__device__ __forceinline__ void issue(const SArgs& a, const Stream& st, long long p) {
-  if (st.cA + st.cB == 0) return;
-  int kind, it;
-  seq_item(st, p, kind, it);
-  const int nc = a.nc, K = 8 * nc;
-  const unsigned char* src;
-  unsigned bytes;
-  if (kind == 0) {
-    const int s = it / a.ipsA, r0 = (it % a.ipsA) * a.rowsA;
-    const int nr = min(a.rowsA, nc - r0);
-    src = a.Af + ((size_t)s * nc + r0) * K * 8;
-    bytes = (unsigned)(nr * K * 8);
-  } else {
-    const int s = it / a.ipsB, r0 = (it % a.ipsB) * a.rowsB;
-    const int nr = min(a.rowsB, nc - r0);
-    src = a.Y + ((size_t)s * nc + r0) * K * a.eszB;
-    bytes = (unsigned)(nr * K * a.eszB);
+// Per-warp state of the link stream: items consumed, and the next one to copy.
+struct Stream {
+  unsigned char* ring;   // this warp's stages
+  uint64_t* full;
+  unsigned t;            // items consumed
+  int kind, it;          // next item to copy: 0 A, 1 B
+};
+
+// lane 0: bulk copy of the next item of the sequence into stage `slot`, and on
+// to the one after it (the warp's B items for b_r, then A and B alternately)
+template <int W>
+__device__ __forceinline__ void issue(const SArgs& a, Stream& st, const Items& A, const Items& B, unsigned slot) {
+  const int wid = threadIdx.x >> 5;
+  for (int tries = 0; tries < 2 && st.it >= (st.kind ? B.i1 : A.i1); tries++) {   // a phase without items is passed over
+    st.kind ^= 1;
+    st.it = (st.kind ? B.i0 : A.i0) + wid;
   }
-  const int stage = (threadIdx.x >> 5) * kStagesPerWarp + (int)(p % kStagesPerWarp);
-  mbar_arrive_expect_tx(&st.full[stage], bytes);
-  bulk_copy_g2s(st.ring + (size_t)stage * a.stage_bytes, src, bytes, &st.full[stage]);
+  if (st.it >= (st.kind ? B.i1 : A.i1)) return;
+  const int nc = a.nc, rows = st.kind ? a.rowsB : a.rowsA, ips = st.kind ? a.ipsB : a.ipsA;
+  size_t row0 = (size_t)st.it * rows;
+  int nr = rows;
+  if (ips * rows != nc) {   // the last item of a site is short
+    const int s = st.it / ips, r0 = (st.it - s * ips) * rows;
+    row0 = (size_t)s * nc + r0;
+    nr = min(rows, nc - r0);
+  }
+  const unsigned per = 8u * nc * (st.kind ? a.eszB : 8);
+  const unsigned bytes = nr * per;
+  mbar_arrive_expect_tx(&st.full[slot], bytes);
+  bulk_copy_g2s(st.ring + (size_t)slot * a.stage_bytes, (st.kind ? a.Y : a.Af) + row0 * per, bytes, &st.full[slot]);
+  st.it += W;
 }
 
 // Gathers the vectors of the block's `ns` sites of a phase: for each site, the
@@ -165,7 +169,8 @@ __device__ __forceinline__ void issue(const SArgs& a, const Stream& st, long lon
 // 16 bytes per lane, the loads of kGather pairs in flight together: one L2
 // round trip for a block of up to eight sites.
 constexpr int kGather = 4;
-__device__ void gather(int nc, int ns, const int* nbr, const float* scale, const float2* in, float2* gv) {
+template <int kWarps>
+__device__ __forceinline__ void gather(int nc, int ns, const int* nbr, const float* scale, const float2* in, float2* gv) {
   const int nc2 = nc >> 1, np = 8 * ns, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float4* g4 = reinterpret_cast<float4*>(gv);
   for (int p0 = w; p0 < np; p0 += kGather * kWarps)
@@ -220,12 +225,8 @@ __device__ __forceinline__ bool item_rows(const unsigned char* stage, int K, con
       acc[2 * r + 1] = fmaf(m.w, x.z, acc[2 * r + 1]);
     }
   };
-  int q = lane;
-  for (; q + 32 < K2; q += 64) {
-    step(q);
-    step(q + 32);
-  }
-  if (q < K2) step(q);
+#pragma unroll 3
+  for (int q = lane; q < K2; q += 32) step(q);
   const float t = warp_transpose_sum<V>(acc);                       // lane l: value (l >> SH) & (V - 1)
   const float im = __shfl_down_sync(0xffffffffu, t, 1 << SH);  // value 2 row + 1
   res = make_float2(t, im);
@@ -233,53 +234,35 @@ __device__ __forceinline__ bool item_rows(const unsigned char* stage, int K, con
   return (lane & ((2 << SH) - 1)) == 0 && row < NR;
 }
 
-template <int ST>
-__device__ __forceinline__ bool item_rows_n(int nr, const unsigned char* stage, int K, const float2* v, float2& res,
-                                            int& row) {
-  switch (nr) {
-    case 1: return item_rows<ST, 1>(stage, K, v, res, row);
-    case 2: return item_rows<ST, 2>(stage, K, v, res, row);
-    case 3: return item_rows<ST, 3>(stage, K, v, res, row);
-    case 4: return item_rows<ST, 4>(stage, K, v, res, row);
-    case 5: return item_rows<ST, 5>(stage, K, v, res, row);
-    case 6: return item_rows<ST, 6>(stage, K, v, res, row);
-    case 7: return item_rows<ST, 7>(stage, K, v, res, row);
-    default: return item_rows<ST, 8>(stage, K, v, res, row);
-  }
-}
-
 // One phase of this warp's items: waits for each staged item, computes its
-// rows, hands row results to epi(kind-specific index, row value) and refills
-// the stage two positions ahead.  false on a timeout (uniform in the block
-// after the closing barrier).
-template <int ST, typename Epi>
-__device__ bool run_items(const SArgs& a, Stream& st, int kind, const float2* gv, Epi epi, int* s_fail) {
-  const int nc = a.nc, K = 8 * nc;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i0 = kind ? st.b0 : st.a0, i1 = kind ? st.b1 : st.a1;
-  const int ips = kind ? a.ipsB : a.ipsA, rows = kind ? a.rowsB : a.rowsA;
-  const int sbase = i0 / ips;
-  bool ok = true;
-  for (int it = i0 + w; it < i1; it += kWarps) {
-    const int stage = w * kStagesPerWarp + (int)(st.t % kStagesPerWarp);
-    const unsigned par = (unsigned)((st.t / kStagesPerWarp) & 1);
-    if (!mbar_wait(&st.full[stage], par)) {
-      ok = false;
+// rows, hands them to epi(element from the block's first site, row value) and
+// refills the stage two items ahead.  false on a timeout (uniform in the block).
+template <int ST, int NR, int W, typename Epi>
+__device__ __forceinline__ bool run_items(const SArgs& a, Stream& st, const Items& A, const Items& B, const Items& g,
+                                          const float2* gv, Epi epi, int* s_fail) {
+  const int nc = a.nc, K = 8 * nc, lane = threadIdx.x & 31;
+  int sl = g.sl, rem = g.rem;
+  for (int it = g.i0 + (threadIdx.x >> 5); it < g.i1; it += W) {
+    const unsigned slot = st.t % kStagesPerWarp;
+    if (!mbar_wait(&st.full[slot], (st.t / kStagesPerWarp) & 1u)) {
+      atomicExch(s_fail, 1);
       break;
     }
-    const int s = it / ips, r0 = (it % ips) * rows;
-    const int nr = min(rows, nc - r0);
+    const int r0 = rem * NR;
     float2 res;
-    int row;
-    const unsigned char* sp = st.ring + (size_t)stage * a.stage_bytes;
-    const float2* vp = gv + (size_t)(s - sbase) * K;
-    const bool mine = kind == 0 ? item_rows_n<kStF32>(nr, sp, K, vp, res, row) : item_rows_n<ST>(nr, sp, K, vp, res, row);
-    if (mine) epi((size_t)s * nc + r0 + row, res);
+    int row;   // rows past the site's last are not copied; what their sums hold is dropped
+    const bool mine = item_rows<ST, NR>(st.ring + (size_t)slot * a.stage_bytes, K, gv + (size_t)sl * K, res, row);
     __syncwarp();
-    if (lane == 0) issue(a, st, st.t + kStagesPerWarp);
+    if (lane == 0) issue<W>(a, st, A, B, slot);
+    if (mine && r0 + row < nc) epi(sl * nc + r0 + row, res);
     st.t++;
+    sl += g.dq;
+    rem += g.dr;
+    if (rem >= g.ips) {
+      rem -= g.ips;
+      sl++;
+    }
   }
-  if (!ok) atomicExch(s_fail, 1);
   __syncthreads();
   return *(volatile int*)s_fail == 0;
 }
@@ -287,7 +270,8 @@ __device__ bool run_items(const SArgs& a, Stream& st, int kind, const float2* gv
 // block partial sums of nq <= 4 per-thread float values v[q]: one transposed
 // warp reduction for the four, then warp q adds the warps' sums of value q;
 // partials[q0 + q][block]
-__device__ void block_partials(const SArgs& a, const float* v, int nq, int q0, df* sred) {
+template <int kWarps>
+__device__ __forceinline__ void block_partials(const SArgs& a, const float* v, int nq, int q0, df* sred) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   df t[4];
 #pragma unroll
@@ -303,12 +287,12 @@ __device__ void block_partials(const SArgs& a, const float* v, int nq, int q0, d
 }
 
 // totals of slots [q0, q0 + nq) after a grid barrier, identical in every
-// block.  Warp w sums slots w, w + 16, ...; each round issues the loads of U
+// block.  Warp w sums slots w, w + kWarps, ...; each round issues the loads of U
 // slots (up to kTotG / 32 per lane and slot) before adding any, so that a
 // round costs one L2 round trip; the U sums leave the warp through one
 // transposing reduction.
 constexpr int kTotG = 160;   // grids up to this size take the one-pass path
-template <int U>
+template <int U, int kWarps>
 __device__ __forceinline__ void totals_rounds(const SArgs& a, int q0, int nq, df* out) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int G = gridDim.x;
@@ -336,16 +320,17 @@ __device__ __forceinline__ void totals_rounds(const SArgs& a, int q0, int nq, df
     if (lane % (32 / U) == 0 && q < nq) out[q] = s;
   }
 }
-__device__ void grid_totals(const SArgs& a, int q0, int nq, df* out) {
+template <int kWarps>
+__device__ __forceinline__ void grid_totals(const SArgs& a, int q0, int nq, df* out) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int G = gridDim.x;
   if (G <= kTotG) {
     if (nq <= kWarps)
-      totals_rounds<1>(a, q0, nq, out);
+      totals_rounds<1, kWarps>(a, q0, nq, out);
     else if (nq <= 4 * kWarps)
-      totals_rounds<4>(a, q0, nq, out);
+      totals_rounds<4, kWarps>(a, q0, nq, out);
     else
-      totals_rounds<8>(a, q0, nq, out);
+      totals_rounds<8, kWarps>(a, q0, nq, out);
   } else {
     for (int q = wid; q < nq; q += kWarps) {
       const float2* p = a.partials + (size_t)(q0 + q) * G;
@@ -361,43 +346,54 @@ __device__ void grid_totals(const SArgs& a, int q0, int nq, df* out) {
   __syncthreads();
 }
 
-template <int ST>
-__global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
+// What the next pass over the links is for: b_r at the start, w = D_r r of an
+// iteration, or the true residual that closes a restart cycle.  One loop and
+// one copy of the two stencil phases serve all three: the code of an iteration
+// is fetched again every time round.
+enum { M_INIT, M_ITER, M_CLOSE };
+
+// W warps, R rows per item of phase A (phase B, 16-bit links: 2 R)
+template <int ST, int W, int R>
+__global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_constant__ SArgs a) {
+  constexpr int kThreads = 32 * W, kUpdThreads = kThreads - 32;   // warp 0 forms the coefficients meanwhile
+  constexpr int RB_ = rows_b(ST, R);
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) uint64_t full[kStages];
+  __shared__ __align__(8) uint64_t full[W * kStagesPerWarp];
   __shared__ float s_coef[4];              // 1/gamma, Re alpha, Im alpha, exact flag
   __shared__ int s_fail;
   const int nc = a.nc, K = 8 * nc, m = a.m;
   const int G = gridDim.x, bid = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float2* gv = reinterpret_cast<float2*>(smem + (size_t)kStages * a.stage_bytes);
+  float2* gv = reinterpret_cast<float2*>(smem + (size_t)W * kStagesPerWarp * a.stage_bytes);
   float2* upd = gv + (size_t)a.gmax * K;                               // [2][kThreads] update partial sums
   float2* wsm = upd + 2 * kThreads;                                    // [m][wsm_ld] when used
-  df* sred = reinterpret_cast<df*>(wsm + (size_t)m * a.wsm_ld);        // [4][kWarps]
-  df* tot = sred + 4 * kWarps;                                         // [kNR]
+  float2* esm = wsm + (size_t)m * a.wsm_ld;                            // [2][esm] when used
+  df* sred = reinterpret_cast<df*>(esm + 2 * (size_t)a.esm);           // [4][W]
+  df* tot = sred + 4 * W;                                              // [kNR]
   int* nbA = reinterpret_cast<int*>(tot + kNR);                        // [gmax][8] neighbours of the A sites,
   int* nbB = nbA + 8 * a.gmax;                                         // of the B sites,
   float* scB = reinterpret_cast<float*>(nbB + 8 * a.gmax);             // and the tile scales of the B sites
 
+  const Items A(bid, G, a.NA, a.ipsA, W, wid), B(bid, G, a.NB, a.ipsB, W, wid);
   Stream st;
-  st.ring = smem;
-  st.full = full;
-  st.a0 = (int)((long long)bid * a.NA / G);
-  st.a1 = (int)((long long)(bid + 1) * a.NA / G);
-  st.b0 = (int)((long long)bid * a.NB / G);
-  st.b1 = (int)((long long)(bid + 1) * a.NB / G);
-  st.cA = st.a1 - st.a0 > wid ? (st.a1 - st.a0 - wid + kWarps - 1) / kWarps : 0;
-  st.cB = st.b1 - st.b0 > wid ? (st.b1 - st.b0 - wid + kWarps - 1) / kWarps : 0;
+  st.ring = smem + (size_t)wid * kStagesPerWarp * a.stage_bytes;
+  st.full = full + wid * kStagesPerWarp;
   st.t = 0;
-  const size_t E0 = item_elem(st.b0, a.ipsB, a.rowsB, nc);
-  const size_t E1 = st.b1 == a.NB ? (size_t)a.half * nc : item_elem(st.b1, a.ipsB, a.rowsB, nc);
-  const int E = (int)(E1 - E0);
-  const size_t n = (size_t)a.half * nc;
+  st.kind = 1;
+  st.it = B.i0 + wid;
+  const int sA = A.site0(), nA = A.sites(), sB = B.site0(), nB = B.sites();
+  const size_t E0 = item_elem(B.i0, a.ipsB, RB_, nc);
+  const size_t E1 = B.i1 == a.NB ? (size_t)a.half * nc : item_elem(B.i1, a.ipsB, RB_, nc);
+  const int E = (int)(E1 - E0), offB = (int)(E0 - (size_t)sB * nc);
+  const size_t n = (size_t)a.half * nc, oA = ((size_t)a.half + sA) * nc;
   // the block's slices of w_j and z_j: element e at Wj(j)[e - E0], Zj(j)[e - E0]
   float2* const wbase = a.wsm_ld > 0 ? wsm : a.W + E0;
   const size_t wld = a.wsm_ld > 0 ? (size_t)a.wsm_ld : n;
   auto Wj = [&](int j) { return wbase + (size_t)j * wld; };
   auto Zj = [&](int j) { return a.Z + (size_t)j * n + E0; };
+  // r and w = D_r r on the owned rows (r also in global memory, for the gathers)
+  float2* const rs = a.esm > 0 ? esm : a.r + E0;
+  float2* const ws = a.esm > 0 ? esm + a.esm : a.w + E0;
   // the j sums of the Gram-Schmidt update are split over ngrp groups of the
   // threads of warps 1 .. when the slice has at most one element per thread
   const int ngrp = (E > 0 && E <= kUpdThreads) ? min(kUpdThreads / E, kMaxGroups) : 0;
@@ -406,268 +402,253 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
   float v[4];
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; s++) mbar_init(&full[s], 1);
+    for (int s = 0; s < W * kStagesPerWarp; s++) mbar_init(&full[s], 1);
     mbar_fence_init();
     s_fail = 0;
   }
-  const int sA = st.a0 / a.ipsA, nA = st.a1 > st.a0 ? (st.a1 - 1) / a.ipsA - sA + 1 : 0;
-  const int sB = st.b0 / a.ipsB, nB = st.b1 > st.b0 ? (st.b1 - 1) / a.ipsB - sB + 1 : 0;
-  for (int i = threadIdx.x; i < 8 * nA; i += blockDim.x) nbA[i] = a.nbr[(size_t)(a.half + sA) * 8 + i];
-  for (int i = threadIdx.x; i < 8 * nB; i += blockDim.x) {
+  for (int i = threadIdx.x; i < 8 * nA; i += kThreads) nbA[i] = a.nbr[(size_t)(a.half + sA) * 8 + i];
+  for (int i = threadIdx.x; i < 8 * nB; i += kThreads) {
     nbB[i] = a.nbr[(size_t)sB * 8 + i];
     scB[i] = a.Ys[(size_t)sB * 8 + i];
   }
   __syncthreads();
   if (lane == 0)
-    for (long long p = 0; p < kStagesPerWarp; p++) issue(a, st, p);
+    for (unsigned p = 0; p < kStagesPerWarp; p++) issue<W>(a, st, A, B, p);
 
-  // ||b||^2 over the full right-hand side (any partition of it)
-  {
-    const size_t nf = 2 * n;
-    const size_t cf = (nf + G - 1) / G;
-    const size_t f0 = (size_t)bid * cf, f1 = f0 + cf < nf ? f0 + cf : nf;
-    v[0] = 0.f;
-    for (size_t e = f0 + threadIdx.x; e < f1; e += blockDim.x) {
-      const float2 q = a.b[e];
-      v[0] = fmaf(q.x, q.x, fmaf(q.y, q.y, v[0]));
-    }
-    block_partials(a, v, 1, RD, sred);
-  }
-  // b_r = b_e - Y_eo X_o^{-1} b_o on the owned rows; r = b_r, y = 0
-  gather(nc, nB, nbB, scB, a.to, gv);
-  ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
-    const float2 bb = a.b[i];
-    const float2 o = make_float2(bb.x - u.x, bb.y - u.y);
-    a.br[i] = o;
-    a.r[i] = o;
-    a.y[i] = make_float2(0.f, 0.f);
-  }, &s_fail);
-  // ||b_r||^2 over the owned rows (written by this block's own items)
-  v[0] = 0.f;
-  for (size_t e = E0 + threadIdx.x; e < E1; e += blockDim.x) {
-    const float2 rr = a.r[e];
-    v[0] = fmaf(rr.x, rr.x, fmaf(rr.y, rr.y, v[0]));
-  }
-  block_partials(a, v, 1, RC, sred);
-  if (ok) ok = grid_barrier(a.bar, a.abort, target);
+  int mode = M_INIT, k = 0;
   long long its = 0;
-  bool done = true;
   df tol2 = df_of(0.f);
-  if (ok) {
-    grid_totals(a, RC, 2, tot + RC);   // ||b_r||^2 (the running ||r||^2) and ||b||^2
-    const df tr = df_of((float)a.tol_rel);
-    tol2 = df_mul(df_mul(tr, tr), tot[RD]);
-    done = !(tot[RD].h > 0.f);
-  }
-  while (ok && !done && its < a.maxit) {
-    int k = 0;
-    while (k < m && its < a.maxit) {
-      float2* wk = Wj(k);
-      // w = D_r r: phase A, barrier, phase B
-      gather(nc, nA, nbA, nullptr, a.r, gv);
-      if (!(ok = run_items<ST>(a, st, 0, gv, [&](size_t i, float2 u) { a.tB[(size_t)a.half * nc + i] = u; }, &s_fail)))
-        break;
-      if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-      gather(nc, nB, nbB, scB, a.tB, gv);
-      if (!(ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
-              const float2 rr = a.r[i];
-              wk[i - E0] = make_float2(rr.x - u.x, rr.y - u.y);
-            }, &s_fail)))
-        break;
-      // beta_j = <w_j, w> (warp wid owns j = wid + 8 u, u < 4), ||w||^2, <w, r>
-      for (int jb = wid; jb < k; jb += 4 * kWarps) {
-        float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int e = lane; e < E; e += 32) {
-          const float2 x = wk[e];
-#pragma unroll
-          for (int u = 0; u < 4; u++) {
-            const int j = jb + u * kWarps;
-            const float2 p = j < k ? Wj(j)[e] : make_float2(0.f, 0.f);
-            re[u] = fmaf(p.x, x.x, fmaf(p.y, x.y, re[u]));
-            im[u] = fmaf(p.x, x.y, fmaf(-p.y, x.x, im[u]));
-          }
+  while (true) {
+    if (mode != M_INIT) {
+      // phase A: A v on the odd sites; in the closing pass v = y, and the odd
+      // half of the solution is x_o = X_o^{-1} b_o - A y
+      gather<W>(nc, nA, nbA, nullptr, mode == M_ITER ? a.r : a.y, gv);
+      ok = run_items<kStF32, R, W>(a, st, A, B, A, gv, [&](int e, float2 u) {
+        a.tB[oA + e] = u;
+        if (mode == M_CLOSE) {
+          const float2 o = a.to[oA + e];
+          a.x[oA + e] = make_float2(o.x - u.x, o.y - u.y);
         }
-        df sv[8];
+      }, &s_fail);
+      if (!ok || !(ok = grid_barrier(a.bar, a.abort, target))) break;
+    }
+    // phase B on the even sites: w = r - Y_eo t, without r outside the iterations
+    gather<W>(nc, nB, nbB, scB, mode == M_INIT ? a.to : a.tB, gv);
+    ok = run_items<ST, RB_, W>(a, st, A, B, B, gv, [&](int e, float2 u) {
+      const float2 o = mode == M_ITER ? rs[e - offB] : make_float2(0.f, 0.f);
+      ws[e - offB] = make_float2(o.x - u.x, o.y - u.y);
+    }, &s_fail);
+    if (!ok) break;
+    if (mode != M_ITER) {
+      // b_r = b_e - Y_eo X_o^{-1} b_o, r = b_r, y = 0; or the true r = b_r - D_r y
+      v[0] = v[1] = 0.f;
+      for (int e = threadIdx.x; e < E; e += kThreads) {
+        const float2 u = ws[e];
+        float2 rr;
+        if (mode == M_INIT) {
+          const float2 bb = a.b[E0 + e];
+          rr = make_float2(bb.x + u.x, bb.y + u.y);
+          a.br[E0 + e] = rr;
+          a.y[E0 + e] = make_float2(0.f, 0.f);
+        } else {
+          const float2 bb = a.br[E0 + e], yy = a.y[E0 + e];
+          rr = make_float2(bb.x - (yy.x + u.x), bb.y - (yy.y + u.y));
+        }
+        rs[e] = rr;
+        a.r[E0 + e] = rr;
+        v[0] = fmaf(rr.x, rr.x, fmaf(rr.y, rr.y, v[0]));
+      }
+      if (mode == M_INIT) {   // ||b||^2 over the full right-hand side (any partition of it)
+        const size_t cf = (2 * n + G - 1) / G;
+        const size_t f0 = (size_t)bid * cf, f1 = f0 + cf < 2 * n ? f0 + cf : 2 * n;
+        for (size_t e = f0 + threadIdx.x; e < f1; e += kThreads) {
+          const float2 q = a.b[e];
+          v[1] = fmaf(q.x, q.x, fmaf(q.y, q.y, v[1]));
+        }
+      }
+      const int nq = mode == M_INIT ? 2 : 1;
+      block_partials<W>(a, v, nq, RC, sred);
+      if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
+      grid_totals<W>(a, RC, nq, tot + RC);   // ||r||^2 restarts the running norm
+      if (mode == M_INIT) {
+        const df tr = df_of((float)a.tol_rel);
+        tol2 = df_mul(df_mul(tr, tr), tot[RD]);
+        if (!(tot[RD].h > 0.f)) break;
+      } else if (tot[RC].h <= tol2.h || !(tot[RC].h == tot[RC].h)) {
+        break;
+      }
+      if (its >= a.maxit) break;
+      mode = M_ITER;
+      k = 0;
+      continue;
+    }
+    float2* wk = Wj(k);
+    // beta_j = <w_j, w> (warp wid owns j = wid + W u, u < 4), ||w||^2, <w, r>
+    for (int jb = wid; jb < k; jb += 4 * W) {
+      float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+      for (int e = lane; e < E; e += 32) {
+        const float2 x = ws[e];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-          sv[2 * u] = df_of(re[u]);
-          sv[2 * u + 1] = df_of(im[u]);
+          const int j = jb + u * W;
+          const float2 p = j < k ? Wj(j)[e] : make_float2(0.f, 0.f);
+          re[u] = fmaf(p.x, x.x, fmaf(p.y, x.y, re[u]));
+          im[u] = fmaf(p.x, x.y, fmaf(-p.y, x.x, im[u]));
         }
-        const df sr = warp_transpose_sum<8>(sv);   // lane l: sum (l >> 2) = 2 u + {re, im}
-        const int j = jb + (lane >> 3) * kWarps;
-        if ((lane & 3) == 0 && j < k) a.partials[(size_t)(RA + 2 * j + ((lane >> 2) & 1)) * G + bid] = make_float2(sr.h, sr.l);
       }
+      df sv[8];
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        sv[2 * u] = df_of(re[u]);
+        sv[2 * u + 1] = df_of(im[u]);
+      }
+      const df sr = warp_transpose_sum<8>(sv);   // lane l: sum (l >> 2) = 2 u + {re, im}
+      const int j = jb + (lane >> 3) * W;
+      if ((lane & 3) == 0 && j < k) a.partials[(size_t)(RA + 2 * j + ((lane >> 2) & 1)) * G + bid] = make_float2(sr.h, sr.l);
+    }
+    v[0] = v[1] = v[2] = 0.f;
+    for (int e = threadIdx.x; e < E; e += kThreads) {
+      const float2 x = ws[e], rr = rs[e];
+      v[0] = fmaf(x.x, x.x, fmaf(x.y, x.y, v[0]));
+      v[1] = fmaf(x.x, rr.x, fmaf(x.y, rr.y, v[1]));
+      v[2] = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, v[2]));
+    }
+    block_partials<W>(a, v, 3, RA + 2 * k, sred);   // after the beta slots: one pass reads all of them
+    if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
+    grid_totals<W>(a, RA, 2 * k + 3, tot);
+    // warp 0: sum_j |beta_j|^2 and the coefficients; the other warps meanwhile
+    // S_w = sum_j beta_j w_j, S_z = sum_j beta_j z_j on the owned rows
+    auto beta = [&](int j) {
+      return make_float2(tot[2 * j].h + tot[2 * j].l, tot[2 * j + 1].h + tot[2 * j + 1].l);
+    };
+    // gamma = ||w''||, alpha = <w'', r> / gamma; with w_k = w'' / gamma of
+    // unit norm, ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2 (the running norm)
+    auto coefficients = [&](df g2, df wr, df wi) {
+      const df g = df_sqrt(g2);
+      const bool gz = !(g.h > 0.f);
+      s_coef[0] = gz ? 1.f : 1.f / g.h;
+      const df ar = gz ? wr : df_div(wr, g);
+      const df ai = gz ? wi : df_div(wi, g);
+      s_coef[1] = ar.h + ar.l;
+      s_coef[2] = ai.h + ai.l;
+      if (!gz) {
+        const df rn = df_add(tot[RC], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
+        tot[RC] = rn.h > 0.f ? rn : df_of(0.f);
+      }
+    };
+    if (wid == 0) {
+      df bb = df_of(0.f);
+      for (int j = lane; j < k; j += 32) {
+        bb = df_add(bb, df_mul(tot[2 * j], tot[2 * j]));
+        bb = df_add(bb, df_mul(tot[2 * j + 1], tot[2 * j + 1]));
+      }
+      bb = df_wsum(bb);
+      if (lane == 0) {
+        const df ww = tot[2 * k], g2 = df_add(ww, df_neg(bb));
+        const bool fine = g2.h > 1e-3f * ww.h;   // otherwise Pythagoras lost more than three digits
+        s_coef[3] = fine ? 0.f : 1.f;
+        if (fine) coefficients(g2, tot[2 * k + 1], tot[2 * k + 2]);
+      }
+    } else if (ngrp) {
+      const int t = threadIdx.x - 32, gi = t / E, ei = t - gi * E;
+      if (gi < ngrp) {
+        float swr = 0.f, swi = 0.f, szr = 0.f, szi = 0.f;
+#pragma unroll 8
+        for (int j = gi; j < k; j += ngrp) {
+          const float2 bj = beta(j);
+          const float2 p = Wj(j)[ei], q = Zj(j)[ei];
+          swr = fmaf(bj.x, p.x, fmaf(-bj.y, p.y, swr));
+          swi = fmaf(bj.x, p.y, fmaf(bj.y, p.x, swi));
+          szr = fmaf(bj.x, q.x, fmaf(-bj.y, q.y, szr));
+          szi = fmaf(bj.x, q.y, fmaf(bj.y, q.x, szi));
+        }
+        upd[gi * E + ei] = make_float2(swr, swi);
+        upd[kThreads + gi * E + ei] = make_float2(szr, szi);
+      }
+    }
+    __syncthreads();
+    const bool exact = s_coef[3] != 0.f;
+    // w'' = w - S_w
+    auto w_orth = [&](int ei) {
+      float2 x = ws[ei];
+      if (ngrp) {
+        for (int g = 0; g < ngrp; g++) {
+          const float2 u = upd[g * E + ei];
+          x.x -= u.x;
+          x.y -= u.y;
+        }
+      } else {
+#pragma unroll 4
+        for (int j = 0; j < k; j++) {
+          const float2 bj = beta(j), p = Wj(j)[ei];
+          x.x -= bj.x * p.x - bj.y * p.y;
+          x.y -= bj.x * p.y + bj.y * p.x;
+        }
+      }
+      return x;
+    };
+    if (exact) {  // uniform: every block took the same decision from the same totals
       v[0] = v[1] = v[2] = 0.f;
-      for (size_t e = E0 + threadIdx.x; e < E1; e += blockDim.x) {
-        const float2 x = wk[e - E0], rr = a.r[e];
+      for (int ei = threadIdx.x; ei < E; ei += kThreads) {
+        const float2 x = w_orth(ei), rr = rs[ei];
         v[0] = fmaf(x.x, x.x, fmaf(x.y, x.y, v[0]));
         v[1] = fmaf(x.x, rr.x, fmaf(x.y, rr.y, v[1]));
         v[2] = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, v[2]));
       }
-      block_partials(a, v, 3, RA + 2 * k, sred);   // after the beta slots: one pass reads all of them
+      block_partials<W>(a, v, 3, RE, sred);
       if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-      grid_totals(a, RA, 2 * k + 3, tot);
-      // warp 0: sum_j |beta_j|^2 and the coefficients; the other warps meanwhile
-      // S_w = sum_j beta_j w_j, S_z = sum_j beta_j z_j on the owned rows
-      auto beta = [&](int j) {
-        return make_float2(tot[2 * j].h + tot[2 * j].l, tot[2 * j + 1].h + tot[2 * j + 1].l);
-      };
-      // gamma = ||w''||, alpha = <w'', r> / gamma; with w_k = w'' / gamma of
-      // unit norm, ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2 (the running norm)
-      auto coefficients = [&](df g2, df wr, df wi) {
-        const df g = df_sqrt(g2);
-        const bool gz = !(g.h > 0.f);
-        s_coef[0] = gz ? 1.f : 1.f / g.h;
-        const df ar = gz ? wr : df_div(wr, g);
-        const df ai = gz ? wi : df_div(wi, g);
-        s_coef[1] = ar.h + ar.l;
-        s_coef[2] = ai.h + ai.l;
-        if (!gz) {
-          const df rn = df_add(tot[RC], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
-          tot[RC] = rn.h > 0.f ? rn : df_of(0.f);
-        }
-      };
-      if (wid == 0) {
-        df bb = df_of(0.f);
-        for (int j = lane; j < k; j += 32) {
-          bb = df_add(bb, df_mul(tot[2 * j], tot[2 * j]));
-          bb = df_add(bb, df_mul(tot[2 * j + 1], tot[2 * j + 1]));
-        }
-        bb = df_wsum(bb);
-        if (lane == 0) {
-          const df ww = tot[2 * k], g2 = df_add(ww, df_neg(bb));
-          const bool fine = g2.h > 1e-3f * ww.h;   // otherwise Pythagoras lost more than three digits
-          s_coef[3] = fine ? 0.f : 1.f;
-          if (fine) coefficients(g2, tot[2 * k + 1], tot[2 * k + 2]);
-        }
-      } else if (ngrp) {
-        const int t = threadIdx.x - 32, gi = t / E, ei = t - gi * E;
-        if (gi < ngrp) {
-          float swr = 0.f, swi = 0.f, szr = 0.f, szi = 0.f;
-#pragma unroll 8
-          for (int j = gi; j < k; j += ngrp) {
-            const float2 bj = beta(j);
-            const float2 p = Wj(j)[ei], q = Zj(j)[ei];
-            swr = fmaf(bj.x, p.x, fmaf(-bj.y, p.y, swr));
-            swi = fmaf(bj.x, p.y, fmaf(bj.y, p.x, swi));
-            szr = fmaf(bj.x, q.x, fmaf(-bj.y, q.y, szr));
-            szi = fmaf(bj.x, q.y, fmaf(bj.y, q.x, szi));
-          }
-          upd[gi * E + ei] = make_float2(swr, swi);
-          upd[kThreads + gi * E + ei] = make_float2(szr, szi);
-        }
-      }
+      grid_totals<W>(a, RE, 3, tot + RB);   // the exact ||w''||^2, <w'', r> replace the estimates
+      if (threadIdx.x == 0) coefficients(tot[RB], tot[RB + 1], tot[RB + 2]);
       __syncthreads();
-      const bool exact = s_coef[3] != 0.f;
-      // w'' = w - S_w
-      auto w_orth = [&](int ei) {
-        float2 x = wk[ei];
-        if (ngrp) {
-          for (int g = 0; g < ngrp; g++) {
-            const float2 u = upd[g * E + ei];
-            x.x -= u.x;
-            x.y -= u.y;
-          }
-        } else {
-#pragma unroll 4
-          for (int j = 0; j < k; j++) {
-            const float2 bj = beta(j), p = Wj(j)[ei];
-            x.x -= bj.x * p.x - bj.y * p.y;
-            x.y -= bj.x * p.y + bj.y * p.x;
-          }
-        }
-        return x;
-      };
-      if (exact) {  // uniform: every block took the same decision from the same totals
-        v[0] = v[1] = v[2] = 0.f;
-        for (int ei = threadIdx.x; ei < E; ei += blockDim.x) {
-          const float2 x = w_orth(ei), rr = a.r[E0 + ei];
-          v[0] = fmaf(x.x, x.x, fmaf(x.y, x.y, v[0]));
-          v[1] = fmaf(x.x, rr.x, fmaf(x.y, rr.y, v[1]));
-          v[2] = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, v[2]));
-        }
-        block_partials(a, v, 3, RE, sred);
-        if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-        grid_totals(a, RE, 3, tot + RB);   // the exact ||w''||^2, <w'', r> replace the estimates
-        if (threadIdx.x == 0) coefficients(tot[RB], tot[RB + 1], tot[RB + 2]);
-        __syncthreads();
-      }
-      // w_k = w'' / gamma, z_k = (r - S_z) / gamma, y += alpha z_k, r -= alpha w_k
-      const float ig = s_coef[0], far = s_coef[1], fai = s_coef[2];
-      v[0] = 0.f;
-      for (int ei = threadIdx.x; ei < E; ei += blockDim.x) {
-        const size_t e = E0 + ei;
-        float2 x = w_orth(ei);
-        x.x *= ig;
-        x.y *= ig;
-        wk[ei] = x;
-        float2 rr = a.r[e];
-        float2 z = rr;
-        if (ngrp) {
-          for (int g = 0; g < ngrp; g++) {
-            const float2 u = upd[kThreads + g * E + ei];
-            z.x -= u.x;
-            z.y -= u.y;
-          }
-        } else {
-#pragma unroll 4
-          for (int j = 0; j < k; j++) {
-            const float2 bj = beta(j), q = Zj(j)[ei];
-            z.x -= bj.x * q.x - bj.y * q.y;
-            z.y -= bj.x * q.y + bj.y * q.x;
-          }
-        }
-        z.x *= ig;
-        z.y *= ig;
-        Zj(k)[ei] = z;
-        float2 yy = a.y[e];
-        yy.x += far * z.x - fai * z.y;
-        yy.y += far * z.y + fai * z.x;
-        a.y[e] = yy;
-        rr.x -= far * x.x - fai * x.y;
-        rr.y -= far * x.y + fai * x.x;
-        a.r[e] = rr;
-      }
-      // r complete on every block before the next iteration's phase A reads it
-      if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-      k++;
-      its++;
-      const df rn2 = tot[RC];
-      if (!(rn2.h == rn2.h)) {
-        if (bid == 0 && threadIdx.x == 0) atomicExch(&a.flags[FLAG_NAN], 1);
-        done = true;
-        break;
-      }
-      if (rn2.h <= tol2.h) break;
     }
-    if (!ok || done) break;
-    // true residual r = b_r - D_r y (y complete on every block after the last barrier)
-    // and the odd half of the solution, x_o = X_o^{-1} b_o - A y
-    gather(nc, nA, nbA, nullptr, a.y, gv);
-    if (!(ok = run_items<ST>(a, st, 0, gv, [&](size_t i, float2 u) {
-            const float2 o = a.to[(size_t)a.half * nc + i];
-            a.tB[(size_t)a.half * nc + i] = u;
-            a.x[(size_t)a.half * nc + i] = make_float2(o.x - u.x, o.y - u.y);
-          }, &s_fail)))
-      break;
-    if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-    gather(nc, nB, nbB, scB, a.tB, gv);
-    if (!(ok = run_items<ST>(a, st, 1, gv, [&](size_t i, float2 u) {
-            const float2 yy = a.y[i], bb = a.br[i];
-            a.r[i] = make_float2(bb.x - (yy.x - u.x), bb.y - (yy.y - u.y));
-          }, &s_fail)))
-      break;
+    // w_k = w'' / gamma, z_k = (r - S_z) / gamma, y += alpha z_k, r -= alpha w_k
+    const float ig = s_coef[0], far = s_coef[1], fai = s_coef[2];
     v[0] = 0.f;
-    for (size_t e = E0 + threadIdx.x; e < E1; e += blockDim.x) {
-      const float2 rr = a.r[e];
-      v[0] = fmaf(rr.x, rr.x, fmaf(rr.y, rr.y, v[0]));
+    for (int ei = threadIdx.x; ei < E; ei += kThreads) {
+      const size_t e = E0 + ei;
+      float2 x = w_orth(ei);
+      x.x *= ig;
+      x.y *= ig;
+      wk[ei] = x;
+      float2 rr = rs[ei];
+      float2 z = rr;
+      if (ngrp) {
+        for (int g = 0; g < ngrp; g++) {
+          const float2 u = upd[kThreads + g * E + ei];
+          z.x -= u.x;
+          z.y -= u.y;
+        }
+      } else {
+#pragma unroll 4
+        for (int j = 0; j < k; j++) {
+          const float2 bj = beta(j), q = Zj(j)[ei];
+          z.x -= bj.x * q.x - bj.y * q.y;
+          z.y -= bj.x * q.y + bj.y * q.x;
+        }
+      }
+      z.x *= ig;
+      z.y *= ig;
+      Zj(k)[ei] = z;
+      float2 yy = a.y[e];
+      yy.x += far * z.x - fai * z.y;
+      yy.y += far * z.y + fai * z.x;
+      a.y[e] = yy;
+      rr.x -= far * x.x - fai * x.y;
+      rr.y -= far * x.y + fai * x.x;
+      rs[ei] = rr;
+      a.r[e] = rr;
     }
-    block_partials(a, v, 1, RC, sred);
+    // r complete on every block before the next phase A reads it
     if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
-    grid_totals(a, RC, 1, tot + RC);   // the true ||r||^2 restarts the running norm
+    k++;
+    its++;
     const df rn2 = tot[RC];
-    if (rn2.h <= tol2.h || !(rn2.h == rn2.h)) done = true;
+    if (!(rn2.h == rn2.h)) {
+      if (bid == 0 && threadIdx.x == 0) atomicExch(&a.flags[FLAG_NAN], 1);
+      break;
+    }
+    if (rn2.h <= tol2.h || k == m || its >= a.maxit) mode = M_CLOSE;
   }
   if (ok && its == 0)   // b = 0: y = 0 and x_o = t_o
     for (size_t e = (size_t)bid * kThreads + threadIdx.x; e < n; e += (size_t)G * kThreads) a.x[n + e] = a.to[n + e];
@@ -676,23 +657,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_stream(SArgs a) {
     atomicExch(a.abort, 1);
   }
   // drain: the copies this warp issued beyond what it consumed land before exit
-  if (lane == 0 && st.cA + st.cB > 0)
-    for (long long p = st.t; p < st.t + kStagesPerWarp; p++)
-      (void)mbar_wait(&full[wid * kStagesPerWarp + (int)(p % kStagesPerWarp)],
-                      (unsigned)((p / kStagesPerWarp) & 1));
+  if (lane == 0 && (A.i1 > A.i0 + wid || B.i1 > B.i0 + wid))
+    for (unsigned p = st.t; p < st.t + kStagesPerWarp; p++)
+      (void)mbar_wait(&st.full[p % kStagesPerWarp], (p / kStagesPerWarp) & 1u);
   if (bid == 0 && threadIdx.x == 0) *a.iters += its;
 }
 
 struct Plan {
-  int grid, stage_bytes, rowsA, rowsB, ipsA, ipsB, NA, NB, gmax, wsm_ld, emax;
+  int grid, warps, stage_bytes, rowsA, rowsB, ipsA, ipsB, NA, NB, gmax, wsm_ld, esm, emax;
   size_t smem;
 };
 
+int pow2_floor(int v) {
+  int p = 1;
+  while (2 * p <= v) p *= 2;
+  return v > 0 ? p : 0;
+}
+
 // items, the sites a block's item ranges touch, and the shared memory they need
-void plan_items(Plan& p, int half, int nc, int esz) {
+void plan_items(Plan& p, int half, int nc, int store) {
   const int K = 8 * nc;
-  p.rowsA = std::min(kMaxRows, std::min(nc, p.stage_bytes / (K * 8)));
-  p.rowsB = std::min(kMaxRows, std::min(nc, p.stage_bytes / (K * esz)));
+  p.rowsA = pow2_floor(std::min(p.warps == 16 ? kMaxRows : 2, std::min(nc, p.stage_bytes / (K * 8))));
+  p.rowsB = rows_b(store == STORE_F32 ? kStF32 : kStF16, p.rowsA);
   p.ipsA = p.rowsA > 0 ? (nc + p.rowsA - 1) / p.rowsA : 0;
   p.ipsB = p.rowsB > 0 ? (nc + p.rowsB - 1) / p.rowsB : 0;
   p.NA = half * p.ipsA;
@@ -712,47 +698,62 @@ void plan_items(Plan& p, int half, int nc, int esz) {
   }
 }
 
-Plan make_plan(const LevelGeom& G, const CoarseOp& C, int grid, int m) {
+Plan plan_warps(const LevelGeom& G, const CoarseOp& C, int grid, int m, int warps) {
   Plan p;
-  const int nc = C.nc, K = 8 * nc;
-  const int esz = C.store == STORE_F32 ? 8 : 4;
+  p.warps = warps;
+  const int nc = C.nc, K = 8 * nc, stages = warps * kStagesPerWarp;
   int dev = 0, optin = 0;
   MG_CUDA(cudaGetDevice(&dev));
   MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t budget = (size_t)optin - 4096;   // static shared memory and slack
-  const size_t fixed = sizeof(float2) * (4 * kWarps + kNR) + sizeof(float2) * 2 * kThreads;
+  const size_t fixed = sizeof(float2) * (4 * warps + kNR) + sizeof(float2) * 2 * 32 * warps;
   const size_t per_site = sizeof(float2) * K + 24 * sizeof(int);   // gathered vector, neighbours, tile scales
   p.grid = grid;
   // the w_j slice in shared memory only when it is small (a sixteenth of the
   // budget): measured on GB300 at Nc = 48, m = 64, a deeper link ring gains
   // more than shared-memory Gram-Schmidt vectors save.  A block's slice has
   // at most ceil(n / grid) elements plus the rows of the partial items at
-  // both ends of its range.
+  // both ends of its range.  r and w of the owned rows: an eighth.
   const size_t n = (size_t)G.half * nc;
   const int gb = std::max(1, grid);
   const int ebound = (int)((n + gb - 1) / gb) + (int)((7LL * G.half + gb - 1) / gb) + 2 * kMaxRows;
   const bool wsmem = (size_t)m * ebound * sizeof(float2) <= budget / 16;
-  const size_t wbytes = wsmem ? (size_t)m * ebound * sizeof(float2) : 0;
+  const bool esmem = 2 * (size_t)ebound * sizeof(float2) <= budget / 8;
+  const size_t wbytes = (wsmem ? (size_t)m * ebound * sizeof(float2) : 0) + (esmem ? 2 * (size_t)ebound * sizeof(float2) : 0);
   int gsites = 4;
   for (int pass = 0; pass < 3; pass++) {
     const size_t other = fixed + wbytes + per_site * (size_t)gsites;
-    p.stage_bytes = budget > other ? (int)(((budget - other) / kStages) / 16 * 16) : 0;
-    plan_items(p, G.half, nc, esz);
+    p.stage_bytes = budget > other ? (int)(((budget - other) / stages) / 16 * 16) : 0;
+    plan_items(p, G.half, nc, C.store);
     if (p.gmax <= gsites) break;
     gsites = p.gmax;
   }
   p.grid = std::min(grid, std::min(p.NA, p.NB));
-  p.smem = (size_t)kStages * p.stage_bytes + fixed + wbytes + per_site * (size_t)std::max(gsites, p.gmax);
+  p.smem = (size_t)stages * p.stage_bytes + fixed + wbytes + per_site * (size_t)std::max(gsites, p.gmax);
   p.gmax = std::max(gsites, p.gmax);
   p.wsm_ld = wsmem ? ebound : 0;
-  if (wsmem && p.emax > ebound) raise(MG_ERR_STATE, "streamed coarse GCR: Krylov slice larger than planned");
+  p.esm = esmem ? ebound : 0;
+  if ((wsmem || esmem) && p.emax > ebound) raise(MG_ERR_STATE, "streamed coarse GCR: slice larger than planned");
   return p;
 }
 
-const void* kernel_for(int store) {
-  return store == STORE_F16    ? (const void*)k_coarse_gcr_stream<kStF16>
-         : store == STORE_BF16 ? (const void*)k_coarse_gcr_stream<kStBF16>
-                               : (const void*)k_coarse_gcr_stream<kStF32>;
+// 16 warps where their 32 stages hold items of two rows or more (Nc up to about
+// 64), 8 beyond: 16 halve the serial chain of a warp, two to three items per
+// phase at 16^3x32.
+Plan make_plan(const LevelGeom& G, const CoarseOp& C, int grid, int m) {
+  const Plan p = plan_warps(G, C, grid, m, 16);
+  return p.rowsA >= 2 ? p : plan_warps(G, C, grid, m, 8);
+}
+
+template <int W, int R>
+const void* kernel_st(int store) {
+  return store == STORE_F16    ? (const void*)k_coarse_gcr_stream<kStF16, W, R>
+         : store == STORE_BF16 ? (const void*)k_coarse_gcr_stream<kStBF16, W, R>
+                               : (const void*)k_coarse_gcr_stream<kStF32, W, R>;
+}
+const void* kernel_for(int store, const Plan& p) {
+  if (p.warps == 16) return p.rowsA == 8 ? kernel_st<16, 8>(store) : p.rowsA == 4 ? kernel_st<16, 4>(store) : kernel_st<16, 2>(store);
+  return p.rowsA >= 2 ? kernel_st<8, 2>(store) : kernel_st<8, 1>(store);
 }
 
 int sm_count() {
@@ -791,9 +792,9 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   const Plan p = make_plan(G, C, grid, m);
   const int sms = sm_count();
   int per = 0;
-  const void* kern = kernel_for(C.store);
+  const void* kern = kernel_for(C.store, p);
   MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
-  MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, p.smem));
+  MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * p.warps, p.smem));
   if (per < 1 || p.grid > per * sms) raise(MG_ERR_CUDA, "streamed coarse GCR cannot be resident");
   const size_t n = (size_t)G.half * C.nc;
   auto need = [&](DBuf& d, size_t bytes) {
@@ -822,6 +823,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   a.stage_bytes = p.stage_bytes;
   a.gmax = p.gmax;
   a.wsm_ld = p.wsm_ld;
+  a.esm = p.esm;
   a.tol_rel = tol_rel;
   a.nbr = G.d_nbr.as<int>();
   a.Y = static_cast<const unsigned char*>(C.Y.get());
@@ -834,6 +836,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   a.r = B.r.as<float2>();
   a.br = B.br.as<float2>();
   a.tB = B.tB.as<float2>();
+  a.w = B.tA.as<float2>();
   a.W = B.W.as<float2>();
   a.Z = B.Z.as<float2>();
   a.partials = B.st_part.as<float2>();
@@ -842,7 +845,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   a.bar = B.st_sync.as<unsigned>();
   a.abort = reinterpret_cast<int*>(B.st_sync.as<unsigned char>() + 128);
   void* params[] = {&a};
-  MG_CUDA(cudaLaunchCooperativeKernel(kern, dim3(p.grid), dim3(kThreads), params, p.smem, s));
+  MG_CUDA(cudaLaunchCooperativeKernel(kern, dim3(p.grid), dim3(32 * p.warps), params, p.smem, s));
   MG_LAUNCH();
   coarse_site_mul(G, C, true, 0, G.half, x, B.y.as<float>(), s);   // x_e = X_e^{-1} y_e; the kernel wrote x_o
 }
