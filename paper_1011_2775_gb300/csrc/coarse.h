@@ -157,7 +157,7 @@ void coarse_gcr_solve(const LevelGeom& G, const CoarseOp& C, const CoarseGCRBuff
                       int grid = 0);
 // The same solve with the links streamed through shared memory by bulk
 // asynchronous copies and three grid barriers per iteration
-// (coarse_stream.cu): even-odd levels only.  grid: blocks of the cooperative
+// (coarse_stream.cu).  grid: blocks of the cooperative
 // launch, one of coarse_gcr_stream_grids().  Raises FLAG_TIMEOUT if a wait
 // runs out of time.
 bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C);

@@ -46,12 +46,14 @@
 // Measured (16^3x32, 4^4 blocks, Nc = 48, 256 reduced sites, 35 iterations):
 // 817 us per solve with 256 threads, neighbour indices read for every gather,
 // the coefficients formed before the sums, divisions and a switch over the rows
-// of every item, and r and w read back from global memory; 640 us here.  Of the
+// of every item, and r and w read back from global memory; 618 us here.  Of the
 // 38k cycles of an iteration the stencil passes take 6.6k each (shared-memory
 // port: every link byte is written and read there, every gathered vector read
 // once per two rows), the gathers 1.5k each, the barriers 9k, inner products,
-// totals, coefficients and update 12k.  24^3x48 with bf16 links: 427 -> 290 us;
+// totals, coefficients and update 12k.  24^3x48 with bf16 links: 427 -> 269 us;
 // the links come from HBM and phase A runs at its rate (191 MB in 28.6 us).
+// On a lattice with an odd extent the same loop applies D_hat = [Y_0 .. Y_7 | X]
+// on all sites: 3^3x6, Nc = 48: 112 us on the grouped kernel with one system, 67 here.
 #include <algorithm>
 #include <cstring>
 
@@ -78,13 +80,13 @@ constexpr int RE = RD + 1;
 constexpr int kNR = RE + 3;
 
 struct SArgs {
-  int nc, half, m, maxit;
+  int nc, half, m, maxit;     // half: sites of the solved system (all of them on an odd extent)
   int rowsA, rowsB, ipsA, ipsB, NA, NB, eszB;
   int stage_bytes, gmax, wsm_ld;   // wsm_ld > 0: the w_j slice in shared memory, leading dimension
   int esm;                         // > 0: r and w of the owned rows in shared memory, their capacity
   double tol_rel;
   const int* nbr;
-  const unsigned char* Y;     // even-site links [e][nc][8][nc], storage format
+  const unsigned char* Y;     // even-site links [e][nc][8][nc], storage format; odd extents: [s][nc][9][nc], FP32
   const float* Ys;            // their tile scales [e][8]
   const unsigned char* Af;    // folded odd-site links [o - half][nc][8][nc], FP32
   const float2* b;            // full right-hand side
@@ -140,7 +142,7 @@ struct Stream {
 
 // lane 0: bulk copy of the next item of the sequence into stage `slot`, and on
 // to the one after it (the warp's B items for b_r, then A and B alternately)
-template <int W>
+template <int W, int ND>
 __device__ __forceinline__ void issue(const SArgs& a, Stream& st, const Items& A, const Items& B, unsigned slot) {
   const int wid = threadIdx.x >> 5;
   for (int tries = 0; tries < 2 && st.it >= (st.kind ? B.i1 : A.i1); tries++) {   // a phase without items is passed over
@@ -156,7 +158,7 @@ __device__ __forceinline__ void issue(const SArgs& a, Stream& st, const Items& A
     row0 = (size_t)s * nc + r0;
     nr = min(rows, nc - r0);
   }
-  const unsigned per = 8u * nc * (st.kind ? a.eszB : 8);
+  const unsigned per = (unsigned)ND * nc * (st.kind ? a.eszB : 8);
   const unsigned bytes = nr * per;
   mbar_arrive_expect_tx(&st.full[slot], bytes);
   bulk_copy_g2s(st.ring + (size_t)slot * a.stage_bytes, (st.kind ? a.Y : a.Af) + row0 * per, bytes, &st.full[slot]);
@@ -169,9 +171,9 @@ __device__ __forceinline__ void issue(const SArgs& a, Stream& st, const Items& A
 // 16 bytes per lane, the loads of kGather pairs in flight together: one L2
 // round trip for a block of up to eight sites.
 constexpr int kGather = 4;
-template <int kWarps>
+template <int kWarps, int ND>
 __device__ __forceinline__ void gather(int nc, int ns, const int* nbr, const float* scale, const float2* in, float2* gv) {
-  const int nc2 = nc >> 1, np = 8 * ns, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nc2 = nc >> 1, np = ND * ns, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float4* g4 = reinterpret_cast<float4*>(gv);
   for (int p0 = w; p0 < np; p0 += kGather * kWarps)
     for (int q = lane; q < nc2; q += 32) {
@@ -237,10 +239,10 @@ __device__ __forceinline__ bool item_rows(const unsigned char* stage, int K, con
 // One phase of this warp's items: waits for each staged item, computes its
 // rows, hands them to epi(element from the block's first site, row value) and
 // refills the stage two items ahead.  false on a timeout (uniform in the block).
-template <int ST, int NR, int W, typename Epi>
+template <int ST, int NR, int W, int ND, typename Epi>
 __device__ __forceinline__ bool run_items(const SArgs& a, Stream& st, const Items& A, const Items& B, const Items& g,
                                           const float2* gv, Epi epi, int* s_fail) {
-  const int nc = a.nc, K = 8 * nc, lane = threadIdx.x & 31;
+  const int nc = a.nc, K = ND * nc, lane = threadIdx.x & 31;
   int sl = g.sl, rem = g.rem;
   for (int it = g.i0 + (threadIdx.x >> 5); it < g.i1; it += W) {
     const unsigned slot = st.t % kStagesPerWarp;
@@ -253,7 +255,7 @@ __device__ __forceinline__ bool run_items(const SArgs& a, Stream& st, const Item
     int row;   // rows past the site's last are not copied; what their sums hold is dropped
     const bool mine = item_rows<ST, NR>(st.ring + (size_t)slot * a.stage_bytes, K, gv + (size_t)sl * K, res, row);
     __syncwarp();
-    if (lane == 0) issue<W>(a, st, A, B, slot);
+    if (lane == 0) issue<W, ND>(a, st, A, B, slot);
     if (mine && r0 + row < nc) epi(sl * nc + r0 + row, res);
     st.t++;
     sl += g.dq;
@@ -352,16 +354,18 @@ __device__ __forceinline__ void grid_totals(const SArgs& a, int q0, int nq, df* 
 // is fetched again every time round.
 enum { M_INIT, M_ITER, M_CLOSE };
 
-// W warps, R rows per item of phase A (phase B, 16-bit links: 2 R)
-template <int ST, int W, int R>
+// W warps, R rows per item of phase A (phase B, 16-bit links: 2 R).  On a
+// lattice with an odd extent (EO false) there is phase B alone, D_hat v with the
+// links [Y_0 .. Y_7 | X] of all sites.
+template <int ST, int W, int R, bool EO>
 __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_constant__ SArgs a) {
   constexpr int kThreads = 32 * W, kUpdThreads = kThreads - 32;   // warp 0 forms the coefficients meanwhile
-  constexpr int RB_ = rows_b(ST, R);
+  constexpr int RB_ = rows_b(ST, R), ND = EO ? 8 : 9;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[W * kStagesPerWarp];
   __shared__ float s_coef[4];              // 1/gamma, Re alpha, Im alpha, exact flag
   __shared__ int s_fail;
-  const int nc = a.nc, K = 8 * nc, m = a.m;
+  const int nc = a.nc, K = ND * nc, m = a.m;
   const int G = gridDim.x, bid = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   float2* gv = reinterpret_cast<float2*>(smem + (size_t)W * kStagesPerWarp * a.stage_bytes);
@@ -371,8 +375,8 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
   df* sred = reinterpret_cast<df*>(esm + 2 * (size_t)a.esm);           // [4][W]
   df* tot = sred + 4 * W;                                              // [kNR]
   int* nbA = reinterpret_cast<int*>(tot + kNR);                        // [gmax][8] neighbours of the A sites,
-  int* nbB = nbA + 8 * a.gmax;                                         // of the B sites,
-  float* scB = reinterpret_cast<float*>(nbB + 8 * a.gmax);             // and the tile scales of the B sites
+  int* nbB = nbA + 8 * a.gmax;                                         // [gmax][ND] of the B sites,
+  float* scB = reinterpret_cast<float*>(nbB + 9 * a.gmax);             // and the tile scales of the B sites
 
   const Items A(bid, G, a.NA, a.ipsA, W, wid), B(bid, G, a.NB, a.ipsB, W, wid);
   Stream st;
@@ -407,23 +411,30 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
     s_fail = 0;
   }
   for (int i = threadIdx.x; i < 8 * nA; i += kThreads) nbA[i] = a.nbr[(size_t)(a.half + sA) * 8 + i];
-  for (int i = threadIdx.x; i < 8 * nB; i += kThreads) {
-    nbB[i] = a.nbr[(size_t)sB * 8 + i];
-    scB[i] = a.Ys[(size_t)sB * 8 + i];
+  if (EO) {
+    for (int i = threadIdx.x; i < 8 * nB; i += kThreads) {
+      nbB[i] = a.nbr[(size_t)sB * 8 + i];
+      scB[i] = a.Ys[(size_t)sB * 8 + i];
+    }
+  } else {
+    for (int i = threadIdx.x; i < 9 * nB; i += kThreads) {
+      const int sl = i / 9, d = i - 9 * sl;
+      nbB[i] = d < 8 ? a.nbr[(size_t)(sB + sl) * 8 + d] : sB + sl;
+    }
   }
   __syncthreads();
   if (lane == 0)
-    for (unsigned p = 0; p < kStagesPerWarp; p++) issue<W>(a, st, A, B, p);
+    for (unsigned p = 0; p < kStagesPerWarp; p++) issue<W, ND>(a, st, A, B, p);
 
   int mode = M_INIT, k = 0;
   long long its = 0;
   df tol2 = df_of(0.f);
   while (true) {
-    if (mode != M_INIT) {
+    if (EO && mode != M_INIT) {
       // phase A: A v on the odd sites; in the closing pass v = y, and the odd
       // half of the solution is x_o = X_o^{-1} b_o - A y
-      gather<W>(nc, nA, nbA, nullptr, mode == M_ITER ? a.r : a.y, gv);
-      ok = run_items<kStF32, R, W>(a, st, A, B, A, gv, [&](int e, float2 u) {
+      gather<W, ND>(nc, nA, nbA, nullptr, mode == M_ITER ? a.r : a.y, gv);
+      ok = run_items<kStF32, R, W, ND>(a, st, A, B, A, gv, [&](int e, float2 u) {
         a.tB[oA + e] = u;
         if (mode == M_CLOSE) {
           const float2 o = a.to[oA + e];
@@ -433,23 +444,32 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
       if (!ok || !(ok = grid_barrier(a.bar, a.abort, target))) break;
     }
     // phase B on the even sites: w = r - Y_eo t, without r outside the iterations
-    gather<W>(nc, nB, nbB, scB, mode == M_INIT ? a.to : a.tB, gv);
-    ok = run_items<ST, RB_, W>(a, st, A, B, B, gv, [&](int e, float2 u) {
-      const float2 o = mode == M_ITER ? rs[e - offB] : make_float2(0.f, 0.f);
-      ws[e - offB] = make_float2(o.x - u.x, o.y - u.y);
-    }, &s_fail);
-    if (!ok) break;
+    // (or w = D_hat v on all sites)
+    if (EO || mode != M_INIT) {
+      if (EO)
+        gather<W, ND>(nc, nB, nbB, scB, mode == M_INIT ? a.to : a.tB, gv);
+      else
+        gather<W, ND>(nc, nB, nbB, nullptr, mode == M_ITER ? a.r : a.y, gv);
+      ok = run_items<ST, RB_, W, ND>(a, st, A, B, B, gv, [&](int e, float2 u) {
+        const float2 o = EO && mode == M_ITER ? rs[e - offB] : make_float2(0.f, 0.f);
+        ws[e - offB] = EO ? make_float2(o.x - u.x, o.y - u.y) : u;
+      }, &s_fail);
+      if (!ok) break;
+    }
     if (mode != M_ITER) {
       // b_r = b_e - Y_eo X_o^{-1} b_o, r = b_r, y = 0; or the true r = b_r - D_r y
       v[0] = v[1] = 0.f;
       for (int e = threadIdx.x; e < E; e += kThreads) {
-        const float2 u = ws[e];
-        float2 rr;
+        float2 rr, u = make_float2(0.f, 0.f);
+        if (EO || mode != M_INIT) u = ws[e];
         if (mode == M_INIT) {
           const float2 bb = a.b[E0 + e];
           rr = make_float2(bb.x + u.x, bb.y + u.y);
-          a.br[E0 + e] = rr;
+          if (EO) a.br[E0 + e] = rr;
           a.y[E0 + e] = make_float2(0.f, 0.f);
+        } else if (!EO) {
+          const float2 bb = a.b[E0 + e];
+          rr = make_float2(bb.x - u.x, bb.y - u.y);
         } else {
           const float2 bb = a.br[E0 + e], yy = a.y[E0 + e];
           rr = make_float2(bb.x - (yy.x + u.x), bb.y - (yy.y + u.y));
@@ -459,8 +479,8 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
         v[0] = fmaf(rr.x, rr.x, fmaf(rr.y, rr.y, v[0]));
       }
       if (mode == M_INIT) {   // ||b||^2 over the full right-hand side (any partition of it)
-        const size_t cf = (2 * n + G - 1) / G;
-        const size_t f0 = (size_t)bid * cf, f1 = f0 + cf < 2 * n ? f0 + cf : 2 * n;
+        const size_t nf = EO ? 2 * n : n, cf = (nf + G - 1) / G;
+        const size_t f0 = (size_t)bid * cf, f1 = f0 + cf < nf ? f0 + cf : nf;
         for (size_t e = f0 + threadIdx.x; e < f1; e += kThreads) {
           const float2 q = a.b[e];
           v[1] = fmaf(q.x, q.x, fmaf(q.y, q.y, v[1]));
@@ -650,7 +670,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
     }
     if (rn2.h <= tol2.h || k == m || its >= a.maxit) mode = M_CLOSE;
   }
-  if (ok && its == 0)   // b = 0: y = 0 and x_o = t_o
+  if (EO && ok && its == 0)   // b = 0: y = 0 and x_o = t_o
     for (size_t e = (size_t)bid * kThreads + threadIdx.x; e < n; e += (size_t)G * kThreads) a.x[n + e] = a.to[n + e];
   if (!ok && threadIdx.x == 0) {
     atomicExch(&a.flags[FLAG_TIMEOUT], 1);
@@ -675,19 +695,19 @@ int pow2_floor(int v) {
 }
 
 // items, the sites a block's item ranges touch, and the shared memory they need
-void plan_items(Plan& p, int half, int nc, int store) {
-  const int K = 8 * nc;
+void plan_items(Plan& p, int sites, int nc, int nd, int store) {
+  const int K = nd * nc;
   p.rowsA = pow2_floor(std::min(p.warps == 16 ? kMaxRows : 2, std::min(nc, p.stage_bytes / (K * 8))));
   p.rowsB = rows_b(store == STORE_F32 ? kStF32 : kStF16, p.rowsA);
   p.ipsA = p.rowsA > 0 ? (nc + p.rowsA - 1) / p.rowsA : 0;
   p.ipsB = p.rowsB > 0 ? (nc + p.rowsB - 1) / p.rowsB : 0;
-  p.NA = half * p.ipsA;
-  p.NB = half * p.ipsB;
+  p.NA = sites * p.ipsA;
+  p.NB = sites * p.ipsB;
   p.gmax = 1;
   p.emax = 0;
   const int G = std::min(p.grid, std::min(p.NA, p.NB));
   auto elem = [&](int i) -> long long {   // item_elem of the kernel
-    return i == p.NB ? (long long)half * nc : (long long)(i / p.ipsB) * nc + (long long)(i % p.ipsB) * p.rowsB;
+    return i == p.NB ? (long long)sites * nc : (long long)(i / p.ipsB) * nc + (long long)(i % p.ipsB) * p.rowsB;
   };
   for (int b = 0; b < G && p.rowsA > 0 && p.rowsB > 0; b++) {
     const int a0 = (int)((long long)b * p.NA / G), a1 = (int)((long long)(b + 1) * p.NA / G);
@@ -701,22 +721,23 @@ void plan_items(Plan& p, int half, int nc, int store) {
 Plan plan_warps(const LevelGeom& G, const CoarseOp& C, int grid, int m, int warps) {
   Plan p;
   p.warps = warps;
-  const int nc = C.nc, K = 8 * nc, stages = warps * kStagesPerWarp;
+  const int nc = C.nc, nd = G.eo ? 8 : 9, K = nd * nc, stages = warps * kStagesPerWarp;
+  const int sites = G.eo ? G.half : G.nsites, store = G.eo ? C.store : STORE_F32;
   int dev = 0, optin = 0;
   MG_CUDA(cudaGetDevice(&dev));
   MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const size_t budget = (size_t)optin - 4096;   // static shared memory and slack
   const size_t fixed = sizeof(float2) * (4 * warps + kNR) + sizeof(float2) * 2 * 32 * warps;
-  const size_t per_site = sizeof(float2) * K + 24 * sizeof(int);   // gathered vector, neighbours, tile scales
+  const size_t per_site = sizeof(float2) * K + 25 * sizeof(int);   // gathered vector, neighbours, tile scales
   p.grid = grid;
   // the w_j slice in shared memory only when it is small (a sixteenth of the
   // budget): measured on GB300 at Nc = 48, m = 64, a deeper link ring gains
   // more than shared-memory Gram-Schmidt vectors save.  A block's slice has
   // at most ceil(n / grid) elements plus the rows of the partial items at
   // both ends of its range.  r and w of the owned rows: an eighth.
-  const size_t n = (size_t)G.half * nc;
+  const size_t n = (size_t)sites * nc;
   const int gb = std::max(1, grid);
-  const int ebound = (int)((n + gb - 1) / gb) + (int)((7LL * G.half + gb - 1) / gb) + 2 * kMaxRows;
+  const int ebound = (int)((n + gb - 1) / gb) + (int)((7LL * sites + gb - 1) / gb) + 2 * kMaxRows;
   const bool wsmem = (size_t)m * ebound * sizeof(float2) <= budget / 16;
   const bool esmem = 2 * (size_t)ebound * sizeof(float2) <= budget / 8;
   const size_t wbytes = (wsmem ? (size_t)m * ebound * sizeof(float2) : 0) + (esmem ? 2 * (size_t)ebound * sizeof(float2) : 0);
@@ -724,7 +745,7 @@ Plan plan_warps(const LevelGeom& G, const CoarseOp& C, int grid, int m, int warp
   for (int pass = 0; pass < 3; pass++) {
     const size_t other = fixed + wbytes + per_site * (size_t)gsites;
     p.stage_bytes = budget > other ? (int)(((budget - other) / stages) / 16 * 16) : 0;
-    plan_items(p, G.half, nc, C.store);
+    plan_items(p, sites, nc, nd, store);
     if (p.gmax <= gsites) break;
     gsites = p.gmax;
   }
@@ -737,23 +758,27 @@ Plan plan_warps(const LevelGeom& G, const CoarseOp& C, int grid, int m, int warp
   return p;
 }
 
-// 16 warps where their 32 stages hold items of two rows or more (Nc up to about
-// 64), 8 beyond: 16 halve the serial chain of a warp, two to three items per
-// phase at 16^3x32.
+// 16 warps where their 32 stages hold items of two rows or more (Nc = 48 with a
+// few sites per block), 8 otherwise: 16 halve the serial chain of a warp, two to
+// three items per phase at 16^3x32.
 Plan make_plan(const LevelGeom& G, const CoarseOp& C, int grid, int m) {
   const Plan p = plan_warps(G, C, grid, m, 16);
   return p.rowsA >= 2 ? p : plan_warps(G, C, grid, m, 8);
 }
 
 template <int W, int R>
-const void* kernel_st(int store) {
-  return store == STORE_F16    ? (const void*)k_coarse_gcr_stream<kStF16, W, R>
-         : store == STORE_BF16 ? (const void*)k_coarse_gcr_stream<kStBF16, W, R>
-                               : (const void*)k_coarse_gcr_stream<kStF32, W, R>;
+const void* kernel_st(int store, bool eo) {
+  return !eo                  ? (const void*)k_coarse_gcr_stream<kStF32, W, R, false>
+         : store == STORE_F16  ? (const void*)k_coarse_gcr_stream<kStF16, W, R, true>
+         : store == STORE_BF16 ? (const void*)k_coarse_gcr_stream<kStBF16, W, R, true>
+                               : (const void*)k_coarse_gcr_stream<kStF32, W, R, true>;
 }
-const void* kernel_for(int store, const Plan& p) {
-  if (p.warps == 16) return p.rowsA == 8 ? kernel_st<16, 8>(store) : p.rowsA == 4 ? kernel_st<16, 4>(store) : kernel_st<16, 2>(store);
-  return p.rowsA >= 2 ? kernel_st<8, 2>(store) : kernel_st<8, 1>(store);
+const void* kernel_for(int store, bool eo, const Plan& p) {
+  if (p.warps == 16)
+    return p.rowsA == 8   ? kernel_st<16, 8>(store, eo)
+           : p.rowsA == 4 ? kernel_st<16, 4>(store, eo)
+                          : kernel_st<16, 2>(store, eo);
+  return p.rowsA >= 2 ? kernel_st<8, 2>(store, eo) : kernel_st<8, 1>(store, eo);
 }
 
 int sm_count() {
@@ -766,7 +791,7 @@ int sm_count() {
 }  // namespace
 
 bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C) {
-  if (!G.eo || C.nc % 2 || !C.A.get()) return false;
+  if (C.nc % 2 || !C.A.get()) return false;
   const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
   return p.rowsA >= 1 && p.rowsB >= 1 && p.smem <= 232448;
 }
@@ -792,11 +817,11 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   const Plan p = make_plan(G, C, grid, m);
   const int sms = sm_count();
   int per = 0;
-  const void* kern = kernel_for(C.store, p);
+  const void* kern = kernel_for(C.store, G.eo, p);
   MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
   MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * p.warps, p.smem));
   if (per < 1 || p.grid > per * sms) raise(MG_ERR_CUDA, "streamed coarse GCR cannot be resident");
-  const size_t n = (size_t)G.half * C.nc;
+  const size_t n = (size_t)(G.eo ? G.half : G.nsites) * C.nc;
   auto need = [&](DBuf& d, size_t bytes) {
     if (d.bytes() < bytes) d.alloc(bytes);
   };
@@ -804,35 +829,37 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   need(B.st_sync, 256);
   if (B.W.bytes() < sizeof(float2) * n * m || B.Z.bytes() < sizeof(float2) * n * m)
     raise(MG_ERR_STATE, "coarse GCR buffers too small for this restart length");
-  need(B.st_to, sizeof(float2) * 2 * n);
-  coarse_site_mul(G, C, true, G.half, G.nsites, B.st_to.as<float>(), b, s);     // t_o = X_o^{-1} b_o
+  if (G.eo) {
+    need(B.st_to, sizeof(float2) * 2 * n);
+    coarse_site_mul(G, C, true, G.half, G.nsites, B.st_to.as<float>(), b, s);     // t_o = X_o^{-1} b_o
+  }
   MG_CUDA(cudaMemsetAsync(B.st_sync.get(), 0, 256, s));
   SArgs a;
   std::memset(&a, 0, sizeof(a));
   a.nc = C.nc;
-  a.half = G.half;
+  a.half = G.eo ? G.half : G.nsites;
   a.m = m;
   a.maxit = maxit;
   a.rowsA = p.rowsA;
   a.rowsB = p.rowsB;
   a.ipsA = p.ipsA;
   a.ipsB = p.ipsB;
-  a.NA = p.NA;
+  a.NA = G.eo ? p.NA : 0;
   a.NB = p.NB;
-  a.eszB = C.store == STORE_F32 ? 8 : 4;
+  a.eszB = !G.eo || C.store == STORE_F32 ? 8 : 4;
   a.stage_bytes = p.stage_bytes;
   a.gmax = p.gmax;
   a.wsm_ld = p.wsm_ld;
   a.esm = p.esm;
   a.tol_rel = tol_rel;
   a.nbr = G.d_nbr.as<int>();
-  a.Y = static_cast<const unsigned char*>(C.Y.get());
+  a.Y = static_cast<const unsigned char*>(G.eo ? C.Y.get() : C.A.get());
   a.Ys = C.Yscale.as<float>();
   a.Af = static_cast<const unsigned char*>(C.A.get());
   a.b = reinterpret_cast<const float2*>(b);
   a.to = B.st_to.as<float2>();
   a.x = reinterpret_cast<float2*>(x);
-  a.y = B.y.as<float2>();
+  a.y = G.eo ? B.y.as<float2>() : a.x;
   a.r = B.r.as<float2>();
   a.br = B.br.as<float2>();
   a.tB = B.tB.as<float2>();
@@ -847,7 +874,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   void* params[] = {&a};
   MG_CUDA(cudaLaunchCooperativeKernel(kern, dim3(p.grid), dim3(32 * p.warps), params, p.smem, s));
   MG_LAUNCH();
-  coarse_site_mul(G, C, true, 0, G.half, x, B.y.as<float>(), s);   // x_e = X_e^{-1} y_e; the kernel wrote x_o
+  if (G.eo) coarse_site_mul(G, C, true, 0, G.half, x, B.y.as<float>(), s);   // x_e = X_e^{-1} y_e; the kernel wrote x_o
 }
 
 }  // namespace mg

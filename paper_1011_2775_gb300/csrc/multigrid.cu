@@ -279,9 +279,9 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
     // batched kernel with one system (row-blocked GEMV: fewer registers, more
     // co-resident CTAs).  The autotuner times them on the first solve of this
     // lattice (the tuning runs do not count towards the iteration statistics).
-    // The streamed kernel (links through shared memory by bulk copies, even-odd
-    // levels) is a third implementation, on the full grid or on the largest
-    // grid that splits its work evenly; candidates 100 + k.
+    // The streamed kernel (links through shared memory by bulk copies) is a third
+    // implementation, on the full grid or on the largest grid that splits its
+    // work evenly; candidates 100 + k.
     const int restart = p.restart_coarse > 0 ? p.restart_coarse : 32;
     long long* d_it = H.d_iters.as<long long>() + l;
     const std::vector<int> smaller = coarse_gcr_smaller_grids(G, W.cg);
@@ -315,8 +315,8 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
       std::vector<int> cands = {0, 1};
       for (size_t k = 0; k < smaller.size(); k++) cands.push_back(2 + (int)k);
       for (size_t k = 0; k < streamed.size(); k++) cands.push_back(100 + (int)k);
-      // the grouped kernel with one system (candidate 300) also takes odd-extent lattices (3^3x6 sites, Nc = 48:
-      // 99 us against 243 us of the single-system kernel); on even-odd lattices it is timed against the streamed one
+      // the grouped kernel with one system (candidate 300) is timed against the streamed one (3^3x6 sites, Nc = 48:
+      // 112 us and 67 us; the single-system kernel takes 243 us)
       if (grouped) cands.push_back(300);
       const int forced = c->params.coarse_impl;
       // one system on tensor cores uses one column of eight of every MMA and
