@@ -36,8 +36,10 @@
 //
 // Measured (16^3x32, 4^4 blocks, Nc = 48, 256 reduced sites, twelve systems,
 // 34 iterations): 10.1 ms per launch on the tensor-core kernel, whose site
-// inverses and Krylov loops ran on a few warps, 2.65 ms here.  One system of a
-// 3^3x6 lattice: 243 us on the single-system kernel, 99 us here.  Reductions
+// inverses and Krylov loops ran on a few warps; 2.33 ms with the next links in
+// flight only within an item, the epilogue's reads after the sums and whole
+// warps on the inner products; 2.20 ms here, 65 us per iteration of which the
+// FMAs of the two stencil phases are 12 and the four barriers 6.  Reductions
 // are double-float and added in a fixed order; every wait is bounded in time
 // (async_copy.cuh); FLAG_TIMEOUT on expiry.
 #include <algorithm>
@@ -90,42 +92,58 @@ struct GArgs {
 // gathered vectors of `ns` sites from s0: gv[(site, p)][K] complex, times the
 // tile scale; nbd neighbours (8, or 9 with the site itself); in: element
 // (storage - base) nc of system p at in + p n.  A warp takes one neighbour of
-// one site for all systems (lanes over its nc / 2 <= 32 pairs): no index
-// arithmetic per element, up to NS loads in flight per lane.
+// one site for all systems (lanes over its nc / 2 <= 32 pairs), 32 neighbours
+// to a round: their indices and scales come in one trip to L2, the vectors of
+// kPairs neighbours in the next.
 template <int NS>
 __device__ void gather(const GArgs& a, size_t n, int store0, int s0, int ns, int nbd, int base, const float2* in,
                        const float* scale, float4* gv) {
-  const int hc = a.nc >> 1, K2 = nbd * hc;
+  constexpr int kPairs = NS <= 4 ? 4 : 2;
+  const int hc = a.nc >> 1, K2 = nbd * hc, nt = ns * nbd;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const size_t n2 = n >> 1;
-  for (int t = w; t < ns * nbd; t += kWarps) {
-    const int sl = t / nbd, d = t - sl * nbd, st = store0 + s0 + sl;
-    const int from = d < 8 ? a.nbr[(size_t)st * 8 + d] : st;
-    const float sc = scale && d < 8 ? scale[(size_t)st * 8 + d] : 1.f;
-    if (lane >= hc) continue;
-    const float4* src = reinterpret_cast<const float4*>(in) + (size_t)(from - base) * hc + lane;
-    float4* dst = gv + (size_t)sl * NS * K2 + d * hc + lane;
-    constexpr int U = NS < 12 ? NS : 12;
+  for (int tb = w; tb < nt; tb += 32 * kWarps) {
+    const int tl = min(tb + lane * kWarps, nt - 1), sll = tl / nbd, dl = tl - sll * nbd, stl = store0 + s0 + sll;
+    const int froml = dl < 8 ? a.nbr[(size_t)stl * 8 + dl] : stl;
+    const float scl = scale && dl < 8 ? scale[(size_t)stl * 8 + dl] : 1.f;
+    const int cnt = min(32, (nt - tb + kWarps - 1) / kWarps);
+    for (int c = 0; c < cnt; c += kPairs) {
+      constexpr int U = NS < 12 ? NS : 12;
 #pragma unroll
-    for (int p0 = 0; p0 < NS; p0 += U) {
-      float4 v[U];
+      for (int p0 = 0; p0 < NS; p0 += U) {
+        float4 v[kPairs][U];
 #pragma unroll
-      for (int u = 0; u < U; u++)
-        v[u] = p0 + u < a.nb ? __ldcg(src + (size_t)(p0 + u) * n2) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int x = 0; x < kPairs; x++) {
+          const int from = __shfl_sync(0xffffffffu, froml, min(c + x, cnt - 1));
+          const float4* src = reinterpret_cast<const float4*>(in) + (size_t)(from - base) * hc + lane;
 #pragma unroll
-      for (int u = 0; u < U; u++)
-        if (p0 + u < NS)
-          dst[(size_t)(p0 + u) * K2] = make_float4(sc * v[u].x, sc * v[u].y, sc * v[u].z, sc * v[u].w);
+          for (int u = 0; u < U; u++)
+            v[x][u] = lane < hc && p0 + u < a.nb ? __ldcg(src + (size_t)(p0 + u) * n2) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int x = 0; x < kPairs; x++) {
+          const int cx_ = min(c + x, cnt - 1);   // past the end the last neighbour is written again
+          const float sc = __shfl_sync(0xffffffffu, scl, cx_);
+          const int t = tb + cx_ * kWarps, sl = t / nbd, d = t - sl * nbd;
+          float4* dst = gv + (size_t)sl * NS * K2 + d * hc + lane;
+#pragma unroll
+          for (int u = 0; u < U; u++)
+            if (lane < hc && p0 + u < NS)
+              dst[(size_t)(p0 + u) * K2] = make_float4(sc * v[x][u].x, sc * v[x][u].y, sc * v[x][u].z, sc * v[x][u].w);
+        }
+      }
     }
   }
   __syncthreads();
 }
 
-// one stencil phase over the block's items [i0, i1): epi(p, element, value) for
-// every row and system; links of site s at links + s nc K entries
-template <int ST, int NS, typename Epi>
+// one stencil phase over the block's items [i0, i1): epi(p, element, value, pre)
+// for every row and system, with pre = pre(p, element) read before the item's
+// arithmetic (in the epilogue it was three more trips to L2 per item); links of
+// site s at links + s nc K entries
+template <int ST, int NS, typename Pre, typename Epi>
 __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int i0, int i1, int store0, int nbd,
-                      int base, const float2* in, const float* scale, float4* gv, Epi epi) {
+                      int base, const float2* in, const float* scale, float4* gv, Pre pre, Epi epi) {
   const int nc = a.nc, K2 = nbd * (nc >> 1);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int sbeg = i0 / a.ips, send = i1 > i0 ? (i1 - 1) / a.ips + 1 : sbeg;
@@ -133,19 +151,42 @@ __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int 
     const int ns = min(a.chunk, send - s0);
     gather<NS>(a, n, store0, s0, ns, nbd, base, in, scale, gv);
     const int c0 = max(i0, s0 * a.ips), c1 = min(i1, (s0 + ns) * a.ips);
-    for (int it = c0 + w; it < c1; it += kWarps) {
+    using raw_t = typename LinkPair<ST>::raw;
+    const unsigned char* row[kRows];
+    auto rows_of = [&](int it) {
       const int s = it / a.ips, r0 = (it - s * a.ips) * kRows;
-      const unsigned char* row[kRows];
 #pragma unroll
       for (int r = 0; r < kRows; r++)   // a row past the end repeats the last one and is dropped
-        row[r] = links + ((size_t)s * nc + min(r0 + r, nc - 1)) * (size_t)(2 * K2) * link_bytes<ST>();
+        row[r] = links + ((size_t)s * nc + min(r0 + r, nc - 1)) * (size_t)K2 * sizeof(raw_t);
+    };
+    auto load = [&](raw_t (&m)[kRows], int q) {
+#pragma unroll
+      for (int r = 0; r < kRows; r++) m[r] = q < K2 ? LinkPair<ST>::load(row[r], q) : LinkPair<ST>::zero();
+    };
+    // several systems: the links of the next step are in flight, across items too
+    raw_t nx[kRows];
+    if (NS > 1 && c0 + w < c1) {
+      rows_of(c0 + w);
+      load(nx, lane);
+    }
+    for (int it = c0 + w; it < c1; it += kWarps) {
+      const int s = it / a.ips, r0 = (it - s * a.ips) * kRows;
+      if (NS == 1) rows_of(it);
+      // value f = (r NS + p) 2 + {re, im}: 32 at a time (8 with one system)
+      constexpr int V = kRows * NS * 2 < 32 ? kRows * NS * 2 : 32, per = 32 / V, NG = kRows * NS * 2 / V;
+      float2 before[NG];
+#pragma unroll
+      for (int g = 0; g < NG; g++) {
+        const int f = g * V + lane / per, r = (f >> 1) / NS, p = (f >> 1) % NS;
+        before[g] = lane % (2 * per) == 0 && p < a.nb && r0 + r < nc ? pre(p, (size_t)s * nc + r0 + r) : make_float2(0.f, 0.f);
+      }
       float acc[kRows][NS][2];
 #pragma unroll
       for (int r = 0; r < kRows; r++)
 #pragma unroll
         for (int p = 0; p < NS; p++) acc[r][p][0] = acc[r][p][1] = 0.f;
       const float4* v = gv + (size_t)(s - s0) * NS * K2;
-      auto step = [&](const typename LinkPair<ST>::raw (&raw)[kRows], int q) {
+      auto step = [&](const raw_t (&raw)[kRows], int q) {
         float4 l[kRows];
 #pragma unroll
         for (int r = 0; r < kRows; r++) l[r] = LinkPair<ST>::decode(raw[r]);
@@ -169,34 +210,29 @@ __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int 
         // one system: bound by the links' way from L2, so a lane keeps up to
         // kDeep steps of all rows in flight (98 KB per SM)
         for (int q0 = lane; q0 < K2; q0 += 32 * kDeep) {
-          typename LinkPair<ST>::raw raw[kDeep][kRows];
+          raw_t raw[kDeep][kRows];
 #pragma unroll
-          for (int u = 0; u < kDeep; u++)
-#pragma unroll
-            for (int r = 0; r < kRows; r++)
-              raw[u][r] = q0 + 32 * u < K2 ? LinkPair<ST>::load(row[r], q0 + 32 * u) : LinkPair<ST>::zero();
+          for (int u = 0; u < kDeep; u++) load(raw[u], q0 + 32 * u);
 #pragma unroll
           for (int u = 0; u < kDeep; u++)
             if (q0 + 32 * u < K2) step(raw[u], q0 + 32 * u);
         }
       } else {
-        typename LinkPair<ST>::raw cur[kRows], nx[kRows];
-#pragma unroll
-        for (int r = 0; r < kRows; r++) nx[r] = lane < K2 ? LinkPair<ST>::load(row[r], lane) : LinkPair<ST>::zero();
-        for (int q = lane; q < K2; q += 32) {
+        raw_t cur[kRows];
+        for (int q0 = 0; q0 < K2; q0 += 32) {
 #pragma unroll
           for (int r = 0; r < kRows; r++) cur[r] = nx[r];
-          if (q + 32 < K2) {
-#pragma unroll
-            for (int r = 0; r < kRows; r++) nx[r] = LinkPair<ST>::load(row[r], q + 32);
+          if (q0 + 32 < K2) {
+            load(nx, q0 + 32 + lane);
+          } else if (it + kWarps < c1) {
+            rows_of(it + kWarps);
+            load(nx, lane);
           }
-          step(cur, q);
+          if (q0 + lane < K2) step(cur, q0 + lane);
         }
       }
-      // value f = (r NS + p) 2 + {re, im}: 32 at a time (8 with one system)
-      constexpr int V = kRows * NS * 2 < 32 ? kRows * NS * 2 : 32, per = 32 / V;
 #pragma unroll
-      for (int g = 0; g < kRows * NS * 2 / V; g++) {
+      for (int g = 0; g < NG; g++) {
         float val[V];
 #pragma unroll
         for (int i = 0; i < V; i++) {
@@ -207,7 +243,7 @@ __device__ void phase(const GArgs& a, size_t n, const unsigned char* links, int 
         const float im = __shfl_down_sync(0xffffffffu, re, per);
         const int f = g * V + lane / per;
         const int r = (f >> 1) / NS, p = (f >> 1) % NS;
-        if (lane % (2 * per) == 0 && p < a.nb && r0 + r < nc) epi(p, (size_t)s * nc + r0 + r, make_float2(re, im));
+        if (lane % (2 * per) == 0 && p < a.nb && r0 + r < nc) epi(p, (size_t)s * nc + r0 + r, make_float2(re, im), before[g]);
       }
     }
     __syncthreads();
@@ -293,14 +329,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
   auto Rk = [&](int k, int p) { return a.R + ((size_t)k * nb + p) * n + E0; };
   auto partial = [&](int p, int q, df s) { a.part[((size_t)p * kSlots + q) * G + bid] = make_float2(s.h, s.l); };
   // w = D v for all systems: t on the odd sites, a barrier, out(p, element, Y_eo t); or out(p, element, D_hat v)
-  auto apply = [&](const float2* in, auto out) -> bool {
+  auto none = [](int, size_t) { return make_float2(0.f, 0.f); };
+  auto apply = [&](const float2* in, auto pre, auto out) -> bool {
     if (EO) {
-      phase<kStF32, NS>(a, n, a.A, i0, i1, a.half, 8, 0, in, nullptr, gv,
-                        [&](int p, size_t e, float2 u) { a.t[(size_t)p * n + e] = u; });
+      phase<kStF32, NS>(a, n, a.A, i0, i1, a.half, 8, 0, in, nullptr, gv, none,
+                        [&](int p, size_t e, float2 u, float2) { a.t[(size_t)p * n + e] = u; });
       if (!grid_barrier(a.bar, a.abort, target)) return false;
-      phase<ST, NS>(a, n, a.Y, i0, i1, 0, 8, a.half, a.t, a.Ys, gv, out);
+      phase<ST, NS>(a, n, a.Y, i0, i1, 0, 8, a.half, a.t, a.Ys, gv, pre, out);
     } else {
-      phase<kStF32, NS>(a, n, a.A, i0, i1, 0, 9, 0, in, nullptr, gv, out);
+      phase<kStF32, NS>(a, n, a.A, i0, i1, 0, 9, 0, in, nullptr, gv, pre, out);
     }
     return true;
   };
@@ -333,8 +370,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
   }
   // r = b_r = b_e - Y_eo X_o^{-1} b_o (or b), y = 0 on the owned elements
   if (EO)
-    phase<ST, NS>(a, n, a.Y, i0, i1, 0, 8, a.half, a.tb, a.Ys, gv, [&](int p, size_t e, float2 u) {
-      const float2 bb = a.b[p][e];
+    phase<ST, NS>(a, n, a.Y, i0, i1, 0, 8, a.half, a.tb, a.Ys, gv, [&](int p, size_t e) { return a.b[p][e]; },
+                  [&](int p, size_t e, float2 u, float2 bb) {
       a.br[(size_t)p * n + e] = make_float2(bb.x - u.x, bb.y - u.y);
     });
   for (int q = threadIdx.x; q < nb * E; q += kThreads) {
@@ -371,59 +408,59 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
     while (k < m && its < a.maxit && s_run) {
       const unsigned run = s_run;
       // w = D r into the history slot, on the owned elements
-      if (!(ok = apply(a.r, [&](int p, size_t e, float2 u) {
-              if (EO) {
-                const float2 rr = a.r[(size_t)p * n + e];
-                u = make_float2(rr.x - u.x, rr.y - u.y);
-              }
+      if (!(ok = apply(a.r, [&](int p, size_t e) { return EO ? a.r[(size_t)p * n + e] : make_float2(0.f, 0.f); },
+                       [&](int p, size_t e, float2 u, float2 rr) {
+              if (EO) u = make_float2(rr.x - u.x, rr.y - u.y);
               a.W[((size_t)k * nb + p) * n + e] = u;
             })))
         break;
-      // <w_j, w> (a warp takes eight j of one system, two elements per load), ||w||^2 and <w, r>
-      const int groups = max(1, (k + 7) >> 3);
+      // <w_j, w> (a half-warp takes four j of one system, two elements per load: 16
+      // lanes leave fewer of them idle on a short slice and half the sums to
+      // reduce per lane), ||w||^2 and <w, r>
+      const int groups = max(1, (k + 7) >> 3), l16 = lane & 15;
       for (int task = wid; task < nb * groups; task += kWarps) {
         const int p = task % nb, gi = task / nb;
         if (!((run >> p) & 1u)) continue;
         const float4* wk = reinterpret_cast<const float4*>(Wk(k, p));
         const float4* rp = reinterpret_cast<const float4*>(a.r + (size_t)p * n + E0);
-        const int j0 = 8 * gi;
-        float re[8], im[8], s0 = 0.f, s1 = 0.f, s2 = 0.f;
+        const int j0 = 8 * gi + 4 * (lane >> 4);
+        float re[4], im[4], s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll
-        for (int u = 0; u < 8; u++) re[u] = im[u] = 0.f;
-#pragma unroll 2
-        for (int e = lane; e < E2; e += 32) {
-          float4 q[8];
+        for (int u = 0; u < 4; u++) re[u] = im[u] = 0.f;
+#pragma unroll 3
+        for (int e = l16; e < E2; e += 16) {
+          float4 q[4];
 #pragma unroll
-          for (int u = 0; u < 8; u++)
+          for (int u = 0; u < 4; u++)
             q[u] = j0 + u < k ? __ldcg(reinterpret_cast<const float4*>(Wk(j0 + u, p)) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
           const float4 x = __ldcg(wk + e);
-          if (gi == 0) {
+          if (gi == 0 && lane < 16) {
             const float4 rr = __ldcg(rp + e);
             s0 = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, s0))));
             s1 = fmaf(x.x, rr.x, fmaf(x.y, rr.y, fmaf(x.z, rr.z, fmaf(x.w, rr.w, s1))));
             s2 = fmaf(x.x, rr.y, fmaf(-x.y, rr.x, fmaf(x.z, rr.w, fmaf(-x.w, rr.z, s2))));
           }
 #pragma unroll
-          for (int u = 0; u < 8; u++) {
+          for (int u = 0; u < 4; u++) {
             re[u] = fmaf(q[u].x, x.x, fmaf(q[u].y, x.y, fmaf(q[u].z, x.z, fmaf(q[u].w, x.w, re[u]))));
             im[u] = fmaf(q[u].x, x.y, fmaf(-q[u].y, x.x, fmaf(q[u].z, x.w, fmaf(-q[u].w, x.z, im[u]))));
           }
         }
         if (k > 0) {
-          df v[16];
+          df v[8];
 #pragma unroll
-          for (int u = 0; u < 8; u++) {
+          for (int u = 0; u < 4; u++) {
             v[2 * u] = df_of(re[u]);
             v[2 * u + 1] = df_of(im[u]);
           }
-          const df t = warp_transpose_sum<16>(v);   // lane l: value l >> 1
-          const int q = 2 * j0 + (lane >> 1);
-          if ((lane & 1) == 0 && q < 2 * k) partial(p, q, t);
+          const df t = warp_transpose_sum<8, 16>(v);   // lane l of a half: value l >> 1
+          const int q = 2 * j0 + (l16 >> 1);
+          if ((l16 & 1) == 0 && q < 2 * k) partial(p, q, t);
         }
         if (gi == 0) {
           df v[4] = {df_of(s0), df_of(s1), df_of(s2), df_of(0.f)};
-          const df t = warp_transpose_sum<4>(v);   // lane l: value l >> 3
-          if ((lane & 7) == 0 && (lane >> 3) < 3) partial(p, QW + (lane >> 3), t);
+          const df t = warp_transpose_sum<4, 16>(v);   // lane l of a half: value l >> 2
+          if ((lane & 3) == 0 && (lane >> 2) < 3) partial(p, QW + (lane >> 2), t);
         }
       }
       if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
@@ -618,7 +655,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
     }
     if (!(ok = grid_barrier(a.bar, a.abort, target))) break;
     // the true residual restarts r and its norm
-    if (!(ok = apply(a.y, [&](int p, size_t e, float2 u) {
+    if (!(ok = apply(a.y, none, [&](int p, size_t e, float2 u, float2) {
             const size_t i = (size_t)p * n + e;
             if (EO) {
               const float2 yy = a.y[i];

@@ -91,10 +91,10 @@ __device__ __forceinline__ df shfl_x(df v, int o) { return df{shfl_x(v.h, o), sh
 __device__ __forceinline__ float add_x(float a, float b) { return a + b; }
 __device__ __forceinline__ double add_x(double a, double b) { return a + b; }
 __device__ __forceinline__ df add_x(df a, df b) { return df_add(a, b); }
-template <int V, typename S>
+template <int V, int LANES = 32, typename S>
 __device__ __forceinline__ S warp_transpose_sum(S (&v)[V]) {
   const int lane = threadIdx.x & 31;
-  int off = 16;
+  int off = LANES / 2;
 #pragma unroll
   for (int half = V / 2; half >= 1; half /= 2, off /= 2) {
     const bool up = (lane & off) != 0;
@@ -107,7 +107,7 @@ __device__ __forceinline__ S warp_transpose_sum(S (&v)[V]) {
   }
   S t = v[0];
 #pragma unroll
-  for (int o = 16 / V; o >= 1; o /= 2) t = add_x(t, shfl_x(t, o));
+  for (int o = LANES / 2 / V; o >= 1; o /= 2) t = add_x(t, shfl_x(t, o));
   return t;
 }
 
