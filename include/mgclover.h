@@ -148,8 +148,8 @@ typedef struct {
                                   /* captured CUDA graph (0: launch its kernels one by one)        */
   int coarse_impl;                /* coarsest-level persistent GCR: 0 chosen by timing on the      */
                                   /* first solve; 1 single-system kernel, 2 batched kernel,        */
-                                  /* 3 links streamed through shared memory (even-odd levels),     */
                                   /* 3 links streamed through shared memory,                       */
+                                  /* 4 tensor cores (even-odd levels, FP16 storage, Nc a multiple  */
                                   /* of 8 up to 64; also the batched cycle's solves); an           */
                                   /* implementation that does not apply falls back to 1            */
   int outer_prec;                 /* MG mode: precision of the outer FGCR's product D_r z inside a */
