@@ -158,36 +158,39 @@ __global__ void k_dot2(const cx<T>* __restrict__ w, const cx<T>* __restrict__ r,
   const acc_t<T> v[3] = {s0, s1, s2};
   grid_reduce<3>(v, partials, counter, out);
 }
-// nrhs pairs (w_q, r_q) at `stride` complex apart: d_out[4q .. 4q+2] per pair,
-// one launch (blockIdx.y = q, a separate reduction per pair)
-template <typename T>
-__global__ void k_dot2_multi(const cx<T>* __restrict__ w, const cx<T>* __restrict__ r, size_t n, size_t stride,
-                             double* partials, unsigned* counters, double* out) {
+// nrhs pairs (w_q, r_q) of FP32 vectors at `stride` floats apart: d_out[4q ..
+// 4q+2] per pair, one launch (blockIdx.y = q, a separate reduction per pair);
+// 16 bytes per load, a sum for the first and one for the second of a pair of
+// complex numbers (n is even)
+__global__ void __launch_bounds__(kBS) k_dot2_multi(const float* __restrict__ w, const float* __restrict__ r, size_t n2,
+                                                    size_t stride, double* partials, unsigned* counters, double* out) {
   const int q = blockIdx.y;
-  w += q * stride;
-  r += q * stride;
-  acc_t<T> s0 = 0, s1 = 0, s2 = 0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    cx<T> a = w[i], b = r[i];
-    s0 = fma((acc_t<T>)a.re, (acc_t<T>)a.re, s0);
-    s0 = fma((acc_t<T>)a.im, (acc_t<T>)a.im, s0);
-    s1 = fma((acc_t<T>)a.re, (acc_t<T>)b.re, s1);
-    s1 = fma((acc_t<T>)a.im, (acc_t<T>)b.im, s1);
-    s2 = fma((acc_t<T>)a.re, (acc_t<T>)b.im, s2);
-    s2 = fma(-(acc_t<T>)a.im, (acc_t<T>)b.re, s2);
+  const float4* w4 = reinterpret_cast<const float4*>(w + q * stride);
+  const float4* r4 = reinterpret_cast<const float4*>(r + q * stride);
+  float s[2][3] = {};
+#pragma unroll 4
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n2; i += (size_t)gridDim.x * kBS) {
+    const float4 a = w4[i], b = r4[i];
+    s[0][0] = fmaf(a.x, a.x, fmaf(a.y, a.y, s[0][0]));
+    s[0][1] = fmaf(a.x, b.x, fmaf(a.y, b.y, s[0][1]));
+    s[0][2] = fmaf(a.x, b.y, fmaf(-a.y, b.x, s[0][2]));
+    s[1][0] = fmaf(a.z, a.z, fmaf(a.w, a.w, s[1][0]));
+    s[1][1] = fmaf(a.z, b.z, fmaf(a.w, b.w, s[1][1]));
+    s[1][2] = fmaf(a.z, b.w, fmaf(-a.w, b.z, s[1][2]));
   }
-  const acc_t<T> v[3] = {s0, s1, s2};
+  df v[3];
+#pragma unroll
+  for (int k = 0; k < 3; k++) v[k] = df_add(df_of(s[0][k]), df_of(s[1][k]));
   grid_reduce<3>(v, partials + (size_t)q * gridDim.x * 3, counters + q, out + 4 * q);
 }
 template <typename T>
 void blas_dot2_multi(const T* w, const T* r, size_t n, size_t stride, int nrhs, double* d_out, Workspace& ws,
                      cudaStream_t s) {
   if (nrhs > Workspace::kMultiCounters) raise(MG_ERR_ARG, "too many vectors for one multi-reduction");
-  int g = red_grid(n);
-  const int cap = Workspace::kMaxBlocks * Workspace::kMaxResults / (3 * nrhs);
-  if (g > cap) g = cap;
-  k_dot2_multi<T><<<dim3(g, nrhs), kBS, 0, s>>>((const cx<T>*)w, (const cx<T>*)r, n, stride / 2,
-                                                 ws.partials.as<double>(), ws.mcounters.as<unsigned>(), d_out);
+  // a wave of CTAs over all pairs: every CTA is a partial sum for the last one of its pair to add
+  const int g = std::max(1, std::min(red_grid(n / 2), 152 * 8 / nrhs));
+  k_dot2_multi<<<dim3(g, nrhs), kBS, 0, s>>>(w, r, n / 2, stride, ws.partials.as<double>(), ws.mcounters.as<unsigned>(),
+                                             d_out);
   MG_LAUNCH();
 }
 
@@ -232,7 +235,38 @@ void blas_dot2(const T* w, const T* r, size_t n, double* d_out, Workspace& ws, c
   MG_LAUNCH();
 }
 
-// d_out[2j..] = <V_j, w>, j < K
+// d_out[2j..] = <V_j, w>, j < K.  FP64: bound by the FP64 pipe (4 K operations
+// per element of 64 cycles per warp), so two CTAs per SM are enough to hide the
+// loads and halve the sums over lanes and blocks, which queue on the same pipe.
+// FP32: pairs of complex numbers, 16 bytes per load, with a sum for the first
+// and one for the second of a pair (n is even: 12 or 2 Nv components a site).
+// Eight vectors: FP64, 0.79 M complex, 57.2 -> 52.3 us (40 us of the pipe); FP32,
+// 1.57 M complex, 47.5 -> 26.1 us (17 us of memory traffic).
+constexpr int kDotGrid64 = 304;
+template <int K>
+__global__ void __launch_bounds__(kBS) k_multidot_pairs(VecPtrs<float> V, const float4* __restrict__ w, size_t n2,
+                                                        double* partials, unsigned* counter, double* out) {
+  float s[2][2 * K];
+#pragma unroll
+  for (int r = 0; r < 2 * K; r++) s[0][r] = s[1][r] = 0.f;
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n2; i += (size_t)gridDim.x * kBS) {
+    float4 a[K];
+#pragma unroll
+    for (int j = 0; j < K; j++) a[j] = reinterpret_cast<const float4*>(V.p[j])[i];
+    const float4 b = w[i];
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      s[0][2 * j] = fmaf(a[j].x, b.x, fmaf(a[j].y, b.y, s[0][2 * j]));
+      s[0][2 * j + 1] = fmaf(a[j].x, b.y, fmaf(-a[j].y, b.x, s[0][2 * j + 1]));
+      s[1][2 * j] = fmaf(a[j].z, b.z, fmaf(a[j].w, b.w, s[1][2 * j]));
+      s[1][2 * j + 1] = fmaf(a[j].z, b.w, fmaf(-a[j].w, b.z, s[1][2 * j + 1]));
+    }
+  }
+  df v[2 * K];
+#pragma unroll
+  for (int r = 0; r < 2 * K; r++) v[r] = df_add(df_of(s[0][r]), df_of(s[1][r]));
+  grid_reduce<2 * K>(v, partials, counter, out);
+}
 template <typename T, int K>
 __global__ void k_multidot(VecPtrs<T> V, const cx<T>* __restrict__ w, size_t n, double* partials, unsigned* counter,
                            double* out) {
@@ -255,48 +289,81 @@ __global__ void k_multidot(VecPtrs<T> V, const cx<T>* __restrict__ w, size_t n, 
 
 template <typename T>
 void blas_multidot(const T* const* V, int k, const T* w, size_t n, double* d_out, Workspace& ws, cudaStream_t s) {
+  double* pa = ws.partials.as<double>();
+  unsigned* ct = ws.counter.as<unsigned>();
   for (int j0 = 0; j0 < k; j0 += 8) {
     const int kk = (k - j0) < 8 ? (k - j0) : 8;
     VecPtrs<T> P;
     for (int j = 0; j < 8; j++) P.p[j] = (const cx<T>*)(j < kk ? V[j0 + j] : V[j0]);
     double* o = d_out + 2 * j0;
-    const int grid = red_grid(n);
-    double* pa = ws.partials.as<double>();
-    unsigned* ct = ws.counter.as<unsigned>();
-    const cx<T>* wp = (const cx<T>*)w;
+    auto run = [&](auto kc) {
+      constexpr int K = decltype(kc)::value;
+      if constexpr (sizeof(T) == 4)
+        k_multidot_pairs<K><<<red_grid(n / 2), kBS, 0, s>>>(P, (const float4*)w, n / 2, pa, ct, o);
+      else
+        k_multidot<T, K><<<std::min(red_grid(n), kDotGrid64), kBS, 0, s>>>(P, (const cx<T>*)w, n, pa, ct, o);
+    };
     switch (kk) {
-      case 1: k_multidot<T, 1><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 2: k_multidot<T, 2><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 3: k_multidot<T, 3><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 4: k_multidot<T, 4><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 5: k_multidot<T, 5><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 6: k_multidot<T, 6><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      case 7: k_multidot<T, 7><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
-      default: k_multidot<T, 8><<<grid, kBS, 0, s>>>(P, wp, n, pa, ct, o); break;
+      case 1: run(std::integral_constant<int, 1>()); break;
+      case 2: run(std::integral_constant<int, 2>()); break;
+      case 3: run(std::integral_constant<int, 3>()); break;
+      case 4: run(std::integral_constant<int, 4>()); break;
+      case 5: run(std::integral_constant<int, 5>()); break;
+      case 6: run(std::integral_constant<int, 6>()); break;
+      case 7: run(std::integral_constant<int, 7>()); break;
+      default: run(std::integral_constant<int, 8>());
     }
     MG_LAUNCH();
   }
 }
 
-// w -= sum_{j<K} beta_j V_j; if RED: {||w||^2, <w, r>} -> out
+// w -= sum_{j<K} beta_j V_j; if RED: {||w||^2, <w, r>} -> out.  FP32 vectors in
+// pairs of complex numbers (16 bytes per load), as above.
+template <int K, bool RED>
+__global__ void __launch_bounds__(kBS) k_orth_update_pairs(float4* w, VecPtrs<float> V,
+                                                           const double* __restrict__ beta,
+                                                           const float4* __restrict__ r, size_t n2, double* partials,
+                                                           unsigned* counter, double* out) {
+  __shared__ Coefs<K> sb;
+  if (K > 0) load_coefs<K>(sb, beta, 1.0);
+  float s[2][3] = {};
+  for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n2; i += (size_t)gridDim.x * kBS) {
+    float4 q[K > 0 ? K : 1], b = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < K; j++) q[j] = reinterpret_cast<const float4*>(V.p[j])[i];
+    float4 a = w[i];
+    if (RED) b = r[i];
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const float br = sb.h[2 * j], bi = sb.h[2 * j + 1];
+      a.x = fmaf(-br, q[j].x, fmaf(bi, q[j].y, a.x));
+      a.y = fmaf(-br, q[j].y, fmaf(-bi, q[j].x, a.y));
+      a.z = fmaf(-br, q[j].z, fmaf(bi, q[j].w, a.z));
+      a.w = fmaf(-br, q[j].w, fmaf(-bi, q[j].z, a.w));
+    }
+    if (K > 0) w[i] = a;
+    if (RED) {
+      s[0][0] = fmaf(a.x, a.x, fmaf(a.y, a.y, s[0][0]));
+      s[0][1] = fmaf(a.x, b.x, fmaf(a.y, b.y, s[0][1]));
+      s[0][2] = fmaf(a.x, b.y, fmaf(-a.y, b.x, s[0][2]));
+      s[1][0] = fmaf(a.z, a.z, fmaf(a.w, a.w, s[1][0]));
+      s[1][1] = fmaf(a.z, b.z, fmaf(a.w, b.w, s[1][1]));
+      s[1][2] = fmaf(a.z, b.w, fmaf(-a.w, b.z, s[1][2]));
+    }
+  }
+  df v[3];
+#pragma unroll
+  for (int q = 0; q < 3; q++) v[q] = df_add(df_of(s[0][q]), df_of(s[1][q]));
+  if (RED) grid_reduce<3>(v, partials, counter, out);
+}
 template <typename T, int K, bool RED>
 __global__ void k_orth_update(cx<T>* w, VecPtrs<T> V, const double* __restrict__ beta, const cx<T>* __restrict__ r,
                               size_t n, double* partials, unsigned* counter, double* out) {
   T br[K > 0 ? K : 1], bi[K > 0 ? K : 1];
-  if constexpr (sizeof(T) == 4) {
-    __shared__ Coefs<K> sb;
-    if (K > 0) load_coefs<K>(sb, beta, 1.0);
 #pragma unroll
-    for (int j = 0; j < K; j++) {
-      br[j] = sb.h[2 * j];
-      bi[j] = sb.h[2 * j + 1];
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < K; j++) {
-      br[j] = (T)beta[2 * j];
-      bi[j] = (T)beta[2 * j + 1];
-    }
+  for (int j = 0; j < K; j++) {
+    br[j] = (T)beta[2 * j];
+    bi[j] = (T)beta[2 * j + 1];
   }
   acc_t<T> s0 = 0, s1 = 0, s2 = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
@@ -325,46 +392,41 @@ __global__ void k_orth_update(cx<T>* w, VecPtrs<T> V, const double* __restrict__
 template <typename T>
 void blas_orth_update(T* w, const T* const* V, const double* d_beta, int k, const T* r, size_t n, double* d_out,
                       Workspace& ws, cudaStream_t s) {
-  const int grid = red_grid(n);
   double* pa = ws.partials.as<double>();
   unsigned* ct = ws.counter.as<unsigned>();
-  cx<T>* wp = (cx<T>*)w;
-  const cx<T>* rp = (const cx<T>*)r;
-  if (k == 0) {
-    VecPtrs<T> P{};
-    k_orth_update<T, 0, true><<<grid, kBS, 0, s>>>(wp, P, d_beta, rp, n, pa, ct, d_out);
+  auto launch = [&](auto kc, auto red, const VecPtrs<T>& P, const double* b) {
+    constexpr int K = decltype(kc)::value;
+    constexpr bool RED = decltype(red)::value;
+    if constexpr (sizeof(T) == 4)
+      k_orth_update_pairs<K, RED><<<red_grid(n / 2), kBS, 0, s>>>((float4*)w, P, b, (const float4*)r, n / 2, pa, ct, d_out);
+    else
+      k_orth_update<T, K, RED><<<red_grid(n), kBS, 0, s>>>((cx<T>*)w, P, b, (const cx<T>*)r, n, pa, ct, d_out);
     MG_LAUNCH();
+  };
+  if (k == 0) {
+    launch(std::integral_constant<int, 0>(), std::true_type(), VecPtrs<T>{}, d_beta);
     return;
   }
   for (int j0 = 0; j0 < k; j0 += 8) {
     const int kk = (k - j0) < 8 ? (k - j0) : 8;
-    const bool last = j0 + kk >= k;
     VecPtrs<T> P;
     for (int j = 0; j < 8; j++) P.p[j] = (const cx<T>*)(j < kk ? V[j0 + j] : V[j0]);
-    const double* b = d_beta + 2 * j0;
-#define MG_ORTH_CASE(KK)                                                                         \
-  case KK:                                                                                       \
-    if (last)                                                                                    \
-      k_orth_update<T, KK, true><<<grid, kBS, 0, s>>>(wp, P, b, rp, n, pa, ct, d_out);           \
-    else                                                                                         \
-      k_orth_update<T, KK, false><<<grid, kBS, 0, s>>>(wp, P, b, rp, n, pa, ct, d_out);          \
-    break;
+    auto run = [&](auto kc) {
+      if (j0 + kk >= k)
+        launch(kc, std::true_type(), P, d_beta + 2 * j0);
+      else
+        launch(kc, std::false_type(), P, d_beta + 2 * j0);
+    };
     switch (kk) {
-      MG_ORTH_CASE(1)
-      MG_ORTH_CASE(2)
-      MG_ORTH_CASE(3)
-      MG_ORTH_CASE(4)
-      MG_ORTH_CASE(5)
-      MG_ORTH_CASE(6)
-      MG_ORTH_CASE(7)
-      default:
-        if (last)
-          k_orth_update<T, 8, true><<<grid, kBS, 0, s>>>(wp, P, b, rp, n, pa, ct, d_out);
-        else
-          k_orth_update<T, 8, false><<<grid, kBS, 0, s>>>(wp, P, b, rp, n, pa, ct, d_out);
+      case 1: run(std::integral_constant<int, 1>()); break;
+      case 2: run(std::integral_constant<int, 2>()); break;
+      case 3: run(std::integral_constant<int, 3>()); break;
+      case 4: run(std::integral_constant<int, 4>()); break;
+      case 5: run(std::integral_constant<int, 5>()); break;
+      case 6: run(std::integral_constant<int, 6>()); break;
+      case 7: run(std::integral_constant<int, 7>()); break;
+      default: run(std::integral_constant<int, 8>());
     }
-#undef MG_ORTH_CASE
-    MG_LAUNCH();
   }
 }
 
@@ -422,26 +484,32 @@ void blas_r_update(T* w, T* r, size_t n, const double* d_in, double* d_alpha, do
 // complex, against 126 MB of traffic).
 template <typename T, typename TZ, int K>
 __global__ void k_lincomb(cx<T>* x, VecPtrs<TZ> Z, const double* __restrict__ c, double scale, size_t n) {
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4) {   // pairs of complex numbers; n is even
     __shared__ Coefs<K> sc;
     load_coefs<K>(sc, c, scale);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-      cx<float> z[K];
+    float4* x4 = reinterpret_cast<float4*>(x);
+    const size_t n2 = n / 2;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n2; i += (size_t)gridDim.x * blockDim.x) {
+      float4 z[K];
 #pragma unroll
-      for (int j = 0; j < K; j++) z[j] = Z.p[j][i];
-      const cx<T> a = x[i];
-      float rh = a.re, rl = 0.f, ih = a.im, il = 0.f;
+      for (int j = 0; j < K; j++) z[j] = reinterpret_cast<const float4*>(Z.p[j])[i];
+      const float4 a = x4[i];
+      float h[4] = {a.x, a.y, a.z, a.w}, l[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int j = 0; j < K; j++) {
         const float cr = sc.h[2 * j], ci = sc.h[2 * j + 1], lr = sc.l[2 * j], li = sc.l[2 * j + 1];
-        dot2_acc(rh, rl, cr, z[j].re);
-        dot2_acc(rh, rl, -ci, z[j].im);
-        rl = fmaf(lr, z[j].re, fmaf(-li, z[j].im, rl));
-        dot2_acc(ih, il, cr, z[j].im);
-        dot2_acc(ih, il, ci, z[j].re);
-        il = fmaf(lr, z[j].im, fmaf(li, z[j].re, il));
+        const float zr[2] = {z[j].x, z[j].z}, zi[2] = {z[j].y, z[j].w};
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          dot2_acc(h[2 * u], l[2 * u], cr, zr[u]);
+          dot2_acc(h[2 * u], l[2 * u], -ci, zi[u]);
+          l[2 * u] = fmaf(lr, zr[u], fmaf(-li, zi[u], l[2 * u]));
+          dot2_acc(h[2 * u + 1], l[2 * u + 1], cr, zi[u]);
+          dot2_acc(h[2 * u + 1], l[2 * u + 1], ci, zr[u]);
+          l[2 * u + 1] = fmaf(lr, zi[u], fmaf(li, zr[u], l[2 * u + 1]));
+        }
       }
-      x[i] = mkc<T>(rh + rl, ih + il);
+      x4[i] = make_float4(h[0] + l[0], h[1] + l[1], h[2] + l[2], h[3] + l[3]);
     }
   } else {
     double cr[K], ci[K];
@@ -472,7 +540,7 @@ void blas_lincomb(T* x, const TZ* const* Z, const double* d_c, int k, double sca
     VecPtrs<TZ> P;
     for (int j = 0; j < 8; j++) P.p[j] = (const cx<TZ>*)(j < kk ? Z[j0 + j] : Z[j0]);
     const double* c = d_c + 2 * j0;
-    const int grid = ew_grid(n);
+    const int grid = ew_grid(sizeof(T) == 4 ? n / 2 : n);
     cx<T>* xp = (cx<T>*)x;
     switch (kk) {
       case 1: k_lincomb<T, TZ, 1><<<grid, kBS, 0, s>>>(xp, P, c, scale, n); break;
