@@ -342,6 +342,8 @@ struct FineOps {
   void reserve_multi(int nrhs);
   int block_for(const char* kernel, int nrhs, const std::function<void(int)>& launch);
   void Dr_multi(T* out_e, const T* in_e, int nrhs, size_t stride);
+  // out_e = x_e + a H_eo A_o^{-1} H_oe m1, packed half vectors
+  void hops_multi(T* out_e, const T* x_e, double a, int nrhs);
   void br_multi(T* out_e, const T* b_e, const T* b_o, int nrhs, size_t stride);
   void reconstruct_multi(T* x_e, T* x_o, const T* y_e, const T* b_o, int nrhs, size_t stride);
   void D_multi(T* oe, T* oo, const T* ie, const T* io, int nrhs, size_t stride);
@@ -424,6 +426,9 @@ class Krylov {
 // last step's inner products
 void mr_post_smooth_fine(Ctx* c, float* z, const float* b, float* e, float* r, float* w, float* s, float* t, int nu,
                          double* d_scr);
+// the same for nb packed right-hand sides (d_scr: 4 nb doubles)
+void mr_post_smooth_multi(Ctx* c, FineOps<float>& F, float* z, const float* b, float* e, float* r, float* w, int nu,
+                          int nb, double* d_scr);
 // MR smoothing: e = MR_nu(A, r) from e = 0 (r is consumed as scratch)
 template <typename T>
 void mr_smooth(Ctx* c, const std::function<void(T*, const T*)>& A, T* e, T* r, T* w, size_t n, int nu,

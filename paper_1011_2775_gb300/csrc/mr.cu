@@ -140,15 +140,24 @@ __global__ void __launch_bounds__(128) k_mr_residual_lanes(Geom g, float* __rest
 }
 
 // e += alpha r (e = alpha r on the first step), r -= alpha w (alpha = in[1..2] /
-// in[0]), and s = A_e^{-1} r of the updated r on even sites
+// in[0]), and s = A_e^{-1} r of the updated r on even sites; nrhs right-hand
+// sides `stride` floats apart (scalars four apart), neighbouring CTAs sharing
+// the sites and so the clover matrices
 template <bool FIRST>
 __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restrict__ e, float* __restrict__ r,
                                                           const float* __restrict__ w, const double* __restrict__ in,
-                                                          const float* __restrict__ clov, float* __restrict__ s) {
+                                                          const float* __restrict__ clov, float* __restrict__ s,
+                                                          int nrhs, size_t stride) {
   __shared__ float s_al[2];   // two FP64 divisions per block, not per thread
+  const int q = blockIdx.x % nrhs;
+  in += 4 * q;
   if (threadIdx.x < 2) s_al[threadIdx.x] = (float)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
   __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x / nrhs) * blockDim.x + threadIdx.x;
+  e += q * stride;
+  r += q * stride;
+  w += q * stride;
+  s += q * stride;
   if (i >= g.Vh) return;
   const float ar = s_al[0], ai = s_al[1];
   cx<float> ev[12], rv[12], wv[12], sv[12];
@@ -169,11 +178,16 @@ __global__ void __launch_bounds__(128) k_mr_update_clover(Geom g, float* __restr
   SpinorIO<float>::store(s, g.Vh, i, sv);
 }
 
-// z += e + alpha r (without e when FIRST), pairs of complex numbers
+// z += e + alpha r (without e when FIRST), pairs of complex numbers; blockIdx.y:
+// right-hand side (packed vectors)
 template <bool FIRST>
 __global__ void __launch_bounds__(256) k_mr_finish(float4* __restrict__ z, const float4* __restrict__ e,
                                                    const float4* __restrict__ r, const double* __restrict__ in, int n2) {
   __shared__ float s_al[2];
+  in += 4 * blockIdx.y;
+  z += (size_t)blockIdx.y * n2;
+  e += (size_t)blockIdx.y * n2;
+  r += (size_t)blockIdx.y * n2;
   if (threadIdx.x < 2) s_al[threadIdx.x] = (float)(in[1 + threadIdx.x] / (in[0] > 0 ? in[0] : 1.0));
   __syncthreads();
   const float ar = s_al[0], ai = s_al[1];
@@ -188,6 +202,23 @@ __global__ void __launch_bounds__(256) k_mr_finish(float4* __restrict__ z, const
     ev.w += ar * rv.w + ai * rv.z;
     z[i] = make_float4(zv.x + ev.x, zv.y + ev.y, zv.z + ev.z, zv.w + ev.w);
   }
+}
+
+// s = A_e^{-1} z and d = b - z for nrhs right-hand sides
+__global__ void __launch_bounds__(128) k_mr_begin(Geom g, float* __restrict__ s, float* __restrict__ d,
+                                                  const float* __restrict__ z, const float* __restrict__ b,
+                                                  const float* __restrict__ clov, int nrhs, size_t stride) {
+  const int q = blockIdx.x % nrhs, i = (blockIdx.x / nrhs) * blockDim.x + threadIdx.x;
+  if (i >= g.Vh) return;
+  const size_t o = q * stride;
+  cx<float> zv[12], bv[12], sv[12];
+  SpinorIO<float>::load(z + o, g.Vh, i, zv);
+  SpinorIO<float>::load(b + o, g.Vh, i, bv);
+#pragma unroll
+  for (int k = 0; k < 12; k++) bv[k] = mkc(bv[k].re - zv[k].re, bv[k].im - zv[k].im);
+  SpinorIO<float>::store(d + o, g.Vh, i, bv);
+  clover_mul<float>(clov, g.Vh, i, zv, sv);
+  SpinorIO<float>::store(s + o, g.Vh, i, sv);
 }
 
 }  // namespace
@@ -234,15 +265,53 @@ void mr_post_smooth_fine(Ctx* c, float* z, const float* b, float* e, float* r, f
     dslash_dot();
     if (it + 1 < nu) {
       if (it == 0)
-        k_mr_update_clover<true><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s);
+        k_mr_update_clover<true><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s, 1, 0);
       else
-        k_mr_update_clover<false><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s);
+        k_mr_update_clover<false><<<sites, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s, 1, 0);
     } else {
       const int n2 = (int)(6 * c->Vh), grid = (int)std::min<long long>(152 * 8, (n2 + 255) / 256);
       if (it == 0)
         k_mr_finish<true><<<grid, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
       else
         k_mr_finish<false><<<grid, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
+    }
+    MG_LAUNCH();
+  }
+}
+
+// The same for nb right-hand sides (packed half vectors) with the multi-RHS
+// hops: d = b - z and s = A^{-1} z in one pass, r = d + H t, then per step the hops, the inner
+// products, and one pass for e, r and the next A^{-1} r.  The passes run at the
+// memory's rate, so what counts is what they do not read and write again.
+void mr_post_smooth_multi(Ctx* c, FineOps<float>& F, float* z, const float* b, float* e, float* r, float* w, int nu,
+                          int nb, double* d_scr) {
+  const Geom& g = c->g;
+  cudaStream_t st = c->stream;
+  if (nu <= 0) return;
+  F.reserve_multi(nb);
+  const size_t hs = 24 * (size_t)c->Vh;
+  const int bs = site_block((long long)c->Vh * nb);
+  const unsigned grid = (unsigned)((c->Vh + bs - 1) / bs) * nb;
+  float* s = F.m1.as<float>();
+  k_mr_begin<<<grid, bs, 0, st>>>(g, s, w, z, b, c->Ainv<float>(0), nb, hs);
+  MG_LAUNCH();
+  F.hops_multi(r, w, 1.0, nb);
+  clover_apply_mrhs<float>(g, nb, hs, s, r, c->Ainv<float>(0), st);
+  for (int it = 0; it < nu; it++) {
+    F.hops_multi(w, r, -1.0, nb);
+    blas_dot2_multi<float>(w, r, hs / 2, hs, nb, d_scr, c->ws, st);
+    if (it + 1 < nu) {
+      if (it == 0)
+        k_mr_update_clover<true><<<grid, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s, nb, hs);
+      else
+        k_mr_update_clover<false><<<grid, bs, 0, st>>>(g, e, r, w, d_scr, c->Ainv<float>(0), s, nb, hs);
+    } else {
+      const int n2 = (int)(6 * c->Vh);
+      const dim3 gf((unsigned)std::min<long long>((152 * 16 + nb - 1) / nb, (n2 + 255) / 256), nb);
+      if (it == 0)
+        k_mr_finish<true><<<gf, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
+      else
+        k_mr_finish<false><<<gf, 256, 0, st>>>((float4*)z, (const float4*)e, (const float4*)r, d_scr, n2);
     }
     MG_LAUNCH();
   }

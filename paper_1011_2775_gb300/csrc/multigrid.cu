@@ -810,16 +810,8 @@ void mg_batch_post(Ctx* c, float* z, const float* r, int nb) {
   } else {
     prolong_vec_multi(T, nb, z, b.hs, ec, b.cs, true, b.s);
   }
-  if (b.p.nu_post > 0) {
-    float* w = bw.w.as<float>();
-    float* res = bw.res.as<float>();
-    float* e = bw.e.as<float>();
-    b.H.F32->Dr_multi(w, z, nb, b.hs);
-    blas_convert<float, float>(res, r, b.n * nb, b.s);
-    blas_axpby<float>(-1.0, w, 1.0, res, b.n * nb, b.s);
-    batch_mr(c, b, e, res, b.p.nu_post, nb);
-    blas_axpby<float>(1.0, e, 1.0, z, b.n * nb, b.s);
-  }
+  mr_post_smooth_multi(c, *b.H.F32, z, r, bw.e.as<float>(), bw.res.as<float>(), bw.w.as<float>(), b.p.nu_post, nb,
+                       bw.scr.as<double>());
 }
 
 void mg_precondition_batch(Ctx* c, float* z, const float* r, int nb) {

@@ -182,16 +182,24 @@ void FineOps<T>::Dr_multi(T* out_e, const T* in_e, int nrhs, size_t stride) {
   const Geom& g = c->g;
   cudaStream_t st = c->stream;
   reserve_multi(nrhs);
-  const size_t ts = 24 * c->Vh;  // temporaries are packed at half-vector stride
-  if (stride != ts) raise(MG_ERR_ARG, "multi-RHS operators take packed half vectors");
+  if (stride != 24 * (size_t)c->Vh) raise(MG_ERR_ARG, "multi-RHS operators take packed half vectors");
+  clover_apply_mrhs<T>(g, nrhs, stride, m1.as<T>(), in_e, c->Ainv<T>(0), st);
+  hops_multi(out_e, in_e, -1.0, nrhs);
+}
+
+// out_e = x_e + a H_eo A_o^{-1} H_oe m1, packed half vectors
+template <typename T>
+void FineOps<T>::hops_multi(T* out_e, const T* x_e, double a, int nrhs) {
+  const Geom& g = c->g;
+  cudaStream_t st = c->stream;
+  const size_t ts = 24 * c->Vh;
   T* s = m1.as<T>();
   T* t = m2.as<T>();
-  clover_apply_mrhs<T>(g, nrhs, stride, s, in_e, c->Ainv<T>(0), st);
   auto k1 = [&](int b) {
     dslash_mrhs<T>(g, EPI_CH, 1, nrhs, ts, t, s, c->gauge<T>(), c->Ainv<T>(1), nullptr, 0.0, 0xff, b, st);
   };
   auto k2 = [&](int b) {
-    dslash_mrhs<T>(g, EPI_XPAY, 0, nrhs, ts, out_e, t, c->gauge<T>(), nullptr, in_e, -1.0, 0xff, b, st);
+    dslash_mrhs<T>(g, EPI_XPAY, 0, nrhs, ts, out_e, t, c->gauge<T>(), nullptr, x_e, a, 0xff, b, st);
   };
   k1(block_for("dslash_ch", nrhs, k1));
   k2(block_for("dslash_xpay", nrhs, k2));
