@@ -113,40 +113,40 @@ TArgs targs(const TransferOp& T) {
 }  // namespace
 
 // --------------------------------------------------------------------------- restriction
-// One CTA per coarse site.  Warp w takes the block's fine sites w, w+8, ...;
-// lane k (and k+32 when Nv > 32) accumulates conj(P[i][c][k]) v[i][c] for the
-// two chiralities.  The site's components are read once by lanes 0..ndof-1
-// and broadcast with shuffles; P rows are read coalesced, several components
-// in flight at a time.  Per-warp sums are combined in FP64 at the end.
+// One CTA per coarse site and chirality.  Warp w takes the block's fine sites w,
+// w+8, ...; lane k (and k+32 when Nv > 32) accumulates conj(P[i][c][k]) v[i][c].
+// The site's components are read once by lanes 0..hd-1 and broadcast with
+// shuffles; P rows are read coalesced, twelve in flight at a time: a coarse
+// level has few blocks (32 of 2^4 sites here), so the time is a warp's chain of
+// trips to L2 (both chiralities in one CTA with four rows in flight: 30 us,
+// 15 us here, at Nc = 48).  Per-warp sums are combined in FP64 at the end.
 template <int ST>
 __global__ void __launch_bounds__(256) k_restrict(TArgs a, float* __restrict__ out, const float* __restrict__ v,
                                                   int even_only, int nrhs, size_t vstride, size_t cstride) {
-  extern __shared__ float2 sacc[];  // [nwarps][2 nv]
+  extern __shared__ float2 sacc[];  // [nwarps][nv]
   // one CTA per (coarse site, rhs), rhs fastest: the CTAs of a site share its P rows in L2
-  const int cc = blockIdx.x / nrhs, rq = blockIdx.x % nrhs;
+  const int cc = blockIdx.x / nrhs, rq = blockIdx.x % nrhs, ch = blockIdx.y;
   v += rq * vstride;
   out += rq * cstride;
   const int nv = a.nv, hd = a.ndof / 2;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  float acc[2][2][2] = {};  // [k-half][chirality][re, im]
+  float acc[2][2] = {};  // [k-half][re, im]
   for (int i = w; i < a.nb; i += nw) {
     const int idx = a.blockmap[cc * a.nb + i];
     if (even_only && idx >= a.fine_half) continue;
-    const cx<float> x0 = lane < a.ndof ? fget(a.fa, v, idx, lane) : mkc(0.f, 0.f);
-    const cx<float> x1 = lane + 32 < a.ndof ? fget(a.fa, v, idx, lane + 32) : mkc(0.f, 0.f);
-    const size_t base = (size_t)(cc * a.nb + i) * a.ndof;
-#pragma unroll 4
-    for (int c = 0; c < a.ndof; c++) {
-      const float xr = __shfl_sync(0xffffffffu, c < 32 ? x0.re : x1.re, c & 31);
-      const float xi = __shfl_sync(0xffffffffu, c < 32 ? x0.im : x1.im, c & 31);
-      const int ch = c >= hd;
+    const cx<float> x = lane < hd ? fget(a.fa, v, idx, ch * hd + lane) : mkc(0.f, 0.f);
+    const size_t base = (size_t)(cc * a.nb + i) * a.ndof + ch * hd;
+#pragma unroll 12
+    for (int c = 0; c < hd; c++) {
+      const float xr = __shfl_sync(0xffffffffu, x.re, c);
+      const float xi = __shfl_sync(0xffffffffu, x.im, c);
 #pragma unroll
       for (int h = 0; h < 2; h++) {
         const int k = lane + 32 * h;
         if (k < nv) {
           const cx<float> p = sget<ST>(a.P, (base + c) * nv + k);
-          acc[h][ch][0] += p.re * xr + p.im * xi;
-          acc[h][ch][1] += p.re * xi - p.im * xr;
+          acc[h][0] += p.re * xr + p.im * xi;
+          acc[h][1] += p.re * xi - p.im * xr;
         }
       }
     }
@@ -154,21 +154,17 @@ __global__ void __launch_bounds__(256) k_restrict(TArgs a, float* __restrict__ o
 #pragma unroll
   for (int h = 0; h < 2; h++) {
     const int k = lane + 32 * h;
-    if (k < nv) {
-      sacc[(size_t)w * 2 * nv + k] = make_float2(acc[h][0][0], acc[h][0][1]);
-      sacc[(size_t)w * 2 * nv + nv + k] = make_float2(acc[h][1][0], acc[h][1][1]);
-    }
+    if (k < nv) sacc[(size_t)w * nv + k] = make_float2(acc[h][0], acc[h][1]);
   }
   __syncthreads();
-  const float s0 = a.Ps[cc * 2], s1 = a.Ps[cc * 2 + 1];
-  for (int t = threadIdx.x; t < 2 * nv; t += blockDim.x) {
+  const float sc = a.Ps[cc * 2 + ch];
+  for (int t = threadIdx.x; t < nv; t += blockDim.x) {
     double re = 0, im = 0;
     for (int q = 0; q < nw; q++) {
-      re += sacc[(size_t)q * 2 * nv + t].x;
-      im += sacc[(size_t)q * 2 * nv + t].y;
+      re += sacc[(size_t)q * nv + t].x;
+      im += sacc[(size_t)q * nv + t].y;
     }
-    const float sc = t < nv ? s0 : s1;
-    reinterpret_cast<float2*>(out)[(size_t)cc * 2 * nv + t] = make_float2((float)(sc * re), (float)(sc * im));
+    reinterpret_cast<float2*>(out)[(size_t)cc * 2 * nv + ch * nv + t] = make_float2((float)(sc * re), (float)(sc * im));
   }
 }
 
@@ -378,8 +374,8 @@ void restrict_vec_multi(const TransferOp& T, int nrhs, float* out_c, size_t cstr
     }
     return;
   }
-  const size_t sm = sizeof(float2) * (kBS / 32) * 2 * (size_t)T.nv;
-  const unsigned grid = (unsigned)((size_t)T.ncoarse * nrhs);
+  const size_t sm = sizeof(float2) * (kBS / 32) * (size_t)T.nv;
+  const dim3 grid((unsigned)((size_t)T.ncoarse * nrhs), 2);
   switch (T.store) {
     case STORE_F32: k_restrict<STORE_F32><<<grid, kBS, sm, s>>>(a, out_c, v, even_only, nrhs, vstride, cstride); break;
     case STORE_F16: k_restrict<STORE_F16><<<grid, kBS, sm, s>>>(a, out_c, v, even_only, nrhs, vstride, cstride); break;
@@ -852,8 +848,9 @@ void galerkin_project(const TransferOp& T, CoarseOp& C, const float* const W[8],
 }
 
 // --------------------------------------------------------------------------- coarse stencil
+// Hops followed by a site matrix (EPI_CH, EPI_CX_PAY): CTA = site.
 struct HopArgs {
-  int nc, s0, dirmask;
+  int nc, s0;
   const int* nbr;
   const void* Y;    // links in the level's storage format
   const float* Ys;
@@ -874,16 +871,11 @@ __global__ void __launch_bounds__(256) k_coarse_hop(HopArgs h) {
   float2* vx = tv + nc;
   for (int t = threadIdx.x; t < 8 * nc; t += blockDim.x) {
     const int d = t / nc, j = t % nc;
-    float2 v = make_float2(0.f, 0.f);
-    if ((h.dirmask >> d) & 1) {
-      const float sc = h.Ys[(size_t)s * 8 + d];
-      v = h.in[(size_t)h.nbr[(size_t)s * 8 + d] * nc + j];
-      v.x *= sc;
-      v.y *= sc;
-    }
-    vin[t] = v;
+    const float sc = h.Ys[(size_t)s * 8 + d];
+    const float2 v = h.in[(size_t)h.nbr[(size_t)s * 8 + d] * nc + j];
+    vin[t] = make_float2(sc * v.x, sc * v.y);
   }
-  if (EPI == EPI_CX_PAY || EPI == EPI_XPAY || EPI == EPI_C_XPAY)
+  if (EPI == EPI_CX_PAY)
     for (int t = threadIdx.x; t < nc; t += blockDim.x) vx[t] = h.x[(size_t)s * nc + t];
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -895,15 +887,8 @@ __global__ void __launch_bounds__(256) k_coarse_hop(HopArgs h) {
 #pragma unroll
     for (int r = 0; r < kGemvMaxRows; r++) {
       const int i = w * rpw + r;
-      if (r < rpw && i < nc) {
-        if (EPI == EPI_H) h.out[(size_t)s * nc + i] = res[r];
-        else if (EPI == EPI_XPAY)
-          h.out[(size_t)s * nc + i] = make_float2(vx[i].x + h.a * res[r].x, vx[i].y + h.a * res[r].y);
-        else if (EPI == EPI_CH || EPI == EPI_CX_PAY) tv[i] = res[r];
-        else tv[i] = make_float2(vx[i].x + h.a * res[r].x, vx[i].y + h.a * res[r].y);  // EPI_C_XPAY
-      }
+      if (r < rpw && i < nc) tv[i] = res[r];
     }
-  if (EPI == EPI_H || EPI == EPI_XPAY) return;
   __syncthreads();
   const float2* src = (EPI == EPI_CX_PAY) ? vx : tv;
   warp_gemv(h.C + (size_t)s * nc * nc, nc, nc, src, w, rpw, lane, res);
@@ -1038,31 +1023,30 @@ void coarse_hop(const LevelGeom& G, const CoarseOp& C, Epilogue epi, bool use_in
                 const float* in, const float* x, float a, int dirmask, cudaStream_t s) {
   if (s1 <= s0) return;
   if (epi == EPI_H || epi == EPI_XPAY) {
-    const bool single = (dirmask & (dirmask - 1)) == 0;
-    if (dirmask == 0xff || (single && dirmask)) {
-      RowArgs r;
-      r.nc = C.nc;
-      r.s0 = s0;
-      r.lbase = 0;
-      int d = 0;
-      while (single && dirmask >> (d + 1)) d++;
-      r.q0 = single ? d * (C.nc / 2) : 0;
-      r.q1 = single ? r.q0 + C.nc / 2 : 4 * C.nc;
-      r.nbr = G.d_nbr.as<int>();
-      r.L = C.Y.get();
-      r.Ls = C.Yscale.as<float>();
-      r.out = (float2*)out;
-      r.in = (const float2*)in;
-      r.x = (const float2*)x;
-      r.a = a;
-      launch_rows(r, s1 - s0, C.store, epi == EPI_XPAY, s);
-      return;
-    }
+    const bool single = dirmask != 0xff;
+    int d = 0;
+    while (single && dirmask >> (d + 1)) d++;
+    if (single && dirmask != 1 << d) raise(MG_ERR_ARG, "coarse hops take all directions or one");
+    RowArgs r;
+    r.nc = C.nc;
+    r.s0 = s0;
+    r.lbase = 0;
+    r.q0 = single ? d * (C.nc / 2) : 0;
+    r.q1 = single ? r.q0 + C.nc / 2 : 4 * C.nc;
+    r.nbr = G.d_nbr.as<int>();
+    r.L = C.Y.get();
+    r.Ls = C.Yscale.as<float>();
+    r.out = (float2*)out;
+    r.in = (const float2*)in;
+    r.x = (const float2*)x;
+    r.a = a;
+    launch_rows(r, s1 - s0, C.store, epi == EPI_XPAY, s);
+    return;
   }
+  if ((epi != EPI_CH && epi != EPI_CX_PAY) || dirmask != 0xff) raise(MG_ERR_ARG, "no such coarse hop");
   HopArgs h;
   h.nc = C.nc;
   h.s0 = s0;
-  h.dirmask = dirmask;
   h.nbr = G.d_nbr.as<int>();
   h.Y = C.Y.get();
   h.Ys = C.Yscale.as<float>();
@@ -1075,13 +1059,10 @@ void coarse_hop(const LevelGeom& G, const CoarseOp& C, Epilogue epi, bool use_in
   const int nb = s1 - s0;
   auto launch = [&](auto st) {
     constexpr int ST = decltype(st)::value;
-    switch (epi) {
-      case EPI_H: k_coarse_hop<EPI_H, ST><<<nb, 256, sm, s>>>(h); break;
-      case EPI_CH: k_coarse_hop<EPI_CH, ST><<<nb, 256, sm, s>>>(h); break;
-      case EPI_XPAY: k_coarse_hop<EPI_XPAY, ST><<<nb, 256, sm, s>>>(h); break;
-      case EPI_CX_PAY: k_coarse_hop<EPI_CX_PAY, ST><<<nb, 256, sm, s>>>(h); break;
-      case EPI_C_XPAY: k_coarse_hop<EPI_C_XPAY, ST><<<nb, 256, sm, s>>>(h); break;
-    }
+    if (epi == EPI_CH)
+      k_coarse_hop<EPI_CH, ST><<<nb, 256, sm, s>>>(h);
+    else
+      k_coarse_hop<EPI_CX_PAY, ST><<<nb, 256, sm, s>>>(h);
   };
   switch (C.store) {
     case STORE_F32: launch(std::integral_constant<int, kStF32>()); break;

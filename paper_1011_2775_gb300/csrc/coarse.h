@@ -119,7 +119,8 @@ void galerkin_project(const TransferOp& T, CoarseOp& C, const float* const W[8],
 
 // ---- coarse stencil kernels
 // out[s] = epi(sum_{d in mask} Y_d(s) in[nbr_d(s)]) for storage sites
-// s in [s0, s1); epilogues as the fine dslash (EPI_*), C = X or Xinv.
+// s in [s0, s1); epilogues as the fine dslash: EPI_H and EPI_XPAY with all
+// directions or a single one, EPI_CH and EPI_CX_PAY (C = X or Xinv) with all.
 void coarse_hop(const LevelGeom& G, const CoarseOp& C, Epilogue epi, bool use_inv, int s0, int s1, float* out,
                 const float* in, const float* x, float a, int dirmask, cudaStream_t s);
 // out_o = A in_e (+ x_o: out_o = x_o + a A in_e) on the odd sites of an even-odd

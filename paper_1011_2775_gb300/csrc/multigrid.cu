@@ -187,8 +187,10 @@ void br_level(Ctx* c, Hierarchy& H, int l, float* br, const float* b) {
 void recon_level(Ctx* c, Hierarchy& H, int l, float* x, const float* y, const float* b) {
   const LevelGeom& G = H.geo[l];
   const CoarseOp& C = H.cop[l];
+  // x_e = X_e^{-1} y, x_o = X_o^{-1} (b_o - Y_oe x_e) = X_o^{-1} b_o - A y
   coarse_site_mul(G, C, true, 0, G.half, x, y, c->stream);
-  coarse_hop(G, C, EPI_C_XPAY, true, G.half, G.nsites, x, x, b, -1.f, 0xff, c->stream);
+  coarse_site_mul(G, C, true, G.half, G.nsites, x, b, c->stream);
+  coarse_folded(G, C, x, y, x, -1.f, c->stream);
 }
 
 void Dfull_level(Ctx* c, Hierarchy& H, int l, float* out, const float* in) {
