@@ -431,7 +431,7 @@ void blas_orth_update(T* w, const T* const* V, const double* d_beta, int k, cons
 }
 
 template <typename T>
-__global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restrict__ in, double* alpha_out,
+__global__ void k_r_update(cx<T>* w, const cx<T>* r, cx<T>* r_out, size_t n, const double* __restrict__ in, double* alpha_out,
                            double* gamma_out, double* partials, unsigned* counter, double* out) {
   // the square root and the divisions by one thread of the block: in every
   // thread they took longer than the pass over the vectors (29.8 us of which
@@ -461,7 +461,7 @@ __global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restric
     cx<T> b = r[i];
     b.re = fma(-a_r, q.re, fma(a_i, q.im, b.re));
     b.im = fma(-a_r, q.im, fma(-a_i, q.re, b.im));
-    r[i] = b;
+    r_out[i] = b;
     s = fma((acc_t<T>)b.re, (acc_t<T>)b.re, s);
     s = fma((acc_t<T>)b.im, (acc_t<T>)b.im, s);
   }
@@ -470,9 +470,10 @@ __global__ void k_r_update(cx<T>* w, cx<T>* r, size_t n, const double* __restric
 }
 
 template <typename T>
-void blas_r_update(T* w, T* r, size_t n, const double* d_in, double* d_alpha, double* d_gamma, double* d_rnorm2,
+void blas_r_update(T* w, const T* r, T* r_out, size_t n, const double* d_in, double* d_alpha, double* d_gamma,
+                   double* d_rnorm2,
                    Workspace& ws, cudaStream_t s) {
-  k_r_update<T><<<red_grid(n), kBS, 0, s>>>((cx<T>*)w, (cx<T>*)r, n, d_in, d_alpha, d_gamma, ws.partials.as<double>(),
+  k_r_update<T><<<red_grid(n), kBS, 0, s>>>((cx<T>*)w, (const cx<T>*)r, (cx<T>*)r_out, n, d_in, d_alpha, d_gamma, ws.partials.as<double>(),
                                             ws.counter.as<unsigned>(), d_rnorm2);
   MG_LAUNCH();
 }
@@ -626,7 +627,7 @@ void blas_normalize(T* x, const double* d_norm2, size_t n, cudaStream_t s) {
   template void blas_multidot<T>(const T* const*, int, const T*, size_t, double*, Workspace&, cudaStream_t);   \
   template void blas_orth_update<T>(T*, const T* const*, const double*, int, const T*, size_t, double*,        \
                                     Workspace&, cudaStream_t);                                                 \
-  template void blas_r_update<T>(T*, T*, size_t, const double*, double*, double*, double*, Workspace&,         \
+  template void blas_r_update<T>(T*, const T*, T*, size_t, const double*, double*, double*, double*, Workspace&, \
                                  cudaStream_t);                                                                \
   template void blas_mr_update<T>(T*, T*, const T*, const double*, size_t, cudaStream_t);                      \
   template void blas_normalize<T>(T*, const double*, size_t, cudaStream_t);

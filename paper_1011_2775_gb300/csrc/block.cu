@@ -280,7 +280,7 @@ int solve_runs(std::vector<Run>& runs, double tol) {
             double* bk = R.beta(q) + 2 * (size_t)m * k;
             if (k > 0) blas_multidot<double>(Wp.data(), k, w, R.n, bk, c->ws, c->stream);
             blas_orth_update<double>(w, Wp.data(), bk, k, r + q * R.hs, R.n, R.orth(q), c->ws, c->stream);
-            blas_r_update<double>(w, r + q * R.hs, R.n, R.orth(q), R.alpha(q) + 2 * k, R.gam(q) + k,
+            blas_r_update<double>(w, r + q * R.hs, r + q * R.hs, R.n, R.orth(q), R.alpha(q) + 2 * k, R.gam(q) + k,
                                   B.rn2.as<double>() + 2 * q, c->ws, c->stream);
           }
         }

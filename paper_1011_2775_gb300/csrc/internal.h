@@ -192,9 +192,10 @@ template <typename T>
 void blas_orth_update(T* w, const T* const* V, const double* d_beta, int k, const T* r, size_t n, double* d_out,
                       Workspace& ws, cudaStream_t s);
 // gamma = sqrt(d_in[0]); alpha = (d_in[1] + i d_in[2]) / gamma; w /= gamma;
-// r -= alpha w; stores alpha (2 doubles), gamma; d_rnorm2 = ||r||^2
+// r_out = r - alpha w (r_out may be r); stores alpha (2 doubles), gamma;
+// d_rnorm2 = ||r_out||^2
 template <typename T>
-void blas_r_update(T* w, T* r, size_t n, const double* d_in, double* d_alpha, double* d_gamma, double* d_rnorm2,
+void blas_r_update(T* w, const T* r, T* r_out, size_t n, const double* d_in, double* d_alpha, double* d_gamma, double* d_rnorm2,
                    Workspace& ws, cudaStream_t s);
 // x += scale * sum_j c_j Z_j (c device complex)
 template <typename T, typename TZ>

@@ -287,7 +287,11 @@ typename GCR<T, TZ>::Result GCR<T, TZ>::solve(const Op& A, const Pre* M, T* x, c
   cudaStream_t s = c_->stream;
   const int m = m_;
   const size_t n = n_;
-  T* r = r_.as<T>();
+  // without a preconditioner the residual is the direction: it lives in the
+  // history, every update writes the next one, and no copy is made
+  const bool in_place = !M && std::is_same<T, TZ>::value;
+  auto slot = [&](int k) { return in_place && k < m ? reinterpret_cast<T*>(Z_[k].as<TZ>()) : r_.as<T>(); };
+  T* r = slot(0);
   T* tmp = tmp_.as<T>();
   double* beta = s_;
   double* alpha = beta + 2 * (size_t)m * m;
@@ -329,7 +333,7 @@ typename GCR<T, TZ>::Result GCR<T, TZ>::solve(const Op& A, const Pre* M, T* x, c
       T* w = W_[k].as<T>();
       if (M)
         (*M)(z, r);
-      else
+      else if (!in_place)
         blas_convert<T, TZ>(z, r, n, s);
       if (Al) {
         (*Al)(w, z);
@@ -341,7 +345,9 @@ typename GCR<T, TZ>::Result GCR<T, TZ>::solve(const Op& A, const Pre* M, T* x, c
       }
       if (k > 0) blas_multidot<T>(Wp.data(), k, w, n, beta + 2 * (size_t)m * k, c_->ws, s);
       blas_orth_update<T>(w, Wp.data(), beta + 2 * (size_t)m * k, k, r, n, orth, c_->ws, s);
-      blas_r_update<T>(w, r, n, orth, alpha + 2 * k, gam + k, rn2, c_->ws, s);
+      T* next = slot(k + 1);
+      blas_r_update<T>(w, r, next, n, orth, alpha + 2 * k, gam + k, rn2, c_->ws, s);
+      r = next;
       k++;
       res.iterations++;
       if (check) {
@@ -357,8 +363,13 @@ typename GCR<T, TZ>::Result GCR<T, TZ>::solve(const Op& A, const Pre* M, T* x, c
     gcr_backsub(beta, m, alpha, gam, k, cc, s);
     blas_lincomb<T, TZ>(x, Zp.data(), cc, k, 1.0, n, s);
     res.restarts++;
-    if (!check) continue;  // recurrence residual carries over
+    if (!check) {  // recurrence residual carries over
+      if (r != slot(0) && res.iterations < maxit) blas_convert<T, T>(slot(0), r, n, s);
+      r = slot(0);
+      continue;
+    }
     // true residual at every restart
+    r = slot(0);
     A(tmp, x);
     blas_convert<T, T>(r, b, n, s);
     blas_axpby<T>(-1.0, tmp, 1.0, r, n, s);
