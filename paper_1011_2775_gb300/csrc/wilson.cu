@@ -219,20 +219,12 @@ __device__ void step(const Geom& g, const int x[4], int mu, int d, int y[4]) {
   for (int k = 0; k < 4; k++) y[k] = x[k];
   y[mu] = (x[mu] + d + g.L[mu]) % g.L[mu];
 }
-// c = a b, a^dag b, a b^dag
+// c = a b, a b^dag, a^dag b^dag
 __device__ void mm(const cd a[9], const cd b[9], cd c[9]) {
   for (int i = 0; i < 3; i++)
     for (int j = 0; j < 3; j++) {
       cd s = mkc(0.0, 0.0);
       for (int k = 0; k < 3; k++) s = cfma(a[i * 3 + k], b[k * 3 + j], s);
-      c[i * 3 + j] = s;
-    }
-}
-__device__ void mdm(const cd a[9], const cd b[9], cd c[9]) {
-  for (int i = 0; i < 3; i++)
-    for (int j = 0; j < 3; j++) {
-      cd s = mkc(0.0, 0.0);
-      for (int k = 0; k < 3; k++) s = cfma_conj(a[k * 3 + i], b[k * 3 + j], s);
       c[i * 3 + j] = s;
     }
 }
@@ -245,96 +237,122 @@ __device__ void mmd(const cd a[9], const cd b[9], cd c[9]) {
     }
 }
 
-// Q_{mu nu}(x): sum of the four counter-clockwise plaquette leaves at x.
-__device__ void clover_leaves(const Geom& g, const double* gauge, const int x[4], int mu, int nu, cd q[9]) {
-  int y[4], z[4];
-  cd a[9], b[9], t1[9], t2[9];
-  for (int e = 0; e < 9; e++) q[e] = mkc(0.0, 0.0);
-  // leaf 1: U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-  link_at(g, gauge, x, mu, a);
-  step(g, x, mu, +1, y); link_at(g, gauge, y, nu, b);
-  mm(a, b, t1);
-  step(g, x, nu, +1, y); link_at(g, gauge, y, mu, a);
-  mmd(t1, a, t2);
-  link_at(g, gauge, x, nu, a);
-  mmd(t2, a, t1);
-  for (int e = 0; e < 9; e++) q[e] = q[e] + t1[e];
-  // leaf 2: U_nu(x) U_mu(x+nu-mu)^dag U_nu(x-mu)^dag U_mu(x-mu)
-  link_at(g, gauge, x, nu, a);
-  step(g, x, nu, +1, y); step(g, y, mu, -1, z); link_at(g, gauge, z, mu, b);
-  mmd(a, b, t1);
-  step(g, x, mu, -1, y); link_at(g, gauge, y, nu, a);
-  mmd(t1, a, t2);
-  link_at(g, gauge, y, mu, a);
-  mm(t2, a, t1);
-  for (int e = 0; e < 9; e++) q[e] = q[e] + t1[e];
-  // leaf 3: U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu)
-  step(g, x, mu, -1, y); link_at(g, gauge, y, mu, a);
-  step(g, y, nu, -1, z); link_at(g, gauge, z, nu, b);
-  // t1 = a^dag b^dag = (b a)^dag
-  mm(b, a, t2);
+__device__ void mdmd(const cd a[9], const cd b[9], cd c[9]) {
   for (int i = 0; i < 3; i++)
-    for (int j = 0; j < 3; j++) t1[i * 3 + j] = conj(t2[j * 3 + i]);
-  link_at(g, gauge, z, mu, a);
-  mm(t1, a, t2);
-  step(g, x, nu, -1, y); link_at(g, gauge, y, nu, a);
-  mm(t2, a, t1);
-  for (int e = 0; e < 9; e++) q[e] = q[e] + t1[e];
-  // leaf 4: U_nu(x-nu)^dag U_mu(x-nu) U_nu(x-nu+mu) U_mu(x)^dag
-  step(g, x, nu, -1, y); link_at(g, gauge, y, nu, a);
-  link_at(g, gauge, y, mu, b);
-  mdm(a, b, t1);
-  step(g, y, mu, +1, z); link_at(g, gauge, z, nu, a);
-  mm(t1, a, t2);
-  link_at(g, gauge, x, mu, a);
-  mmd(t2, a, t1);
-  for (int e = 0; e < 9; e++) q[e] = q[e] + t1[e];
+    for (int j = 0; j < 3; j++) {
+      cd s = mkc(0.0, 0.0);
+      for (int k = 0; k < 3; k++) s = cfma(b[j * 3 + k], a[k * 3 + i], s);   // (b a)_{j i}
+      c[i * 3 + j] = conj(s);
+    }
 }
 
-// In-place inverse of a 6x6 complex matrix by Gauss-Jordan with partial
-// pivoting; returns false if a pivot falls below 1e-12 of the largest entry.
-__device__ bool invert6(cd m[36], cd inv[36]) {
+// G with G - G^dag = Q_{mu nu}(x) - Q_{mu nu}(x)^dag, Q the sum of the four
+// counter-clockwise plaquette leaves at x.  The leaves that run through
+// U_nu(x - nu) enter as minus their daggers, so that two leaves at a time share
+// their first or last link: ten products instead of twelve.
+__device__ void clover_leaves(const Geom& g, const double* gauge, const int x[4], int mu, int nu, cd q[9]) {
+  int xm[4], xn[4], y[4];
+  cd a[9], b[9], t[9], u[9];
+  // U_mu(x) [U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x-nu+mu)^dag U_mu(x-nu)^dag U_nu(x-nu)]
+  step(g, x, mu, +1, xm); link_at(g, gauge, xm, nu, a);
+  step(g, x, nu, +1, y); link_at(g, gauge, y, mu, b);
+  mmd(a, b, t);
+  link_at(g, gauge, x, nu, a);
+  mmd(t, a, u);
+  step(g, xm, nu, -1, y); link_at(g, gauge, y, nu, a);
+  step(g, x, nu, -1, xn); link_at(g, gauge, xn, mu, b);
+  mdmd(a, b, t);
+  link_at(g, gauge, xn, nu, a);
+  mm(t, a, b);
+  for (int e = 0; e < 9; e++) u[e] = u[e] - b[e];
+  link_at(g, gauge, x, mu, a);
+  mm(a, u, q);
+  // [U_nu(x) U_mu(x+nu-mu)^dag U_nu(x-mu)^dag - U_nu(x-nu)^dag U_mu(x-mu-nu)^dag U_nu(x-mu-nu)] U_mu(x-mu)
+  step(g, x, mu, -1, xm);
+  link_at(g, gauge, x, nu, a);
+  step(g, xm, nu, +1, y); link_at(g, gauge, y, mu, b);
+  mmd(a, b, t);
+  link_at(g, gauge, xm, nu, a);
+  mmd(t, a, u);
+  link_at(g, gauge, xn, nu, a);
+  step(g, xm, nu, -1, y); link_at(g, gauge, y, mu, b);
+  mdmd(a, b, t);
+  link_at(g, gauge, y, nu, a);
+  mm(t, a, b);
+  for (int e = 0; e < 9; e++) u[e] = u[e] - b[e];
+  link_at(g, gauge, xm, mu, a);
+  mm(u, a, t);
+  for (int e = 0; e < 9; e++) q[e] = q[e] + t[e];
+}
+
+// Inverse of a 6x6 complex matrix by Gauss-Jordan with partial pivoting, in
+// place (the columns of the inverse replace the eliminated ones, the row
+// exchanges become column exchanges at the end) and in registers: every index
+// is a constant, an exchange is a select.  Returns false if a pivot falls below
+// 1e-12 of the largest entry.
+__device__ __forceinline__ bool invert6(cd (&m)[36]) {
   double amax = 0;
+#pragma unroll
   for (int e = 0; e < 36; e++) amax = fmax(amax, fabs(m[e].re) + fabs(m[e].im));
-  for (int i = 0; i < 6; i++)
-    for (int j = 0; j < 6; j++) inv[i * 6 + j] = mkc(i == j ? 1.0 : 0.0, 0.0);
   bool ok = amax > 0;
+  int perm[6];
+#pragma unroll
   for (int col = 0; col < 6; col++) {
     int piv = col;
     double best = -1;
+#pragma unroll
     for (int r = col; r < 6; r++) {
-      double v = m[r * 6 + col].re * m[r * 6 + col].re + m[r * 6 + col].im * m[r * 6 + col].im;
+      const double v = fma(m[r * 6 + col].re, m[r * 6 + col].re, m[r * 6 + col].im * m[r * 6 + col].im);
       if (v > best) { best = v; piv = r; }
     }
+    perm[col] = piv;
     if (!(sqrt(best) > 1e-12 * amax)) { ok = false; best = 1.0; }
-    if (piv != col)
-      for (int j = 0; j < 6; j++) {
-        cd t = m[col * 6 + j]; m[col * 6 + j] = m[piv * 6 + j]; m[piv * 6 + j] = t;
-        t = inv[col * 6 + j]; inv[col * 6 + j] = inv[piv * 6 + j]; inv[piv * 6 + j] = t;
+#pragma unroll
+    for (int r = col + 1; r < 6; r++)
+      if (piv == r) {
+#pragma unroll
+        for (int j = 0; j < 6; j++) {
+          const cd t = m[col * 6 + j];
+          m[col * 6 + j] = m[r * 6 + j];
+          m[r * 6 + j] = t;
+        }
       }
-    cd p = m[col * 6 + col];
-    double den = p.re * p.re + p.im * p.im;
+    const cd p = m[col * 6 + col];
+    double den = fma(p.re, p.re, p.im * p.im);
     if (den == 0) den = 1;
-    cd pinv = mkc(p.re / den, -p.im / den);
-    for (int j = 0; j < 6; j++) {
-      m[col * 6 + j] = pinv * m[col * 6 + j];
-      inv[col * 6 + j] = pinv * inv[col * 6 + j];
-    }
+    const double di = 1.0 / den;
+    const cd pinv = mkc(p.re * di, -p.im * di);
+#pragma unroll
+    for (int j = 0; j < 6; j++) m[col * 6 + j] = j == col ? pinv : pinv * m[col * 6 + j];
+#pragma unroll
     for (int r = 0; r < 6; r++) {
       if (r == col) continue;
-      cd f = m[r * 6 + col];
-      for (int j = 0; j < 6; j++) {
-        m[r * 6 + j] = m[r * 6 + j] - f * m[col * 6 + j];
-        inv[r * 6 + j] = inv[r * 6 + j] - f * inv[col * 6 + j];
-      }
+      const cd f = m[r * 6 + col], nf = mkc(-f.re, -f.im);
+#pragma unroll
+      for (int j = 0; j < 6; j++) m[r * 6 + j] = j == col ? nf * m[col * 6 + j] : cfma(nf, m[col * 6 + j], m[r * 6 + j]);
     }
   }
+#pragma unroll
+  for (int col = 5; col >= 0; col--)
+#pragma unroll
+    for (int r = col + 1; r < 6; r++)
+      if (perm[col] == r) {
+#pragma unroll
+        for (int i = 0; i < 6; i++) {
+          const cd t = m[i * 6 + col];
+          m[i * 6 + col] = m[i * 6 + r];
+          m[i * 6 + r] = t;
+        }
+      }
   return ok;
 }
 
-__device__ void pack_herm(const cd m[36], double r[36]) {
+__device__ __forceinline__ void pack_herm(const cd (&m)[36], double (&r)[36]) {
+#pragma unroll
   for (int i = 0; i < 6; i++) r[i] = m[i * 6 + i].re;
+#pragma unroll
   for (int i = 1; i < 6; i++)
+#pragma unroll
     for (int j = 0; j < i; j++) {
       const int k = i * (i - 1) / 2 + j;
       r[6 + 2 * k] = m[i * 6 + j].re;
@@ -343,8 +361,14 @@ __device__ void pack_herm(const cd m[36], double r[36]) {
 }
 }  // namespace
 
-__global__ void k_build_clover(Geom g, const double* __restrict__ gauge, CloverCoef cf, double m0, double* A64,
-                               double* Ainv64, float* A32, float* Ainv32, int* flags) {
+// One thread per site, bound by the FP64 pipe: per plane ten 3x3 products, per
+// spin entry of sigma one product with F (the zero entries are skipped, the
+// condition is the same for all threads), and two inversions in place.  With
+// twelve products, two complex products per entry and the inversion of the
+// augmented matrix in local memory 131072 sites took 4.11 ms, 2.41 here.
+__global__ void __launch_bounds__(64) k_build_clover(Geom g, const double* __restrict__ gauge, CloverCoef cf, double m0,
+                                                     double* A64, double* Ainv64, float* A32, float* Ainv32,
+                                                     int* flags) {
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= 2 * g.Vh) return;
   const int par = gid / g.Vh, i = gid % g.Vh;
@@ -352,32 +376,53 @@ __global__ void k_build_clover(Geom g, const double* __restrict__ gauge, CloverC
   cb_coords(g, i, par, x);
   // lower triangles (i >= j) of the two chiral blocks
   cd L[2][21];
+#pragma unroll
   for (int b = 0; b < 2; b++)
+#pragma unroll
     for (int e = 0; e < 21; e++) L[b][e] = mkc(0.0, 0.0);
   int plane = 0;
+#pragma unroll 1
   for (int mu = 0; mu < 4; mu++)
+#pragma unroll 1
     for (int nu = mu + 1; nu < 4; nu++, plane++) {
       cd q[9], F[9];
       clover_leaves(g, gauge, x, mu, nu, q);
+#pragma unroll
       for (int a = 0; a < 3; a++)
+#pragma unroll
         for (int c = 0; c < 3; c++) F[a * 3 + c] = 0.125 * (q[a * 3 + c] - conj(q[c * 3 + a]));
-      cd tr = mkc((F[0].re + F[4].re + F[8].re) / 3.0, (F[0].im + F[4].im + F[8].im) / 3.0);
+      const cd tr = mkc((F[0].re + F[4].re + F[8].re) / 3.0, (F[0].im + F[4].im + F[8].im) / 3.0);
       F[0] = F[0] - tr; F[4] = F[4] - tr; F[8] = F[8] - tr;
       // sum over mu != nu of both orders gives 2x the mu < nu term:
       // A += (i c_{mu nu} / 2) sigma_{mu nu} (x) F_{mu nu}, c = csw_t for the planes
       // that contain t, csw_s for the spatial ones (one csw when isotropic)
-      const cd pre = mkc(0.0, 0.5 * (nu == 3 ? cf.csw_t : cf.csw_s));
+      const double pre = 0.5 * (nu == 3 ? cf.csw_t : cf.csw_s);
+#pragma unroll
       for (int b = 0; b < 2; b++)
-        for (int ii = 0; ii < 6; ii++)
-          for (int jj = 0; jj <= ii; jj++) {
-            const int si = ii / 3, ci = ii % 3, sj = jj / 3, cj = jj % 3;
-            cd sg = mkc(c_sigma[plane][b][si][sj][0], c_sigma[plane][b][si][sj][1]);
-            L[b][ii * (ii + 1) / 2 + jj] = L[b][ii * (ii + 1) / 2 + jj] + pre * (sg * F[ci * 3 + cj]);
+#pragma unroll
+        for (int si = 0; si < 2; si++)
+#pragma unroll
+          for (int sj = 0; sj <= si; sj++) {
+            const cd sg = mkc(-pre * c_sigma[plane][b][si][sj][1], pre * c_sigma[plane][b][si][sj][0]);   // i pre sigma
+            if (sg.re == 0.0 && sg.im == 0.0) continue;
+#pragma unroll
+            for (int ci = 0; ci < 3; ci++)
+#pragma unroll
+              for (int cj = 0; cj < 3; cj++) {
+                const int ii = 3 * si + ci, jj = 3 * sj + cj;
+                if (jj > ii) continue;
+                cd& e = L[b][ii * (ii + 1) / 2 + jj];
+                e = cfma(sg, F[ci * 3 + cj], e);
+              }
           }
     }
+  bool ok = true;
+#pragma unroll
   for (int b = 0; b < 2; b++) {
-    cd M[36], Minv[36];
+    cd M[36];
+#pragma unroll
     for (int ii = 0; ii < 6; ii++)
+#pragma unroll
       for (int jj = 0; jj <= ii; jj++) {
         cd v = L[b][ii * (ii + 1) / 2 + jj];
         if (ii == jj) v = mkc(v.re + (g.w[0] + g.w[1] + g.w[2] + g.w[3]) + m0, 0.0);   // 4 + m0 when isotropic
@@ -385,23 +430,28 @@ __global__ void k_build_clover(Geom g, const double* __restrict__ gauge, CloverC
         M[jj * 6 + ii] = conj(v);
       }
     double r[36];
+    float rf[36];
     pack_herm(M, r);
     CloverIO<double>::store_block(A64 + (size_t)par * 72 * g.Vh, g.Vh, i, b, r);
-    float rf[36];
+#pragma unroll
     for (int e = 0; e < 36; e++) rf[e] = (float)r[e];
     CloverIO<float>::store_block(A32 + (size_t)par * 72 * g.Vh, g.Vh, i, b, rf);
-    if (!invert6(M, Minv)) atomicExch(&flags[FLAG_SINGULAR], 1);
+    ok &= invert6(M);
     // symmetrise: store the Hermitian part of the inverse
+#pragma unroll
     for (int ii = 0; ii < 6; ii++)
+#pragma unroll
       for (int jj = 0; jj <= ii; jj++) {
-        cd a = Minv[ii * 6 + jj], c = conj(Minv[jj * 6 + ii]);
-        Minv[ii * 6 + jj] = mkc(0.5 * (a.re + c.re), 0.5 * (a.im + c.im));
+        const cd a = M[ii * 6 + jj], c = conj(M[jj * 6 + ii]);
+        M[ii * 6 + jj] = mkc(0.5 * (a.re + c.re), 0.5 * (a.im + c.im));
       }
-    pack_herm(Minv, r);
+    pack_herm(M, r);
     CloverIO<double>::store_block(Ainv64 + (size_t)par * 72 * g.Vh, g.Vh, i, b, r);
+#pragma unroll
     for (int e = 0; e < 36; e++) rf[e] = (float)r[e];
     CloverIO<float>::store_block(Ainv32 + (size_t)par * 72 * g.Vh, g.Vh, i, b, rf);
   }
+  if (!ok) atomicExch(&flags[FLAG_SINGULAR], 1);
 }
 
 void build_clover(const Geom& g, const double* g64, CloverCoef cf, double m0, double* A64, double* Ainv64,
