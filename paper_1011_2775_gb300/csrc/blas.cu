@@ -2,7 +2,8 @@
 // (section "Adaptive multigrid": GCR is the outer solver; section
 // "Implementation": GCR again on every coarse level).
 //
-// All inner products accumulate in FP64 regardless of the vector precision.
+// Inner products of FP64 vectors accumulate in FP64; of FP32 vectors in FP32 over
+// the few elements of a thread and in double-float across threads.
 // Reductions are deterministic: a fixed grid (a function of n only), per-block
 // partials written to the workspace, and an ordered final sum by the last
 // block to finish (grid_sum in dfloat.cuh).  The GCR kernels fuse the

@@ -21,7 +21,7 @@
 //    arrive while the block waits at a grid barrier.  A warp computes all
 //    rows of its item: every lane strides along the row, the gathered vector
 //    element is loaded once for all rows, and one transposing shuffle
-//    reduction finishes up to eight rows.
+//    reduction finishes an item's rows (two, four or eight of them).
 //  * The element-wise work belongs to the block that computed those rows in
 //    phase B, so the Gram-Schmidt dots follow phase B without a barrier:
 //    one iteration is phase A | barrier | phase B + dots | barrier |
@@ -30,7 +30,7 @@
 //    reduction when that subtraction loses more than three digits; <w', r>
 //    = <w, r> / gamma because r is orthogonal to the w_j.  The block's slice
 //    of the Krylov vectors w_j stays in shared memory when it is small.
-//  * Every inner product is reduced deterministically (per-block FP64
+//  * Every inner product is reduced deterministically (per-block double-float
 //    partials summed in the same order by every block), so all blocks take
 //    identical decisions and the result is reproducible bit for bit.
 //  * Every wait (mbarrier, grid barrier) is bounded in time; a block that
