@@ -61,10 +61,10 @@ REFERENCE_OUTER_PER_SOLVE = 42
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the FP32 fused
 # dslash on 32^3x64, from the ncu capture in profiles/dslash_fp32_32x32x32x64.md
 # (set to None whenever that kernel changes)
-DSLASH_TRAFFIC_BYTES = 1.125e9
+DSLASH_TRAFFIC_BYTES = 1.124e9
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the streamed
 # coarsest-level solve on this workload (None whenever that kernel changes)
-COARSE_TRAFFIC_BYTES = 79.13e6        # profiles/coarse_gcr_stream_4x4x4x8.md: 76.46 MB read + 2.67 MB written
+COARSE_TRAFFIC_BYTES = 78.58e6        # profiles/coarse_gcr_stream_4x4x4x8.md: 76.24 MB read + 2.34 MB written
                                       # per launch of COARSE_PROFILE_ITERS iterations (the links' first touch
                                       # after the fine-level work; L2 hits afterwards)
 DSLASH_FLOPS_PER_SITE = 1824        # fused hop + clover inverse, per output site
