@@ -147,6 +147,15 @@ struct CoarseGCRBuffers {
   DBuf tc_y, tc_r, tc_br, tc_s, tc_sy, tc_t, tc_tb, tc_W, tc_Z, tc_part, tc_sync;
   // grouped solve (coarse_group.cu; grown on demand)
   DBuf gp_v, gp_W, gp_R, gp_part, gp_sync;
+  // Grows a buffer.  A captured cycle holds the buffers' addresses, and a solve of
+  // more systems moves them: `regrown` counts the moves, and the graph is captured
+  // again when it has changed (mg_precondition_graph).
+  long long regrown = 0;
+  void grow(DBuf& d, size_t bytes) {
+    if (d.bytes() >= bytes) return;
+    regrown++;
+    d.alloc(bytes);
+  }
   void init(const LevelGeom& G, int nc, int m);
 };
 // x = D_hat^{-1} b to ||b - D_hat x|| <= tol_rel ||b|| (or maxit iterations) by

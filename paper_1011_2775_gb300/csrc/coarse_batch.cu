@@ -654,20 +654,17 @@ void coarse_gcr_solve_multi(const std::vector<CoarseSystem>& sys, CoarseGCRBuffe
   if (A.Gp < 1) raise(MG_ERR_ARG, "batch larger than the co-resident grid");
   // buffers (grown on demand)
   A.nscal = scalars_per_system(m);
-  auto grow = [&](DBuf& d, size_t bytes) {
-    if (d.bytes() < bytes) d.alloc(bytes);
-  };
-  grow(Bf.bx_r, sizeof(float2) * ntot);
-  grow(Bf.bx_y, sizeof(float2) * ntot);
-  grow(Bf.bx_br, sizeof(float2) * ntot);
+  Bf.grow(Bf.bx_r, sizeof(float2) * ntot);
+  Bf.grow(Bf.bx_y, sizeof(float2) * ntot);
+  Bf.grow(Bf.bx_br, sizeof(float2) * ntot);
   if (Bf.bx_tB.bytes() < sizeof(float2) * nftot) {
-    Bf.bx_tB.alloc(sizeof(float2) * nftot);
+    Bf.grow(Bf.bx_tB, sizeof(float2) * nftot);
     MG_CUDA(cudaMemsetAsync(Bf.bx_tB.get(), 0, sizeof(float2) * nftot, s));
   }
-  grow(Bf.bx_W, sizeof(float2) * ntot * m);
-  grow(Bf.bx_Z, sizeof(float2) * ntot * m);
-  grow(Bf.bx_part, sizeof(double) * (size_t)kNR * nb * A.Gp);
-  grow(Bf.bx_scal, sizeof(double) * A.nscal * nb);
+  Bf.grow(Bf.bx_W, sizeof(float2) * ntot * m);
+  Bf.grow(Bf.bx_Z, sizeof(float2) * ntot * m);
+  Bf.grow(Bf.bx_part, sizeof(double) * (size_t)kNR * nb * A.Gp);
+  Bf.grow(Bf.bx_scal, sizeof(double) * A.nscal * nb);
   A.r = Bf.bx_r.as<float2>();
   A.y = Bf.bx_y.as<float2>();
   A.br = Bf.bx_br.as<float2>();

@@ -813,14 +813,11 @@ void coarse_gcr_group_solve(const std::vector<CoarseSystem>& sys, CoarseGCRBuffe
   a.items = p.items;
   a.chunk = p.chunk;
   const size_t n = (size_t)a.rows_sites * nc;
-  auto need = [&](DBuf& d, size_t bytes) {
-    if (d.bytes() < bytes) d.alloc(bytes);
-  };
-  need(B.gp_v, sizeof(float2) * n * nb * 5);
-  need(B.gp_W, sizeof(float2) * n * nb * (size_t)m);
-  need(B.gp_R, sizeof(float2) * n * nb * (size_t)m);
-  need(B.gp_part, sizeof(float2) * (size_t)nb * kSlots * p.grid);
-  need(B.gp_sync, 512 + sizeof(float2) * (kMaxSys * (size_t)(kSlots + 2 * kMaxRestart + kMaxRestart * kMaxRestart)));
+  B.grow(B.gp_v, sizeof(float2) * n * nb * 5);
+  B.grow(B.gp_W, sizeof(float2) * n * nb * (size_t)m);
+  B.grow(B.gp_R, sizeof(float2) * n * nb * (size_t)m);
+  B.grow(B.gp_part, sizeof(float2) * (size_t)nb * kSlots * p.grid);
+  B.grow(B.gp_sync, 512 + sizeof(float2) * (kMaxSys * (size_t)(kSlots + 2 * kMaxRestart + kMaxRestart * kMaxRestart)));
   float2* v = B.gp_v.as<float2>();
   a.y = v;
   a.r = v + n * nb;

@@ -822,15 +822,12 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
   MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 32 * p.warps, p.smem));
   if (per < 1 || p.grid > per * sms) raise(MG_ERR_CUDA, "streamed coarse GCR cannot be resident");
   const size_t n = (size_t)(G.eo ? G.half : G.nsites) * C.nc;
-  auto need = [&](DBuf& d, size_t bytes) {
-    if (d.bytes() < bytes) d.alloc(bytes);
-  };
-  need(B.st_part, sizeof(float2) * (size_t)kNR * p.grid);
-  need(B.st_sync, 256);
+  B.grow(B.st_part, sizeof(float2) * (size_t)kNR * p.grid);
+  B.grow(B.st_sync, 256);
   if (B.W.bytes() < sizeof(float2) * n * m || B.Z.bytes() < sizeof(float2) * n * m)
     raise(MG_ERR_STATE, "coarse GCR buffers too small for this restart length");
   if (G.eo) {
-    need(B.st_to, sizeof(float2) * 2 * n);
+    B.grow(B.st_to, sizeof(float2) * 2 * n);
     coarse_site_mul(G, C, true, G.half, G.nsites, B.st_to.as<float>(), b, s);     // t_o = X_o^{-1} b_o
   }
   MG_CUDA(cudaMemsetAsync(B.st_sync.get(), 0, 256, s));

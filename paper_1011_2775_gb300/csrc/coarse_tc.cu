@@ -801,22 +801,19 @@ void coarse_gcr_tc_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuffers
   MG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, p.smem));
   if (per < 1 || p.grid > per * sms) raise(MG_ERR_CUDA, "tensor-core coarse GCR cannot be resident");
   const size_t n = (size_t)G.half * C.nc;
-  auto need = [&](DBuf& d, size_t bytes) {
-    if (d.bytes() < bytes) d.alloc(bytes);
-  };
   const size_t vb = sizeof(float2) * n * nb;
-  need(B.tc_y, vb);
-  need(B.tc_r, vb);
-  need(B.tc_br, vb);
-  need(B.tc_s, vb);
-  need(B.tc_sy, vb);
-  need(B.tc_t, vb);
-  need(B.tc_tb, vb);
-  need(B.tc_W, vb * m);
-  need(B.tc_Z, vb * m);
+  B.grow(B.tc_y, vb);
+  B.grow(B.tc_r, vb);
+  B.grow(B.tc_br, vb);
+  B.grow(B.tc_s, vb);
+  B.grow(B.tc_sy, vb);
+  B.grow(B.tc_t, vb);
+  B.grow(B.tc_tb, vb);
+  B.grow(B.tc_W, vb * m);
+  B.grow(B.tc_Z, vb * m);
   const int Gp = p.grid / nb;
-  need(B.tc_part, sizeof(float2) * (size_t)kSlots * kMaxSys * Gp);
-  need(B.tc_sync, 512);
+  B.grow(B.tc_part, sizeof(float2) * (size_t)kSlots * kMaxSys * Gp);
+  B.grow(B.tc_sync, 512);
   TArgs a;
   std::memset(&a, 0, sizeof(a));
   a.nc = C.nc;

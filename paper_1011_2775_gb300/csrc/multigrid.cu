@@ -107,6 +107,7 @@ struct CycleGraph {
   cudaStream_t cap = nullptr;   // private stream the capture runs on
   const double* r = nullptr;    // the input the graph was captured for
   float* r32 = nullptr;
+  long long regrown = 0;        // CoarseGCRBuffers::regrown of the coarsest level at the capture
   bool failed = false;
   long long dslash = 0, kernels = 0;   // launches one replay executes (for the statistics)
   DBuf zc;                      // the graph's output
@@ -855,7 +856,8 @@ bool mg_precondition_graph(Ctx* c, float* z_e, const double* r_e, float* r32) {
   CycleGraph& G = H.graph;
   if (H.L != 2 || G.failed || H.work[1].coarse_impl < 0) return false;
   const size_t n = half_n(H, 0);
-  if (!G.exec || G.r != r_e || G.r32 != r32) {
+  // captured for other vectors, or the coarsest solver's buffers have moved since
+  if (!G.exec || G.r != r_e || G.r32 != r32 || G.regrown != H.work[1].cg.regrown) {
     if (G.exec) {
       cudaGraphExecDestroy(G.exec);
       G.exec = nullptr;
@@ -893,6 +895,7 @@ bool mg_precondition_graph(Ctx* c, float* z_e, const double* r_e, float* r32) {
     }
     G.r = r_e;
     G.r32 = r32;
+    G.regrown = H.work[1].cg.regrown;
   }
   MG_CUDA(cudaGraphLaunch(G.exec, c->stream));
   c->dslash_launches += G.dslash;
