@@ -121,6 +121,34 @@ void read_norms(Run& R, const double* ve, const double* vo, const std::vector<ch
   c->sync();
 }
 
+// Puts the coarsest solves of several contexts in order, whatever their streams:
+// a persistent solver's grid waits for all of its blocks at grid barriers, and of
+// two such grids in flight on different streams each could become resident in part.
+class OneAtATime {
+ public:
+  OneAtATime() = default;
+  OneAtATime(const OneAtATime&) = delete;
+  OneAtATime& operator=(const OneAtATime&) = delete;
+  ~OneAtATime() {
+    for (cudaEvent_t e : ev_) cudaEventDestroy(e);   // one still pending is released when it completes
+  }
+  // what `s` is given from here on starts after the solves queued so far
+  void begin(cudaStream_t s) {
+    if (!ev_.empty() && s != last_) MG_CUDA(cudaStreamWaitEvent(s, ev_.back(), 0));
+  }
+  void end(cudaStream_t s) {
+    cudaEvent_t e;
+    MG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    ev_.push_back(e);
+    MG_CUDA(cudaEventRecord(e, s));
+    last_ = s;
+  }
+
+ private:
+  std::vector<cudaEvent_t> ev_;
+  cudaStream_t last_ = nullptr;
+};
+
 // the cycle for every run, with the coarsest solves of the joinable runs in
 // shared launches (the others solve their own)
 void precondition_all(std::vector<Run*>& runs, int k) {
@@ -151,11 +179,17 @@ void precondition_all(std::vector<Run*>& runs, int k) {
     blas_convert<double, float>(r32, R->B->r.as<double>(), R->n * R->nb, R->c->stream);
     mg_batch_pre(R->c, zk, r32, R->nb);
   }
-  for (Run* R : alone) mg_batch_coarse(R->c, R->nb);
+  OneAtATime turn;
+  for (Run* R : alone) {
+    turn.begin(R->c->stream);
+    mg_batch_coarse(R->c, R->nb);
+    if (alone.size() + shared.size() > 1) turn.end(R->c->stream);
+  }
   if (!shared.empty()) {
     // all systems, in groups the persistent kernel accepts; the first context's stream
     // runs the shared launches after every participant's restriction
     Ctx* c0 = shared[0]->c;
+    turn.begin(c0->stream);
     std::vector<CoarseSystem> sys;
     std::vector<std::vector<CoarseSystem>> launches;
     std::vector<const void*> lattices;
