@@ -349,10 +349,12 @@ MG_API int mg_solve(void* ctx, void* psi, const void* eta, int nrhs, double tol,
  * lattice) to tolerance tol, by multigrid-preconditioned FGCR, one per
  * right-hand side, run in lock-step: each iteration applies the fine
  * operators of every context to all of its right-hand sides in multi-RHS
- * launches, and puts the coarsest-level solves of all right-hand sides of all
- * 2-level contexts into shared persistent launches (up to 16 systems and 8
- * lattices each; contexts whose hierarchy is deeper, or whose coarse storage,
- * restart or cap differ from the first's, solve their own).  Right-hand sides
+ * launches.  The coarsest-level solves of many small 2-level lattices go into
+ * shared persistent launches (up to 16 systems and 8 lattices each); larger
+ * lattices, or few, take a launch each for all of their right-hand sides, and
+ * so do contexts whose hierarchy is deeper or whose coarse storage, restart or
+ * cap differ from the first's.  One such launch is in flight at a time,
+ * whatever the contexts' streams.  Right-hand sides
  * are taken in context order in groups of at most the first context's
  * rhs_block (a context's right-hand sides are not split when they fit in a
  * fresh group).

@@ -5,10 +5,10 @@
 // "Red-black preconditioning"; section "Implementation"), run for every
 // right-hand side in lock-step: every iteration applies the multigrid cycle to
 // all residuals of a context at once (multi-RHS D_r in the smoother) and the
-// FP64 D_r to all its new directions in one multi-RHS launch, and the
-// coarsest-level solves of ALL right-hand sides of all contexts go into one
-// persistent launch (coarse_gcr_solve_multi: one coarse lattice per context,
-// systems of one lattice sharing link reads).  The Krylov space, scalars,
+// FP64 D_r to all its new directions in one multi-RHS launch.  The
+// coarsest-level solves of a context's right-hand sides go into one persistent
+// launch, or those of several small lattices share one (coarse_gcr_solve_multi;
+// the rule is mg_batch_own_launch).  The Krylov space, scalars,
 // convergence test and restarts of every right-hand side are its own; a
 // right-hand side that has converged stops updating (its slot in the
 // multi-RHS launches is carried along).  Vectors are packed half vectors: rhs
@@ -153,9 +153,10 @@ class OneAtATime {
 // shared launches (the others solve their own)
 void precondition_all(std::vector<Run*>& runs, int k) {
   std::vector<Run*> joint, own;
-  // a lattice whose systems the grouped solver takes together is faster by itself than
-  // in a launch shared with other lattices
-  for (Run* R : runs) (mg_batch_joinable(R->c) && !mg_batch_grouped(R->c, R->nb) ? joint : own).push_back(R);
+  int joinable = 0;
+  for (Run* R : runs) joinable += mg_batch_joinable(R->c);
+  for (Run* R : runs)
+    (mg_batch_joinable(R->c) && !mg_batch_own_launch(R->c, R->nb, joinable) ? joint : own).push_back(R);
   // runs that can share a launch: same device, coarse storage, restart, cap and even-odd structure
   std::vector<Run*> shared, alone = own;
   for (Run* R : joint) {

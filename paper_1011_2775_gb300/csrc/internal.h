@@ -478,6 +478,9 @@ void mg_batch_post(Ctx* c, float* z_e, const float* r_e, int nb);
 bool mg_batch_joinable(Ctx* c);
 // the coarsest solves of nb right-hand sides of this context take the grouped solver by themselves
 bool mg_batch_grouped(Ctx* c, int nb);
+// of `contexts` 2-level contexts solved together, this one takes a launch of its own
+// rather than a share of one over all lattices
+bool mg_batch_own_launch(Ctx* c, int nb, int contexts);
 // MG_OP_CYCLE of level 0 for nb ABI vectors through mg_precondition_batch
 void mg_cycle_batch(Ctx* c, double* out_abi, const double* in_abi, int nb);
 void mg_apply_level(Ctx* c, int op, int level, double* out_abi, const double* in_abi);

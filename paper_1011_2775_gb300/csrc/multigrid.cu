@@ -728,6 +728,24 @@ bool mg_batch_grouped(Ctx* c, int nb) {
   return coarse_gcr_group_ok(c->mg->geo[1], c->mg->cop[1], std::min(nb, coarse_gcr_batch_max()));
 }
 
+// Several lattices: a launch for each takes its links at the grouped solver's
+// rate, one shared launch has its barriers once for all.  Solves of L lattices with
+// n sources each, a launch each against shared (reduced sites, Nc of the coarsest
+// level):
+//   256, 48: 30 / 52 ms (L 2, n 1), 118 / 164 (8, 1), 197 / 234 (8, 2)
+//   128, 48: 27 / 38 (3, 1), 72 / 85 (8, 1), 110 / 116 (8, 2)
+//    64, 48: 31 / 34 (4, 1), 62 / 64 (8, 1), 84 / 82.5 (8, 2)
+//    32, 48: 25 / 27 (4, 1), 50.5 / 48.8 (8, 1), 33 / 31 (4, 2), 66 / 57.5 (8, 2)
+//    16, 48: 11.2 / 14.2 (2, 1), 46.7 / 42.5 (8, 1), 15.0 / 16.6 (2, 2), 31 / 27.6 (4, 2)
+//   128, 16: 22.5 / 24 (4, 1), 46 / 45.3 (8, 1), 14.3 / 16.1 (2, 2), 59 / 55 (8, 2)
+// so small lattices share unless they are few.
+bool mg_batch_own_launch(Ctx* c, int nb, int contexts) {
+  if (!mg_batch_grouped(c, nb)) return false;
+  const LevelGeom& G = c->mg->geo[1];
+  const long long sites = G.eo ? G.half : G.nsites, nc = c->mg->cop[1].nc;
+  return contexts <= 2 || (nb == 1 && contexts <= 4) || (sites >= 64 && sites * nc * nc >= 65536);
+}
+
 void mg_batch_systems(Ctx* c, int nb, std::vector<CoarseSystem>& out) {
   if (!mg_batch_joinable(c)) raise(MG_ERR_STATE, "only 2-level hierarchies join a shared coarsest solve");
   Hierarchy& H = *c->mg;

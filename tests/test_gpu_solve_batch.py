@@ -20,7 +20,8 @@ LATTICES = [((8, 8, 8, 8), (2, 2, 2, 2), 8, 0.3, -0.1, 8101),
 
 
 # sources per context, coarse_impl
-@pytest.mark.parametrize("nrhs,impl", [((3, 2, 2), 0)], ids=["grouped"])
+@pytest.mark.parametrize("nrhs,impl", [((3, 2, 2), 0), ((1, 1, 1), 0), ((3, 2, 2), 2)],
+                         ids=["shared_launch", "a_launch_each", "forced_shared"])
 def test_contexts_on_their_own_streams(nrhs, impl):
     lib_built()
     torch = pytest.importorskip("torch")
