@@ -790,20 +790,30 @@ int sm_count() {
 
 }  // namespace
 
-bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C) {
-  if (C.nc % 2 || !C.A.get()) return false;
-  const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
-  return p.rowsA >= 1 && p.rowsB >= 1 && p.smem <= 232448;
+// A stage holds a row of links, and the block fits with its static shared memory
+// (below 512 bytes).  A smaller grid has more sites to gather per block and a shorter
+// restart may place Krylov vectors in shared memory, so every (grid, m) is asked.
+static bool plan_ok(const Plan& p) {
+  int dev = 0, optin = 0;
+  MG_CUDA(cudaGetDevice(&dev));
+  MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  return p.rowsA >= 1 && p.rowsB >= 1 && p.grid >= 1 && p.smem + 512 <= (size_t)optin;
 }
 
-std::vector<int> coarse_gcr_stream_grids(const LevelGeom& G, const CoarseOp& C) {
+bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C, int m) {
+  if (C.nc % 2 || !C.A.get()) return false;
+  const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
+  return plan_ok(p) && plan_ok(make_plan(G, C, p.grid, m));
+}
+
+std::vector<int> coarse_gcr_stream_grids(const LevelGeom& G, const CoarseOp& C, int m) {
   const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
   std::vector<int> out = {p.grid};
   // the largest grid that splits both item lists evenly (no block waits at a
   // barrier for a neighbour with one more item)
   for (int g = p.grid - 1; g >= p.grid / 2 && g >= 1; g--)
     if (p.NA % g == 0 && p.NB % g == 0) {
-      out.push_back(g);
+      if (plan_ok(make_plan(G, C, g, m))) out.push_back(g);
       break;
     }
   return out;
@@ -813,8 +823,9 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
                              double tol_rel, const float* b, float* x, long long* d_iters, int* flags, cudaStream_t s,
                              int grid) {
   if (m > kMaxRestart) raise(MG_ERR_ARG, "coarse restart too long for the persistent solver");
-  if (!coarse_gcr_stream_ok(G, C)) raise(MG_ERR_STATE, "streamed coarse solve not applicable to this level");
+  if (!coarse_gcr_stream_ok(G, C, m)) raise(MG_ERR_STATE, "streamed coarse solve not applicable to this level");
   const Plan p = make_plan(G, C, grid, m);
+  if (!plan_ok(p)) raise(MG_ERR_STATE, "streamed coarse solve not applicable on this grid");
   const int sms = sm_count();
   int per = 0;
   const void* kern = kernel_for(C.store, G.eo, p);
