@@ -1556,18 +1556,34 @@ struct GSArgs {
   int L;                // nb * ndof / 2
 };
 
+// The orthonormal vectors do not depend on the vectors' scales, the float-pair
+// products do: below about 2^-50 their low halves underflow, above 2^60 the sums
+// of squares overflow.  A vector whose largest entry in a block lies outside
+// 2^-24 .. 2^24 is multiplied by a power of two there (exactly).
 __global__ void k_gs_gather(GSArgs g) {
+  __shared__ int s_max[64];   // [chirality][k], bits of the largest |Re|, |Im|
   const int cc = blockIdx.x;
   const int nv = g.a.nv, hd = g.a.ndof / 2, L = g.L;
   const size_t per = (size_t)2 * nv * L;
+  if (threadIdx.x < 2 * nv) s_max[threadIdx.x] = 0;
+  __syncthreads();
   for (size_t t = threadIdx.x; t < per; t += blockDim.x) {
-    const int ch = (int)(t / ((size_t)nv * L));
-    const int k = (int)((t / L) % nv);
+    const int ck = (int)(t / L), ch = ck / nv;
     const int l = (int)(t % L);
     const int i = l / hd, c = ch * hd + l % hd;
     const int idx = g.a.blockmap[cc * g.a.nb + i];
-    const cx<float> z = fget(g.a.fa, g.V + (size_t)k * g.vstride, idx, c);
+    const cx<float> z = fget(g.a.fa, g.V + (size_t)(ck % nv) * g.vstride, idx, c);
     g.Q[(size_t)cc * per + t] = make_float4(z.re, 0.f, z.im, 0.f);
+    const int m = max(__float_as_int(fabsf(z.re)), __float_as_int(fabsf(z.im)));
+    if (m > *(volatile int*)&s_max[ck]) atomicMax(&s_max[ck], m);
+  }
+  __syncthreads();
+  for (int ck = 0; ck < 2 * nv; ck++) {
+    const float m = __int_as_float(s_max[ck]);
+    if (!(m > 0.f && m <= 3.4e38f) || (m >= 0x1p-24f && m <= 0x1p24f)) continue;
+    const int e = ilogbf(m);
+    float4* q = g.Q + (size_t)cc * per + (size_t)ck * L;
+    for (int l = threadIdx.x; l < L; l += blockDim.x) q[l] = make_float4(ldexpf(q[l].x, -e), 0.f, ldexpf(q[l].z, -e), 0.f);
   }
 }
 
