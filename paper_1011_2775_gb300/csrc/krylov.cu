@@ -61,8 +61,8 @@ inline int sum_grid(size_t n) {   // blocks of the fused passes with sums
 }
 
 // device scalars of an iteration (doubles): <rh, v>; <t, t>, <t, s>, ||s||^2;
-// <rh, r>, <r, r>; alpha; omega
-enum { S_RV = 0, S_TT = 2, S_TS = 3, S_SS = 5, S_RHO = 6, S_RR = 8, S_AL = 10, S_OM = 12, S_COUNT = 14 };
+// <rh, r>, <r, r>; alpha; omega; 1 if <rh, v> broke down
+enum { S_RV = 0, S_TT = 2, S_TS = 3, S_SS = 5, S_RHO = 6, S_RR = 8, S_AL = 10, S_OM = 12, S_BROKE = 14, S_COUNT = 15 };
 
 // a complex coefficient and a running sum c z: FP64, or for FP32 vectors the
 // coefficient as float pairs and the sum in compensated FP32 (about 48 bits,
@@ -109,15 +109,13 @@ struct Sum<float> {
   __device__ cx<float> value() const { return mkc(rh + rl, ih + il); }
 };
 
-// |z|^2 <= 1e-60 rn^4, the breakdown test |z| <= 1e-30 rn^2 without a square root
-__device__ __forceinline__ bool tiny(double re, double im, double rn) {
-  return re * re + im * im <= 1e-60 * (rn * rn) * (rn * rn);
-}
-__device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double& re, double& im) {
-  const double d = 1.0 / (br * br + bi * bi);
-  re = (ar * br + ai * bi) * d;
-  im = (ai * br - ar * bi) * d;
-}
+// Scalars are products of two vectors and are taken relative to rn^2 (irn = 1 / rn)
+// before anything is squared: vectors of any scale that FP64 norms hold.
+struct Scaled {
+  double re, im;
+  __device__ Scaled(double r, double i, double irn) : re((r * irn) * irn), im((i * irn) * irn) {}
+  __device__ double abs2() const { return re * re + im * im; }
+};
 
 // p = r + beta p - (beta omega) v
 template <typename T>
@@ -134,16 +132,24 @@ __global__ void __launch_bounds__(kBS) k_bicg_p(cx<T>* __restrict__ p, const cx<
 // s = r - alpha v, alpha = rho / <rh, v> (0 on a breakdown, which the host sees too)
 template <typename T>
 __global__ void __launch_bounds__(kBS) k_bicg_s(cx<T>* __restrict__ sv, const cx<T>* __restrict__ r,
-                                                const cx<T>* __restrict__ v, double rho_re, double rho_im, double rn,
+                                                const cx<T>* __restrict__ v, double rho_re, double rho_im, double irn,
                                                 double* sc, size_t n) {
   __shared__ Coef<T> ma;
   if (threadIdx.x == 0) {
+    const Scaled rv(sc[S_RV], sc[S_RV + 1], irn), rho(rho_re, rho_im, irn);
+    const double a2 = rv.abs2();
+    const bool broke = a2 <= 1e-60;   // |<rh, v>| <= 1e-30 rn^2
     double re = 0.0, im = 0.0;
-    if (!tiny(sc[S_RV], sc[S_RV + 1], rn)) cdiv(rho_re, rho_im, sc[S_RV], sc[S_RV + 1], re, im);
+    if (!broke) {
+      const double d = 1.0 / a2;
+      re = (rho.re * rv.re + rho.im * rv.im) * d;
+      im = (rho.im * rv.re - rho.re * rv.im) * d;
+    }
     ma = Coef<T>::of(-re, -im);
     if (blockIdx.x == 0) {
       sc[S_AL] = re;
       sc[S_AL + 1] = im;
+      sc[S_BROKE] = broke ? 1.0 : 0.0;
     }
   }
   __syncthreads();
@@ -176,7 +182,7 @@ __global__ void __launch_bounds__(kBS) k_bicg_dots(const cx<T>* __restrict__ t, 
 template <typename T>
 __global__ void __launch_bounds__(kBS) k_bicg_xr(cx<T>* __restrict__ x, cx<T>* __restrict__ r,
                                                  const cx<T>* __restrict__ p, const cx<T>* __restrict__ sv,
-                                                 const cx<T>* __restrict__ t, const cx<T>* __restrict__ rh, double rn,
+                                                 const cx<T>* __restrict__ t, const cx<T>* __restrict__ rh, double irn,
                                                  double tol_abs, size_t n, double* partials, unsigned* counter,
                                                  double* sc) {
   __shared__ Coef<T> s_al, s_om, s_mom;
@@ -185,11 +191,12 @@ __global__ void __launch_bounds__(kBS) k_bicg_xr(cx<T>* __restrict__ x, cx<T>* _
     const bool half = sqrt(sc[S_SS]) <= tol_abs || sc[S_TT] == 0.0;
     double re = 0.0, im = 0.0;
     if (!half) {
-      const double d = 1.0 / sc[S_TT];
-      re = sc[S_TS] * d;
-      im = sc[S_TS + 1] * d;
+      const Scaled ts(sc[S_TS], sc[S_TS + 1], irn);
+      const double d = 1.0 / ((sc[S_TT] * irn) * irn);
+      re = ts.re * d;
+      im = ts.im * d;
     }
-    s_skip = tiny(sc[S_RV], sc[S_RV + 1], rn);
+    s_skip = sc[S_BROKE] != 0.0;
     s_al = Coef<T>::of(sc[S_AL], sc[S_AL + 1]);
     s_om = Coef<T>::of(re, im);
     s_mom = Coef<T>::of(-re, -im);
@@ -275,17 +282,16 @@ typename Krylov<T>::Result Krylov<T>::bicgstab(const Op& A, T* x, const T* b, bo
     fresh = false;
     A(v, p);
     blas_cdot<T>(rh, v, n, d + S_RV, c_->ws, s);
-    k_bicg_s<T><<<wide, kBS, 0, s>>>(cv(sv), cv(r), cv(v), rho_new.real(), rho_new.imag(), rn, d, n);
+    k_bicg_s<T><<<wide, kBS, 0, s>>>(cv(sv), cv(r), cv(v), rho_new.real(), rho_new.imag(), 1.0 / rn, d, n);
     MG_LAUNCH();
     A(t, sv);
     k_bicg_dots<T><<<grid, kBS, 0, s>>>(cv(t), cv(sv), n, part, cnt, d);
     MG_LAUNCH();
-    k_bicg_xr<T><<<grid, kBS, 0, s>>>(cv(x), cv(r), cv(p), cv(sv), cv(t), cv(rh), rn, tol_abs, n, part, cnt, d);
+    k_bicg_xr<T><<<grid, kBS, 0, s>>>(cv(x), cv(r), cv(p), cv(sv), cv(t), cv(rh), 1.0 / rn, tol_abs, n, part, cnt, d);
     MG_LAUNCH();
     c_->read_scalars(d, h, S_COUNT);
     if (!std::isfinite(h[S_RV]) || !std::isfinite(h[S_RV + 1])) raise(MG_ERR_NAN, "non-finite scalar in BiCGStab");
-    const double rv2 = h[S_RV] * h[S_RV] + h[S_RV + 1] * h[S_RV + 1];
-    if (rv2 <= 1e-60 * (rn * rn) * (rn * rn)) {   // the kernels' breakdown test
+    if (h[S_BROKE] != 0.0) {
       // breakdown: restart from the current residual, unless this step already
       // was the restart (<r, A r> = 0: no progress possible from here)
       if (restarted) break;
