@@ -18,6 +18,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdio>
+#include <algorithm>
 #include <type_traits>
 #include <vector>
 
@@ -152,26 +153,39 @@ __global__ void __launch_bounds__(kUnpack) k_unpack_spinor(Geom g, const T* __re
   for (int t = threadIdx.x; t < n; t += kUnpack) dst[t] = sm[(t / 12) * 13 + t % 12];
 }
 
+// vectors of one launch: the limit of gridDim.y
+constexpr int kMaxVectors = 65535;
+
 void pack_spinors(const Geom& g, int nrhs, const double* abi, void* even, void* odd, size_t stride, bool even_only,
                   bool fp32, cudaStream_t s) {
-  const dim3 grid((g.Vh + kPack - 1) / kPack, nrhs, even_only ? 1 : 2);
+  auto run = [&](auto* e, auto* o) {
+    for (int r0 = 0; r0 < nrhs; r0 += kMaxVectors) {
+      const dim3 grid((g.Vh + kPack - 1) / kPack, std::min(nrhs - r0, kMaxVectors), even_only ? 1 : 2);
+      k_pack_spinor<<<grid, kPack, 0, s>>>(g, (const double2*)abi + (size_t)r0 * 24 * g.Vh, e + r0 * stride, o + r0 * stride,
+                                           stride);
+      MG_LAUNCH();
+    }
+  };
   if (fp32)
-    k_pack_spinor<float><<<grid, kPack, 0, s>>>(g, (const double2*)abi, (float*)even, (float*)odd, stride);
+    run((float*)even, (float*)odd);
   else
-    k_pack_spinor<double><<<grid, kPack, 0, s>>>(g, (const double2*)abi, (double*)even, (double*)odd, stride);
-  MG_LAUNCH();
+    run((double*)even, (double*)odd);
 }
 
 void unpack_spinors(const Geom& g, int nrhs, const void* even, const void* odd, size_t stride, bool zero_odd, bool fp32,
                     double* abi, cudaStream_t s) {
-  const dim3 grid((2 * g.Vh + kUnpack - 1) / kUnpack, nrhs);
+  auto run = [&](auto* e, auto* o) {
+    for (int r0 = 0; r0 < nrhs; r0 += kMaxVectors) {
+      const dim3 grid((2 * g.Vh + kUnpack - 1) / kUnpack, std::min(nrhs - r0, kMaxVectors));
+      k_unpack_spinor<<<grid, kUnpack, 0, s>>>(g, e + r0 * stride, o + r0 * stride, (double2*)abi + (size_t)r0 * 24 * g.Vh,
+                                               stride, zero_odd);
+      MG_LAUNCH();
+    }
+  };
   if (fp32)
-    k_unpack_spinor<float><<<grid, kUnpack, 0, s>>>(g, (const float*)even, (const float*)odd, (double2*)abi, stride,
-                                                    zero_odd);
+    run((const float*)even, (const float*)odd);
   else
-    k_unpack_spinor<double><<<grid, kUnpack, 0, s>>>(g, (const double*)even, (const double*)odd, (double2*)abi, stride,
-                                                     zero_odd);
-  MG_LAUNCH();
+    run((const double*)even, (const double*)odd);
 }
 
 void pack_spinor(const Geom& g, const double* abi, void* even, void* odd, bool fp32, cudaStream_t s) {
