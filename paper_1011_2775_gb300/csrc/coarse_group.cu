@@ -394,6 +394,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
       s_tol2[p] = a.tol_rel[p] * a.tol_rel[p] * (b2.h + b2.l);
       s_rn[p] = tot[p * kSlots + QE];
       if (b2.h > 0.f) act |= 1u << p;
+      if (!(s_rn[p].h == s_rn[p].h)) {   // NaN or infinity in b: nothing to iterate on
+        act &= ~(1u << p);
+        atomicExch(&a.flags[FLAG_NAN], 1);
+      }
     }
     s_act = act;
   }
@@ -507,13 +511,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
         if (threadIdx.x < nb && ((run >> threadIdx.x) & 1u)) {
           const int p = threadIdx.x;
           const df* d = tot + (size_t)p * kSlots + (exact ? QE + 1 : QW + 1);
-          const df g = df_sqrt(exact ? tot[(size_t)p * kSlots + QE] : s_g2[p]);
+          const df g2 = exact ? tot[(size_t)p * kSlots + QE] : s_g2[p];
+          const df g = df_sqrt(g2);
           const bool gz = !(g.h > 0.f);
           const df ar = gz ? d[0] : df_div(d[0], g), ai = gz ? d[1] : df_div(d[1], g);
           s_ig[p] = gz ? 1.f : 1.f / g.h;
           s_ar[p] = ar.h + ar.l;
           s_ai[p] = ai.h + ai.l;
-          if (!gz) {   // ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2
+          if (!(g2.h == g2.h)) {   // NaN in w: the system ends with this step
+            s_rn[p] = g2;
+          } else if (!gz) {   // ||r - alpha w_k||^2 = ||r||^2 - |alpha|^2
             const df rn = df_add(s_rn[p], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
             s_rn[p] = rn.h > 0.f ? rn : df_of(rn.h == rn.h ? 0.f : rn.h);
           }
@@ -673,6 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_coarse_gcr_group(GArgs a) {
     if (threadIdx.x < nb && ((act >> threadIdx.x) & 1u)) {
       const int p = threadIdx.x;
       s_rn[p] = tot[(size_t)p * kSlots + QN];
+      if (!(s_rn[p].h == s_rn[p].h)) atomicExch(&a.flags[FLAG_NAN], 1);
       if (!(s_rn[p].h > s_tol2[p])) atomicAnd(&s_act, ~(1u << p));
     }
     __syncthreads();

@@ -493,8 +493,12 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
       if (mode == M_INIT) {
         const df tr = df_of((float)a.tol_rel);
         tol2 = df_mul(df_mul(tr, tr), tot[RD]);
-        if (!(tot[RD].h > 0.f)) break;
-      } else if (tot[RC].h <= tol2.h || !(tot[RC].h == tot[RC].h)) {
+        if (!(tot[RD].h > 0.f) && tot[RC].h == tot[RC].h) break;
+      } else if (tot[RC].h <= tol2.h) {
+        break;
+      }
+      if (!(tot[RC].h == tot[RC].h)) {
+        if (bid == 0 && threadIdx.x == 0) atomicExch(&a.flags[FLAG_NAN], 1);
         break;
       }
       if (its >= a.maxit) break;
@@ -552,9 +556,11 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
       const df ai = gz ? wi : df_div(wi, g);
       s_coef[1] = ar.h + ar.l;
       s_coef[2] = ai.h + ai.l;
-      if (!gz) {
+      if (!(g2.h == g2.h)) {   // NaN in w: the running norm carries it to the test below
+        tot[RC] = g2;
+      } else if (!gz) {
         const df rn = df_add(tot[RC], df_neg(df_add(df_mul(ar, ar), df_mul(ai, ai))));
-        tot[RC] = rn.h > 0.f ? rn : df_of(0.f);
+        tot[RC] = rn.h > 0.f || !(rn.h == rn.h) ? rn : df_of(0.f);
       }
     };
     if (wid == 0) {

@@ -1052,6 +1052,8 @@ void mg_benchmark_coarse_solve(Ctx* c, int warmup, int iters, double* avg_ms, do
 void mg_reset_counters(Ctx* c) {
   if (!c->mg) return;
   c->mg->iters.assign(c->mg->L, 0);
+  // a NaN that an earlier call's cycle met (mg_apply) is not this solve's
+  MG_CUDA(cudaMemsetAsync(c->ws.flags.as<int>() + FLAG_NAN, 0, sizeof(int), c->stream));
   MG_CUDA(cudaMemsetAsync(c->mg->d_iters.get(), 0, sizeof(long long) * MG_MAX_LEVELS, c->stream));
 }
 
