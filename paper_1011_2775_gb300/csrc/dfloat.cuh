@@ -8,6 +8,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace mg {
 
 struct df {
@@ -116,8 +118,9 @@ __device__ __forceinline__ S warp_transpose_sum(S (&v)[V]) {
 // warps of a block added in order, block sums in partials[r][block], and the
 // last block to finish adds them, one warp per value.  FP64 additions are the
 // scarce resource here (1/62 of the FP32 rate): with a whole butterfly per
-// value the tree took longer than the memory pass it closes.  THREADS = block
-// size; the counter is 0 at launch and left at 0.
+// value the tree took longer than the memory pass it closes.  A block whose
+// float-pair sum leaves FP32's range adds its threads' sums again in FP64.
+// THREADS = block size; the counter is 0 at launch and left at 0.
 __device__ __forceinline__ double sum_to_double(double v) { return v; }
 __device__ __forceinline__ double sum_to_double(df v) { return (double)v.h + (double)v.l; }
 __device__ __forceinline__ double sum_of(double v) { return v; }
@@ -129,9 +132,10 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, uns
   constexpr int W = THREADS / 32;
   constexpr int V = NR <= 1 ? 1 : NR <= 2 ? 2 : NR <= 4 ? 4 : NR <= 8 ? 8 : 16;
   static_assert(NR <= 16, "at most 16 values");
-  __shared__ S sm[NR][W];
+  __shared__ __align__(8) S sm[NR][W];
   __shared__ bool is_last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  bool over = false;
   S t[V];
 #pragma unroll
   for (int r = 0; r < V; r++) t[r] = r < NR ? sum_of(v[r < NR ? r : 0]) : sum_of(T{});
@@ -153,8 +157,28 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, uns
 #pragma unroll
     for (int w = 1; w < W; w++) s = add_x(s, sm[threadIdx.x][w]);
     partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = sum_to_double(s);
+    if constexpr (!std::is_same<T, double>::value) over = !(fabsf(s.h) <= 3.402823466e38f);
   }
-  __syncthreads();
+  if constexpr (std::is_same<T, double>::value) {
+    __syncthreads();
+  } else if (__syncthreads_or(over)) {
+    // finite sums of threads beyond FP32's range in the block: again in FP64
+    double* sd = reinterpret_cast<double*>(&sm[0][0]);
+#pragma unroll
+    for (int r = 0; r < NR; r++) {
+      double d = sum_to_double(sum_of(v[r]));
+#pragma unroll
+      for (int o = 16; o >= 1; o /= 2) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if (lane == 0) sd[r * W + wid] = d;
+    }
+    __syncthreads();
+    if (threadIdx.x < NR) {
+      double d = 0.0;
+      for (int w = 0; w < W; w++) d += sd[threadIdx.x * W + w];
+      partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = d;
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
     __threadfence();   // the block's partials before its ticket
     is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
