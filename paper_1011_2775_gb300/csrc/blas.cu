@@ -161,27 +161,28 @@ __global__ void k_dot2(const cx<T>* __restrict__ w, const cx<T>* __restrict__ r,
 }
 // nrhs pairs (w_q, r_q) of FP32 vectors at `stride` floats apart: d_out[4q ..
 // 4q+2] per pair, one launch (blockIdx.y = q, a separate reduction per pair);
-// 16 bytes per load, a sum for the first and one for the second of a pair of
-// complex numbers (n is even)
+// 16 bytes per load (n is even).  With many pairs a thread has many elements, so
+// its running sums are float pairs: the FP32 part of a sum is the two products of
+// one complex number.
 __global__ void __launch_bounds__(kBS) k_dot2_multi(const float* __restrict__ w, const float* __restrict__ r, size_t n2,
                                                     size_t stride, double* partials, unsigned* counters, double* out) {
   const int q = blockIdx.y;
   const float4* w4 = reinterpret_cast<const float4*>(w + q * stride);
   const float4* r4 = reinterpret_cast<const float4*>(r + q * stride);
-  float s[2][3] = {};
+  float h[3] = {}, l[3] = {};
 #pragma unroll 4
   for (size_t i = blockIdx.x * (size_t)kBS + threadIdx.x; i < n2; i += (size_t)gridDim.x * kBS) {
     const float4 a = w4[i], b = r4[i];
-    s[0][0] = fmaf(a.x, a.x, fmaf(a.y, a.y, s[0][0]));
-    s[0][1] = fmaf(a.x, b.x, fmaf(a.y, b.y, s[0][1]));
-    s[0][2] = fmaf(a.x, b.y, fmaf(-a.y, b.x, s[0][2]));
-    s[1][0] = fmaf(a.z, a.z, fmaf(a.w, a.w, s[1][0]));
-    s[1][1] = fmaf(a.z, b.z, fmaf(a.w, b.w, s[1][1]));
-    s[1][2] = fmaf(a.z, b.w, fmaf(-a.w, b.z, s[1][2]));
+    df_acc(h[0], l[0], fmaf(a.x, a.x, a.y * a.y));
+    df_acc(h[1], l[1], fmaf(a.x, b.x, a.y * b.y));
+    df_acc(h[2], l[2], fmaf(a.x, b.y, -a.y * b.x));
+    df_acc(h[0], l[0], fmaf(a.z, a.z, a.w * a.w));
+    df_acc(h[1], l[1], fmaf(a.z, b.z, a.w * b.w));
+    df_acc(h[2], l[2], fmaf(a.z, b.w, -a.w * b.z));
   }
   df v[3];
 #pragma unroll
-  for (int k = 0; k < 3; k++) v[k] = df_add(df_of(s[0][k]), df_of(s[1][k]));
+  for (int k = 0; k < 3; k++) v[k] = df_norm(h[k], l[k]);
   grid_reduce<3>(v, partials + (size_t)q * gridDim.x * 3, counters + q, out + 4 * q);
 }
 template <typename T>
