@@ -18,6 +18,10 @@
  *   bound to one CUDA device and one stream, is single-stream and is not
  *   thread-safe.  Calls return after the stream has drained (the results are
  *   visible to the caller on any stream).
+ * - A context keeps solver workspaces and, up to 8 GiB in all, the buffers of
+ *   mg_apply, mg_force and mg_solve_dagger between calls.  Those 8 GiB are given
+ *   back when an allocation of a call on the context does not fit, and with
+ *   everything else by mg_destroy.
  * - Caller buffers are plain pointers.  `where` says whether they are host
  *   (MG_HOST) or device (MG_DEVICE) memory; the library never keeps them.
  * - Lattice dims are {Lx, Ly, Lz, Lt}; all four must be even (even-odd
@@ -289,7 +293,10 @@ MG_API int mg_get_null_vectors(void* ctx, int level, void* V, int nv, int where)
  *                   NULL) as mg_setup, setup_ms being the whole call.
  *   mg_update_mass: sets a new bare mass (same csw) and rebuilds the
  *                   hierarchy from the current null vectors -- setup reuse
- *                   across masses.
+ *                   across masses.  As after mg_set_null_vectors, the vectors
+ *                   stay with the context (in device memory) for later setups
+ *                   until the setup parameters change, others are set or the
+ *                   context is destroyed; mg_adapt_setup does the same.
  * Errors: MG_ERR_ARG (unreadable or foreign file), MG_ERR_DIMS (another
  * lattice), MG_ERR_STATE (no setup / no clover), MG_ERR_GS_BREAKDOWN,
  * MG_ERR_SINGULAR_CLOVER, MG_ERR_CUDA. */
@@ -410,8 +417,9 @@ MG_API int mg_apply(void* ctx, int op, int level, void* out, const void* in, int
  * device memory is owned by another allocator (a framework's caching
  * allocator or a fixed pool) and latency-critical loops that cannot afford
  * the implicit device synchronisation of cudaMalloc/cudaFree.  mg_apply
- * allocates staging buffers and temporaries on every call; this entry point
- * allocates nothing.
+ * allocates its buffers on the first call, on one of more vectors and on calls
+ * that need more than a context keeps, and staging buffers for host memory on
+ * every call; this entry point allocates nothing.
  *
  * Applies op (MG_OP_D, MG_OP_DP, MG_OP_DR, MG_OP_BR, MG_OP_M, MG_OP_MINV or
  * MG_OP_HOP) of the fine level to ONE vector: `in` and `out` are DEVICE

@@ -20,6 +20,7 @@ thread_local std::string g_last_error;
 
 template <typename F>
 int guarded(F&& f) {
+  mg::CallScope scope;
   try {
     g_last_error.clear();
     return f();
@@ -39,6 +40,7 @@ mg::Ctx* as_ctx(void* p) {
   if (!p) mg::raise(MG_ERR_ARG, "null context");
   mg::Ctx* c = static_cast<mg::Ctx*>(p);
   MG_CUDA(cudaSetDevice(c->device));
+  mg::call_uses(c);
   return c;
 }
 
@@ -86,15 +88,14 @@ void stage_out_finish(mg::Ctx* c, Staged& st, void* user, size_t bytes, int wher
 
 // mg_apply's fine-level buffers, kept with the context between calls: at
 // 6x4x8x10 the ten cudaMalloc and cudaFree calls of one application took 100 of
-// its 153 us.  Buffers above kApplyKeep bytes are given back after the call.
-constexpr size_t kApplyKeep = (size_t)8 << 30;
-struct ApplyWork {
+// its 153 us.
+struct ApplyWork : mg::KeptWork {
   mg::DBuf in, out, tmp;
   std::unique_ptr<mg::FineOps<double>> F64;
   std::unique_ptr<mg::FineOps<float>> F32;
   template <typename T>
   mg::FineOps<T>& ops(mg::Ctx* c);
-  size_t bytes() const {
+  size_t bytes() const override {
     size_t n = in.bytes() + out.bytes() + tmp.bytes();
     if (F64) n += F64->bytes();
     if (F32) n += F32->bytes();
@@ -119,6 +120,12 @@ void check_where(int where) {
   if (where != MG_HOST && where != MG_DEVICE) mg::raise(MG_ERR_ARG, "where must be MG_HOST or MG_DEVICE");
 }
 
+// gamma_5-rotated copy of a device source
+struct AdjointWork : mg::KeptWork {
+  mg::DBuf src;
+  size_t bytes() const override { return src.bytes(); }
+};
+
 // mg_solve / mg_solve_dagger.  The dagger form solves D^dag psi = eta as
 // psi = gamma_5 D^{-1} gamma_5 eta (D^dag = gamma_5 D gamma_5).
 int solve_impl(void* ctx, void* psi, const void* eta, int nrhs, double tol, int mode, int where,
@@ -139,10 +146,12 @@ int solve_impl(void* ctx, void* psi, const void* eta, int nrhs, double tol, int 
   const long long kernels0 = mg::launches_so_far();
   const size_t per = sizeof(double) * 24 * c->V;
   Staged si, so;
+  std::unique_ptr<AdjointWork> adj;
   if (dagger && where == MG_DEVICE) {
     // gamma_5 must not touch the caller's source: work on a copy
-    if (c->dagger_src.bytes() < per * nrhs) c->dagger_src.alloc(per * nrhs);
-    si.ptr = c->dagger_src.as<double>();
+    adj = c->take<AdjointWork>(mg::KEEP_ADJOINT);
+    grow(adj->src, per * nrhs);
+    si.ptr = adj->src.as<double>();
     MG_CUDA(cudaMemcpyAsync(si.ptr, eta, per * nrhs, cudaMemcpyDeviceToDevice, c->stream));
   } else {
     stage_in(c, si, eta, per * nrhs, where);
@@ -160,6 +169,7 @@ int solve_impl(void* ctx, void* psi, const void* eta, int nrhs, double tol, int 
   }
   if (dagger) mg::gamma5_abi(so.ptr, c->V * nrhs, c->stream);
   stage_out_finish(c, so, psi, per * nrhs, where);
+  if (adj) c->leave(mg::KEEP_ADJOINT, std::move(adj));
   mg::mg_read_counters(c, local.coarse_iterations);
   mg::level_times(c, local.level_ms);
   local.dslash_launches = c->dslash_launches - launches0;
@@ -749,8 +759,8 @@ int mg_apply(void* ctx, int op, int level, void* out, const void* in, int nrhs, 
       const bool f32 = prec == MG_FP32;
       const size_t es = f32 ? sizeof(float) : sizeof(double);
       const size_t half = 24 * c->Vh;  // reals per half vector
-      if (!c->apply_work) c->apply_work = std::make_shared<ApplyWork>();
-      ApplyWork& aw = *static_cast<ApplyWork*>(c->apply_work.get());
+      std::unique_ptr<ApplyWork> work = c->take<ApplyWork>(mg::KEEP_APPLY);
+      ApplyWork& aw = *work;
       grow(aw.in, es * 2 * half * nrhs);
       grow(aw.out, es * 2 * half * nrhs);
       char* ie = aw.in.as<char>();
@@ -798,10 +808,7 @@ int mg_apply(void* ctx, int op, int level, void* out, const void* in, int nrhs, 
       else
         run((double*)nullptr);
       mg::unpack_spinors(c->g, nrhs, oe, oo, half, writes_even, f32, so.ptr, c->stream);
-      if (aw.bytes() > kApplyKeep) {
-        c->sync();
-        c->apply_work.reset();
-      }
+      c->leave(mg::KEEP_APPLY, std::move(work));
     }
     stage_out_finish(c, so, out, sizeof(double) * 2 * nout * nrhs, where);
     return MG_OK;

@@ -414,12 +414,19 @@ void gamma5_abi(double* v, size_t sites, cudaStream_t s) {
   MG_LAUNCH();
 }
 
+// packed vectors, insertions, plaquette contributions: kept between calls
+struct ForceWork : KeptWork {
+  DBuf vec, W, R;
+  size_t bytes() const override { return vec.bytes() + W.bytes() + R.bytes(); }
+};
+
 template <typename T>
 void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double* psi_abi, int kind) {
   const Geom& g = c->g;
   const size_t half = 24 * c->Vh;   // reals per half vector
-  DBuf& vec = c->force_vec;
-  DBuf& W = c->force_W;
+  std::unique_ptr<ForceWork> work = c->take<ForceWork>(KEEP_FORCE);
+  DBuf& vec = work->vec;
+  DBuf& W = work->W;
   if (vec.bytes() < sizeof(T) * 4 * half) vec.alloc(sizeof(T) * 4 * half);
   if (W.bytes() < sizeof(T) * 2 * 6 * 9 * c->V) W.alloc(sizeof(T) * 2 * 6 * 9 * c->V);
   T* lam_e = vec.as<T>();
@@ -437,7 +444,7 @@ void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double*
   // all planes in one pass, or one by one where their contributions would take more than 4 GiB
   const size_t per_plane = sizeof(V2) * 72 * (size_t)c->Vh;
   const int np = per_plane * 6 <= ((size_t)4 << 30) ? 6 : 1;
-  DBuf& R = c->force_R;
+  DBuf& R = work->R;
   if (R.bytes() < per_plane * np) R.alloc(per_plane * np);
   for (int p0 = 0; p0 < 6; p0 += np) {
     k_force_plaquettes<T><<<dim3(nb, np), bs, 0, c->stream>>>(g, c->gauge<T>(), W.as<V2>(), p0, R.as<V2>());
@@ -446,6 +453,7 @@ void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double*
                                                         p0 == 0, p0 + np == 6, kind, (double2*)out_abi);
     MG_LAUNCH();
   }   // the caller waits for the stream
+  c->leave(KEEP_FORCE, std::move(work));
 }
 
 void gauge_force(Ctx* c, double* out_abi, const double* lam_abi, const double* psi_abi, int kind) {

@@ -88,6 +88,29 @@ class DBuf {
   size_t bytes_ = 0;
 };
 
+// Contexts that the entry point running on this thread works with.  When one of
+// its allocations fails, what these contexts keep between calls is given back
+// and the allocation is tried once more.
+struct CallScope {
+  CallScope();
+  ~CallScope();
+  CallScope(const CallScope&) = delete;
+  CallScope& operator=(const CallScope&) = delete;
+  size_t mark;
+};
+void call_uses(Ctx* c);
+
+// Device buffers that an entry point leaves with its context for the next call
+// (Ctx::take, Ctx::leave)
+struct KeptWork {
+  virtual ~KeptWork() {}
+  virtual size_t bytes() const = 0;
+};
+enum { KEEP_APPLY, KEEP_FORCE, KEEP_ADJOINT, KEEP_COUNT };
+// All that a context keeps this way: 3 % of the device.  The operators on twelve
+// FP32 vectors of 32^3x64 take 7.3 GB of it.
+constexpr size_t kKeepBytes = (size_t)8 << 30;
+
 // --------------------------------------------------------------------------- workspace
 // Reduction scratch, device scalars and error flags shared by all kernels of
 // one context.  Reductions are deterministic: fixed grid, per-block FP64
@@ -266,9 +289,18 @@ struct Ctx {
   std::vector<std::vector<double>> injected;
   std::vector<std::shared_ptr<DBuf>> injected_dev;
 
-  DBuf dagger_src;                       // gamma_5-rotated copy of a device source (adjoint solves)
-  DBuf force_vec, force_W, force_R;      // mg_force: packed vectors, insertions, plaquette contributions
-  std::shared_ptr<void> apply_work;      // mg_apply's buffers (api.cu), kept between calls
+  // kept between calls: mg_apply's buffers, mg_force's, the rotated source of adjoint
+  // solves.  A call takes its own and leaves them when it has succeeded.
+  std::unique_ptr<KeptWork> kept[KEEP_COUNT];
+  template <typename W>
+  std::unique_ptr<W> take(int slot) {
+    std::unique_ptr<W> w(static_cast<W*>(kept[slot].release()));
+    if (!w) w.reset(new W());
+    return w;
+  }
+  void leave(int slot, std::unique_ptr<KeptWork> w);   // frees it, or the others, beyond kKeepBytes
+  DBuf* spare = nullptr;                 // scratch of a running setup that is not needed at the moment
+  bool give_back();                      // frees all that is kept; false: there was nothing
   long long dslash_launches = 0;
   // mg_params.level_timing: CUDA event pairs around each level's work, per level
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> level_events[MG_MAX_LEVELS];

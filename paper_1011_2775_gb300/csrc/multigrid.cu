@@ -652,7 +652,15 @@ void mg_build(Ctx* c, mg_setup_info* info) {
     for (int k = 0; k < T.nv; k++) V[k] = H->nullvecs[l]->as<float>() + (size_t)k * 2 * full_n(*H, l);
     block_orthonormalize(T, V.data(), H->gs_scratch, c->ws.flags.as<int>(), c->stream);
     if (c->read_flag(FLAG_GS_BREAKDOWN, true)) raise(MG_ERR_GS_BREAKDOWN, "block Gram-Schmidt breakdown");
-    build_coarse_links(c, *H, l);
+    {
+      // the Gram-Schmidt scratch gives way if the projection's buffers do not fit beside it
+      struct Spare {
+        Ctx* c;
+        ~Spare() { c->spare = nullptr; }
+      } lent{c};
+      c->spare = &H->gs_scratch;
+      build_coarse_links(c, *H, l);
+    }
     if (info) info->coarse_sites[l] = Gc.nsites;
   }
   H->gs_scratch.release();

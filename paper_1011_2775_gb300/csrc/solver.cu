@@ -41,10 +41,51 @@ long long launches_so_far() { return g_launches.load(std::memory_order_relaxed);
 
 void add_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+namespace {
+thread_local std::vector<Ctx*> t_call;   // contexts of the entry point running on this thread
+}
+CallScope::CallScope() : mark(t_call.size()) {}
+CallScope::~CallScope() { t_call.resize(mark); }
+void call_uses(Ctx* c) { t_call.push_back(c); }
+
+bool Ctx::give_back() {
+  bool any = spare && spare->get();
+  for (auto& k : kept) any |= k != nullptr;
+  if (!any) return false;
+  sync();
+  if (spare) spare->release();
+  for (auto& k : kept) k.reset();
+  return true;
+}
+
+void Ctx::leave(int slot, std::unique_ptr<KeptWork> w) {
+  size_t others = 0;
+  for (int k = 0; k < KEEP_COUNT; k++)
+    if (k != slot && kept[k]) others += kept[k]->bytes();
+  if (w->bytes() > kKeepBytes) {
+    sync();
+    return;
+  }
+  if (others + w->bytes() > kKeepBytes) {
+    sync();
+    for (auto& k : kept) k.reset();
+  }
+  kept[slot] = std::move(w);
+}
+
 void DBuf::alloc(size_t bytes) {
   release();
   if (bytes == 0) return;
-  MG_CUDA(cudaMalloc(&p_, bytes));
+  cudaError_t e = cudaMalloc(&p_, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();   // reported here, not by the next launch
+    bool any = false;
+    for (Ctx* c : t_call) any |= c->give_back();
+    if (any) e = cudaMalloc(&p_, bytes);
+    if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+  }
+  if (e != cudaSuccess) p_ = nullptr;
+  MG_CUDA(e);
   bytes_ = bytes;
 }
 
