@@ -23,12 +23,12 @@
 // every site ([parity][plane][9][Vh]); k_force_plaquettes the four links'
 // contributions R of every plaquette; k_force_links adds the hopping part and
 // the six plaquettes of every link and writes K (or the force) in the ABI
-// gauge layout (complex128).  The FP64 work is bound by the FP64 pipes: taken
+// gauge layout (complex128), at once or in passes by plane and parity.  The FP64 work is bound by the FP64 pipes: taken
 // plaquette by plaquette the four links share their partial products, 22 3x3
 // products instead of the 32 of a link-by-link evaluation (5.17 ms for 16^3x32
 // at 91 % of the FP64 rate; 3.15 ms now, k_force_links 0.60), for 3456 bytes per
 // site of contributions written and read once.
-// Both run in FP64 or, on request, in FP32 (FP32 gauge copy, vectors and W,
+// All run in FP64 or, on request, in FP32 (FP32 gauge copy, vectors and W,
 // FP32 arithmetic; the result is widened to complex128 on output).  With the
 // anisotropic reading every hop carries its direction's weight w_mu and the
 // planes containing t their own clover coefficient csw_t.
@@ -125,6 +125,10 @@ __device__ __forceinline__ void gamma_dyn(int mu, const cx<T> in[12], cx<T> out[
 }
 
 __device__ __forceinline__ int plane_of(int a, int b) { return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5); }
+__device__ __forceinline__ void plane_dirs(int p, int& a, int& b) {
+  a = p < 3 ? 0 : (p < 5 ? 1 : 2);
+  b = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+}
 
 __device__ __forceinline__ void step(const Geom& g, int c[4], int mu, int d) {
   c[mu] += d;
@@ -196,7 +200,8 @@ __global__ void __launch_bounds__(128) k_force_insertion(Geom g, const T* lam_e,
 }
 
 // Contributions of every plaquette to the derivatives of its four links, planes
-// p0 + blockIdx.y, thread = (base corner, plane); R[plane - p0][parity][j][9][Vh].
+// p0 + blockIdx.y, base corners of parity par0 + blockIdx.z, thread = (base corner,
+// plane); R[plane - p0][parity - par0][j][9][Vh].
 //   L0 = U_al(b), L1 = U_be(b + al), L2 = U_al(b + be)^dag, L3 = U_be(b)^dag, W_k at the corner where L_k begins:
 //   R_j = W_{j+1} L_{j+1} L_{j+2} L_{j+3} + L_{j+1} W_{j+2} L_{j+2} L_{j+3} + L_{j+1} L_{j+2} W_{j+3} L_{j+3}
 //       + L_{j+1} L_{j+2} L_{j+3} W_j,
@@ -204,13 +209,14 @@ __global__ void __launch_bounds__(128) k_force_insertion(Geom g, const T* lam_e,
 template <typename T>
 __global__ void __launch_bounds__(128) k_force_plaquettes(Geom g, const T* __restrict__ gauge,
                                                           const typename V2of<T>::type* __restrict__ W, int p0,
-                                                          typename V2of<T>::type* __restrict__ R) {
+                                                          int par0, typename V2of<T>::type* __restrict__ R) {
   typedef cx<T> cd;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= 2 * g.Vh) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.Vh) return;
   const int p = p0 + blockIdx.y;
-  const int al = p < 3 ? 0 : (p < 5 ? 1 : 2), be = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
-  const int par = t >= g.Vh, i = t - par * g.Vh;
+  int al, be;
+  plane_dirs(p, al, be);
+  const int par = par0 + blockIdx.z;
   int c0[4], c1[4], c2[4], c3[4];
   cb_coords(g, i, par, c0);
 #pragma unroll
@@ -220,7 +226,7 @@ __global__ void __launch_bounds__(128) k_force_plaquettes(Geom g, const T* __res
 #pragma unroll
   for (int m = 0; m < 4; m++) c2[m] = c1[m];
   step(g, c2, be, +1);
-  typename V2of<T>::type* out = R + (size_t)(blockIdx.y * 2 + par) * 36 * g.Vh + i;
+  typename V2of<T>::type* out = R + (size_t)(blockIdx.y * gridDim.z + blockIdx.z) * 36 * g.Vh + i;
   auto store = [&](int j, const cd m[9]) {
 #pragma unroll
     for (int e = 0; e < 9; e++) out[(size_t)(9 * j + e) * g.Vh] = mk2<T>(m[e].re, m[e].im);
@@ -280,19 +286,25 @@ __global__ void __launch_bounds__(128) k_force_plaquettes(Geom g, const T* __res
   store(2, S);
 }
 
-// K_mu(x) (or the force) of every link; thread = (site, mu = blockIdx.y).  The
-// plaquettes of the planes p0 .. p0 + np - 1 are added; `first` starts from the
-// hopping part, otherwise K so far is read back from `out`; `last` writes the
-// result in the requested form, otherwise K.
-template <typename T>
+// K_mu(x) (or the force) of links; thread = (site, mu): all four directions, or the
+// two of plane `p0` when it is a pass over plaquettes of one plane and base parity.
+// FORCE_ALL: hopping part, the plaquettes of all planes and parities, result.
+// In passes: FORCE_HOP writes the hopping part to `out`, FORCE_ADD adds the
+// plaquettes of plane p0 whose base has parity par0 to it, FORCE_FORM gives it the
+// requested form.
+enum ForcePass { FORCE_ALL, FORCE_HOP, FORCE_ADD, FORCE_FORM };
+template <typename T, int PASS>
 __global__ void __launch_bounds__(128) k_force_links(Geom g, const T* lam_e, const T* lam_o, const T* psi_e,
                                                      const T* psi_o, const T* gauge,
-                                                     const typename V2of<T>::type* R, int p0, int np, int first,
-                                                     int last, int kind, double2* out) {
+                                                     const typename V2of<T>::type* R, int p0, int par0, int kind,
+                                                     double2* out) {
+  constexpr bool first = PASS == FORCE_ALL || PASS == FORCE_HOP, last = PASS == FORCE_ALL || PASS == FORCE_FORM;
   typedef cx<T> cd;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * g.Vh) return;
-  const int mu = blockIdx.y;
+  int al, be;
+  plane_dirs(p0, al, be);
+  const int mu = PASS == FORCE_ADD ? (blockIdx.y ? be : al) : blockIdx.y;
   const int par = t >= g.Vh;
   const int i = t - par * g.Vh;
   int x[4];
@@ -348,21 +360,30 @@ __global__ void __launch_bounds__(128) k_force_links(Geom g, const T* lam_e, con
       }
   }
 
-  // ---- clover part: two plaquettes per plane containing mu
-  for (int nu = 0; nu < 4; nu++) {
-    if (nu == mu) continue;
-    const int p = plane_of(mu < nu ? mu : nu, mu < nu ? nu : mu);
-    if (p < p0 || p >= p0 + np) continue;
-    // U_mu(x) is L0 of the plaquette at x and L2 of the one at x - nu (mu < nu), or L3 and L1
-    const typename V2of<T>::type* Rp = R + (size_t)(p - p0) * 72 * g.Vh;
-    const typename V2of<T>::type* r0 = Rp + (size_t)par * 36 * g.Vh + (size_t)(mu < nu ? 0 : 27) * g.Vh + i;
-    int y[4] = {x[0], x[1], x[2], x[3]};
-    step(g, y, nu, -1);
-    const typename V2of<T>::type* r1 = Rp + (size_t)(1 - par) * 36 * g.Vh + (size_t)(mu < nu ? 18 : 9) * g.Vh + cb_index(g, y);
+  // ---- clover part: U_mu(x) is L0 of the plaquette at x and L2 of the one at x - nu (mu < nu), or L3 and L1
+  auto add = [&](const typename V2of<T>::type* r) {
 #pragma unroll
     for (int e = 0; e < 9; e++) {
-      const typename V2of<T>::type u = r0[(size_t)e * g.Vh], v = r1[(size_t)e * g.Vh];
-      K[e] = K[e] + mkc(u.x, u.y) + mkc(v.x, v.y);
+      const typename V2of<T>::type u = r[(size_t)e * g.Vh];
+      K[e] = K[e] + mkc(u.x, u.y);
+    }
+  };
+  if (PASS == FORCE_ALL) {
+    for (int nu = 0; nu < 4; nu++) {
+      if (nu == mu) continue;
+      const typename V2of<T>::type* Rp = R + (size_t)plane_of(mu < nu ? mu : nu, mu < nu ? nu : mu) * 72 * g.Vh;
+      int y[4] = {x[0], x[1], x[2], x[3]};
+      step(g, y, nu, -1);
+      add(Rp + (size_t)par * 36 * g.Vh + (size_t)(mu < nu ? 0 : 27) * g.Vh + i);
+      add(Rp + (size_t)(1 - par) * 36 * g.Vh + (size_t)(mu < nu ? 18 : 9) * g.Vh + cb_index(g, y));
+    }
+  } else if (PASS == FORCE_ADD) {   // the plaquette at x, or the one at x - nu, whose parity is the other
+    if (par == par0) {
+      add(R + (size_t)(mu == al ? 0 : 27) * g.Vh + i);
+    } else {
+      int y[4] = {x[0], x[1], x[2], x[3]};
+      step(g, y, mu == al ? be : al, -1);
+      add(R + (size_t)(mu == al ? 18 : 9) * g.Vh + cb_index(g, y));
     }
   }
 
@@ -420,6 +441,12 @@ struct ForceWork : KeptWork {
   size_t bytes() const override { return vec.bytes() + W.bytes() + R.bytes(); }
 };
 
+// The contributions of all plaquettes in one pass up to this many bytes (1.24 M sites
+// in FP64) and where they can be allocated.  The passes by plane and parity need no
+// memory beyond the vectors and insertions and cost 2 %: 32^3x64 FP64 68.3 ms, 67.2
+// plane by plane with 1.2 GB for a plane's contributions.
+constexpr size_t kForceR = (size_t)4 << 30;
+
 template <typename T>
 void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double* psi_abi, int kind) {
   const Geom& g = c->g;
@@ -441,17 +468,39 @@ void gauge_force_t(Ctx* c, double* out_abi, const double* lam_abi, const double*
   typedef typename V2of<T>::type V2;
   k_force_insertion<T><<<nb, bs, 0, c->stream>>>(g, lam_e, lam_o, psi_e, psi_o, (T)c->csw, (T)c->csw_t, W.as<V2>());
   MG_LAUNCH();
-  // all planes in one pass, or one by one where their contributions would take more than 4 GiB
-  const size_t per_plane = sizeof(V2) * 72 * (size_t)c->Vh;
-  const int np = per_plane * 6 <= ((size_t)4 << 30) ? 6 : 1;
+  const T* U = c->gauge<T>();
+  auto links = [&](auto pass, int nmu, const V2* r, int p, int par) {
+    k_force_links<T, decltype(pass)::value><<<dim3(nb, nmu), bs, 0, c->stream>>>(g, lam_e, lam_o, psi_e, psi_o, U, r, p, par,
+                                                                                 kind, (double2*)out_abi);
+    MG_LAUNCH();
+  };
+  const int nh = (int)((c->Vh + bs - 1) / bs);
+  const size_t need = sizeof(V2) * 72 * 6 * c->Vh;
   DBuf& R = work->R;
-  if (R.bytes() < per_plane * np) R.alloc(per_plane * np);
-  for (int p0 = 0; p0 < 6; p0 += np) {
-    k_force_plaquettes<T><<<dim3(nb, np), bs, 0, c->stream>>>(g, c->gauge<T>(), W.as<V2>(), p0, R.as<V2>());
+  bool whole = need <= kForceR;
+  if (whole && R.bytes() < need) {
+    try {
+      R.alloc(need);
+    } catch (const Error& e) {
+      if (e.code != MG_ERR_ALLOC) throw;
+      whole = false;
+    }
+  }
+  if (whole) {
+    k_force_plaquettes<T><<<dim3(nh, 6, 2), bs, 0, c->stream>>>(g, U, W.as<V2>(), 0, 0, R.as<V2>());
     MG_LAUNCH();
-    k_force_links<T><<<dim3(nb, 4), bs, 0, c->stream>>>(g, lam_e, lam_o, psi_e, psi_o, c->gauge<T>(), R.as<V2>(), p0, np,
-                                                        p0 == 0, p0 + np == 6, kind, (double2*)out_abi);
-    MG_LAUNCH();
+    links(std::integral_constant<int, FORCE_ALL>(), 4, R.as<V2>(), 0, 0);
+  } else {
+    // by plane and parity of the base, in the memory of the packed vectors, which only the hopping part reads
+    V2* r = vec.as<V2>();
+    links(std::integral_constant<int, FORCE_HOP>(), 4, nullptr, 0, 0);
+    for (int p = 0; p < 6; p++)
+      for (int par = 0; par < 2; par++) {
+        k_force_plaquettes<T><<<dim3(nh, 1, 1), bs, 0, c->stream>>>(g, U, W.as<V2>(), p, par, r);
+        MG_LAUNCH();
+        links(std::integral_constant<int, FORCE_ADD>(), 2, r, p, par);
+      }
+    links(std::integral_constant<int, FORCE_FORM>(), 4, nullptr, 0, 0);
   }   // the caller waits for the stream
   c->leave(KEEP_FORCE, std::move(work));
 }
