@@ -448,7 +448,9 @@ MG_API int mg_apply_noalloc(void* ctx, int op, void* out, const void* in, int pr
  *   DSLASH_CLOVER: Vh * (8 links * 18 + 24 spinor + 72 clover + 24 out) reals,
  *   DSLASH_XPAY:   Vh * (8 * 18 + 24 + 24 x + 24 out) reals,
  *   DR:            the sum of its three kernels,
- *   COARSE_DR:     Vc/2 * (18 Nc^2 link/inverse entries + 7 Nc vector entries) complex,
+ *   COARSE_DR:     Vc/2 * (8 Nc^2 entries of the links with the site inverses folded in, FP32,
+ *                  + 8 Nc^2 link entries of the storage format + 5 Nc vector entries), as the
+ *                  solver of an intermediate level applies it,
  *   RESTRICT, PROLONG: the P rows of the even fine sites (Vh * 12 * Nv entries
  *                  of the storage format: 8 bytes FP32, 4 bytes FP16/BF16) + the
  *                  even half of the fine vector (24 Vh floats) + the coarse
