@@ -252,6 +252,7 @@ struct TuneKey {
   int dims[4];
   int nrhs;
   int prec;   // 0 FP64, 1 FP32
+  int nc = 0; // components per coarse site, where the choice also depends on something else in nrhs
 };
 // CTA size for `k`: looked up, or chosen by timing `launch(block)` for every
 // candidate on stream `s` (the launches must be idempotent: no output aliases

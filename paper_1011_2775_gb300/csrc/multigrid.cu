@@ -807,7 +807,7 @@ void mg_batch_coarse(Ctx* c, int nb) {
         long long* d_it = b.H.d_iters.as<long long>();
         DBuf keep(sizeof(long long) * MG_MAX_LEVELS);
         MG_CUDA(cudaMemcpyAsync(keep.get(), d_it, sizeof(long long) * MG_MAX_LEVELS, cudaMemcpyDeviceToDevice, b.s));
-        choice = tuned_block(TuneKey{"coarse_group", {G1.L[0], G1.L[1], G1.L[2], G1.L[3]}, nb, C1.store}, {0, 1},
+        choice = tuned_block(TuneKey{"coarse_group", {G1.L[0], G1.L[1], G1.L[2], G1.L[3]}, nb, C1.store, C1.nc}, {0, 1},
                              [&](int which) {
                                if (which)
                                  one_by_one();

@@ -6,7 +6,9 @@
 // operands) and keeps the fastest; later launches look the choice up.  The
 // table lives for the process and, when MGCLOVER_TUNE_CACHE names a file, is
 // read from and appended to that file (one line per entry:
-// "kernel Lx Ly Lz Lt nrhs prec gpu block ms").
+// "kernel Lx Ly Lz Lt nrhs prec gpu block ms"; a kernel whose choice also depends
+// on Nc is written as "kernel.Nc", and a line of the file without it stands for
+// every Nc that has no line of its own).
 #include <cstdio>
 #include <cstdlib>
 #include <fstream>
@@ -35,9 +37,11 @@ std::string gpu_name() {
   return n;
 }
 
-std::string key_of(const TuneKey& k) {
+std::string key_of(const TuneKey& k, bool with_nc = true) {
   std::ostringstream o;
-  o << k.kernel << ' ' << k.dims[0] << ' ' << k.dims[1] << ' ' << k.dims[2] << ' ' << k.dims[3] << ' ' << k.nrhs << ' '
+  o << k.kernel;
+  if (k.nc > 0 && with_nc) o << '.' << k.nc;
+  o << ' ' << k.dims[0] << ' ' << k.dims[1] << ' ' << k.dims[2] << ' ' << k.dims[3] << ' ' << k.nrhs << ' '
     << k.prec << ' ' << gpu_name();
   return o.str();
 }
@@ -77,6 +81,7 @@ int tuned_block(const TuneKey& k, const std::vector<int>& candidates, const std:
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     if (!g_loaded) load_file();
     auto it = g_table.find(key);
+    if (it == g_table.end() && k.nc > 0) it = g_table.find(key_of(k, false));
     if (it != g_table.end()) return it->second;
   }
   cudaEvent_t e0, e1;
