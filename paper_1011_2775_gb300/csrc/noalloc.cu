@@ -49,15 +49,13 @@ void run_op(mg::Ctx* c, int op, T* base) {
   cudaStream_t s = c->stream;
   switch (op) {
     case MG_OP_D:
-      mg::dslash<T>(g, mg::EPI_CX_PAY, 0, oe, io, c->gauge<T>(), c->A<T>(0), ie, 1.0, 0xff, s);
-      mg::dslash<T>(g, mg::EPI_CX_PAY, 1, oo, ie, c->gauge<T>(), c->A<T>(1), io, 1.0, 0xff, s);
+      mg::dslash_full<T>(g, mg::EPI_CX_PAY, oe, oo, ie, io, c->gauge<T>(), c->A<T>(0), c->A<T>(1), ie, io, 1.0, s);
       c->dslash_launches += 2;
       break;
     case MG_OP_DP:
       mg::clover_apply<T>(g, t1, ie, c->Ainv<T>(0), s);
       mg::clover_apply<T>(g, t2, io, c->Ainv<T>(1), s);
-      mg::dslash<T>(g, mg::EPI_XPAY, 0, oe, t2, c->gauge<T>(), nullptr, ie, 1.0, 0xff, s);
-      mg::dslash<T>(g, mg::EPI_XPAY, 1, oo, t1, c->gauge<T>(), nullptr, io, 1.0, 0xff, s);
+      mg::dslash_full<T>(g, mg::EPI_XPAY, oe, oo, t1, t2, c->gauge<T>(), nullptr, nullptr, ie, io, 1.0, s);
       c->dslash_launches += 2;
       break;
     case MG_OP_DR:
@@ -81,8 +79,7 @@ void run_op(mg::Ctx* c, int op, T* base) {
       break;
     }
     case MG_OP_HOP:
-      mg::dslash<T>(g, mg::EPI_H, 0, oe, io, c->gauge<T>(), nullptr, nullptr, 0.0, 0xff, s);
-      mg::dslash<T>(g, mg::EPI_H, 1, oo, ie, c->gauge<T>(), nullptr, nullptr, 0.0, 0xff, s);
+      mg::dslash_full<T>(g, mg::EPI_H, oe, oo, ie, io, c->gauge<T>(), nullptr, nullptr, nullptr, nullptr, 0.0, s);
       c->dslash_launches += 2;
       break;
     default:

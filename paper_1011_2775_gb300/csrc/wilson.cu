@@ -689,19 +689,21 @@ __global__ void __launch_bounds__(BS, MINB) k_dslash_mrhs(Geom g, int par, int n
 // 960 sites).
 int site_block(long long sites) { return sites >= 128 * 152 * 6 ? 128 : sites >= 64 * 152 * 6 ? 64 : 32; }
 
-// Four lanes per site: in FP64 by the length of the busiest scheduler's chain
-// (608 schedulers; a warp of 32 sites is about 1320 FP64 instructions of 64
-// cycles each, one of 8 sites and four lanes each about 366: 43.6 -> 15.8 us for
-// both parities of 6x4x8x10).  In FP32 up to kLanesF32 sites of a parity, where
-// latency and not bandwidth sets the time: A^{-1} H takes 6.2 us with a thread
-// per site and 4.8 with four lanes at 4096 sites, 7.3 and 6.7 at 20736, 8.8 and
-// 9.6 at 32768, 13.8 and 19.2 at 65536.
+// Four lanes per site, by the sites of a launch (both parities where it has both).
+// FP64: by the length of the busiest scheduler's chain (608 schedulers; a warp of 32
+// sites is about 1320 FP64 instructions of 64 cycles each, one of 8 sites and four
+// lanes each about 380).  Lanes / a thread per site: 15.8 / 43.5 us at 1920 sites,
+// 35 / 44 at 12288, 50 / 46 at 18432, 111 / 117 at 41472, 256 / 260 at 98304, 329 / 303
+// at 131072; one parity 21.8 / 35.7 at 9216, 52 / 57 at 20736, 72 / 66 at 32768, 111 /
+// 101 at 49152.  FP32, up to kLanesF32 sites, where latency and not bandwidth sets the
+// time: 5.2 / 7.0 us at 8192 sites, 6.3 / 7.7 at 18432, 7.9 / 7.8 at 27648, 11.6 / 8.9
+// at 41472; one parity 4.3 / 5.8 at 4096, 6.1 / 6.9 at 20736, 7.7 / 7.3 at 32768.
 constexpr int kLanesF32 = 24576;
 template <typename T>
-bool lanes_per_site(int Vh) {
-  if (sizeof(T) == 4) return Vh <= kLanesF32;
-  const int warps = (Vh + 31) / 32;
-  return ((4 * warps + 607) / 608) * 366 < ((warps + 607) / 608) * 1320;
+bool lanes_per_site(int sites) {
+  if (sizeof(T) == 4) return sites <= kLanesF32;
+  const int warps = (sites + 31) / 32;
+  return ((4 * warps + 607) / 608) * 380 < ((warps + 607) / 608) * 1320;
 }
 
 bool dslash_lanes_f32(int Vh) { return lanes_per_site<float>(Vh); }
@@ -709,7 +711,7 @@ bool dslash_lanes_f32(int Vh) { return lanes_per_site<float>(Vh); }
 template <typename T>
 void dslash_halves(const Geom& g, Epilogue epi, int par0, int npar, const HalfArgs<T>& h, const T* gauge, double a,
                    int dirmask, cudaStream_t s) {
-  if (dirmask == 0xff && lanes_per_site<T>(g.Vh)) {
+  if (dirmask == 0xff && lanes_per_site<T>(npar * g.Vh)) {
     const int bl = site_block((long long)g.Vh * 4);
     const dim3 nl((4 * g.Vh + bl - 1) / bl, npar);
     switch (epi) {
