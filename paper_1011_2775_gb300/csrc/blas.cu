@@ -61,9 +61,10 @@ struct VecPtrs {
 };
 
 // Per-thread accumulation type: a thread sums only its few grid-stride
-// elements, in the vectors' own precision (FP64 for FP64 vectors); the
-// cross-thread tree is always FP64.  On GB300 this keeps the FP32 reductions
-// off the (slow) FP64 pipe.
+// elements, in the vectors' own precision.  Across the threads of a block FP64
+// sums are added in FP64 and FP32 sums as float pairs (about 48 bits; in FP64
+// where the pairs leave FP32's range), across blocks in FP64 (grid_sum).  On
+// GB300 this keeps the FP32 reductions off the (slow) FP64 pipe.
 template <typename T>
 using acc_t = typename std::conditional<sizeof(T) == 4, float, double>::type;
 }  // namespace

@@ -674,8 +674,9 @@ void mg_build(Ctx* c, mg_setup_info* info) {
 // The cycle of level 0 for nb right-hand sides at once (packed half vectors,
 // stride 24 Vh floats): multi-RHS D_r in the smoother, all coarsest-level
 // solves in one persistent launch per group of up to coarse_gcr_batch_max().
-// Each rhs gets exactly the arithmetic of mg_precondition.  It is split around
-// the coarsest solve so that several contexts can share that launch:
+// Each rhs gets the method of mg_precondition, with the rounding of the batched
+// kernels.  It is split around the coarsest solve so that several contexts can
+// share that launch:
 // mg_batch_pre (pre-smoothing, restriction to bw.rc), the coarse solve
 // (bw.rc -> bw.ec), mg_batch_post (prolongation, post-smoothing).
 namespace {
