@@ -133,9 +133,16 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, uns
   constexpr int V = NR <= 1 ? 1 : NR <= 2 ? 2 : NR <= 4 ? 4 : NR <= 8 ? 8 : 16;
   static_assert(NR <= 16, "at most 16 values");
   __shared__ __align__(8) S sm[NR][W];
-  __shared__ bool is_last;
+  __shared__ int state;   // 0: not the last block, 1: the last one, 2: out of range
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  bool over = false;
+  // the block's sums, written by lanes of the first warp, then its ticket
+  auto ticket = [&]() {
+    __syncwarp();
+    if (lane == 0) {
+      __threadfence();   // the block's partials before its ticket
+      state = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+  };
   S t[V];
 #pragma unroll
   for (int r = 0; r < V; r++) t[r] = r < NR ? sum_of(v[r < NR ? r : 0]) : sum_of(T{});
@@ -152,39 +159,45 @@ __device__ __forceinline__ void grid_sum(const T (&v)[NR], double* partials, uns
     if (lane % per == 0 && r < NR) sm[r][wid] = sum;
   }
   __syncthreads();
-  if (threadIdx.x < NR) {
-    S s = sm[threadIdx.x][0];
+  if (wid == 0) {
+    bool over = false;
+    if (lane < NR) {
+      S s = sm[lane][0];
 #pragma unroll
-    for (int w = 1; w < W; w++) s = add_x(s, sm[threadIdx.x][w]);
-    partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = sum_to_double(s);
-    if constexpr (!std::is_same<T, double>::value) over = !(fabsf(s.h) <= 3.402823466e38f);
-  }
-  if constexpr (std::is_same<T, double>::value) {
-    __syncthreads();
-  } else if (__syncthreads_or(over)) {
-    // finite sums of threads beyond FP32's range in the block: again in FP64
-    double* sd = reinterpret_cast<double*>(&sm[0][0]);
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-      double d = sum_to_double(sum_of(v[r]));
-#pragma unroll
-      for (int o = 16; o >= 1; o /= 2) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if (lane == 0) sd[r * W + wid] = d;
+      for (int w = 1; w < W; w++) s = add_x(s, sm[lane][w]);
+      partials[(size_t)lane * gridDim.x + blockIdx.x] = sum_to_double(s);
+      if constexpr (!std::is_same<T, double>::value) over = !(fabsf(s.h) <= 3.402823466e38f);
     }
-    __syncthreads();
-    if (threadIdx.x < NR) {
-      double d = 0.0;
-      for (int w = 0; w < W; w++) d += sd[threadIdx.x * W + w];
-      partials[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = d;
+    if (!std::is_same<T, double>::value && __any_sync(0xffffffffu, over)) {
+      if (lane == 0) state = 2;
+    } else {
+      ticket();
     }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();   // the block's partials before its ticket
-    is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (!is_last) return;
+  if constexpr (!std::is_same<T, double>::value) {
+    if (state == 2) {   // finite sums of threads beyond FP32's range in the block: again in FP64
+      double* sd = reinterpret_cast<double*>(&sm[0][0]);
+#pragma unroll
+      for (int r = 0; r < NR; r++) {
+        double d = sum_to_double(sum_of(v[r]));
+#pragma unroll
+        for (int o = 16; o >= 1; o /= 2) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (lane == 0) sd[r * W + wid] = d;
+      }
+      __syncthreads();
+      if (wid == 0) {
+        if (lane < NR) {
+          double d = 0.0;
+          for (int w = 0; w < W; w++) d += sd[lane * W + w];
+          partials[(size_t)lane * gridDim.x + blockIdx.x] = d;
+        }
+        ticket();
+      }
+      __syncthreads();
+    }
+  }
+  if (!state) return;
   __threadfence();
   if constexpr (NR <= 4) {   // every thread takes blocks, all values in flight together
     __shared__ double fin[NR][W];
