@@ -165,17 +165,17 @@ struct CoarseGCRBuffers {
 void coarse_gcr_solve(const LevelGeom& G, const CoarseOp& C, const CoarseGCRBuffers& B, int m, int maxit,
                       double tol_rel, const float* b, float* x, long long* d_iters, int* flags, cudaStream_t s,
                       int grid = 0);
-// The same solve with the links streamed through shared memory by bulk
-// asynchronous copies and three grid barriers per iteration
-// (coarse_stream.cu).  m: restart length; grid: blocks of the cooperative
-// launch, one of coarse_gcr_stream_grids() for this m.  Raises FLAG_TIMEOUT if
-// a wait runs out of time.
-bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C, int m);
 // floors of one coarsest-level GCR iteration on `grid` CTAs: the time of one
 // grid barrier and of streaming the iteration's links (A and the even-site Y)
 // L2 -> shared memory without arithmetic (floor.cu)
 void coarse_floor(const LevelGeom& G, const CoarseOp& C, int grid, int* flags, cudaStream_t s, double* barrier_us,
                   double* stream_us, double* stream_bytes);
+// The same solve with the links streamed through shared memory by bulk
+// asynchronous copies and three grid barriers per iteration
+// (coarse_stream.cu).  m: restart length; grid: blocks of the cooperative
+// launch, one of coarse_gcr_stream_grids() for this m.  Raises FLAG_TIMEOUT if
+// a wait runs out of time.
+// the grids to choose from (the full one first); none where the kernel does not apply
 std::vector<int> coarse_gcr_stream_grids(const LevelGeom& G, const CoarseOp& C, int m);
 void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuffers& B, int m, int maxit,
                              double tol_rel, const float* b, float* x, long long* d_iters, int* flags, cudaStream_t s,

@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(32 * W, 1) k_coarse_gcr_stream(const __grid_co
 }
 
 struct Plan {
-  int grid, warps, stage_bytes, rowsA, rowsB, ipsA, ipsB, NA, NB, gmax, wsm_ld, esm, emax;
+  int optin, grid, warps, stage_bytes, rowsA, rowsB, ipsA, ipsB, NA, NB, gmax, wsm_ld, esm, emax;
   size_t smem;
 };
 
@@ -732,6 +732,7 @@ Plan plan_warps(const LevelGeom& G, const CoarseOp& C, int grid, int m, int warp
   int dev = 0, optin = 0;
   MG_CUDA(cudaGetDevice(&dev));
   MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  p.optin = optin;
   const size_t budget = (size_t)optin - 4096;   // static shared memory and slack
   const size_t fixed = sizeof(float2) * (4 * warps + kNR) + sizeof(float2) * 2 * 32 * warps;
   const size_t per_site = sizeof(float2) * K + 25 * sizeof(int);   // gathered vector, neighbours, tile scales
@@ -800,21 +801,15 @@ int sm_count() {
 // (below 512 bytes).  A smaller grid has more sites to gather per block and a shorter
 // restart may place Krylov vectors in shared memory, so every (grid, m) is asked.
 static bool plan_ok(const Plan& p) {
-  int dev = 0, optin = 0;
-  MG_CUDA(cudaGetDevice(&dev));
-  MG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  return p.rowsA >= 1 && p.rowsB >= 1 && p.grid >= 1 && p.smem + 512 <= (size_t)optin;
-}
-
-bool coarse_gcr_stream_ok(const LevelGeom& G, const CoarseOp& C, int m) {
-  if (C.nc % 2 || !C.A.get()) return false;
-  const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
-  return plan_ok(p) && plan_ok(make_plan(G, C, p.grid, m));
+  return p.rowsA >= 1 && p.rowsB >= 1 && p.grid >= 1 && p.smem + 512 <= (size_t)p.optin;
 }
 
 std::vector<int> coarse_gcr_stream_grids(const LevelGeom& G, const CoarseOp& C, int m) {
+  std::vector<int> out;
+  if (C.nc % 2 || !C.A.get()) return out;
   const Plan p = make_plan(G, C, sm_count(), kMaxRestart);
-  std::vector<int> out = {p.grid};
+  if (!plan_ok(p) || (m != kMaxRestart && !plan_ok(make_plan(G, C, p.grid, m)))) return out;
+  out.push_back(p.grid);
   // the largest grid that splits both item lists evenly (no block waits at a
   // barrier for a neighbour with one more item)
   for (int g = p.grid - 1; g >= p.grid / 2 && g >= 1; g--)
@@ -829,7 +824,7 @@ void coarse_gcr_stream_solve(const LevelGeom& G, const CoarseOp& C, CoarseGCRBuf
                              double tol_rel, const float* b, float* x, long long* d_iters, int* flags, cudaStream_t s,
                              int grid) {
   if (m > kMaxRestart) raise(MG_ERR_ARG, "coarse restart too long for the persistent solver");
-  if (!coarse_gcr_stream_ok(G, C, m)) raise(MG_ERR_STATE, "streamed coarse solve not applicable to this level");
+  if (C.nc % 2 || !C.A.get()) raise(MG_ERR_STATE, "streamed coarse solve not applicable to this level");
   const Plan p = make_plan(G, C, grid, m);
   if (!plan_ok(p)) raise(MG_ERR_STATE, "streamed coarse solve not applicable on this grid");
   const int sms = sm_count();

@@ -290,8 +290,7 @@ void coarse_solve(Ctx* c, Hierarchy& H, int l, float* x, const float* b) {
     const int restart = p.restart_coarse > 0 ? p.restart_coarse : 32;
     long long* d_it = H.d_iters.as<long long>() + l;
     const std::vector<int> smaller = coarse_gcr_smaller_grids(G, W.cg);
-    const std::vector<int> streamed =
-        coarse_gcr_stream_ok(G, H.cop[l], restart) ? coarse_gcr_stream_grids(G, H.cop[l], restart) : std::vector<int>();
+    const std::vector<int> streamed = coarse_gcr_stream_grids(G, H.cop[l], restart);
     const std::vector<int> tensor =
         coarse_gcr_tc_ok(G, H.cop[l], 1) ? coarse_gcr_tc_grids(G, H.cop[l], 1) : std::vector<int>();
     const bool grouped = coarse_gcr_group_ok(G, H.cop[l], 1);
@@ -1016,9 +1015,9 @@ void mg_benchmark_coarse_floor(Ctx* c, double* barrier_us, double* stream_us, do
   Hierarchy& H = *c->mg;
   const int l = H.L - 1;
   const int restart = c->params.restart_coarse > 0 ? c->params.restart_coarse : 32;
-  if (!coarse_gcr_stream_ok(H.geo[l], H.cop[l], restart))
-    raise(MG_ERR_STATE, "the coarsest level has no streamed solver");
-  *grid = coarse_gcr_stream_grids(H.geo[l], H.cop[l], restart)[0];
+  const std::vector<int> grids = coarse_gcr_stream_grids(H.geo[l], H.cop[l], restart);
+  if (grids.empty()) raise(MG_ERR_STATE, "the coarsest level has no streamed solver");
+  *grid = grids[0];
   coarse_floor(H.geo[l], H.cop[l], *grid, c->ws.flags.as<int>(), c->stream, barrier_us, stream_us, stream_bytes);
   if (c->read_flag(FLAG_TIMEOUT, true)) raise(MG_ERR_CUDA, "a wait in the coarse floor benchmark ran out of time");
 }
